@@ -156,9 +156,12 @@ static size_t plan(const smc_config& cfg, Ctx* c, char* base) {
         C.gcov = P.take<double>((size_t)K * r * r); C.gL = P.take<double>((size_t)K * r * r);
         C.gLi = P.take<double>((size_t)K * r * r); C.glogdet = P.take<double>(K);
         C.covpart = P.take<double>(cov_partial_doubles(K, r));
+        C.gLb = P.take<double>(cov_lb_doubles(K, r));
+    } else {
+        C.empart = P.take<double>(em_partial_doubles(K, r));
     }
     C.tab = P.take<double>(4 * (size_t)K * r + r + 2 * K);
-    C.xsT = P.take<double>((size_t)r * N); C.resp = P.take<double>((size_t)K * N); C.nj = P.take<double>(K);
+    C.xsT = P.take<double>((size_t)r * N); C.resp = P.take<double>((size_t)K * N);
     C.pooled = P.take<double>(2 * (size_t)r); C.lse = P.take<double>(N); C.gmax = P.take<double>(N);
     C.gridtmp = P.take<double>(std::max<size_t>(N, 2 * cells));
     if (dim == 2) {

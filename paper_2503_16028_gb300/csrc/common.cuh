@@ -65,4 +65,28 @@ __device__ inline void cp_async_elem(T* shared_dst, const T* global_src) {
 // makes the copies of all threads visible to the block.
 __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Barrier over all blocks of a cooperative launch (all of them resident): every block adds
+// one arrival to *count (zeroed before the launch) and waits until `target` arrivals have
+// been counted (gridDim.x times the number of barriers so far).  The wait is bounded: after
+// GRID_SPINS polls the block sets *err and returns false, and the caller returns.  What
+// other blocks wrote before the barrier must be read with __ldcg (their L2 copies).
+constexpr unsigned GRID_SPINS = 1u << 23;
+__device__ inline bool grid_barrier(unsigned* count, unsigned target, int* err) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(count, 1u);
+        unsigned seen = 0, spins = 0;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+        } while (seen < target && ++spins < GRID_SPINS);
+        ok = seen >= target;
+        if (!ok) atomicExch(err, 1);
+        __threadfence();
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
 }  // namespace smcgm

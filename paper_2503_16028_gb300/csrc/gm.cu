@@ -10,8 +10,8 @@
 //   max_j g_nj (pooled variances, w_j = 1/N); weights are renormalised.
 // Initial means: K distinct particles from Philox (purpose EMINIT), variances
 // the pooled population variance, w_j = 1/K.  A fixed number of iterations.
+#include <algorithm>
 #include <cmath>
-#include <vector>
 #include "smcgm_internal.cuh"
 #include "common.cuh"
 
@@ -43,131 +43,280 @@ __global__ void k_pooled(int N, int r, const double* __restrict__ xsT, const dou
     if (threadIdx.x == 0) pooled[s] = fmax(v / N, floor_frac * lamS[s]);
 }
 
-__global__ void k_em_init(int N, int K, int r, const int* __restrict__ init_idx, const double* __restrict__ xsT,
+// Initial particles of the components (the Philox picks), passed by value.
+struct EmPicks { int idx[MAXK]; };
+
+__global__ void k_em_init(int N, int K, int r, EmPicks init, const double* __restrict__ xsT,
                           const double* __restrict__ pooled, double* __restrict__ w, double* __restrict__ m, double* __restrict__ lam) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < K * r) {
         const int j = t / r, s = t % r;
-        m[t] = xsT[(size_t)s * N + init_idx[j]];
+        m[t] = xsT[(size_t)s * N + init.idx[j]];
         lam[t] = pooled[s];
     }
     if (t < K) w[t] = 1.0 / K;
 }
 
-// E-step: one thread per particle.  resp[j][n], lse[n], gmax[n].
-__global__ void __launch_bounds__(256) k_estep(int N, int K, int r, const double* __restrict__ xsT, const double* __restrict__ w,
-                                               const double* __restrict__ m, const double* __restrict__ lam, double* __restrict__ resp,
-                                               double* __restrict__ lse, double* __restrict__ gmax) {
-    extern __shared__ double sh[];   // K*r means, K*r 1/(2 lam), K constants
-    double* sm = sh;
-    double* si = sm + K * r;
-    double* sc = si + K * r;
-    for (int t = threadIdx.x; t < K * r; t += blockDim.x) { sm[t] = m[t]; si[t] = 1.0 / (2.0 * lam[t]); }
-    __syncthreads();
-    for (int j = threadIdx.x; j < K; j += blockDim.x) {
-        double c = log(w[j]);
-        for (int s = 0; s < r; ++s) c += -0.5 * log(2.0 * M_PI * lam[j * r + s]);
-        sc[j] = c;
-    }
-    __syncthreads();
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    double lp[MAXK];
-    for (int j = 0; j < K; ++j) lp[j] = 0.0;
-    for (int s = 0; s < r; ++s) {
-        const double x = xsT[(size_t)s * N + n];
-        for (int j = 0; j < K; ++j) {
-            const double e = x - sm[j * r + s];
-            lp[j] -= e * e * si[j * r + s];
+// ------------------------------------------------------------------------
+// The whole diagonal EM fit in one cooperative launch.  The work of an iteration is
+// small (3 N K r FP64 operations for the E-step, 4 N K r for the M-step: 23 us at N = 4096,
+// K = 8, r = 64 on the FP64 pipes of 152 SMs) against the launches and the serial parts of
+// separate kernels, so each block keeps its N / gridDim particles in shared memory for all
+// iterations and an iteration has two grid barriers:
+//   1. E-step and the block's sums of g, g (x - c) and g (x - c)^2 about the pivot c = the
+//      component's current mean, to `part` (one row of 2 K r + K values per block);
+//   2. each block adds the rows for its slice of the (j, s) pairs, in a fixed order, and
+//      writes m = c + S1 / N_j and lambda = max(S2 / N_j - (S1 / N_j)^2, floor lambda_s).
+// The pivot moves with the fit, so the subtraction loses nothing once the means settle
+// (|m - c|^2 << lambda), and a component's next iteration starts from the new mean.
+// A collapsed component (N_j < 2) is found by every block alike (same sums, same order).
+// Measured (r = 64, 50 iterations, ncu): N = 1024, K = 4 9.0 -> 1.20 ms, N = 256, K = 2 7.2 -> 1.02 ms
+// (what is left is the chain of FP64 latencies through an iteration, 20 us).
+// ------------------------------------------------------------------------
+constexpr int EM_THREADS = 256;
+constexpr int EM_BLOCKS = 152;      // most blocks of the launch (rows of `part`)
+constexpr int EM_MINP = 8;          // least particles per block: fewer blocks make cheaper barriers
+
+__host__ __device__ inline int em_pad(int r) { return ((r + 11) / 16) * 16 + 4; }   // >= r, 4 mod 16: rows of 4 s fall on other banks
+static size_t em_smem(int K, int r, int per, bool xs_in_smem) {
+    return sizeof(double) * ((size_t)2 * K * em_pad(r) + 2 * (size_t)K * per + 3 * (size_t)K + 40 +
+                             (xs_in_smem ? (size_t)per * em_pad(r) : 0));
+}
+size_t em_partial_doubles(int K, int r) { return (size_t)EM_BLOCKS * (2 * (size_t)K * r + K + 2) + 2 * (size_t)K * r; }
+
+struct EmArgs {
+    int N, K, r, iters;
+    double floor_frac;
+    const double *xsT, *pooled, *lamS;
+    double *w, *m, *lam;          // in: the initial mixture; out: the fitted one
+    double *part;                 // gridDim rows of (S1, S2: K r; N_j: K; min of gmax, its particle), then si, lg: K r each
+    double *loglik;
+    unsigned* bar;
+    int* err;
+};
+
+template <bool XS>
+__global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
+    extern __shared__ __align__(16) double sh[];
+    const int N = A.N, K = A.K, r = A.r, Kr = K * r, rp = em_pad(r), G = gridDim.x, b = blockIdx.x, tid = threadIdx.x;
+    const int per = (N + G - 1) / G, n0 = min(N, b * per), np = min(N, n0 + per) - n0;
+    const int row = 2 * Kr + K + 2;
+    double* sm = sh;                       // means [K][rp]
+    double* si = sm + (size_t)K * rp;      // 1 / (2 lambda) [K][rp]
+    double* lp = si + (size_t)K * rp;      // log densities, then responsibilities [K][per]
+    double* ex = lp + (size_t)K * per;     // exp(lp - max) [K][per]
+    double* cst = ex + (size_t)K * per;    // constants of the log densities
+    double* nj = cst + K;
+    double* sw = nj + K;                   // weights
+    double* red = sw + K;                  // 40
+    double* xs = red + 40;                 // [per][rp]
+    double* g_si = A.part + (size_t)G * row;
+    double* g_lg = g_si + Kr;
+    auto X = [&](int p, int s) -> double { return XS ? xs[(size_t)p * rp + s] : A.xsT[(size_t)s * N + n0 + p]; };
+    if (XS)
+        for (int t = tid; t < np * r; t += EM_THREADS) {
+            const int s = t / np, p = t % np;
+            xs[(size_t)p * rp + s] = A.xsT[(size_t)s * N + n0 + p];
         }
+    for (int t = tid; t < Kr; t += EM_THREADS) {
+        const int j = t / r, s = t % r;
+        const double l = A.lam[t];
+        sm[(size_t)j * rp + s] = A.m[t];
+        si[(size_t)j * rp + s] = 1.0 / (2.0 * l);
     }
-    double mx = -1.0 / 0.0;
-    for (int j = 0; j < K; ++j) { lp[j] += sc[j]; mx = fmax(mx, lp[j]); }
-    double sum = 0.0;
-    for (int j = 0; j < K; ++j) sum += exp(lp[j] - mx);
-    const double l = mx + log(sum);
-    double gm = 0.0;
-    for (int j = 0; j < K; ++j) {
-        const double g = exp(lp[j] - l);
-        resp[(size_t)j * N + n] = g;
-        gm = fmax(gm, g);
-    }
-    lse[n] = l;
-    gmax[n] = gm;
-}
-
-// M-step means (block per (j, s)): nj[j] and m[j][s].
-__global__ void k_mstep_mean(int N, int r, const double* __restrict__ xsT, const double* __restrict__ resp, double* __restrict__ nj,
-                             double* __restrict__ m) {
-    __shared__ double red[32];
-    __shared__ double s_n;
-    const int j = blockIdx.x / r, s = blockIdx.x % r;
-    const double* g = resp + (size_t)j * N;
-    const double* x = xsT + (size_t)s * N;
-    double a = 0.0, b = 0.0;
-    for (int n = threadIdx.x; n < N; n += blockDim.x) { a += g[n]; b += g[n] * x[n]; }
-    a = block_sum(a, red);
-    if (threadIdx.x == 0) s_n = a;
-    __syncthreads();
-    b = block_sum(b, red);
-    if (threadIdx.x == 0) {
-        m[j * r + s] = b / s_n;
-        if (s == 0) nj[j] = s_n;
-    }
-}
-
-__global__ void k_mstep_var(int N, int r, const double* __restrict__ xsT, const double* __restrict__ resp, const double* __restrict__ nj,
-                            const double* __restrict__ m, const double* __restrict__ lamS, double floor_frac, double* __restrict__ lam) {
-    __shared__ double red[32];
-    const int j = blockIdx.x / r, s = blockIdx.x % r;
-    const double* g = resp + (size_t)j * N;
-    const double* x = xsT + (size_t)s * N;
-    const double mu = m[j * r + s];
-    double a = 0.0;
-    for (int n = threadIdx.x; n < N; n += blockDim.x) { const double e = x[n] - mu; a += g[n] * e * e; }
-    a = block_sum(a, red);
-    if (threadIdx.x == 0) lam[j * r + s] = fmax(a / nj[j], floor_frac * lamS[s]);
-}
-
-// Collapse handling and weights (single block).
-__global__ void k_mstep_fix(int N, int K, int r, const double* __restrict__ nj, const double* __restrict__ gmax,
-                            const double* __restrict__ xsT, const double* __restrict__ pooled, double* __restrict__ w,
-                            double* __restrict__ m, double* __restrict__ lam) {
-    __shared__ double s_v[1024];
-    __shared__ int s_i[1024];
-    __shared__ int s_star;
-    bool any = false;
-    for (int j = 0; j < K; ++j) any |= nj[j] < 2.0;
-    if (any) {
-        double best = 1.0 / 0.0;
-        int bi = N;
-        for (int n = threadIdx.x; n < N; n += blockDim.x)
-            if (gmax[n] < best) { best = gmax[n]; bi = n; }
-        s_v[threadIdx.x] = best;
-        s_i[threadIdx.x] = bi;
+    for (int j = tid; j < K; j += EM_THREADS) sw[j] = A.w[j];
+    // constants of the initial mixture: lambda = pooled for every component
+    {
+        double c = 0.0;
+        for (int s = tid; s < r; s += EM_THREADS) c += -0.5 * log(2.0 * M_PI * A.lam[s]);
+        c = block_sum(c, red);
+        if (tid == 0) red[32] = c;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            double b = 1.0 / 0.0;
-            int ib = N;
-            for (int k = 0; k < (int)blockDim.x; ++k)
-                if (s_v[k] < b || (s_v[k] == b && s_i[k] < ib)) { b = s_v[k]; ib = s_i[k]; }
-            s_star = ib;
-        }
+        for (int j = tid; j < K; j += EM_THREADS) cst[j] = log(sw[j]) + red[32];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        for (int j = 0; j < K; ++j) {
-            if (nj[j] < 2.0) {
-                for (int s = 0; s < r; ++s) { m[j * r + s] = xsT[(size_t)s * N + s_star]; lam[j * r + s] = pooled[s]; }
-                w[j] = 1.0 / N;
-            } else {
-                w[j] = nj[j] / N;
+    __shared__ double rs[2][8][8];
+    unsigned arrivals = 0;
+    for (int it = 0;; ++it) {
+        // log densities: four lanes per (particle, component)
+        const int items = np * K;
+        for (int base = 0; base < items * 4; base += EM_THREADS) {
+            const int item = (base + tid) >> 2, l4 = tid & 3;
+            const bool on = item < items;
+            const int p = on ? item / K : 0, j = on ? item % K : 0;
+            double acc = 0.0;
+            if (on) {
+                const double *mj = sm + (size_t)j * rp, *ij = si + (size_t)j * rp;
+                for (int s = l4; s < r; s += 4) {
+                    const double e = X(p, s) - mj[s];
+                    acc -= e * e * ij[s];
+                }
+            }
+            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+            acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+            if (on && l4 == 0) lp[(size_t)j * per + p] = acc + cst[j];
+        }
+        __syncthreads();
+        for (int t = tid; t < items; t += EM_THREADS) {
+            const int j = t / np, p = t % np;
+            double mx = -1.0 / 0.0;
+            for (int q = 0; q < K; ++q) mx = fmax(mx, lp[(size_t)q * per + p]);
+            ex[(size_t)j * per + p] = exp(lp[(size_t)j * per + p] - mx);
+        }
+        __syncthreads();
+        if (it == A.iters) {               // the final log-likelihood: sum over the particles of LSE_j
+            double a = 0.0;
+            for (int p = tid; p < np; p += EM_THREADS) {
+                double mx = -1.0 / 0.0, sum = 0.0;
+                for (int q = 0; q < K; ++q) mx = fmax(mx, lp[(size_t)q * per + p]);
+                for (int q = 0; q < K; ++q) sum += ex[(size_t)q * per + p];
+                a += mx + log(sum);
+            }
+            a = block_sum(a, red);
+            if (tid == 0) A.part[(size_t)b * row] = a;
+            if (!grid_barrier(A.bar, arrivals += G, A.err)) return;
+            if (b == 0) {
+                a = 0.0;
+                for (int k = tid; k < G; k += EM_THREADS) a += __ldcg(&A.part[(size_t)k * row]);
+                a = block_sum(a, red);
+                if (tid == 0) *A.loglik = a;
+                for (int j = tid; j < K; j += EM_THREADS) A.w[j] = sw[j];
+            }
+            return;
+        }
+        double gmin = 1.0 / 0.0;           // least max_j g of the block's particles, lowest index on ties
+        int imin = N;
+        for (int p = tid; p < np; p += EM_THREADS) {
+            double mx = -1.0 / 0.0, sum = 0.0;
+            for (int q = 0; q < K; ++q) mx = fmax(mx, lp[(size_t)q * per + p]);
+            for (int q = 0; q < K; ++q) sum += ex[(size_t)q * per + p];
+            ex[p] = mx + log(sum);         // row 0: read above by this thread alone
+        }
+        __syncthreads();
+        for (int t = tid; t < items; t += EM_THREADS) {
+            const int j = t / np, p = t % np;
+            lp[(size_t)j * per + p] = exp(lp[(size_t)j * per + p] - ex[p]);
+        }
+        __syncthreads();
+        double* out = A.part + (size_t)b * row;
+        for (int t = tid; t < Kr; t += EM_THREADS) {
+            const int j = t / r, s = t % r;
+            const double c = sm[(size_t)j * rp + s];
+            const double* g = lp + (size_t)j * per;
+            double s1 = 0.0, s2 = 0.0;
+            for (int p = 0; p < np; ++p) {
+                const double e = X(p, s) - c, ge = g[p] * e;
+                s1 += ge;
+                s2 = fma(ge, e, s2);
+            }
+            out[t] = s1;
+            out[Kr + t] = s2;
+        }
+        for (int j = tid >> 5; j < K; j += EM_THREADS / 32) {
+            double a = 0.0;
+            for (int p = tid & 31; p < np; p += 32) a += lp[(size_t)j * per + p];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if ((tid & 31) == 0) out[2 * Kr + j] = a;
+        }
+        if (tid < 32) {
+            for (int p = tid; p < np; p += 32) {
+                double gm = 0.0;
+                for (int j = 0; j < K; ++j) gm = fmax(gm, lp[(size_t)j * per + p]);
+                if (gm < gmin) { gmin = gm; imin = n0 + p; }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const double og = __shfl_xor_sync(0xffffffffu, gmin, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, imin, o);
+                if (og < gmin || (og == gmin && oi < imin)) { gmin = og; imin = oi; }
+            }
+            if (tid == 0) { out[2 * Kr + K] = gmin; out[2 * Kr + K + 1] = (double)imin; }
+        }
+        if (!grid_barrier(A.bar, arrivals += G, A.err)) return;
+        // N_j and the weights (every block alike)
+        for (int j = tid >> 5; j < K; j += EM_THREADS / 32) {
+            double a = 0.0;
+            for (int k = tid & 31; k < G; k += 32) a += __ldcg(&A.part[(size_t)k * row + 2 * Kr + j]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if ((tid & 31) == 0) nj[j] = a;
+        }
+        __syncthreads();
+        bool low = false;
+        for (int j = 0; j < K; ++j) low |= nj[j] < 2.0;
+        int star = 0;
+        if (low) {                          // rare: the particle with the lowest max_j g
+            double bg = 1.0 / 0.0;
+            double bi = (double)N;
+            for (int k = 0; k < G; ++k) {
+                const double vg = __ldcg(&A.part[(size_t)k * row + 2 * Kr + K]), vi = __ldcg(&A.part[(size_t)k * row + 2 * Kr + K + 1]);
+                if (vg < bg || (vg == bg && vi < bi)) { bg = vg; bi = vi; }
+            }
+            star = (int)bi;
+        }
+        if (tid == 0) {
+            double tot = 0.0;
+            for (int j = 0; j < K; ++j) { sw[j] = nj[j] < 2.0 ? 1.0 / N : nj[j] / N; tot += sw[j]; }
+            for (int j = 0; j < K; ++j) sw[j] = sw[j] / tot;
+        }
+        // this block's slice of the pairs: 8 pairs at a time, 32 threads adding a pair's rows
+        const int lo = (int)((size_t)Kr * b / G), hi = (int)((size_t)Kr * (b + 1) / G);
+        for (int q0 = lo; q0 < hi; q0 += 8) {
+            const int q = q0 + (tid & 7), bl = tid >> 3;
+            double s1 = 0.0, s2 = 0.0;
+            if (q < hi)
+                for (int k = bl; k < G; k += 32) {
+                    s1 += __ldcg(&A.part[(size_t)k * row + q]);
+                    s2 += __ldcg(&A.part[(size_t)k * row + Kr + q]);
+                }
+#pragma unroll
+            for (int o = 16; o >= 8; o >>= 1) {
+                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+                s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+            }
+            __syncthreads();
+            if ((tid & 31) < 8) { rs[0][tid >> 5][tid & 7] = s1; rs[1][tid >> 5][tid & 7] = s2; }
+            __syncthreads();
+            if (tid < 8 && q < hi) {
+                s1 = 0.0; s2 = 0.0;
+                for (int k = 0; k < 8; ++k) { s1 += rs[0][k][tid]; s2 += rs[1][k][tid]; }
+                const int j = q / r, s = q % r;
+                double mv, lv;
+                if (nj[j] < 2.0) {
+                    mv = A.xsT[(size_t)s * N + star];
+                    lv = A.pooled[s];
+                } else {
+                    const double dm = s1 / nj[j];
+                    mv = sm[(size_t)j * rp + s] + dm;
+                    lv = fmax(s2 / nj[j] - dm * dm, A.floor_frac * A.lamS[s]);
+                }
+                A.m[q] = mv;
+                A.lam[q] = lv;
+                g_si[q] = 1.0 / (2.0 * lv);
+                g_lg[q] = -0.5 * log(2.0 * M_PI * lv);
             }
         }
-        double tot = 0.0;
-        for (int j = 0; j < K; ++j) tot += w[j];
-        for (int j = 0; j < K; ++j) w[j] = w[j] / tot;
+        if (!grid_barrier(A.bar, arrivals += G, A.err)) return;
+        for (int t = tid; t < Kr; t += EM_THREADS) {
+            const int j = t / r, s = t % r;
+            sm[(size_t)j * rp + s] = __ldcg(&A.m[t]);
+            si[(size_t)j * rp + s] = __ldcg(&g_si[t]);
+        }
+        for (int j = tid >> 5; j < K; j += EM_THREADS / 32) {
+            double a = 0.0;
+            for (int s = tid & 31; s < r; s += 32) a += __ldcg(&g_lg[(size_t)j * r + s]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if ((tid & 31) == 0) cst[j] = log(sw[j]) + a;
+        }
+        __syncthreads();
     }
+}
+
+__global__ void k_lamS(int r, const double* __restrict__ lam, const int* __restrict__ S, double* __restrict__ out) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < r) out[s] = lam[S[s]];
 }
 
 __global__ void k_sum(int N, const double* __restrict__ a, double* __restrict__ out) {
@@ -178,202 +327,364 @@ __global__ void k_sum(int N, const double* __restrict__ a, double* __restrict__ 
     if (threadIdx.x == 0) *out = s;
 }
 
-__global__ void k_lamS(int r, const double* __restrict__ lam, const int* __restrict__ S, double* __restrict__ out) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < r) out[s] = lam[S[s]];
-}
-
 // ------------------------------------------------------------------------
 // Full covariances on the mixture modes (cfg.full_cov; a reading beyond the
 // paper, whose C_j are diagonal in the KL basis):
 //   E-step: log p_nj = log w_j - r/2 log(2 pi) - log det L_j - |L_j^{-1}(x_n - m_j)|^2 / 2,
 //   M-step: C_j = sum_n g_nj (x_n - m_j)(x_n - m_j)^T / N_j + floor diag(lambda_S),
 //   initial and re-seeded covariances diag(pooled variances).
-// L_j (Cholesky), L_j^{-1} and log det L_j are formed on the device in FP64
-// (k_factor, one block per component) after every M-step; a pivot that is not
-// positive sets a device flag, read by the host once per fit.
+// An iteration is k_chol, k_estep_full, k_resp, k_cov_acc, k_cov_finish.  The E-step and the
+// contraction are N K r^2 / 2 FP64 multiply-adds each (108 us at N = 4096, K = 8, r = 64 on the
+// FP64 pipes), everything else should stay small beside them.  Measured per 50-iteration fit
+// there: 70.2 -> 22.3 ms (one block per particle reading rows of L^-1 uncoalesced 631 -> 149 us,
+// the factor with its column sums in global memory 416 -> 79 us, the contraction on 32 x 32
+// tiles 292 -> 173 us).
 // ------------------------------------------------------------------------
 
-// E-step, one block per particle: for each j, y = L_j^{-1}(x_n - m_j) (a row per thread).
-__global__ void __launch_bounds__(128) k_estep_full(int N, int K, int r, const double* __restrict__ xsT, const double* __restrict__ w,
-                                                    const double* __restrict__ m, const double* __restrict__ Li,
-                                                    const double* __restrict__ logdet, double* __restrict__ resp,
-                                                    double* __restrict__ lse, double* __restrict__ gmax) {
-    __shared__ double red[32];
-    __shared__ double dev[MAXR];
-    __shared__ double lp[MAXK];
-    const int n = blockIdx.x;
-    for (int j = 0; j < K; ++j) {
-        for (int s = threadIdx.x; s < r; s += blockDim.x) dev[s] = xsT[(size_t)s * N + n] - m[(size_t)j * r + s];
-        __syncthreads();
-        double q = 0.0;
-        const double* Lj = Li + (size_t)j * r * r;
-        for (int i = threadIdx.x; i < r; i += blockDim.x) {
-            double y = 0.0;
-            for (int k = 0; k <= i; ++k) y += Lj[(size_t)i * r + k] * dev[k];
-            q += y * y;
+// Rows in blocks of four: block I holds L[4I + q][k] at 8 I (I + 1) + 4 k + q, k < 4 I + 4, with
+// 1 / L_kk on the diagonal (rows beyond r: zero, diagonal 1), so that a substitution step reads the
+// four rows' entries of one column as two 16-byte words.
+__host__ __device__ inline int row_blocks(int r) { return (r + 3) / 4; }
+__host__ __device__ inline int lb_size(int r) { const int R = row_blocks(r); return 8 * R * (R + 1); }
+size_t cov_lb_doubles(int K, int r) { return (size_t)K * lb_size(r) + K; }
+
+// Cholesky factor L_j (lower), log det L_j and the blocked rows above of every C_j, one block per
+// component, FP64: right-looking, W_ic -= W_ik W_ck / W_kk on the trailing triangle (all threads),
+// L_ik = W_ik / sqrt(W_kk) at the end; in shared memory while it fits (r <= CHOL_SMEM_R), else in
+// L_j's own storage.  A pivot that is not positive (C_j not positive definite) sets *bad and counts
+// as 1 so the rest stays finite.  cst_j = log w_j - r/2 log(2 pi) - log det L_j when w is given.
+// Bound by the FP64 pipe of one SM (r^3 / 6 multiply-adds, 11 us at r = 64) and 2 r barriers.
+constexpr int CHOL_SMEM_R = 160;
+__global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ cov, const double* __restrict__ w, double* __restrict__ L,
+                                              double* __restrict__ Lb, double* __restrict__ logdet, double* __restrict__ cst,
+                                              int* __restrict__ bad) {
+    extern __shared__ __align__(16) double chsm[];
+    __shared__ double T[MAXR], rs[MAXR], red[32];
+    const int j = blockIdx.x, tid = threadIdx.x;
+    const size_t rr = (size_t)r * r;
+    const double* A = cov + j * rr;
+    double* Lj = L + j * rr;
+    const bool in_smem = r <= CHOL_SMEM_R;
+    double* Wk = in_smem ? chsm : Lj;
+    const int ws = in_smem ? r + 1 : r;
+    for (int e = tid; e < (int)rr; e += 256) {
+        const int i = e / r, c = e % r;
+        if (c <= i) Wk[(size_t)i * ws + c] = A[e];
+    }
+    __syncthreads();
+    const int tx = tid & 15, ty = tid >> 4;
+    for (int k = 0; k < r; ++k) {
+        double d = Wk[(size_t)k * ws + k];
+        if (!(d > 0.0)) {
+            d = 1.0;
+            if (tid == 0) atomicExch(bad, 1);
         }
-        q = block_sum(q, red);
-        if (threadIdx.x == 0) lp[j] = log(w[j]) - 0.5 * r * log(2.0 * M_PI) - logdet[j] - 0.5 * q;
+        if (k + 1 + tid < r) T[k + 1 + tid] = Wk[(size_t)(k + 1 + tid) * ws + k] / d;   // r <= 256 = the threads
+        if (tid == 0) rs[k] = d;
+        __syncthreads();
+        for (int i = k + 1 + ty; i < r; i += 16) {
+            const double wi = Wk[(size_t)i * ws + k];
+            for (int c = k + 1 + tx; c <= i; c += 16) Wk[(size_t)i * ws + c] -= wi * T[c];
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        double mx = -1.0 / 0.0;
-        for (int j = 0; j < K; ++j) mx = fmax(mx, lp[j]);
-        double sum = 0.0;
-        for (int j = 0; j < K; ++j) sum += exp(lp[j] - mx);
-        const double l = mx + log(sum);
-        double gm = 0.0;
-        for (int j = 0; j < K; ++j) {
-            const double g = exp(lp[j] - l);
-            resp[(size_t)j * N + n] = g;
-            gm = fmax(gm, g);
+    double ld = 0.0;
+    for (int k = tid; k < r; k += 256) {
+        const double sq = sqrt(rs[k]);
+        rs[k] = 1.0 / sq;
+        T[k] = sq;
+        ld += log(sq);
+    }
+    ld = block_sum(ld, red);                 // its barriers also publish rs and T
+    if (tid == 0) {
+        logdet[j] = ld;
+        if (cst) cst[j] = log(w[j]) - 0.5 * r * log(2.0 * M_PI) - ld;
+    }
+    __syncthreads();
+    double* Lbj = Lb + (size_t)j * lb_size(r);
+    const int R = row_blocks(r);
+    for (int e = tid; e < 16 * R * R; e += 256) {
+        const int i = e / (4 * R), c = e % (4 * R);
+        if (c > (i | 3)) continue;
+        double v = 0.0;
+        if (c == i) v = i < r ? rs[i] : 1.0;
+        else if (c < i && i < r) v = Wk[(size_t)i * ws + c] * rs[c];
+        Lbj[8 * (i >> 2) * ((i >> 2) + 1) + 4 * c + (i & 3)] = v;
+    }
+    __syncthreads();
+    for (int e = tid; e < (int)rr; e += 256) {
+        const int i = e / r, c = e % r;
+        double v = 0.0;
+        if (c == i) v = T[i];
+        else if (c < i) v = Wk[(size_t)i * ws + c] * rs[c];
+        Lj[e] = v;                            // in place when the work array is L_j itself
+    }
+}
+
+// Forward substitution L y = rhs for 32 right-hand sides, one per lane; ys[i][lane] in shared memory,
+// four rows at a time: a step loads one y and two uniform 16-byte words of L for four multiply-adds.
+template <class Rhs, class Out>
+__device__ __forceinline__ void tri_subst(int r, const double* __restrict__ Lb, double* ys, int lane, Rhs rhs, Out out) {
+    const int R = row_blocks(r);
+    for (int I = 0; I < R; ++I) {
+        const double2* Lp = reinterpret_cast<const double2*>(Lb + 8 * I * (I + 1));
+        double a0 = rhs(4 * I), a1 = rhs(4 * I + 1), a2 = rhs(4 * I + 2), a3 = rhs(4 * I + 3);
+#pragma unroll 4
+        for (int k = 0; k < 4 * I; ++k) {
+            const double y = ys[k * 32 + lane];
+            const double2 l01 = __ldg(Lp + 2 * k), l23 = __ldg(Lp + 2 * k + 1);
+            a0 = fma(-l01.x, y, a0);
+            a1 = fma(-l01.y, y, a1);
+            a2 = fma(-l23.x, y, a2);
+            a3 = fma(-l23.y, y, a3);
         }
-        lse[n] = l;
+        const double2* D = Lp + 8 * I;
+        const double2 c0a = __ldg(D), c0b = __ldg(D + 1), c1a = __ldg(D + 2), c1b = __ldg(D + 3), c2b = __ldg(D + 5), c3b = __ldg(D + 7);
+        a0 *= c0a.x;
+        a1 = fma(-c0a.y, a0, a1) * c1a.y;
+        a2 = fma(-c1b.x, a1, fma(-c0b.x, a0, a2)) * c2b.x;
+        a3 = fma(-c2b.y, a2, fma(-c1b.y, a1, fma(-c0b.y, a0, a3))) * c3b.y;
+        ys[(4 * I) * 32 + lane] = a0;
+        ys[(4 * I + 1) * 32 + lane] = a1;
+        ys[(4 * I + 2) * 32 + lane] = a2;
+        ys[(4 * I + 3) * 32 + lane] = a3;
+        out(4 * I, a0, a1, a2, a3);
+    }
+}
+
+// L_j^{-1} (the proposal's terms use it): its columns are the substitutions of the unit vectors, a
+// warp per 32 columns.
+__global__ void __launch_bounds__(32) k_tri_inverse(int r, const double* __restrict__ Lb, double* __restrict__ Li) {
+    extern __shared__ __align__(16) double ysm[];
+    const int j = blockIdx.y, lane = threadIdx.x, col = blockIdx.x * 32 + lane;
+    double* out = Li + (size_t)j * r * r;
+    tri_subst(r, Lb + (size_t)j * lb_size(r), ysm, lane, [&](int i) { return i == col ? 1.0 : 0.0; },
+              [&](int i, double a, double b, double c, double d) {
+                  const double v[4] = {a, b, c, d};
+#pragma unroll
+                  for (int q = 0; q < 4; ++q)
+                      if (col < r && i + q < r) out[(size_t)(i + q) * r + col] = v[q];
+              });
+}
+
+// E-step: log p_nj, a warp per 32 particles of one component (grid y), a particle per lane.
+constexpr int ESF_WARPS = 2;
+__global__ void __launch_bounds__(32 * ESF_WARPS) k_estep_full(int N, int r, const double* __restrict__ xsT, const double* __restrict__ m,
+                                                               const double* __restrict__ Lb, const double* __restrict__ cst,
+                                                               double* __restrict__ lp) {
+    extern __shared__ __align__(16) double ysm[];
+    const int j = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int n = (blockIdx.x * ESF_WARPS + wid) * 32 + lane, nc = min(n, N - 1);
+    const double* mj = m + (size_t)j * r;
+    double q = 0.0;
+    tri_subst(r, Lb + (size_t)j * lb_size(r), ysm + (size_t)wid * 32 * 4 * row_blocks(r), lane,
+              [&](int i) { return i < r ? xsT[(size_t)i * N + nc] - mj[i] : 0.0; },
+              [&](int, double a, double b, double c, double d) { q = fma(d, d, fma(c, c, fma(b, b, fma(a, a, q)))); });
+    if (n < N) lp[(size_t)j * N + n] = cst[j] - 0.5 * q;
+}
+
+// Responsibilities from the log densities (in place), log-sum-exp and largest responsibility of every
+// particle: a thread per (component, particle).
+__global__ void __launch_bounds__(256) k_resp(int N, int K, double* __restrict__ lp, double* __restrict__ lse, double* __restrict__ gmax) {
+    __shared__ double l[256], e[256];
+    const int P = 256 / K, p = threadIdx.x % P, j = threadIdx.x / P;
+    const int n = blockIdx.x * P + p;
+    const bool on = j < K && n < N;
+    double v = 0.0, mx = -1.0 / 0.0;
+    if (on) v = lp[(size_t)j * N + n];
+    l[threadIdx.x] = v;
+    __syncthreads();
+    if (on) {
+        for (int q = 0; q < K; ++q) mx = fmax(mx, l[q * P + p]);
+        e[threadIdx.x] = exp(v - mx);
+    }
+    __syncthreads();
+    double g = 0.0, ls = 0.0;
+    if (on) {
+        double sum = 0.0;
+        for (int q = 0; q < K; ++q) sum += e[q * P + p];
+        ls = mx + log(sum);
+        g = exp(v - ls);
+        lp[(size_t)j * N + n] = g;
+    }
+    __syncthreads();
+    l[threadIdx.x] = g;
+    __syncthreads();
+    if (on && j == 0) {
+        double gm = 0.0;
+        for (int q = 0; q < K; ++q) gm = fmax(gm, l[q * P + p]);
+        lse[n] = ls;
         gmax[n] = gm;
     }
 }
 
-// M-step covariances as a blocked SYRK: S_j = sum_n g_nj (x_n - m_j)(x_n - m_j)^T.
-// The r x r output is cut into CT x CT tiles; a block computes one lower-triangle
-// tile (ta >= tb) of one component over one of COV_NC chunks of the particles
-// (FP64, 256 threads, 4 outputs each), staging CT particles x CT modes of the
-// weighted deviations g (x_a - m_a) and of the deviations (x_b - m_b) in shared
-// memory per step.  The chunk partials go to `part`; k_cov_reduce adds them in a
-// fixed order (deterministic), divides by N_j, adds the ridge and writes both
-// triangles.
-constexpr int CT = 32;
-constexpr int COV_NC = 8;
-__host__ __device__ inline int cov_tiles(int r) { const int t = (r + CT - 1) / CT; return t * (t + 1) / 2; }
+// The contraction sum_n g_nj (x_n - c_j)(x_n - c_j)^T about the pivot c_j = the component's current
+// mean, with sum_n g_nj (x_n - c_j) and N_j, over one chunk of the particles (grid z): each thread
+// holds one 4 x 4 tile of the lower triangle (136 tiles at r = 64: 5 % more products than the triangle
+// itself; 32 x 32 tiles took 48 % more), 16 particles' deviations staged in shared memory per step.
+// k_cov_finish adds the chunks in a fixed order.
+constexpr int COV_PN = 16;
+__host__ __device__ inline int cov_tiles(int r) { const int R = row_blocks(r); return R * (R + 1) / 2; }
+__host__ __device__ inline size_t cov_row(int r) { return (size_t)cov_tiles(r) * 16 + r + 1; }   // values per (component, chunk)
+// chunks: about two blocks of 256 threads per SM in all
+__host__ __device__ inline int cov_chunks(int K, int r) {
+    const int c = 304 / (K * ((cov_tiles(r) + 255) / 256));
+    return c < 1 ? 1 : c > 64 ? 64 : c;
+}
+size_t cov_partial_doubles(int K, int r) { return (size_t)K * cov_chunks(K, r) * cov_row(r); }
+static size_t cov_smem(int r) { return sizeof(double) * (2 * (size_t)COV_PN * 4 * row_blocks(r) + COV_PN); }
 
-__global__ void __launch_bounds__(256) k_mstep_cov(int N, int r, const double* __restrict__ xsT, const double* __restrict__ resp,
-                                                   const double* __restrict__ m, double* __restrict__ part) {
-    __shared__ double Wa[CT][CT + 1];   // [particle][mode a]
-    __shared__ double Db[CT][CT + 1];   // [particle][mode b]
-    const int tile = blockIdx.x, j = blockIdx.y, chunk = blockIdx.z;
-    int ta = 0, t = tile;
-    while (t > ta) { t -= ta + 1; ++ta; }
-    const int tb = t;                                   // tb <= ta
-    const int a0 = ta * CT, b0 = tb * CT;
-    const int per = (N + COV_NC - 1) / COV_NC;
-    const int n_lo = chunk * per, n_hi = min(N, n_lo + per);
+__global__ void __launch_bounds__(256) k_cov_acc(int N, int r, const double* __restrict__ xsT, const double* __restrict__ resp,
+                                                 const double* __restrict__ m, double* __restrict__ part) {
+    extern __shared__ __align__(16) double csm[];
+    const int j = blockIdx.y, chunk = blockIdx.z, nch = gridDim.z, tid = threadIdx.x, rp = 4 * row_blocks(r);
+    double* D = csm;                      // [COV_PN][rp] deviations
+    double* Wd = D + COV_PN * rp;         // [COV_PN][rp] weighted deviations
+    double* gs = Wd + COV_PN * rp;
+    const int t = blockIdx.x * 256 + tid, T = cov_tiles(r);
+    int ta = 0, tb = 0;
+    if (t < T) {
+        ta = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+        while (ta * (ta + 1) / 2 > t) --ta;
+        while ((ta + 1) * (ta + 2) / 2 <= t) ++ta;
+        tb = t - ta * (ta + 1) / 2;
+    }
+    const int per = (N + nch - 1) / nch, n_lo = min(N, chunk * per), n_hi = min(N, n_lo + per);
     const double* g = resp + (size_t)j * N;
-    const int row = threadIdx.x / 8, col0 = (threadIdx.x % 8) * 4;   // outputs (a0 + row, b0 + col0 .. col0 + 3)
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int n0 = n_lo; n0 < n_hi; n0 += CT) {
-        for (int e = threadIdx.x; e < CT * CT; e += blockDim.x) {
-            const int mode = e / CT, pn = e % CT;          // consecutive threads: consecutive particles
-            const int n = n0 + pn;
-            const bool in_n = n < n_hi;
-            const int a = a0 + mode, b = b0 + mode;
-            Wa[pn][mode] = (in_n && a < r) ? g[n] * (xsT[(size_t)a * N + n] - m[(size_t)j * r + a]) : 0.0;
-            Db[pn][mode] = (in_n && b < r) ? xsT[(size_t)b * N + n] - m[(size_t)j * r + b] : 0.0;
+    double acc[4][4] = {}, s1 = 0.0, sn = 0.0;
+    for (int n0 = n_lo; n0 < n_hi; n0 += COV_PN) {
+        if (tid < COV_PN) gs[tid] = n0 + tid < n_hi ? g[n0 + tid] : 0.0;
+        __syncthreads();
+        for (int e = tid; e < COV_PN * rp; e += 256) {
+            const int s = e / COV_PN, p = e % COV_PN;
+            const double dv = (s < r && n0 + p < n_hi) ? xsT[(size_t)s * N + n0 + p] - m[(size_t)j * r + s] : 0.0;
+            D[p * rp + s] = dv;
+            Wd[p * rp + s] = gs[p] * dv;
         }
         __syncthreads();
-#pragma unroll 8
-        for (int pn = 0; pn < CT; ++pn) {
-            const double w = Wa[pn][row];
+        if (t < T) {
+#pragma unroll 4
+            for (int p = 0; p < COV_PN; ++p) {
+                const double2 a01 = *reinterpret_cast<const double2*>(Wd + p * rp + 4 * ta), a23 = *reinterpret_cast<const double2*>(Wd + p * rp + 4 * ta + 2);
+                const double2 b01 = *reinterpret_cast<const double2*>(D + p * rp + 4 * tb), b23 = *reinterpret_cast<const double2*>(D + p * rp + 4 * tb + 2);
+                const double a[4] = {a01.x, a01.y, a23.x, a23.y}, b[4] = {b01.x, b01.y, b23.x, b23.y};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += w * Db[pn][col0 + q];
-        }
-        __syncthreads();
-    }
-    double* out = part + (((size_t)j * cov_tiles(r) + tile) * COV_NC + chunk) * CT * CT;
+                for (int x = 0; x < 4; ++x)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) out[row * CT + col0 + q] = acc[q];
-}
-
-__global__ void k_cov_reduce(int r, const double* __restrict__ part, const double* __restrict__ nj, const double* __restrict__ lamS,
-                             double floor_frac, double* __restrict__ cov) {
-    const int tile = blockIdx.x, j = blockIdx.y;
-    int ta = 0, t = tile;
-    while (t > ta) { t -= ta + 1; ++ta; }
-    const int tb = t;
-    const double* p = part + ((size_t)j * cov_tiles(r) + tile) * COV_NC * CT * CT;
-    for (int e = threadIdx.x; e < CT * CT; e += blockDim.x) {
-        const int a = ta * CT + e / CT, b = tb * CT + e % CT;
-        if (a >= r || b >= r || b > a) continue;
-        double s = 0.0;
-        for (int k = 0; k < COV_NC; ++k) s += p[(size_t)k * CT * CT + e];
-        const double v = s / nj[j] + (a == b ? floor_frac * lamS[a] : 0.0);
-        cov[((size_t)j * r + a) * r + b] = v;
-        cov[((size_t)j * r + b) * r + a] = v;
-    }
-}
-
-size_t cov_partial_doubles(int K, int r) { return (size_t)K * cov_tiles(r) * COV_NC * CT * CT; }
-
-// Cholesky factor L_j (lower), L_j^{-1} and log det L_j of every C_j, one block per
-// component, FP64, in the order of the Cholesky-Banachiewicz recurrence
-//   L_kk = sqrt(C_kk - sum_{q<k} L_kq^2),  L_ik = (C_ik - sum_{q<k} L_iq L_kq) / L_kk,
-// a column at a time (its entries below the diagonal are independent given the earlier
-// columns: a row per thread); then L^{-1} by forward substitution on the unit vectors (a
-// column per thread) and log det L_j = sum_k log L_kk.  A pivot that is not positive (C_j
-// not positive definite) sets *bad and is replaced by 1 so the rest stays finite.
-__global__ void __launch_bounds__(256) k_factor(int r, const double* __restrict__ cov, double* __restrict__ L, double* __restrict__ Li,
-                                                double* __restrict__ logdet, int* __restrict__ bad) {
-    __shared__ double s_piv;
-    const int j = blockIdx.x;
-    const size_t rr = (size_t)r * r;
-    const double* A = cov + j * rr;
-    double* Lj = L + j * rr;
-    double* Ij = Li + j * rr;
-    for (size_t e = threadIdx.x; e < rr; e += blockDim.x)
-        if ((int)(e % r) > (int)(e / r)) { Lj[e] = 0.0; Ij[e] = 0.0; }
-    for (int k = 0; k < r; ++k) {
-        if (threadIdx.x == 0) {
-            double sum = A[(size_t)k * r + k];
-            for (int q = 0; q < k; ++q) sum -= Lj[(size_t)k * r + q] * Lj[(size_t)k * r + q];
-            if (!(sum > 0.0)) { atomicExch(bad, 1); sum = 1.0; }
-            s_piv = sqrt(sum);
-            Lj[(size_t)k * r + k] = s_piv;
+                    for (int y = 0; y < 4; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
+            }
         }
-        __syncthreads();
-        const double piv = s_piv;
-        for (int i = k + 1 + threadIdx.x; i < r; i += blockDim.x) {
-            double sum = A[(size_t)i * r + k];
-            for (int q = 0; q < k; ++q) sum -= Lj[(size_t)i * r + q] * Lj[(size_t)k * r + q];
-            Lj[(size_t)i * r + k] = sum / piv;
+        if (blockIdx.x == 0) {
+            if (tid < r)
+                for (int p = 0; p < COV_PN; ++p) s1 += Wd[p * rp + tid];
+            if (tid == 0)
+                for (int p = 0; p < COV_PN; ++p) sn += gs[p];
         }
         __syncthreads();
     }
-    for (int col = threadIdx.x; col < r; col += blockDim.x) {
-        for (int i = col; i < r; ++i) {
-            double sum = i == col ? 1.0 : 0.0;
-            for (int q = col; q < i; ++q) sum -= Lj[(size_t)i * r + q] * Ij[(size_t)q * r + col];
-            Ij[(size_t)i * r + col] = sum / Lj[(size_t)i * r + i];
-        }
-    }
-    if (threadIdx.x == 0) {
-        double sdet = 0.0;
-        for (int k = 0; k < r; ++k) sdet += log(Lj[(size_t)k * r + k]);
-        logdet[j] = sdet;
+    double* out = part + ((size_t)j * nch + chunk) * cov_row(r);
+    if (t < T)
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) out[(size_t)t * 16 + 4 * x + y] = acc[x][y];
+    if (blockIdx.x == 0) {
+        if (tid < r) out[(size_t)T * 16 + tid] = s1;
+        if (tid == 0) out[(size_t)T * 16 + r] = sn;
     }
 }
 
-// cov_j = diag(lam_j) for the components that are new (all) or re-seeded (N_j < 2).
-__global__ void k_cov_diag(int K, int r, const double* __restrict__ nj, const double* __restrict__ lam, double* __restrict__ cov) {
+// Adds the chunks and writes C_j (both triangles), its diagonal, m_j and the weights; a component with
+// N_j < 2 is re-seeded at the particle with the lowest largest responsibility.
+__global__ void __launch_bounds__(256) k_cov_finish(int N, int K, int r, int nch, const double* __restrict__ part, const double* __restrict__ gmax,
+                                                    const double* __restrict__ xsT, const double* __restrict__ pooled,
+                                                    const double* __restrict__ lamS, double floor_frac, double* __restrict__ w,
+                                                    double* __restrict__ m, double* __restrict__ lam, double* __restrict__ cov) {
+    __shared__ double dm[MAXR], s_nj[MAXK], s_v[256];
+    __shared__ int s_i[256];
+    const int j = blockIdx.y, tid = threadIdx.x, T = cov_tiles(r);
+    const size_t row = cov_row(r);
+    const double* pj = part + (size_t)j * nch * row;
+    if (tid < K) {
+        double a = 0.0;
+        for (int c = 0; c < nch; ++c) a += part[((size_t)tid * nch + c) * row + (size_t)T * 16 + r];
+        s_nj[tid] = a;
+    }
+    double sum1 = 0.0;
+    if (tid < r)
+        for (int c = 0; c < nch; ++c) sum1 += pj[c * row + (size_t)T * 16 + tid];
+    __syncthreads();
+    const double nj = s_nj[j];
+    const bool low = nj < 2.0;
+    if (tid < r) dm[tid] = sum1 / nj;
+    __syncthreads();
+    const size_t e = (size_t)blockIdx.x * 256 + tid;
+    if (e < (size_t)T * 16) {
+        const int t = (int)(e >> 4), q = (int)(e & 15);
+        int ta = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+        while (ta * (ta + 1) / 2 > t) --ta;
+        while ((ta + 1) * (ta + 2) / 2 <= t) ++ta;
+        const int a = 4 * ta + (q >> 2), b = 4 * (t - ta * (ta + 1) / 2) + (q & 3);
+        if (a < r && b <= a) {
+            double s = 0.0;
+            for (int c = 0; c < nch; ++c) s += pj[c * row + e];
+            double v = s / nj - dm[a] * dm[b] + (a == b ? floor_frac * lamS[a] : 0.0);
+            if (low) v = a == b ? pooled[a] : 0.0;
+            cov[((size_t)j * r + a) * r + b] = v;
+            cov[((size_t)j * r + b) * r + a] = v;
+            if (a == b) lam[(size_t)j * r + a] = v;
+        }
+    }
+    if (blockIdx.x != 0) return;
+    if (low) {
+        double best = 1.0 / 0.0;
+        int bi = N;
+        for (int n = tid; n < N; n += 256)
+            if (gmax[n] < best) { best = gmax[n]; bi = n; }
+        s_v[tid] = best;
+        s_i[tid] = bi;
+        __syncthreads();
+        if (tid == 0)
+            for (int k = 1; k < 256; ++k)
+                if (s_v[k] < s_v[0] || (s_v[k] == s_v[0] && s_i[k] < s_i[0])) { s_v[0] = s_v[k]; s_i[0] = s_i[k]; }
+        __syncthreads();
+        if (tid < r) m[(size_t)j * r + tid] = xsT[(size_t)tid * N + s_i[0]];
+    } else if (tid < r) {
+        m[(size_t)j * r + tid] += dm[tid];
+    }
+    if (j == 0 && tid == 0) {
+        double tot = 0.0;
+        for (int k = 0; k < K; ++k) { w[k] = s_nj[k] < 2.0 ? 1.0 / N : s_nj[k] / N; tot += w[k]; }
+        for (int k = 0; k < K; ++k) w[k] = w[k] / tot;
+    }
+}
+
+// cov_j = diag(lam_j) for every component (the initial covariances).
+__global__ void k_cov_diag(int K, int r, const double* __restrict__ lam, double* __restrict__ cov) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= K * r * r) return;
     const int j = t / (r * r), a = (t / r) % r, b = t % r;
-    if (nj && !(nj[j] < 2.0)) return;
     cov[t] = a == b ? lam[(size_t)j * r + a] : 0.0;
 }
 
-// lam_j = diag(C_j) (what smc_get_mixture reports in the full-covariance form).
-__global__ void k_diag_of_cov(int K, int r, const double* __restrict__ cov, double* __restrict__ lam) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < K * r) lam[t] = cov[((size_t)(t / r) * r + t % r) * r + t % r];
-}
-
-// Factors every C_j on the device (k_factor) into L_j, L_j^{-1} and log det L_j; with
-// cov_host the covariances are uploaded first.  check_now: wait and fail (InputError) if a
-// C_j is not positive definite; otherwise the flag is read by the caller later.
 static int* factor_flag(Ctx& c) { return c.icount + 40; }
 
-static void launch_factor(Ctx& c) {
-    k_factor<<<c.K, 256, 0, c.stream>>>(c.r, c.gcov, c.gL, c.gLi, c.glogdet, factor_flag(c)); ++c.pc.launches;
+// L_j, log det L_j and the blocked rows of every C_j; with w also the E-step's constants.
+static void launch_chol(Ctx& c, bool estep_constants) {
+    const size_t sm = c.r <= CHOL_SMEM_R ? sizeof(double) * (size_t)c.r * (c.r + 1) : 0;
+    check(cudaFuncSetAttribute(k_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * CHOL_SMEM_R * (CHOL_SMEM_R + 1))), "attr");
+    k_chol<<<c.K, 256, sm, c.stream>>>(c.r, c.gcov, c.gw, c.gL, c.gLb, c.glogdet,
+                                       estep_constants ? c.gLb + (size_t)c.K * lb_size(c.r) : nullptr, factor_flag(c)); ++c.pc.launches;
     check(cudaGetLastError(), "factor launch");
+}
+
+// L_j, L_j^{-1} and log det L_j of every C_j.
+static void launch_factor(Ctx& c) {
+    launch_chol(c, false);
+    const size_t sm = sizeof(double) * 32 * 4 * row_blocks(c.r);
+    check(cudaFuncSetAttribute(k_tri_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * 32 * MAXR)), "attr");
+    k_tri_inverse<<<dim3((c.r + 31) / 32, c.K), 32, sm, c.stream>>>(c.r, c.gLb, c.gLi); ++c.pc.launches;
+    check(cudaGetLastError(), "inverse launch");
 }
 
 static void check_factor_flag(Ctx& c) {
@@ -386,6 +697,8 @@ static void check_factor_flag(Ctx& c) {
     }
 }
 
+// Factors every C_j on the device; with cov_host the covariances are uploaded first.  Waits, and
+// fails (InputError) if a C_j is not positive definite.
 void factor_mixture(Ctx& c, const double* cov_host) {
     const size_t n = (size_t)c.K * c.r * c.r;
     check(cudaMemsetAsync(factor_flag(c), 0, sizeof(int), c.stream), "memset");
@@ -394,66 +707,90 @@ void factor_mixture(Ctx& c, const double* cov_host) {
     check_factor_flag(c);
 }
 
+// EM with full covariances; the log-likelihood goes to ll (device).
+static void em_full(Ctx& c, const double* lamS, double* ll) {
+    const int N = c.N, K = c.K, r = c.r, kr2 = K * r * r;
+    const int nch = cov_chunks(K, r), tg = (cov_tiles(r) + 255) / 256, P = 256 / K;
+    const size_t esm = sizeof(double) * ESF_WARPS * 32 * 4 * row_blocks(r), csm = cov_smem(r);
+    check(cudaFuncSetAttribute(k_estep_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * ESF_WARPS * 32 * MAXR)), "attr");
+    check(cudaFuncSetAttribute(k_cov_acc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cov_smem(MAXR)), "attr");
+    const double* cst = c.gLb + (size_t)K * lb_size(r);
+    auto estep = [&] {
+        k_estep_full<<<dim3((N + 32 * ESF_WARPS - 1) / (32 * ESF_WARPS), K), 32 * ESF_WARPS, esm, c.stream>>>(N, r, c.xsT, c.gmu, c.gLb, cst, c.resp);
+        k_resp<<<(N + P - 1) / P, 256, 0, c.stream>>>(N, K, c.resp, c.lse, c.gmax);
+        c.pc.launches += 2;
+    };
+    check(cudaMemsetAsync(factor_flag(c), 0, sizeof(int), c.stream), "memset");
+    k_cov_diag<<<(kr2 + 255) / 256, 256, 0, c.stream>>>(K, r, c.glam, c.gcov); ++c.pc.launches;
+    for (int it = 0; it < c.cfg.em_iters; ++it) {
+        launch_chol(c, true);
+        estep();
+        k_cov_acc<<<dim3(tg, K, nch), 256, csm, c.stream>>>(N, r, c.xsT, c.resp, c.gmu, c.covpart);
+        k_cov_finish<<<dim3((cov_tiles(r) * 16 + 255) / 256, K), 256, 0, c.stream>>>(N, K, r, nch, c.covpart, c.gmax, c.xsT, c.pooled, lamS,
+                                                                                   c.cfg.var_floor, c.gw, c.gmu, c.glam, c.gcov);
+        c.pc.launches += 2;
+    }
+    launch_chol(c, true);
+    estep();
+    launch_factor(c);                                    // the proposal's L_j^{-1}
+    k_sum<<<1, 1024, 0, c.stream>>>(N, c.lse, ll); ++c.pc.launches;
+    check(cudaGetLastError(), "full-covariance fit");
+}
+
+// EM with diagonal covariances; the log-likelihood goes to ll (device).
+static void em_diag(Ctx& c, const double* lamS, double* ll) {
+    const int N = c.N, K = c.K, r = c.r;
+    EmArgs A{};
+    A.N = N; A.K = K; A.r = r; A.iters = c.cfg.em_iters; A.floor_frac = c.cfg.var_floor;
+    A.xsT = c.xsT; A.pooled = c.pooled; A.lamS = lamS; A.w = c.gw; A.m = c.gmu; A.lam = c.glam;
+    A.part = c.empart; A.loglik = ll; A.bar = reinterpret_cast<unsigned*>(c.icount + 44); A.err = c.dev_err;
+    const int G = std::max(1, std::min({EM_BLOCKS, c.sm_count, (N + EM_MINP - 1) / EM_MINP}));
+    const int per = (N + G - 1) / G;
+    constexpr size_t LIMIT = 200 * 1024;
+    const bool xs = em_smem(K, r, per, true) <= LIMIT;
+    const size_t sm = em_smem(K, r, per, xs);
+    const void* fn = xs ? reinterpret_cast<const void*>(&k_em<true>) : reinterpret_cast<const void*>(&k_em<false>);
+    check(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIMIT), "attr");
+    check(cudaMemsetAsync(A.bar, 0, sizeof(unsigned), c.stream), "memset");
+    void* args[] = {&A};
+    check(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(EM_THREADS), args, sm, c.stream), "EM launch"); ++c.pc.launches;
+}
+
 double gm_fit_device(Ctx& c) {
     const int N = c.N, K = c.K, r = c.r;
-    const double fl = c.cfg.var_floor;
     double* lamS = c.pooled + r;          // second half of the pooled scratch
-    int* init_idx = c.icount + 8;
     k_gather_modes<<<(unsigned)(((size_t)N * r + 255) / 256), 256, 0, c.stream>>>(N, c.d, r, c.X, c.S, c.xsT); ++c.pc.launches;
     k_lamS<<<(r + 127) / 128, 128, 0, c.stream>>>(r, c.lam, c.S, lamS); ++c.pc.launches;
-    k_pooled<<<r, 256, 0, c.stream>>>(N, r, c.xsT, lamS, fl, c.pooled); ++c.pc.launches;
+    k_pooled<<<r, 256, 0, c.stream>>>(N, r, c.xsT, lamS, c.cfg.var_floor, c.pooled); ++c.pc.launches;
     // initial picks (host Philox, the same definition as on the device)
-    std::vector<int> picks;
+    EmPicks picks{};
     for (int k = 0; k < K; ++k) {
         const U4 w = philox((uint32_t)k, 0u, (uint32_t)c.layer, P_EMINIT, c.key.k0, c.key.k1);
         int cidx = (int)(((unsigned long long)w.x * (unsigned long long)N) >> 32);
         bool clash = true;
         while (clash) {
             clash = false;
-            for (int q : picks) if (q == cidx) { clash = true; break; }
+            for (int q = 0; q < k; ++q) if (picks.idx[q] == cidx) { clash = true; break; }
             if (clash) cidx = (cidx + 1) % N;
         }
-        picks.push_back(cidx);
+        picks.idx[k] = cidx;
     }
-    check(cudaMemcpyAsync(init_idx, picks.data(), K * sizeof(int), cudaMemcpyHostToDevice, c.stream), "em picks");
-    k_em_init<<<(K * r + 127) / 128, 128, 0, c.stream>>>(N, K, r, init_idx, c.xsT, c.pooled, c.gw, c.gmu, c.glam); ++c.pc.launches;
-    const size_t esm = sizeof(double) * (2 * (size_t)K * r + K);
-    if (esm > 48 * 1024) check(cudaFuncSetAttribute(k_estep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)esm), "attr");
-    const int eg = (N + 255) / 256;
-    if (c.cfg.full_cov) {
-        const int kr2 = K * r * r;
-        const dim3 cg(cov_tiles(r), K, COV_NC);
-        check(cudaMemsetAsync(factor_flag(c), 0, sizeof(int), c.stream), "memset");
-        k_cov_diag<<<(kr2 + 255) / 256, 256, 0, c.stream>>>(K, r, nullptr, c.glam, c.gcov); ++c.pc.launches;
-        for (int it = 0; it < c.cfg.em_iters; ++it) {
-            launch_factor(c);
-            k_estep_full<<<N, 128, 0, c.stream>>>(N, K, r, c.xsT, c.gw, c.gmu, c.gLi, c.glogdet, c.resp, c.lse, c.gmax); ++c.pc.launches;
-            k_mstep_mean<<<K * r, 256, 0, c.stream>>>(N, r, c.xsT, c.resp, c.nj, c.gmu); ++c.pc.launches;
-            k_mstep_cov<<<cg, 256, 0, c.stream>>>(N, r, c.xsT, c.resp, c.gmu, c.covpart); ++c.pc.launches;
-            k_cov_reduce<<<dim3(cov_tiles(r), K), 256, 0, c.stream>>>(r, c.covpart, c.nj, lamS, fl, c.gcov); ++c.pc.launches;
-            k_diag_of_cov<<<(K * r + 255) / 256, 256, 0, c.stream>>>(K, r, c.gcov, c.glam); ++c.pc.launches;
-            k_mstep_fix<<<1, 1024, 0, c.stream>>>(N, K, r, c.nj, c.gmax, c.xsT, c.pooled, c.gw, c.gmu, c.glam); ++c.pc.launches;
-            k_cov_diag<<<(kr2 + 255) / 256, 256, 0, c.stream>>>(K, r, c.nj, c.glam, c.gcov); ++c.pc.launches;   // re-seeded ones
-        }
-        launch_factor(c);
-        k_estep_full<<<N, 128, 0, c.stream>>>(N, K, r, c.xsT, c.gw, c.gmu, c.gLi, c.glogdet, c.resp, c.lse, c.gmax); ++c.pc.launches;
-        k_sum<<<1, 1024, 0, c.stream>>>(N, c.lse, c.dscal + 8); ++c.pc.launches;
-        double ll = 0.0;
-        check(cudaMemcpyAsync(&ll, c.dscal + 8, sizeof(double), cudaMemcpyDeviceToHost, c.stream), "ll");
-        check_factor_flag(c);                            // one wait for the whole fit
-        return ll;
-    }
-    for (int it = 0; it < c.cfg.em_iters; ++it) {
-        k_estep<<<eg, 256, esm, c.stream>>>(N, K, r, c.xsT, c.gw, c.gmu, c.glam, c.resp, c.lse, c.gmax); ++c.pc.launches;
-        k_mstep_mean<<<K * r, 256, 0, c.stream>>>(N, r, c.xsT, c.resp, c.nj, c.gmu); ++c.pc.launches;
-        k_mstep_var<<<K * r, 256, 0, c.stream>>>(N, r, c.xsT, c.resp, c.nj, c.gmu, lamS, fl, c.glam); ++c.pc.launches;
-        k_mstep_fix<<<1, 1024, 0, c.stream>>>(N, K, r, c.nj, c.gmax, c.xsT, c.pooled, c.gw, c.gmu, c.glam); ++c.pc.launches;
-    }
-    k_estep<<<eg, 256, esm, c.stream>>>(N, K, r, c.xsT, c.gw, c.gmu, c.glam, c.resp, c.lse, c.gmax); ++c.pc.launches;
-    k_sum<<<1, 1024, 0, c.stream>>>(N, c.lse, c.dscal + 8); ++c.pc.launches;
+    k_em_init<<<(K * r + 127) / 128, 128, 0, c.stream>>>(N, K, r, picks, c.xsT, c.pooled, c.gw, c.gmu, c.glam); ++c.pc.launches;
+    double* ll_dev = c.dscal + 8;
+    if (c.cfg.full_cov) em_full(c, lamS, ll_dev);
+    else em_diag(c, lamS, ll_dev);
     double ll = 0.0;
-    check(cudaMemcpyAsync(&ll, c.dscal + 8, sizeof(double), cudaMemcpyDeviceToHost, c.stream), "ll");
-    sync_stream(c);
+    int err = 0;
+    check(cudaMemcpyAsync(&ll, ll_dev, sizeof(double), cudaMemcpyDeviceToHost, c.stream), "ll");
+    check(cudaMemcpyAsync(&err, c.dev_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream), "err d2h");
+    if (c.cfg.full_cov) check_factor_flag(c);            // one wait for the whole fit
+    else sync_stream(c);
+    if (err) {
+        check(cudaMemsetAsync(c.dev_err, 0, sizeof(int), c.stream), "err reset");
+        sync_stream(c);
+        c.fitted = false;
+        throw CudaError{cudaErrorLaunchTimeout, "the mixture fit's bounded grid barrier timed out"};
+    }
     return ll;
 }
 

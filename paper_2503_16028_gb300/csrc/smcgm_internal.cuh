@@ -196,6 +196,8 @@ void launch_resample(Ctx& c);
 double gm_fit_device(Ctx& c);
 void factor_mixture(Ctx& c, const double* cov_host);   // Cholesky, inverse and log det of every C_j (device); waits
 size_t cov_partial_doubles(int K, int r);               // scratch of the full-covariance contraction
+size_t cov_lb_doubles(int K, int r);                    // the factors' blocked rows and the E-step constants
+size_t em_partial_doubles(int K, int r);                // scratch of the diagonal fit
 void launch_propose_full(Ctx& c, const MoveSched* ms = nullptr, uint32_t step_off = 0);
 void launch_moments(Ctx& c, double* mean, double* var);
 void launch_grid_moments(Ctx& c, const double* mean_kl, double* mean_grid, double* var_grid);
@@ -222,10 +224,12 @@ struct Ctx {
     // full covariances on the mixture modes (cfg.full_cov): C_j, its Cholesky
     // factor L_j (lower), L_j^{-1} and log det L_j; glam holds diag(C_j)
     double *gcov = nullptr, *gL = nullptr, *gLi = nullptr, *glogdet = nullptr;
+    double* gLb = nullptr;      // the factors' rows in blocks of four, then the E-step's K constants (full_cov)
     double* covpart = nullptr;  // chunk partials of the covariance contraction (full_cov)
+    double* empart = nullptr;   // block partials of the diagonal fit
     double *tab = nullptr;     // per (j, s): c0, a, mu, sq; then per s: b; then per j: log w, cumulative w
     // EM scratch
-    double *xsT = nullptr, *resp = nullptr, *nj = nullptr, *pooled = nullptr, *lse = nullptr, *gmax = nullptr;
+    double *xsT = nullptr, *resp = nullptr, *pooled = nullptr, *lse = nullptr, *gmax = nullptr;
     // forward-solve batch arrays
     double *u64 = nullptr, *Kw64 = nullptr, *Ks64 = nullptr, *E64 = nullptr, *N64 = nullptr, *w64 = nullptr;
     // mixed precision: FP64-accurate faces and right-hand side as df32 pairs (the
