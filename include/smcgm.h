@@ -301,7 +301,7 @@ smc_status smc_profile_query(smc_ctx* ctx, int enable, smc_profile* out, int res
 smc_status smc_copy_to_host(smc_ctx* ctx, void* dst, const void* src, size_t bytes);
 
 /* Largest particle count smc_resample_indices_static() accepts: its scratch is
- * a fixed device array of this many 64-bit words (256 KiB). */
+ * a fixed device array of this many 64-bit words (256 KiB) and 7 KiB of block partials. */
 #define SMC_STATIC_RESAMPLE_MAX 32768
 
 /* Systematic-resampling indices without any allocation.  The paper has no

@@ -25,6 +25,17 @@ void sync_stream(Ctx& c) {
     check(cudaStreamSynchronize(c.stream), "sync");
 }
 
+void sync_and_check_barrier(Ctx& c) {
+    int err = 0;
+    check(cudaMemcpyAsync(&err, c.dev_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream), "err d2h");
+    sync_stream(c);
+    if (err) {   // cleared in stream order, so the context stays usable
+        check(cudaMemsetAsync(c.dev_err, 0, sizeof(int), c.stream), "err reset");
+        sync_stream(c);
+        throw CudaError{cudaErrorLaunchTimeout, "a kernel's bounded wait timed out"};
+    }
+}
+
 NvtxRange::NvtxRange(const char* name) { nvtxRangePushA(name); }
 NvtxRange::~NvtxRange() { nvtxRangePop(); }
 
@@ -148,6 +159,7 @@ static size_t plan(const smc_config& cfg, Ctx* c, char* base) {
     C.logw = P.take<double>(N); C.logalpha = P.take<double>(N);
     C.lfwd = P.take<double>((size_t)N * K); C.lrev = P.take<double>((size_t)N * K);
     C.acc = P.take<unsigned char>(N); C.idx = P.take<int>(N);
+    C.smcpart = P.take<double>(smc_partial_doubles());
     C.icount = P.take<int>(64); C.dscal = P.take<double>(64); C.dev_err = P.take<int>(4);
     C.gcnt = P.take<GraphCounters>(1); C.gouter = P.take<int>(2); C.msched = P.take<MoveSched>(1); C.gsteps = P.take<int>(1);
     C.normtab = P.take<float>(2 * NORMAL_TAB);
@@ -524,7 +536,7 @@ smc_status smc_temper_step(smc_ctx* ctx, double* h, double* ess, double* logZ_in
     double out[4];
     launch_temper(c, c.dscal);
     check(cudaMemcpyAsync(out, c.dscal, 4 * sizeof(double), cudaMemcpyDeviceToHost, c.stream), "d2h");
-    sync_stream(c);
+    sync_and_check_barrier(c);
     if (h) *h = out[0];
     if (ess) *ess = out[1];
     if (logZ_inc) *logZ_inc = out[2];
@@ -543,7 +555,7 @@ smc_status smc_resample(smc_ctx* ctx) {
     if (c.stage != 2) return fail(ctx, SMC_ESTATE, "smc_resample: expected after smc_temper_step");
     API_BEGIN
     launch_resample(c);
-    sync_stream(c);
+    sync_and_check_barrier(c);
     c.stage = 3;
     return SMC_OK;
     API_END(ctx)

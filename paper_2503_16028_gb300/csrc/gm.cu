@@ -780,17 +780,9 @@ double gm_fit_device(Ctx& c) {
     if (c.cfg.full_cov) em_full(c, lamS, ll_dev);
     else em_diag(c, lamS, ll_dev);
     double ll = 0.0;
-    int err = 0;
     check(cudaMemcpyAsync(&ll, ll_dev, sizeof(double), cudaMemcpyDeviceToHost, c.stream), "ll");
-    check(cudaMemcpyAsync(&err, c.dev_err, sizeof(int), cudaMemcpyDeviceToHost, c.stream), "err d2h");
     if (c.cfg.full_cov) check_factor_flag(c);            // one wait for the whole fit
-    else sync_stream(c);
-    if (err) {
-        check(cudaMemsetAsync(c.dev_err, 0, sizeof(int), c.stream), "err reset");
-        sync_stream(c);
-        c.fitted = false;
-        throw CudaError{cudaErrorLaunchTimeout, "the mixture fit's bounded grid barrier timed out"};
-    }
+    else sync_and_check_barrier(c);
     return ll;
 }
 

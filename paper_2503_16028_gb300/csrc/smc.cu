@@ -11,158 +11,274 @@
 // prefix sums CDF_i; particle k takes min{i : N CDF_i > k T + u48} with u48 one
 // Philox draw.  Integer arithmetic makes the indices independent of summation
 // order.
+#include <algorithm>
 #include "smcgm_internal.cuh"
 #include "common.cuh"
 
 namespace smcgm {
 
-constexpr int SB = 1024;   // threads of the single-block kernels
+// Both kernels are cooperative launches over up to SMC_BLOCKS blocks with grid barriers: their
+// cost is FP64 exponentials (some 30 FP64 operations each, and one SM's FP64 pipe does two lanes a
+// cycle), so one block took 2.0 ms for the 66 x 4096 exponentials of a tempering step and 3.5 ms
+// for 8192 particles, however fast its reductions, and resampling 8192 another 206 us.  Reweighting
+// and resampling 8192 particles of 1024 modes, as called: 3.85 -> 0.44 ms.
+constexpr int SMC_BLOCKS = 152;
+constexpr int SMC_THREADS = 256;
+constexpr int TEMPER_MINP = 32;    // particles per block and round: 32 x 8 candidates, one exponential per thread
 
-__device__ double ess_at(const double* phi, int N, double phimin, double h, double* red) {
-    double s1 = 0.0, s2 = 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const double e = exp(-h * (phi[i] - phimin));
-        s1 += e;
-        s2 += e * e;
+static int smc_grid(int N, int per_block, int sms) {
+    return std::max(1, std::min({SMC_BLOCKS, sms, (N + per_block - 1) / per_block}));
+}
+size_t smc_partial_doubles() { return 2 * SMC_BLOCKS * 16 + 2 * SMC_BLOCKS; }
+
+// Value v (of 16) of all blocks' partials, added in a fixed order; every thread of every block
+// gets the same 16 sums in `tot`.
+__device__ inline void sum_partials16(const double* part, int G, double* scr, double* tot) {
+    const int v = threadIdx.x & 15, ch = threadIdx.x >> 4;
+    double a = 0.0;
+    for (int g = ch; g < G; g += SMC_THREADS / 16) a += __ldcg(&part[(size_t)g * 16 + v]);
+    a += __shfl_xor_sync(0xffffffffu, a, 16);
+    __syncthreads();
+    if ((threadIdx.x & 16) == 0) scr[(threadIdx.x >> 5) * 16 + v] = a;
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        a = 0.0;
+        for (int k = 0; k < SMC_THREADS / 32; ++k) a += scr[k * 16 + threadIdx.x];
+        tot[threadIdx.x] = a;
     }
-    __shared__ double out[2];
-    double a = block_sum(s1, red);
-    if (threadIdx.x == 0) out[0] = a;
-    double b = block_sum(s2, red);
-    if (threadIdx.x == 0) out[1] = b;
     __syncthreads();
-    const double r = out[0] * out[0] / out[1];
-    __syncthreads();
-    return r;
 }
 
+// Tempering.  The 64 bisection decisions are taken three at a time: a round evaluates the ESS at
+// the seven points that the next three halvings can visit (the same midpoints, formed the same
+// way) and then walks down, so 22 rounds of one barrier replace 64; the eighth lane of the first
+// round evaluates h = 1 - t.  More points per round cost more exponentials than the barriers saved.
 // out: [0] h, [1] ESS(h), [2] log Z increment, [3] new t
-__global__ void __launch_bounds__(SB) k_temper(int N, const double* __restrict__ phi, double t, double target, double* __restrict__ logw,
-                                               double* __restrict__ out) {
-    __shared__ double red[32];
-    __shared__ double s_min, s_max, s_sum;
+__global__ void __launch_bounds__(SMC_THREADS) k_temper(int N, const double* __restrict__ phi, double t, double target,
+                                                        double* __restrict__ logw, double* __restrict__ out, double* part, unsigned* bar,
+                                                        int* err) {
+    __shared__ double red[32], scr[SMC_THREADS / 32 * 16], tot[16], cand[8];
+    const int G = gridDim.x, tid = threadIdx.x;
+    const int per = (N + G - 1) / G, n0 = min(N, (int)blockIdx.x * per), n1 = min(N, n0 + per);
+    double* pmin = part + 2 * SMC_BLOCKS * 16;
+    unsigned arrivals = 0;
     double mn = 1.0 / 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) mn = fmin(mn, phi[i]);
+    for (int i = n0 + tid; i < n1; i += SMC_THREADS) mn = fmin(mn, phi[i]);
     mn = -block_max(-mn, red);
-    if (threadIdx.x == 0) s_min = mn;
+    if (tid == 0) pmin[blockIdx.x] = mn;
+    if (!grid_barrier(bar, arrivals += G, err)) return;
+    mn = 1.0 / 0.0;
+    for (int g = tid; g < G; g += SMC_THREADS) mn = fmin(mn, __ldcg(&pmin[g]));
+    mn = -block_max(-mn, red);
+    if (tid == 0) tot[0] = mn;
     __syncthreads();
-    const double phimin = s_min;
+    const double phimin = tot[0];
     const double rest = 1.0 - t;
-    double h;
-    double e = ess_at(phi, N, phimin, rest, red);
-    if (e >= target) {
-        h = rest;
-    } else {
-        double lo = 0.0, hi = rest;
-        for (int it = 0; it < 64; ++it) {
-            const double mid = 0.5 * (lo + hi);
-            if (ess_at(phi, N, phimin, mid, red) >= target) lo = mid;
-            else hi = mid;
+    double lo = 0.0, hi = rest, ess_lo = (double)N, h;
+    int done = 0;
+    for (int round = 0;; ++round) {
+        const double c4 = 0.5 * (lo + hi), c2 = 0.5 * (lo + c4), c6 = 0.5 * (c4 + hi);
+        __syncthreads();
+        if (tid == 0) {
+            cand[0] = 0.5 * (lo + c2); cand[1] = c2; cand[2] = 0.5 * (c2 + c4); cand[3] = c4;
+            cand[4] = 0.5 * (c4 + c6); cand[5] = c6; cand[6] = 0.5 * (c6 + hi); cand[7] = rest;
         }
-        h = lo;
-        e = ess_at(phi, N, phimin, h, red);
+        __syncthreads();
+        const int k = tid & 7;
+        const bool on = round == 0 || (done + 3 <= 64 ? k < 7 : k == 3);
+        const double hk = cand[k];
+        double s1 = 0.0, s2 = 0.0;
+        if (on)
+            for (int i = n0 + (tid >> 3); i < n1; i += SMC_THREADS / 8) {
+                const double e = exp(-hk * (phi[i] - phimin));
+                s1 += e;
+                s2 += e * e;
+            }
+#pragma unroll
+        for (int o = 16; o >= 8; o >>= 1) {
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+        if ((tid & 31) < 8) { scr[(tid >> 5) * 16 + k] = s1; scr[(tid >> 5) * 16 + 8 + k] = s2; }
+        __syncthreads();
+        double* pr = part + (size_t)(round & 1) * SMC_BLOCKS * 16;   // the other half is still being read
+        if (tid < 16) {
+            double a = 0.0;
+            for (int w = 0; w < SMC_THREADS / 32; ++w) a += scr[w * 16 + tid];
+            pr[(size_t)blockIdx.x * 16 + tid] = a;
+        }
+        if (!grid_barrier(bar, arrivals += G, err)) return;
+        sum_partials16(pr, G, scr, tot);
+        auto ess = [&](int q) { return tot[q] * tot[q] / tot[8 + q]; };
+        if (round == 0) {
+            const double e = ess(7);
+            if (e >= target) { h = rest; ess_lo = e; break; }
+        }
+        int at = 3, step = 2;                   // walk down: c4, then c2 or c6, then the quarter points
+        const int levels = min(3, 64 - done);
+        for (int l = 0; l < levels; ++l) {
+            const double e = ess(at);
+            if (e >= target) { lo = cand[at]; ess_lo = e; at += step; }
+            else { hi = cand[at]; at -= step; }
+            step >>= 1;
+        }
+        done += levels;
+        if (done == 64) { h = lo; break; }
     }
-    // log weights -h Phi, their LSE, normalised weights; log Z increment = LSE - log N
-    double mx = -1.0 / 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) mx = fmax(mx, -h * phi[i]);
-    mx = block_max(mx, red);
-    if (threadIdx.x == 0) s_max = mx;
-    __syncthreads();
+    // log weights -h Phi, their LSE (the largest is -h min Phi), normalised weights; log Z increment = LSE - log N
+    const double mx = -h * phimin;
     double s = 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) s += exp(-h * phi[i] - s_max);
+    for (int i = n0 + tid; i < n1; i += SMC_THREADS) s += exp(-h * phi[i] - mx);
     s = block_sum(s, red);
-    if (threadIdx.x == 0) s_sum = s;
+    if (tid == 0) pmin[SMC_BLOCKS + blockIdx.x] = s;
+    if (!grid_barrier(bar, arrivals += G, err)) return;
+    s = 0.0;
+    for (int g = tid; g < G; g += SMC_THREADS) s += __ldcg(&pmin[SMC_BLOCKS + g]);
+    s = block_sum(s, red);
+    if (tid == 0) tot[0] = mx + log(s);
     __syncthreads();
-    const double lse = s_max + log(s_sum);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) logw[i] = -h * phi[i] - lse;
-    if (threadIdx.x == 0) {
+    const double lse = tot[0];
+    for (int i = n0 + tid; i < n1; i += SMC_THREADS) logw[i] = -h * phi[i] - lse;
+    if (blockIdx.x == 0 && tid == 0) {
         out[0] = h;
-        out[1] = e;
+        out[1] = ess_lo;
         out[2] = lse - log((double)N);
         out[3] = (h == rest) ? 1.0 : t + h;
     }
 }
 
 void launch_temper(Ctx& c, double* out) {
-    k_temper<<<1, SB, 0, c.stream>>>(c.N, c.Phi, c.t, c.cfg.ess_frac * c.N, c.logw, out); ++c.pc.launches;
-    check(cudaGetLastError(), "temper");
+    unsigned* bar = reinterpret_cast<unsigned*>(c.icount + 44);
+    int N = c.N;
+    const double* phi = c.Phi;
+    double t = c.t, target = c.cfg.ess_frac * c.N;
+    void* args[] = {&N, &phi, &t, &target, &c.logw, &out, &c.smcpart, &bar, &c.dev_err};
+    check(cudaMemsetAsync(bar, 0, sizeof(unsigned), c.stream), "memset");
+    check(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_temper), dim3(smc_grid(N, TEMPER_MINP, c.sm_count)), dim3(SMC_THREADS),
+                                      args, 0, c.stream), "temper"); ++c.pc.launches;
 }
 
-// Systematic resampling on the 2^48 fixed-point CDF; writes idx[N].
-__global__ void __launch_bounds__(SB) k_resample(int N, const double* __restrict__ logw, unsigned long long u48,
-                                                 unsigned long long* __restrict__ cdf, int* __restrict__ idx) {
-    __shared__ double red[32];
-    __shared__ double s_max, s_sum;
-    __shared__ unsigned long long s_part[SB];
-    __shared__ double s_wmax[SB];
-    __shared__ int s_imax[SB];
+// Systematic resampling on the 2^48 fixed-point CDF; writes idx[N].  A particle per thread: q_i =
+// floor(w_i T), the remainder to the largest weight (lowest index on ties), inclusive prefix sums
+// (integers: any order), then a binary search per output.
+__global__ void __launch_bounds__(SMC_THREADS) k_resample(int N, const double* __restrict__ logw, unsigned long long u48,
+                                                          unsigned long long* cdf, int* __restrict__ idx, double* part, unsigned* bar,
+                                                          int* err) {
+    __shared__ double red[32], s_w[SMC_THREADS / 32], s_b;
+    __shared__ unsigned long long s_q[SMC_THREADS / 32], s_off, s_tot;
+    __shared__ int s_i[SMC_THREADS / 32], s_ib;
     const unsigned long long T = 1ull << 48;
-    double mx = -1.0 / 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) mx = fmax(mx, logw[i]);
-    mx = block_max(mx, red);
-    if (threadIdx.x == 0) s_max = mx;
-    __syncthreads();
-    double s = 0.0;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) s += exp(logw[i] - s_max);
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) s_sum = s;
-    __syncthreads();
-    const double lse = s_max + log(s_sum);
-    // contiguous chunk per thread: q_i = floor(w_i T), local argmax (lowest index on ties)
-    const int chunk = (N + blockDim.x - 1) / blockDim.x;
-    const int b0 = threadIdx.x * chunk, b1 = min(N, b0 + chunk);
-    unsigned long long loc = 0;
-    double wbest = -1.0;
-    int ibest = N;
-    for (int i = b0; i < b1; ++i) {
-        const double w = exp(logw[i] - lse);
-        const unsigned long long q = (unsigned long long)floor(w * (double)T);
-        cdf[i] = q;
-        loc += q;
-        if (w > wbest) { wbest = w; ibest = i; }
-    }
-    s_part[threadIdx.x] = loc;
-    s_wmax[threadIdx.x] = wbest;
-    s_imax[threadIdx.x] = ibest;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long tot = 0;
-        double wb = -1.0;
-        int ib = N;
-        for (int k = 0; k < (int)blockDim.x; ++k) {
-            tot += s_part[k];
-            if (s_wmax[k] > wb || (s_wmax[k] == wb && s_imax[k] < ib)) { wb = s_wmax[k]; ib = s_imax[k]; }
+    const int G = gridDim.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int i = blockIdx.x * SMC_THREADS + tid;
+    const bool on = i < N;
+    unsigned arrivals = 0;
+    const double lw = on ? logw[i] : -1.0 / 0.0;
+    auto gather = [&](const double* p, bool maximum) {      // the blocks' values p[g], combined alike in every block
+        double a = maximum ? -1.0 / 0.0 : 0.0;
+        for (int g = tid; g < G; g += SMC_THREADS) { const double v = __ldcg(&p[g]); a = maximum ? fmax(a, v) : a + v; }
+        a = maximum ? block_max(a, red) : block_sum(a, red);
+        if (tid == 0) s_b = a;
+        __syncthreads();
+        const double r = s_b;
+        __syncthreads();
+        return r;
+    };
+    double v = block_max(lw, red);
+    if (tid == 0) part[blockIdx.x] = v;
+    if (!grid_barrier(bar, arrivals += G, err)) return;
+    const double mx = gather(part, true);
+    v = block_sum(on ? exp(lw - mx) : 0.0, red);
+    if (tid == 0) part[SMC_BLOCKS + blockIdx.x] = v;
+    if (!grid_barrier(bar, arrivals += G, err)) return;
+    const double lse = mx + log(gather(part + SMC_BLOCKS, false));
+    const double w = on ? exp(lw - lse) : -1.0;
+    unsigned long long q = on ? (unsigned long long)floor(w * (double)T) : 0;
+    {
+        unsigned long long qs = q;
+        double wb = w;
+        int ib = on ? i : N;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            qs += __shfl_xor_sync(0xffffffffu, qs, o);
+            const double ow = __shfl_xor_sync(0xffffffffu, wb, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, ib, o);
+            if (ow > wb || (ow == wb && oi < ib)) { wb = ow; ib = oi; }
         }
-        cdf[ib] = (unsigned long long)((long long)cdf[ib] + ((long long)T - (long long)tot));
-        // exclusive prefix of the chunk sums (recomputed after the fix-up)
-        s_imax[0] = ib;
+        if (lane == 0) { s_q[wid] = qs; s_w[wid] = wb; s_i[wid] = ib; }
+        __syncthreads();
+        if (tid == 0) {
+            for (int k = 1; k < SMC_THREADS / 32; ++k) {
+                qs += s_q[k];
+                if (s_w[k] > wb || (s_w[k] == wb && s_i[k] < ib)) { wb = s_w[k]; ib = s_i[k]; }
+            }
+            double* pb = part + 2 * SMC_BLOCKS + 4 * blockIdx.x;
+            pb[0] = __longlong_as_double((long long)qs);
+            pb[1] = wb;
+            pb[2] = (double)ib;
+        }
+    }
+    if (!grid_barrier(bar, arrivals += G, err)) return;
+    if (wid == 0) {                              // total, prefix of the earlier blocks, and the largest weight
+        unsigned long long tot = 0, off = 0;
+        double wb = -2.0;
+        int ib = N;
+        for (int g = lane; g < G; g += 32) {
+            const double* pb = part + 2 * SMC_BLOCKS + 4 * g;
+            const unsigned long long qg = (unsigned long long)__double_as_longlong(__ldcg(&pb[0]));
+            const double ow = __ldcg(&pb[1]);
+            const int oi = (int)__ldcg(&pb[2]);
+            tot += qg;
+            if (g < (int)blockIdx.x) off += qg;
+            if (ow > wb || (ow == wb && oi < ib)) { wb = ow; ib = oi; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+            off += __shfl_xor_sync(0xffffffffu, off, o);
+            const double ow = __shfl_xor_sync(0xffffffffu, wb, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, ib, o);
+            if (ow > wb || (ow == wb && oi < ib)) { wb = ow; ib = oi; }
+        }
+        if (lane == 0) {
+            s_tot = tot;
+            s_ib = ib;
+            s_off = off + (ib < (int)blockIdx.x * SMC_THREADS ? T - tot : 0);   // the remainder, modulo 2^64
+        }
     }
     __syncthreads();
-    // recompute chunk sums after the remainder fix-up, then exclusive scan
-    loc = 0;
-    for (int i = b0; i < b1; ++i) loc += cdf[i];
-    __syncthreads();
-    s_part[threadIdx.x] = loc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long run = 0;
-        for (int k = 0; k < (int)blockDim.x; ++k) { unsigned long long v = s_part[k]; s_part[k] = run; run += v; }
+    if (i == s_ib) q += T - s_tot;
+    unsigned long long run = q;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long u = __shfl_up_sync(0xffffffffu, run, o);
+        if (lane >= o) run += u;
     }
+    if (lane == 31) s_q[wid] = run;
     __syncthreads();
-    unsigned long long run = s_part[threadIdx.x];
-    for (int i = b0; i < b1; ++i) { run += cdf[i]; cdf[i] = run; }
-    __syncthreads();
+    run += s_off;
+    for (int k = 0; k < wid; ++k) run += s_q[k];
+    if (on) cdf[i] = run;
+    if (!grid_barrier(bar, arrivals += G, err)) return;
     // particle k: smallest i with N * CDF_i > k T + u48
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        const unsigned long long target = (unsigned long long)k * T + u48;
+    if (on) {
+        const unsigned long long target = (unsigned long long)i * T + u48;
         int lo = 0, hi = N - 1;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
-            if ((unsigned long long)N * cdf[mid] > target) hi = mid;
+            if ((unsigned long long)N * __ldcg(&cdf[mid]) > target) hi = mid;
             else lo = mid + 1;
         }
-        idx[k] = lo;
+        idx[i] = lo;
     }
+}
+
+// Issues k_resample; a block per 256 particles (N <= 32768: 128 blocks, all resident).
+static void launch_resample_indices(int N, const double* logw, unsigned long long u48, unsigned long long* cdf, int* idx, double* part,
+                                    unsigned* bar, int* err, cudaStream_t stream) {
+    void* args[] = {&N, &logw, &u48, &cdf, &idx, &part, &bar, &err};
+    check(cudaMemsetAsync(bar, 0, sizeof(unsigned), stream), "memset");
+    check(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_resample), dim3((N + SMC_THREADS - 1) / SMC_THREADS), dim3(SMC_THREADS),
+                                      args, 0, stream), "k_resample launch");
 }
 
 __global__ void k_gather(int d, const int* __restrict__ idx, const double* __restrict__ X, double* __restrict__ X2,
@@ -178,7 +294,8 @@ __global__ void k_gather(int d, const int* __restrict__ idx, const double* __res
 void launch_resample(Ctx& c) {
     const U4 w = philox(0u, 0u, (uint32_t)c.layer, P_RESAMPLE, c.key.k0, c.key.k1);
     const unsigned long long u48 = ((unsigned long long)w.x << 16) | (unsigned long long)(w.y >> 16);
-    k_resample<<<1, SB, 0, c.stream>>>(c.N, c.logw, u48, reinterpret_cast<unsigned long long*>(c.gridtmp), c.idx); ++c.pc.launches;
+    launch_resample_indices(c.N, c.logw, u48, reinterpret_cast<unsigned long long*>(c.gridtmp), c.idx, c.smcpart,
+                            reinterpret_cast<unsigned*>(c.icount + 44), c.dev_err, c.stream); ++c.pc.launches;
     k_gather<<<c.N, 256, 0, c.stream>>>(c.d, c.idx, c.X, c.X2, c.Phi, c.Phi2); ++c.pc.launches;
     check(cudaGetLastError(), "resample");
     std::swap(c.X, c.X2);
@@ -255,15 +372,17 @@ void launch_grid_moments(Ctx& c, const double* mean_kl, double* mean_grid, doubl
 // the process exits.  The caller passes the log weights and the output array;
 // the library allocates nothing.
 // ---------------------------------------------------------------------------
-static __device__ __align__(256) unsigned long long g_static_cdf[SMC_STATIC_RESAMPLE_MAX];
+constexpr int STATIC_PART = 6 * SMC_BLOCKS;   // the blocks' partials
+// the CDF, the partials, then the grid barrier's counter and its error flag
+static __device__ __align__(256) unsigned long long g_static_scratch[SMC_STATIC_RESAMPLE_MAX + STATIC_PART + 1];
 
-// Device address of g_static_cdf on the current device.  It is looked up on every
+// Device address of g_static_scratch on the current device.  It is looked up on every
 // call (the lookup allocates nothing): a cached address would go stale if the
 // process reset the device, which unloads the library's module there.  The first
 // lookup on a device also loads the module's copy of the array onto it.
-static unsigned long long* static_cdf_ptr() {
+static unsigned long long* static_scratch_ptr() {
     void* p = nullptr;
-    check(cudaGetSymbolAddress(&p, g_static_cdf), "cudaGetSymbolAddress(g_static_cdf)");
+    check(cudaGetSymbolAddress(&p, g_static_scratch), "cudaGetSymbolAddress(g_static_scratch)");
     return reinterpret_cast<unsigned long long*>(p);
 }
 
@@ -285,13 +404,16 @@ extern "C" smc_status smc_resample_indices_static(const double* d_logw, int n_pa
         return SMC_EINVAL;
     }
     try {
-        unsigned long long* cdf = static_cdf_ptr();
+        unsigned long long* scratch = static_scratch_ptr();
+        unsigned long long* cdf = scratch;
+        unsigned* counters = reinterpret_cast<unsigned*>(scratch + SMC_STATIC_RESAMPLE_MAX + STATIC_PART);
         const Key key = key_of(seed);
         const U4 w = philox(0u, 0u, (uint32_t)layer, P_RESAMPLE, key.k0, key.k1);
         const unsigned long long u48 = ((unsigned long long)w.x << 16) | (unsigned long long)(w.y >> 16);
-        // every entry of the CDF scratch below n_particles is written before it is read; nothing needs clearing
-        k_resample<<<1, SB, 0, reinterpret_cast<cudaStream_t>(stream)>>>(n_particles, d_logw, u48, cdf, d_indices);
-        check(cudaGetLastError(), "k_resample launch");
+        // every entry of the CDF scratch below n_particles is written before it is read; only the barrier's counter is cleared
+        launch_resample_indices(n_particles, d_logw, u48, cdf, d_indices, reinterpret_cast<double*>(scratch + SMC_STATIC_RESAMPLE_MAX),
+                                counters, reinterpret_cast<int*>(counters + 1),
+                                reinterpret_cast<cudaStream_t>(stream));
     } catch (const CudaError& ce) {
         set_global_error((std::string(ce.what) + ": " + cudaGetErrorString(ce.e)).c_str());
         return SMC_ECUDA;

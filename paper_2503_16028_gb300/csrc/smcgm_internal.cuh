@@ -197,6 +197,7 @@ double gm_fit_device(Ctx& c);
 void factor_mixture(Ctx& c, const double* cov_host);   // Cholesky, inverse and log det of every C_j (device); waits
 size_t cov_partial_doubles(int K, int r);               // scratch of the full-covariance contraction
 size_t cov_lb_doubles(int K, int r);                    // the factors' blocked rows and the E-step constants
+size_t smc_partial_doubles();                           // scratch of tempering and resampling
 size_t em_partial_doubles(int K, int r);                // scratch of the diagonal fit
 void launch_propose_full(Ctx& c, const MoveSched* ms = nullptr, uint32_t step_off = 0);
 void launch_moments(Ctx& c, double* mean, double* var);
@@ -218,6 +219,7 @@ struct Ctx {
     unsigned char* acc = nullptr;
     int* idx = nullptr;
     int* icount = nullptr;     // small device integer scratch
+    double* smcpart = nullptr; // block partials of tempering and resampling
     double* dscal = nullptr;   // small device double scratch (temper outputs etc.)
     // mixture and proposal tables
     double *gw = nullptr, *gmu = nullptr, *glam = nullptr;
@@ -291,6 +293,8 @@ std::string& global_error();
 void check(cudaError_t e, const char* what);   // throws CudaError
 // Waits for the context's stream (counted in smc_profile::host_syncs).
 void sync_stream(Ctx& c);
+// The same, and throws if a kernel's bounded wait timed out since the last check.
+void sync_and_check_barrier(Ctx& c);
 // An NVTX range named after a kernel family (set-up, solve, proposal, ...) for the
 // duration of a scope, so that profiler timelines group the library's launches.
 struct NvtxRange {
