@@ -151,7 +151,7 @@ static size_t plan(const smc_config& cfg, Ctx* c, char* base) {
     C.dim = dim; C.n = n; C.Km = Km; C.d = d; C.N = N; C.K = K; C.r = r; C.B = B; C.nobs = cfg.n_obs;
     C.lam = P.take<double>(d); C.sqrtlam = P.take<double>(d);
     C.basis = P.take<double>((size_t)n * Km);
-    C.b64 = P.take<double>(dim == 2 ? cells : (size_t)(n - 1));
+    C.b64 = P.take<double>(dim == 2 ? cells : (size_t)(2 * n - 1));   // 1D: b_1 .. b_{n-1}, then B_0 .. B_{n-1}
     C.obs = P.take<double>((size_t)cfg.n_obs * dim); C.data = P.take<double>(cfg.n_obs);
     C.S = P.take<int>(r); C.slot = P.take<int>(d);
     C.X = P.take<double>((size_t)N * d); C.X2 = P.take<double>((size_t)N * d); C.V = P.take<double>((size_t)N * d);
@@ -269,6 +269,8 @@ static void host_tables(Ctx& c, std::vector<double>& lam, std::vector<double>& b
             if (cfg.source_kind == 1) f = cfg.src_amp * std::exp(-cfg.src_width * (x - 0.5) * (x - 0.5));
             b[i - 1] = f / ((double)n * n);
         }
+        b.push_back(0.0);                              // the partial sums B_m = b_1 + .. + b_m, m = 0 .. n - 1
+        for (int i = 1; i < n; ++i) b.push_back(b.back() + b[i - 1]);
         S.resize(c.r);
         std::iota(S.begin(), S.end(), 0);
     }

@@ -582,50 +582,94 @@ void launch_observe(Ctx& c, const double* w, int count, double* Phi) {
 }
 
 // ------------------------------------------------------------------------
-// 1D forward map, one thread per particle: u at the n midpoints from the sine
-// KL expansion, K = e^u, tridiagonal system of the nodal FD scheme solved by
-// the Thomas algorithm (forward elimination, back substitution), linear
-// interpolation at the observation points, Phi.  FP64 throughout.
-// The basis table holds S[i][k] = sqrt(2) sin((k+1) pi (i+1/2)/n).
+// 1D forward map, one block per particle: u at the n midpoints from the sine KL
+// expansion (the basis table holds S[i][k] = sqrt(2) sin((k+1) pi (i+1/2)/n)), then
+// the nodal FD system.  With the flux D_i = K_{i+1/2} (w_{i+1} - w_i) its equations
+// read D_{i-1} - D_i = b_i, so D_i = g - B_i with B_i = b_1 + .. + b_i (a table) and,
+// from w_0 = w_n = 0 and R_i = 1 / K_{i+1/2} = e^{-u_i},
+//   g = sum_i B_i R_i / sum_i R_i,   w_i = sum_{m < i} (g - B_m) R_m.
+// Sums and scans over the block replace the elimination along the grid, which one
+// thread per particle did with n dependent divisions after n Km products of its own:
+// 256 particles, n = 128, 64 modes: 737 -> 15.7 us.  w is summed from the nearer
+// wall, so values next to either wall keep their relative accuracy.  FP64 throughout.
 // ------------------------------------------------------------------------
-__global__ void k_forward1d(int n, int Km, int count, const double* __restrict__ X, const double* __restrict__ S,
-                            const double* __restrict__ b, int nobs, const double* __restrict__ obs, const double* __restrict__ data,
-                            double inv2s2, double* __restrict__ Phi, double* __restrict__ wout, double* __restrict__ scratch) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= count) return;
-    const double* v = X + (size_t)p * Km;
-    // scratch per particle: K[n], cp[n], w[n+1]
-    double* K = scratch + (size_t)p * (3 * n + 2);
-    double* cp = K + n;
-    double* w = cp + n;       // w[0..n], w[0] = w[n] = 0
-    for (int i = 0; i < n; ++i) {
-        double u = 0.0;
-        const double* Si = S + (size_t)i * Km;
-        for (int k = 0; k < Km; ++k) u = fma(v[k], Si[k], u);
-        K[i] = exp(u);
+constexpr int F1_THREADS = 128;
+constexpr int F1_SMEM_N = 8192;    // larger grids keep R and w in the batch's global scratch (and more modes stay in X)
+
+// Exclusive scan of v over the block in thread order (REV: from the last thread down).
+template <bool REV>
+__device__ inline double block_scan_excl(double v, double* sh) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    double x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double y = REV ? __shfl_down_sync(0xffffffffu, x, o) : __shfl_up_sync(0xffffffffu, x, o);
+        if (REV ? lane + o < 32 : lane >= o) x += y;
     }
-    // unknowns w_1..w_{n-1}: diag K_{i-1/2} + K_{i+1/2} = K[i-1] + K[i]; off-diagonal -K[i]
-    // Thomas: forward sweep
-    const int m = n - 1;
-    double dprev = 0.0;
-    for (int r = 0; r < m; ++r) {
-        const int node = r + 1;
-        const double diag = K[node - 1] + K[node];
-        const double lower = r > 0 ? -K[node - 1] : 0.0;
-        const double upper = r < m - 1 ? -K[node] : 0.0;
-        const double denom = diag - lower * (r > 0 ? cp[r - 1] : 0.0);
-        cp[r] = upper / denom;
-        const double rhs = b[r];
-        dprev = (rhs - lower * (r > 0 ? w[r] : 0.0)) / denom;   // w[r] holds d'_{r-1}
-        w[r + 1] = dprev;                                       // temporarily d'_r at w[r+1]
+    __syncthreads();
+    if (lane == (REV ? 0 : 31)) sh[wid] = x;
+    double e = REV ? __shfl_down_sync(0xffffffffu, x, 1) : __shfl_up_sync(0xffffffffu, x, 1);
+    if (lane == (REV ? 31 : 0)) e = 0.0;
+    __syncthreads();
+    double base = 0.0;
+    if (REV) { for (int k = F1_THREADS / 32 - 1; k > wid; --k) base += sh[k]; }
+    else { for (int k = 0; k < wid; ++k) base += sh[k]; }
+    return base + e;
+}
+
+__global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const double* __restrict__ X, const double* __restrict__ S,
+                                                          const double* __restrict__ bsum, int nobs, const double* __restrict__ obs,
+                                                          const double* __restrict__ data, double inv2s2, double* __restrict__ Phi,
+                                                          double* __restrict__ wout, double* __restrict__ scratch) {
+    extern __shared__ __align__(16) double f1sm[];
+    __shared__ double red[32], s_g;
+    const int p = blockIdx.x, tid = threadIdx.x;
+    const int kv = Km <= F1_SMEM_N ? Km : 0;       // modes held in shared memory
+    const double* v = kv ? f1sm : X + (size_t)p * Km;
+    double* R = n <= F1_SMEM_N ? f1sm + kv : scratch + (size_t)p * (3 * n + 2);   // [n]
+    double* w = R + n;                             // [n + 1], w[0] = w[n] = 0
+    for (int k = tid; k < kv; k += F1_THREADS) f1sm[k] = X[(size_t)p * Km + k];
+    __syncthreads();
+    double t1 = 0.0, t2 = 0.0;
+    for (int i = tid; i < n; i += F1_THREADS) {
+        const double2* Si = reinterpret_cast<const double2*>(S + (size_t)i * Km);   // Km is even
+        double u0 = 0.0, u1 = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < Km / 2; ++k) {
+            const double2 sv = Si[k];
+            u0 = fma(v[2 * k], sv.x, u0);
+            u1 = fma(v[2 * k + 1], sv.y, u1);
+        }
+        const double r = exp(-(u0 + u1));
+        R[i] = r;
+        t1 += r;
+        t2 = fma(bsum[i], r, t2);
     }
-    // back substitution: x_{m-1} = d'_{m-1}; x_r = d'_r - c'_r x_{r+1}
-    w[0] = 0.0;
-    w[n] = 0.0;
-    for (int r = m - 2; r >= 0; --r) w[r + 1] = w[r + 1] - cp[r] * w[r + 2];
-    if (wout) for (int i = 0; i < m; ++i) wout[(size_t)p * m + i] = w[i + 1];
+    t1 = block_sum(t1, red);
+    t2 = block_sum(t2, red);
+    if (tid == 0) s_g = t2 / t1;
+    __syncthreads();
+    const double g = s_g;
+    // thread t's cells are [m0, m1): the sum of its increments, the sums of all before and after it
+    const int ch = (n + F1_THREADS - 1) / F1_THREADS, m0 = min(n, tid * ch), m1 = min(n, m0 + ch);
+    double loc = 0.0;
+    for (int m = m0; m < m1; ++m) loc = fma(g - bsum[m], R[m], loc);
+    double L = block_scan_excl<false>(loc, red);
+    double Q = block_scan_excl<true>(loc, red);
+    for (int m = m0; m < m1 && m <= n / 2; ++m) {   // left half: w_m = sum of the increments before m
+        w[m] = L;
+        L = fma(g - bsum[m], R[m], L);
+    }
+    for (int m = m1 - 1; m >= m0 && m > n / 2; --m) {
+        Q = fma(g - bsum[m], R[m], Q);
+        w[m] = -Q;
+    }
+    if (tid == 0) w[n] = 0.0;
+    __syncthreads();
+    if (wout)
+        for (int i = tid; i < n - 1; i += F1_THREADS) wout[(size_t)p * (n - 1) + i] = w[i + 1];
     double acc = 0.0;
-    for (int o = 0; o < nobs; ++o) {
+    for (int o = tid; o < nobs; o += F1_THREADS) {
         const double s = obs[o] * n;
         int i0 = (int)floor(s);
         if (i0 > n - 1) i0 = n - 1;
@@ -635,16 +679,19 @@ __global__ void k_forward1d(int n, int Km, int count, const double* __restrict__
         const double rr = y - data[o];
         acc += rr * rr;
     }
-    Phi[p] = acc * inv2s2;
+    acc = block_sum(acc, red);
+    if (tid == 0) Phi[p] = acc * inv2s2;
 }
 
 void launch_forward1d(Ctx& c, const double* X, int count, double* Phi, double* w_out) {
     const double inv2s2 = 1.0 / (2.0 * c.cfg.sigma * c.cfg.sigma);
+    const size_t sm = sizeof(double) * ((c.Km <= F1_SMEM_N ? (size_t)c.Km : 0) + (c.n <= F1_SMEM_N ? 2 * (size_t)c.n + 1 : 0));
+    if (sm > 48 * 1024) check(cudaFuncSetAttribute(k_forward1d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm), "attr");
     for (int off = 0; off < count; off += c.B) {
         const int cnt = std::min(c.B, count - off);
-        k_forward1d<<<(cnt + 63) / 64, 64, 0, c.stream>>>(c.n, c.Km, cnt, X + (size_t)off * c.d, c.basis, c.b64, c.nobs, c.obs,
-                                                          c.data, inv2s2, Phi + off, w_out ? w_out + (size_t)off * (c.n - 1) : nullptr,
-                                                          c.u64); ++c.pc.launches;
+        k_forward1d<<<cnt, F1_THREADS, sm, c.stream>>>(c.n, c.Km, X + (size_t)off * c.d, c.basis, c.b64 + (c.n - 1), c.nobs, c.obs, c.data,
+                                                       inv2s2, Phi + off, w_out ? w_out + (size_t)off * (c.n - 1) : nullptr,
+                                                       c.u64); ++c.pc.launches;
     }
     check(cudaGetLastError(), "forward1d");
 }
