@@ -17,7 +17,8 @@
  *   - Host input arrays are copied during the call; host output pointers are
  *     caller-owned and may be NULL where stated.
  *   - Work is issued on the CUDA stream given to smc_init().  Calls that
- *     return host scalars synchronise that stream; smc_move() and
+ *     return host scalars synchronise that stream; where the solver runs in
+ *     passes over all particles (see cfg.tile_kernel), smc_move() and
  *     smc_forward() also synchronise once per solver iteration to stop as
  *     soon as every particle has converged.
  *   - Calls must follow the SMC order (init -> [temper -> resample -> fit ->
@@ -127,7 +128,9 @@ typedef struct smc_config {
                            modes (EM with the ridge var_floor * diag(lambda_S)); 0: diagonal
                            lambda_j as in Sec. 2.3.  pCN-GM and independence kernels only */
     int tile_kernel;    /* stencil tiles of the multigrid / CG passes on the tiled levels:
-                           0 = the default (2); 1 = 32 x 32 tiles, one thread block each;
+                           0 = the default: the mixed-precision solver on grids of 64^2
+                           and 128^2 keeps each particle's whole solve on chip (FP32
+                           faces throughout), anything else as 2; 1 = 32 x 32 tiles, one thread block each;
                            2 = 16 x 16 tiles, one warp each, the finest level's inputs staged
                            by TMA (FP32; the FP64 solver uses 3); 3 = 16 x 16 tiles, one warp
                            each, loading from global memory; 4 = the finest level as 2, the

@@ -162,6 +162,7 @@ int gradient_batch(Ctx& c, const double* X, int count, double* Phi_out, double* 
     const size_t nn = (size_t)n * n;
     const bool mixed = mixed_precision(c.cfg);
     int itmax = 0;
+    OnchipCounters counters(c);
     for (int off = 0; off < count; off += c.B) {
         const int cnt = std::min(c.B, count - off);
         // 1. forward: field, coefficients, w, Phi
@@ -193,7 +194,7 @@ int gradient_batch(Ctx& c, const double* X, int count, double* Phi_out, double* 
         launch_analysis2d(c, c.rhs, cnt, grad_out + (size_t)off * c.d);
     }
     check(cudaGetLastError(), "gradient");
-    return itmax;
+    return std::max(itmax, counters.finish());
 }
 
 }  // namespace smcgm

@@ -493,6 +493,7 @@ smc_status smc_init(const smc_config* cfg, void* d_ws, size_t bytes, void* strea
     if (c.dim == 2) {
         if (mixed_precision(c.cfg)) build_tma_maps<float>(c, c.s32);
         else build_tma_maps<double>(c, c.s64);
+        c.onchip = onchip_supported(c);
     }
     set_prior_mixture(c);
     c.fitted = (c.cfg.kernel == SMC_K_PCN || c.cfg.kernel == SMC_K_PCNL);
@@ -594,6 +595,7 @@ smc_status smc_move(smc_ctx* ctx, int steps, double* accept_rate, int* iters_max
     const long long nc0 = c.nonconv;
     int itmax = 0;
     long long solves = (long long)c.N * steps;
+    OnchipCounters counters(c);              // on-chip solves: no wait until the last step
     if (c.cfg.kernel == SMC_K_PCNL) {
         itmax = gradient_batch(c, c.X, c.N, c.Phi2, c.G);   // DPhi of the current particles (Phi2: scratch)
         for (int s = 0; s < steps; ++s) {
@@ -625,6 +627,7 @@ smc_status smc_move(smc_ctx* ctx, int steps, double* accept_rate, int* iters_max
             ++c.step;
         }
     }
+    itmax = std::max(itmax, counters.finish());
     int hacc = 0;
     check(cudaMemcpyAsync(&hacc, accn, sizeof(int), cudaMemcpyDeviceToHost, c.stream), "d2h");
     sync_stream(c);

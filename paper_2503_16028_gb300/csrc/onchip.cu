@@ -1,0 +1,1106 @@
+// The mixed-precision solve of a batch of particles on chip: one launch runs every refinement
+// phase, CG iteration and V-cycle of a particle in one thread block (64^2), or in a cluster of
+// 2 x 2 (128^2) or 4 x 4 blocks (256^2) that exchange tile edges through distributed shared memory.
+//
+// Why: the multi-pass solver (solver.cu) reads and writes every vector of the finest grid three
+// times per CG iteration (82 bytes a cell: 4.6 TB/s at 4096 particles of 256^2), pays a launch
+// for each pass of each level and waits for the host after each iteration; on 64^2 and 128^2
+// grids the launches and the coarse levels' barriers are most of its time.  Here a cell's faces,
+// residual and correction stay in registers for the whole solve, CG's p and the reciprocal
+// diagonals in shared memory, and only the solution's three FP32 parts and x go through L2.
+//
+// Layout: a block covers 64 x 64 cells with 16 x 16 threads, a 4 x 4 patch each; a thread also
+// owns the 2 x 2 cells below its patch on the next level and the one cell on the level after
+// that, so restriction and prolongation over those levels need no exchange, and their Galerkin
+// faces are sums of the patch's.  Neighbours exchange the edge values of one colour per
+// half-sweep; a block's edge threads also store them into the neighbouring block's guard slots
+// (guards at the domain's walls stay zero: the wall faces only enter the diagonal).  Below that
+// every block of a cluster holds the whole coarse problem (32^2 for 4 x 4 blocks, 16^2 for
+// 2 x 2) and solves it redundantly, which costs less than the cluster barriers of sharing it;
+// the 8^2 level is solved with its dense inverse, formed once per solve.
+//
+// The V-cycle is otherwise that of solver.cu (symmetric red-black Gauss-Seidel, the same sweeps,
+// Galerkin coarsening, scaled correction).  The residual after a pre-smoothing that ends with the
+// black cells vanishes there, so only the red cells are restricted.
+//
+// What bounds it: the latency of about 30 barrier-separated phases per CG iteration, not HBM; two
+// blocks per SM (128 registers a thread, 113 KB) overlap them.
+#include <cstdio>
+#include "smcgm_internal.cuh"
+#include "common.cuh"
+#include "df32.cuh"
+
+namespace smcgm {
+
+constexpr int OC_T = 256;
+
+struct OcArgs {
+    int n, max_outer, maxit, nu_f, nu_c;
+    float cc, tol2, floor2, tolout2;
+    double b2const;
+    const double* b2pp;
+    const float *Kw, *Ks, *E, *Nn, *Kwl, *Ksl, *El, *Nl;   // faces: high and low parts
+    const float2* bdf;
+    size_t bstride;
+    float4 *x, *wh, *wm, *wl;    // per particle n^2 floats, [block][patch row][thread]
+    double* W;
+    const int* badp;
+    GraphCounters* cnt;
+    int* err;
+};
+
+// Shared-memory offsets (floats).
+template <int C>
+struct OcMem {
+    static constexpr int CC = C * C;
+    static constexpr int P4 = 0;                            // p: 4 float4 slots
+    static constexpr int INVF = P4 + 16 * OC_T;             // 1/D of the patch: 2 float4 per colour
+    static constexpr int INVH = INVF + 16 * OC_T;           // float4
+    static constexpr int INVQ = INVH + 4 * OC_T;
+    static constexpr int LF = INVQ + OC_T;                  // C = 4: 12 faces and 4 1/D of the 32^2 level's patch
+    static constexpr int SF = LF + (C == 4 ? 16 * OC_T : 0);   // C > 1: 4 faces and 1/D of the 16^2 level's cell
+    static constexpr int INV8 = SF + (C > 1 ? 5 * OC_T : 0);   // dense inverse of the 8^2 level, [k][row]
+    static constexpr int R8 = INV8 + 4096;
+    static constexpr int PART8 = R8 + 64;
+    static constexpr int RED = PART8 + 256;                 // 3 slots of 8 CC warp sums
+    static constexpr int RB = RED + 3 * 8 * CC;             // gathered right-hand side of the first local level
+    static constexpr int SIDE = RB + (C == 4 ? 1024 : C == 2 ? 256 : 0);   // 4 sides x 2 colours x 272 float2
+    static constexpr int HP = SIDE + 8 * 544;               // 4 planes of 18 x 18: cell (i, j) of each 2 x 2 patch
+    static constexpr int QP = HP + 4 * 324;
+    static constexpr int LP = QP + 324;                     // C = 4: as HP for the 32^2 level
+    static constexpr int SP = LP + (C == 4 ? 4 * 324 : 0);  // C > 1: as QP for the 16^2 level
+    static constexpr int BARS = SP + (C > 1 ? 324 : 0);     // C > 1: 2 + 4 mbarriers (8 bytes each)
+    static constexpr int TOTAL = BARS + (C > 1 ? 12 : 0);
+    static constexpr size_t BYTES = (size_t)TOTAL * 4;
+};
+
+__device__ __forceinline__ uint32_t oc_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Barrier of the cluster (of the block when it is alone), ordering shared, distributed shared and
+// global memory among its threads.
+template <int C>
+__device__ __forceinline__ void oc_sync() {
+    if (C == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    }
+}
+// The address of a shared-memory location of this block in block `rank` of the cluster.
+__device__ __forceinline__ uint32_t oc_map(const float* p, uint32_t rank) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+// Asynchronous stores into another block; the receiver's mbarrier counts their bytes, so an
+// exchange needs neither a cluster barrier nor the memory fence that one implies (the fence's
+// wait was the largest stall of the cluster form: 2048 solves at 256^2 62 ms with cluster barriers).
+__device__ __forceinline__ void oc_push(float* p, uint32_t rank, float v, const float* bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(oc_map(p, rank)), "f"(v),
+                 "r"(oc_map(bar, rank))
+                 : "memory");
+}
+__device__ __forceinline__ void oc_push2(float* p, uint32_t rank, float2 v, const float* bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(oc_map(p, rank)), "f"(v.x),
+                 "f"(v.y), "r"(oc_map(bar, rank))
+                 : "memory");
+}
+
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Where a thread stands.
+template <int C>
+struct OcPos {
+    int tid, tx, ty, cx, cy;
+    uint32_t rank;
+    // exchanges (C > 1): edge exchanges alternate between two mbarriers (a neighbour can be at most one
+    // exchange ahead, since it needs this block's edges to go on), the all-to-all ones have one each
+    // (a block can be at most one all-to-all exchange ahead of any other)
+    unsigned seq, par;
+    bool dead;               // a bounded wait ran out
+    int neighbours;
+};
+enum OcAll { OC_RR = 0, OC_RZ = 1, OC_PQ = 2, OC_GATHER = 3 };
+constexpr int OC_POLLS = 1 << 20;
+
+template <int C>
+__device__ __forceinline__ float* nb_bar(float* sm, const OcPos<C>& t) { return sm + OcMem<C>::BARS + 2 * (t.seq & 1); }
+template <int C>
+__device__ __forceinline__ float* all_bar(float* sm, int which) { return sm + OcMem<C>::BARS + 4 + 2 * which; }
+__device__ __forceinline__ void oc_expect(const float* bar, int bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(bar)), "r"(bytes) : "memory");
+}
+template <int C>
+__device__ __forceinline__ void oc_wait(OcPos<C>& t, const float* bar, unsigned parity) {
+    if (t.dead) return;
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(bar);
+    uint32_t ok = 0;
+    for (int k = 0; k < OC_POLLS && !ok; ++k)
+        asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}"
+                     : "=r"(ok)
+                     : "r"(a), "r"(parity)
+                     : "memory");
+    if (!ok) t.dead = true;
+}
+// After the pushes of an edge exchange (`bytes` from each neighbour): the block's own stores and the
+// neighbours' are visible.
+template <int C>
+__device__ __forceinline__ void nb_sync(float* sm, OcPos<C>& t, int bytes) {
+    if (C > 1 && t.tid == 0) oc_expect(nb_bar(sm, t), bytes * t.neighbours);
+    __syncthreads();
+    if (C > 1) {
+        oc_wait<C>(t, nb_bar(sm, t), (t.seq >> 1) & 1);
+        ++t.seq;
+    }
+}
+// The same for an all-to-all exchange (`bytes` from all blocks together).
+template <int C>
+__device__ __forceinline__ void all_sync(float* sm, OcPos<C>& t, int which, int bytes) {
+    if (C > 1 && t.tid == 0) oc_expect(all_bar<C>(sm, which), bytes);
+    __syncthreads();
+    if (C > 1) {
+        oc_wait<C>(t, all_bar<C>(sm, which), (t.par >> which) & 1);
+        t.par ^= 1u << which;
+    }
+}
+
+// The exchange that starts an iteration: |r|^2 and the first red edges.  True if a wait ran out in any thread
+// of the block, which then leaves the loops alike (threads must not decide on sums that others did not see).
+template <int C>
+__device__ __forceinline__ bool rr_sync(float* sm, OcPos<C>& t) {
+    if (C == 1) {
+        __syncthreads();
+        return false;
+    }
+    if (t.tid == 0) {
+        oc_expect(nb_bar(sm, t), 128 * t.neighbours);
+        oc_expect(all_bar<C>(sm, OC_RR), 32 * OcMem<C>::CC);
+    }
+    oc_wait<C>(t, nb_bar(sm, t), (t.seq >> 1) & 1);
+    oc_wait<C>(t, all_bar<C>(sm, OC_RR), (t.par >> OC_RR) & 1);
+    ++t.seq;
+    t.par ^= 1u << OC_RR;
+    return __syncthreads_or(t.dead);
+}
+
+// ---- sums over the particle's cells: every thread of every block ends with the same bits ----
+template <int C>
+__device__ __forceinline__ void red_put(float* sm, const OcPos<C>& t, int slot, float v) {
+    using M = OcMem<C>;
+    v = warp_sum(v);
+    const int lane = t.tid & 31, wid = t.tid >> 5;
+    float* dst = sm + M::RED + slot * 8 * M::CC + (int)t.rank * 8 + wid;
+    if (C == 1) {
+        if (lane == 0) *dst = v;
+    } else if (lane < M::CC) {
+        oc_push(dst, (uint32_t)lane, v, all_bar<C>(sm, slot));
+    }
+}
+template <int C>
+__device__ __forceinline__ float red_get(const float* sm, const OcPos<C>& t, int slot) {
+    using M = OcMem<C>;
+    const float* s = sm + M::RED + slot * 8 * M::CC;
+    if (C == 1) {
+        const float4 a = *reinterpret_cast<const float4*>(s), b = *reinterpret_cast<const float4*>(s + 4);
+        return ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
+    }
+    const int lane = t.tid & 31;
+    float v;
+    if (C == 2) {
+        v = s[lane];
+    } else {
+        const float4 a = *reinterpret_cast<const float4*>(s + 4 * lane);
+        v = (a.x + a.y) + (a.z + a.w);
+    }
+    return warp_sum(v);
+}
+
+// ---- the finest level: a 4 x 4 patch, e[4 j + i] of cell (i, j); red: i + j even ----
+// Sides of colour col: W, E (rows of 17), S, N (17 rows of 16); the pair holds the side's two cells of
+// that colour in ascending order.
+template <int C>
+__device__ __forceinline__ float2* side(float* sm, int s, int col) {
+    return reinterpret_cast<float2*>(sm + OcMem<C>::SIDE) + (s * 2 + col) * 272;
+}
+
+template <int C, int COL>
+__device__ __forceinline__ void pub_f(float* sm, const OcPos<C>& t, const float (&e)[16]) {
+    const float2 w = COL == 0 ? make_float2(e[0], e[8]) : make_float2(e[4], e[12]);
+    const float2 ea = COL == 0 ? make_float2(e[7], e[15]) : make_float2(e[3], e[11]);
+    const float2 s = COL == 0 ? make_float2(e[0], e[2]) : make_float2(e[1], e[3]);
+    const float2 n = COL == 0 ? make_float2(e[13], e[15]) : make_float2(e[12], e[14]);
+    float2 *W = side<C>(sm, 0, COL), *E = side<C>(sm, 1, COL), *S = side<C>(sm, 2, COL), *N = side<C>(sm, 3, COL);
+    W[t.ty * 17 + t.tx] = w;
+    E[t.ty * 17 + t.tx + 1] = ea;
+    S[t.ty * 16 + t.tx] = s;
+    N[(t.ty + 1) * 16 + t.tx] = n;
+    if (C > 1) {
+        const float* bar = nb_bar(sm, t);
+        if (t.tx == 0 && t.cx > 0) oc_push2(reinterpret_cast<float*>(W + t.ty * 17 + 16), t.rank - 1, w, bar);
+        if (t.tx == 15 && t.cx < C - 1) oc_push2(reinterpret_cast<float*>(E + t.ty * 17), t.rank + 1, ea, bar);
+        if (t.ty == 0 && t.cy > 0) oc_push2(reinterpret_cast<float*>(S + 16 * 16 + t.tx), t.rank - C, s, bar);
+        if (t.ty == 15 && t.cy < C - 1) oc_push2(reinterpret_cast<float*>(N + t.tx), t.rank + C, n, bar);
+    }
+}
+
+struct HaloF { float2 w, e, s, n; };
+template <int C>
+__device__ __forceinline__ HaloF halo_f(float* sm, const OcPos<C>& t, int col) {   // the neighbours' cells of colour col
+    HaloF h;
+    h.w = side<C>(sm, 1, col)[t.ty * 17 + t.tx];
+    h.e = side<C>(sm, 0, col)[t.ty * 17 + t.tx + 1];
+    h.s = side<C>(sm, 3, col)[t.ty * 16 + t.tx];
+    h.n = side<C>(sm, 2, col)[(t.ty + 1) * 16 + t.tx];
+    return h;
+}
+__device__ __forceinline__ float pick(float2 v, int k) { return k ? v.y : v.x; }
+
+// Neighbours of cell (i, j), from the patch or the halo of the other colour.
+#define OC_NB_F(i, j, e, h, w_, e_, s_, n_)                                  \
+    const float w_ = (i) > 0 ? e[4 * (j) + (i) - 1] : pick(h.w, (j) >> 1);   \
+    const float e_ = (i) < 3 ? e[4 * (j) + (i) + 1] : pick(h.e, (j) >> 1);   \
+    const float s_ = (j) > 0 ? e[4 * (j) - 4 + (i)] : pick(h.s, (i) >> 1);   \
+    const float n_ = (j) < 3 ? e[4 * (j) + 4 + (i)] : pick(h.n, (i) >> 1);
+
+template <int C, int COL>
+__device__ __forceinline__ void inv_f(const float* sm, const OcPos<C>& t, float (&v)[8]) {
+    const float4* p = reinterpret_cast<const float4*>(sm + OcMem<C>::INVF) + 2 * COL * OC_T + t.tid;
+    const float4 a = p[0], b = p[OC_T];
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+
+template <int C, int COL>
+__device__ __forceinline__ void sweep_f(float* sm, const OcPos<C>& t, const float (&kw)[20], const float (&ks)[20], const float (&r)[16],
+                                        float (&e)[16], bool pointwise) {
+    float inv[8];
+    inv_f<C, COL>(sm, t, inv);
+    if (pointwise) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = (j + COL) & 1; i < 4; i += 2) e[4 * j + i] = r[4 * j + i] * inv[2 * j + (i >> 1)];
+        return;
+    }
+    const HaloF h = halo_f<C>(sm, t, 1 - COL);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = (j + COL) & 1; i < 4; i += 2) {
+            OC_NB_F(i, j, e, h, ew, ee, es, en)
+            const float num = fmaf(ks[4 * (j + 1) + i], en, fmaf(ks[4 * j + i], es, fmaf(kw[5 * j + i + 1], ee, fmaf(kw[5 * j + i], ew, r[4 * j + i]))));
+            e[4 * j + i] = num * inv[2 * j + (i >> 1)];
+        }
+}
+
+// ---- a level with a 2 x 2 patch per thread: cells 0 (0,0), 1 (1,0), 2 (0,1), 3 (1,1); red: 0 and 3 ----
+struct Patch2 { float w[6], s[6]; };   // west faces [j][0..2], south faces [0..2][i]
+template <int C, bool SHARED>
+__device__ __forceinline__ void pub_h(float* sm, float* pl, const OcPos<C>& t, int col, const float (&e)[4]) {
+    const int at = (t.ty + 1) * 18 + t.tx + 1;
+    const int a = col ? 1 : 0, b = col ? 2 : 3;
+    pl[a * 324 + at] = e[col ? 1 : 0];
+    pl[b * 324 + at] = e[col ? 2 : 3];
+    if (SHARED && C > 1) {
+        const float* bar = nb_bar(sm, t);
+        if (t.tx == 0 && t.cx > 0) oc_push(pl + (col ? 2 : 0) * 324 + (t.ty + 1) * 18 + 17, t.rank - 1, col ? e[2] : e[0], bar);
+        if (t.tx == 15 && t.cx < C - 1) oc_push(pl + (col ? 1 : 3) * 324 + (t.ty + 1) * 18, t.rank + 1, col ? e[1] : e[3], bar);
+        if (t.ty == 0 && t.cy > 0) oc_push(pl + (col ? 1 : 0) * 324 + 17 * 18 + t.tx + 1, t.rank - C, col ? e[1] : e[0], bar);
+        if (t.ty == 15 && t.cy < C - 1) oc_push(pl + (col ? 2 : 3) * 324 + t.tx + 1, t.rank + C, col ? e[2] : e[3], bar);
+    }
+}
+// Sum of k e over the four neighbours of the two cells of a colour (0: cells 0 and 3, 1: cells 1 and 2).
+template <int C>
+__device__ __forceinline__ void nb_h(const float* pl, const OcPos<C>& t, int col, const Patch2& k, const float (&e)[4], float& a, float& b) {
+    const int at = (t.ty + 1) * 18 + t.tx + 1;
+    const float *p0 = pl + at, *p1 = p0 + 324, *p2 = p1 + 324, *p3 = p2 + 324;
+    if (col == 0) {
+        a = fmaf(k.w[0], p1[-1], fmaf(k.s[0], p2[-18], fmaf(k.w[1], e[1], k.s[2] * e[2])));
+        b = fmaf(k.w[5], p2[1], fmaf(k.s[5], p1[18], fmaf(k.w[4], e[2], k.s[3] * e[1])));
+    } else {
+        a = fmaf(k.w[2], p0[1], fmaf(k.s[1], p3[-18], fmaf(k.w[1], e[0], k.s[3] * e[3])));
+        b = fmaf(k.w[3], p3[-1], fmaf(k.s[4], p0[18], fmaf(k.w[4], e[3], k.s[2] * e[0])));
+    }
+}
+__device__ __forceinline__ void diag_h(const Patch2& k, float (&d)[4]) {
+    d[0] = (k.w[0] + k.w[1]) + (k.s[0] + k.s[2]);
+    d[1] = (k.w[1] + k.w[2]) + (k.s[1] + k.s[3]);
+    d[2] = (k.w[3] + k.w[4]) + (k.s[2] + k.s[4]);
+    d[3] = (k.w[4] + k.w[5]) + (k.s[3] + k.s[5]);
+}
+
+// Pre-smoothing from e = 0 and the sum of the red cells' residuals (the black ones' are zero).
+template <int C, bool SHARED>
+__device__ __forceinline__ float pre_h(float* sm, float* pl, OcPos<C>& t, int nu, const Patch2& k, const float4 inv, const float (&r)[4], float (&e)[4]) {
+    float a, b;
+    for (int sw = 0; sw < nu; ++sw) {
+        if (sw == 0) {
+            e[0] = r[0] * inv.x;
+            e[3] = r[3] * inv.w;
+        } else {
+            nb_h<C>(pl, t, 0, k, e, a, b);
+            e[0] = (r[0] + a) * inv.x;
+            e[3] = (r[3] + b) * inv.w;
+        }
+        pub_h<C, SHARED>(sm, pl, t, 0, e);
+        if (SHARED) nb_sync<C>(sm, t, 64); else __syncthreads();
+        nb_h<C>(pl, t, 1, k, e, a, b);
+        e[1] = (r[1] + a) * inv.y;
+        e[2] = (r[2] + b) * inv.z;
+        pub_h<C, SHARED>(sm, pl, t, 1, e);
+        if (SHARED) nb_sync<C>(sm, t, 64); else __syncthreads();
+    }
+    nb_h<C>(pl, t, 0, k, e, a, b);
+    float d[4];
+    diag_h(k, d);
+    return (r[0] + fmaf(-d[0], e[0], a)) + (r[3] + fmaf(-d[3], e[3], b));
+}
+// e already holds the corrected values; post-smoothing (black, red); the last red values are not published.
+template <int C, bool SHARED>
+__device__ __forceinline__ void post_h(float* sm, float* pl, OcPos<C>& t, int nu, const Patch2& k, const float4 inv, const float (&r)[4], float (&e)[4]) {
+    float a, b;
+    for (int sw = 0; sw < nu; ++sw) {
+        pub_h<C, SHARED>(sm, pl, t, 0, e);
+        if (SHARED) nb_sync<C>(sm, t, 64); else __syncthreads();
+        nb_h<C>(pl, t, 1, k, e, a, b);
+        e[1] = (r[1] + a) * inv.y;
+        e[2] = (r[2] + b) * inv.z;
+        pub_h<C, SHARED>(sm, pl, t, 1, e);
+        if (SHARED) nb_sync<C>(sm, t, 64); else __syncthreads();
+        nb_h<C>(pl, t, 0, k, e, a, b);
+        e[0] = (r[0] + a) * inv.x;
+        e[3] = (r[3] + b) * inv.w;
+    }
+}
+
+// ---- a level with one cell per thread; red: tx + ty even ----
+struct Cell1 { float w, e, s, n; };
+template <int C, bool SHARED>
+__device__ __forceinline__ void pub_q(float* sm, float* pl, const OcPos<C>& t, float e) {
+    pl[(t.ty + 1) * 18 + t.tx + 1] = e;
+    if (SHARED && C > 1) {
+        const float* bar = nb_bar(sm, t);
+        if (t.tx == 0 && t.cx > 0) oc_push(pl + (t.ty + 1) * 18 + 17, t.rank - 1, e, bar);
+        if (t.tx == 15 && t.cx < C - 1) oc_push(pl + (t.ty + 1) * 18, t.rank + 1, e, bar);
+        if (t.ty == 0 && t.cy > 0) oc_push(pl + 17 * 18 + t.tx + 1, t.rank - C, e, bar);
+        if (t.ty == 15 && t.cy < C - 1) oc_push(pl + t.tx + 1, t.rank + C, e, bar);
+    }
+}
+__device__ __forceinline__ float nb_q(const float* pl, int tx, int ty, const Cell1& k) {
+    const float* p = pl + (ty + 1) * 18 + tx + 1;
+    return fmaf(k.w, p[-1], fmaf(k.e, p[1], fmaf(k.s, p[-18], k.n * p[18])));
+}
+// Pre-smoothing from e = 0; returns the residual of a red cell, 0 for a black one.
+template <int C, bool SHARED>
+__device__ __forceinline__ float pre_q(float* sm, float* pl, OcPos<C>& t, int nu, const Cell1& k, float inv, float r, float& e) {
+    const bool red = ((t.tx + t.ty) & 1) == 0;
+    for (int sw = 0; sw < nu; ++sw) {
+        if (red) {
+            e = (sw == 0 ? r : r + nb_q(pl, t.tx, t.ty, k)) * inv;
+            pub_q<C, SHARED>(sm, pl, t, e);
+        }
+        if (SHARED) nb_sync<C>(sm, t, 32); else __syncthreads();
+        if (!red) {
+            e = (r + nb_q(pl, t.tx, t.ty, k)) * inv;
+            pub_q<C, SHARED>(sm, pl, t, e);
+        }
+        if (SHARED) nb_sync<C>(sm, t, 32); else __syncthreads();
+    }
+    return red ? r + fmaf(-((k.w + k.e) + (k.s + k.n)), e, nb_q(pl, t.tx, t.ty, k)) : 0.f;
+}
+template <int C, bool SHARED>
+__device__ __forceinline__ void post_q(float* sm, float* pl, OcPos<C>& t, int nu, const Cell1& k, float inv, float r, float& e) {
+    const bool red = ((t.tx + t.ty) & 1) == 0;
+    for (int sw = 0; sw < nu; ++sw) {
+        if (red) pub_q<C, SHARED>(sm, pl, t, e);
+        if (SHARED) nb_sync<C>(sm, t, 32); else __syncthreads();
+        if (!red) {
+            e = (r + nb_q(pl, t.tx, t.ty, k)) * inv;
+            pub_q<C, SHARED>(sm, pl, t, e);
+        }
+        if (SHARED) nb_sync<C>(sm, t, 32); else __syncthreads();
+        if (red) e = (r + nb_q(pl, t.tx, t.ty, k)) * inv;
+    }
+}
+
+// Sum over the 2 x 2 threads that share a coarse cell (all in one warp).
+__device__ __forceinline__ float quad_sum(float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 16);
+}
+
+// Faces of the 2 x 2-thread coarse cell: the sums of the fine faces on its sides.
+__device__ __forceinline__ Cell1 coarse_faces(const Cell1& k, int tx, int ty) {
+    const Cell1 a{k.w + __shfl_xor_sync(0xffffffffu, k.w, 16), k.e + __shfl_xor_sync(0xffffffffu, k.e, 16),
+                  k.s + __shfl_xor_sync(0xffffffffu, k.s, 1), k.n + __shfl_xor_sync(0xffffffffu, k.n, 1)};
+    const float w1 = __shfl_xor_sync(0xffffffffu, a.w, 1), e1 = __shfl_xor_sync(0xffffffffu, a.e, 1);
+    const float s1 = __shfl_xor_sync(0xffffffffu, a.s, 16), n1 = __shfl_xor_sync(0xffffffffu, a.n, 16);
+    return Cell1{(tx & 1) ? w1 : a.w, (tx & 1) ? a.e : e1, (ty & 1) ? s1 : a.s, (ty & 1) ? a.n : n1};
+}
+
+// Dense inverse of the 8^2 level from its faces (each held by the four threads of its cell), by
+// Gauss-Jordan elimination in registers: thread (row, quarter) holds 16 columns of a row, the
+// pivot row and column go through shared memory, one barrier per step.  Stored symmetrised.
+template <int C>
+__device__ __forceinline__ void build_inv8(float* sm, const OcPos<C>& t, const Cell1& k8) {
+    using M = OcMem<C>;
+    float* M8 = sm + M::INV8;
+    float* fa = M8;                                         // 4 x 64 faces first
+    if (((t.tx | t.ty) & 1) == 0) {
+        const int c = (t.ty >> 1) * 8 + (t.tx >> 1);
+        fa[c] = k8.w; fa[64 + c] = k8.e; fa[128 + c] = k8.s; fa[192 + c] = k8.n;
+    }
+    __syncthreads();
+    const int row = t.tid & 63, q = t.tid >> 6;
+    float a[16];
+    {
+        const float w = fa[row], e = fa[64 + row], s = fa[128 + row], n = fa[192 + row];
+        const int I = row & 7, J = row >> 3;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+            const int col = 16 * q + c;
+            float v = 0.f;
+            if (col == row) v = (w + e) + (s + n);
+            if (I > 0 && col == row - 1) v = -w;
+            if (I < 7 && col == row + 1) v = -e;
+            if (J > 0 && col == row - 8) v = -s;
+            if (J < 7 && col == row + 8) v = -n;
+            a[c] = v;
+        }
+    }
+    __syncthreads();
+    float* buf = M8;                                        // two buffers of (row 64, column 64)
+    for (int q0 = 0; q0 < 4; ++q0) {
+#pragma unroll
+        for (int kk = 0; kk < 16; ++kk) {
+            const int k = 16 * q0 + kk;
+            float* rb = buf + (kk & 1) * 128;
+            if (row == k) {
+#pragma unroll
+                for (int c = 0; c < 16; ++c) rb[16 * q + c] = a[c];
+            }
+            if (q == q0) rb[64 + row] = a[kk];
+            __syncthreads();
+            const float p = 1.f / rb[k], f = rb[64 + row];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const float rk = rb[16 * q + c] * p;
+                a[c] = row == k ? rk : fmaf(-f, rk, a[c]);
+            }
+            if (q == q0) a[kk] = row == k ? p : -f * p;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 16; ++c) M8[(16 * q + c) * 64 + row] = a[c];
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 16; ++c) a[c] = 0.5f * (a[c] + M8[row * 64 + 16 * q + c]);
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 16; ++c) M8[(16 * q + c) * 64 + row] = a[c];
+    __syncthreads();
+}
+
+// The 16^2 level (one cell per thread, its plane pl) with the dense solve of the 8^2 level below it.
+template <int C, bool SHARED>
+__device__ __forceinline__ void level16(float* sm, float* pl, OcPos<C>& t, int nu, float cc, const Cell1& k, float inv, float r, float& e) {
+    using M = OcMem<C>;
+    const float res = quad_sum(pre_q<C, SHARED>(sm, pl, t, nu, k, inv, r, e));
+    if (((t.tx | t.ty) & 1) == 0) sm[M::R8 + (t.ty >> 1) * 8 + (t.tx >> 1)] = res;
+    __syncthreads();
+    {
+        const int row = t.tid & 63, q = t.tid >> 6;
+        const float* m = sm + M::INV8 + 16 * q * 64 + row;
+        const float4* r8 = reinterpret_cast<const float4*>(sm + M::R8 + 16 * q);
+        float a = 0.f, b = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float4 v = r8[c];
+            a = fmaf(m[(4 * c) * 64], v.x, a);
+            b = fmaf(m[(4 * c + 1) * 64], v.y, b);
+            a = fmaf(m[(4 * c + 2) * 64], v.z, a);
+            b = fmaf(m[(4 * c + 3) * 64], v.w, b);
+        }
+        sm[M::PART8 + 64 * q + row] = a + b;
+    }
+    __syncthreads();
+    const float* p8 = sm + M::PART8 + (t.ty >> 1) * 8 + (t.tx >> 1);
+    e = fmaf(cc, (p8[0] + p8[64]) + (p8[128] + p8[192]), e);
+    post_q<C, SHARED>(sm, pl, t, nu, k, inv, r, e);
+}
+
+__device__ __forceinline__ Patch2 coarsen_f(const float (&kw)[20], const float (&ks)[20]) {
+    Patch2 h;
+#pragma unroll
+    for (int J = 0; J < 2; ++J)
+#pragma unroll
+        for (int I = 0; I < 3; ++I) h.w[3 * J + I] = kw[5 * (2 * J) + 2 * I] + kw[5 * (2 * J + 1) + 2 * I];
+#pragma unroll
+    for (int J = 0; J < 3; ++J)
+#pragma unroll
+        for (int I = 0; I < 2; ++I) h.s[2 * J + I] = ks[4 * (2 * J) + 2 * I] + ks[4 * (2 * J) + 2 * I + 1];
+    return h;
+}
+__device__ __forceinline__ Cell1 coarsen_h(const Patch2& h) {
+    return Cell1{h.w[0] + h.w[3], h.w[2] + h.w[5], h.s[0] + h.s[1], h.s[4] + h.s[5]};
+}
+
+// ---- the solution as three FP32 parts (72 bits): no FP64 instruction, whose rate is 1/64 of FP32 ----
+__device__ __forceinline__ void tri_add(float& h, float& m, float& l, float x) {
+    float s, e1, u, e2;
+    two_sum(h, x, s, e1);
+    two_sum(m, e1, u, e2);
+    const float l2 = __fadd_rn(l, e2);
+    float u2;
+    fast_two_sum(s, u, h, u2);
+    fast_two_sum(u2, l2, m, l);
+}
+// a - b as df32 (exact to ~2^-47 of the difference of neighbouring values).
+__device__ __forceinline__ df32 tri_diff(float ah, float am, float al, float bh, float bm, float bl) {
+    float s, e, s2, e2, u, u2;
+    two_sum(ah, -bh, s, e);
+    two_sum(am, -bm, s2, e2);
+    two_sum(s, s2, u, u2);
+    const float low = __fadd_rn(__fadd_rn(u2, e), __fadd_rn(e2, __fsub_rn(al, bl)));
+    df32 r;
+    fast_two_sum(u, low, r.hi, r.lo);
+    return r;
+}
+// (h + m + l) 2^add, rounded to FP64 with one integer conversion.
+__device__ __forceinline__ double tri_to_double(float h, float m, float l, int add) {
+    const int bh = __float_as_int(h), bm = __float_as_int(m), bl = __float_as_int(l);
+    const int eh = (bh >> 23) & 255, em = (bm >> 23) & 255, el = (bl >> 23) & 255;
+    if (eh < 64 || eh > 250) return ((double)h + ((double)m + (double)l)) * exp2((double)add);
+    auto mant = [](int b, int e) -> long long {
+        const int v = e ? (b & 0x7fffff) | 0x800000 : 0;
+        return (long long)(b < 0 ? -v : v);
+    };
+    long long I = mant(bh, eh) << 36;                       // unit 2^(eh - 150 - 36)
+    auto shifted = [&](int b, int e) -> long long {
+        const int s = 36 - (eh - e);
+        const long long v = mant(b, e);
+        return s >= 0 ? v << min(s, 38) : s > -40 ? v >> (-s) : 0ll;
+    };
+    I += shifted(bm, em) + shifted(bl, el);
+    const double d = __ll2double_rn(I);
+    return I ? __hiloint2double(__double2hiint(d) + ((eh - 186 + add) << 20), __double2loint(d)) : 0.0;
+}
+
+// One particle per cluster of C x C blocks, n = 64 C.
+template <int C>
+__global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
+    using M = OcMem<C>;
+    extern __shared__ __align__(16) float sm[];
+    const int n = 64 * C;
+    const int p = blockIdx.x / M::CC;
+    OcPos<C> t;
+    t.tid = threadIdx.x; t.tx = t.tid & 15; t.ty = t.tid >> 4;
+    t.rank = C == 1 ? 0u : oc_rank();
+    t.cx = (int)t.rank % C; t.cy = (int)t.rank / C;
+    t.seq = 0; t.par = 0; t.dead = false;
+    t.neighbours = (t.cx > 0) + (t.cx < C - 1) + (t.cy > 0) + (t.cy < C - 1);
+    const int gx = 64 * t.cx + 4 * t.tx, gy = 64 * t.cy + 4 * t.ty;
+    const size_t base = (size_t)p * n * n;
+    const double b2 = A.b2pp ? A.b2pp[p] : A.b2const;
+    if (!(b2 > 0.0) || (A.badp && A.badp[p])) {             // not solved: w = 0 (the whole cluster alike)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            double2* o = reinterpret_cast<double2*>(A.W + base + (size_t)(gy + j) * n + gx);
+            o[0] = o[1] = make_double2(0.0, 0.0);
+        }
+        return;
+    }
+    // the system scaled by a power of two so that |b| is in [1, 2): squares stay in range in FP32
+    int sexp = -((int)((__double2hiint(b2) >> 20) & 0x7ff) - 1023 >> 1);
+    sexp = max(-100, min(100, sexp));
+    const float scale = __int_as_float((127 + sexp) << 23);
+    const float b2s = (float)(b2 * (double)scale * (double)scale);
+    // guards and planes
+    for (int i = M::SIDE + t.tid; i < M::BARS; i += OC_T) sm[i] = 0.f;
+    if (C > 1 && t.tid == 0) {
+        for (int k = 0; k < 6; ++k)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(sm + M::BARS + 2 * k)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // faces of the patch: west faces 4 x 5, south faces 5 x 4
+    float kw[20], ks[20];
+    {
+        const float *Kw = A.Kw + base, *Ks = A.Ks + base;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float4 v = *reinterpret_cast<const float4*>(Kw + (size_t)(gy + j) * n + gx);
+            kw[5 * j] = v.x; kw[5 * j + 1] = v.y; kw[5 * j + 2] = v.z; kw[5 * j + 3] = v.w;
+            kw[5 * j + 4] = gx + 4 < n ? Kw[(size_t)(gy + j) * n + gx + 4] : A.E[(size_t)p * n + gy + j];
+        }
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const float4 v = gy + j < n ? *reinterpret_cast<const float4*>(Ks + (size_t)(gy + j) * n + gx)
+                                        : *reinterpret_cast<const float4*>(A.Nn + (size_t)p * n + gx);
+            ks[4 * j] = v.x; ks[4 * j + 1] = v.y; ks[4 * j + 2] = v.z; ks[4 * j + 3] = v.w;
+        }
+    }
+    float4* const P4 = reinterpret_cast<float4*>(sm + M::P4) + t.tid;
+    {
+        float4* q = reinterpret_cast<float4*>(sm + M::INVF) + t.tid;
+        float inv[2][8];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                inv[(i + j) & 1][2 * j + (i >> 1)] = 1.f / ((kw[5 * j + i] + kw[5 * j + i + 1]) + (ks[4 * j + i] + ks[4 * j + 4 + i]));
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            q[(2 * c) * OC_T] = make_float4(inv[c][0], inv[c][1], inv[c][2], inv[c][3]);
+            q[(2 * c + 1) * OC_T] = make_float4(inv[c][4], inv[c][5], inv[c][6], inv[c][7]);
+        }
+    }
+    {
+        const Patch2 h = coarsen_f(kw, ks);
+        float d[4];
+        diag_h(h, d);
+        reinterpret_cast<float4*>(sm + M::INVH)[t.tid] = make_float4(1.f / d[0], 1.f / d[1], 1.f / d[2], 1.f / d[3]);
+        const Cell1 k = coarsen_h(h);
+        sm[M::INVQ + t.tid] = 1.f / ((k.w + k.e) + (k.s + k.n));
+        const Cell1 kc = coarse_faces(k, t.tx, t.ty);
+        oc_sync<C>();                                       // every block of the cluster runs: its shared memory may be written
+        if (C == 1) {
+            build_inv8<C>(sm, t, kc);
+        } else {
+            // gather the next level's faces in every block (through the inverse's storage)
+            constexpr int m = C * 8;
+            float* fb = sm + M::INV8;
+            const int cell = (t.cy * 8 + (t.ty >> 1)) * m + t.cx * 8 + (t.tx >> 1);
+            for (uint32_t d0 = (t.tx & 1) + 2 * (t.ty & 1); d0 < (uint32_t)M::CC; d0 += 4) {
+                const float* bar = all_bar<C>(sm, OC_GATHER);
+                oc_push(fb + cell, d0, kc.w, bar);
+                oc_push(fb + m * m + cell, d0, kc.e, bar);
+                oc_push(fb + 2 * m * m + cell, d0, kc.s, bar);
+                oc_push(fb + 3 * m * m + cell, d0, kc.n, bar);
+            }
+            all_sync<C>(sm, t, OC_GATHER, M::CC * 64 * 16);
+            Cell1 k16;
+            if (C == 4) {
+                float* lf = sm + M::LF + t.tid;
+                Patch2 l;
+#pragma unroll
+                for (int J = 0; J < 2; ++J) {
+                    const int c = (2 * t.ty + J) * m + 2 * t.tx;
+                    l.w[3 * J] = fb[c]; l.w[3 * J + 1] = fb[c + 1]; l.w[3 * J + 2] = fb[m * m + c + 1];
+                    l.s[2 * J] = fb[2 * m * m + c]; l.s[2 * J + 1] = fb[2 * m * m + c + 1];
+                    if (J == 1) { l.s[4] = fb[3 * m * m + c]; l.s[5] = fb[3 * m * m + c + 1]; }
+                }
+                diag_h(l, d);
+#pragma unroll
+                for (int q = 0; q < 6; ++q) { lf[q * OC_T] = l.w[q]; lf[(6 + q) * OC_T] = l.s[q]; }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) lf[(12 + q) * OC_T] = 1.f / d[q];
+                k16 = coarsen_h(l);
+            } else {
+                k16 = Cell1{fb[t.tid], fb[m * m + t.tid], fb[2 * m * m + t.tid], fb[3 * m * m + t.tid]};
+            }
+            float* sf = sm + M::SF + t.tid;
+            sf[0] = k16.w; sf[OC_T] = k16.e; sf[2 * OC_T] = k16.s; sf[3 * OC_T] = k16.n;
+            sf[4 * OC_T] = 1.f / ((k16.w + k16.e) + (k16.s + k16.n));
+            const Cell1 k8 = coarse_faces(k16, t.tx, t.ty);
+            __syncthreads();
+            build_inv8<C>(sm, t, k8);
+        }
+    }
+    // r = scaled b
+    const float2* B = A.bdf + (size_t)p * A.bstride;
+    float r[16], e[16];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 v = B[(size_t)(gy + j) * n + gx + i];
+            r[4 * j + i] = __fadd_rn(v.x, v.y) * scale;
+        }
+    const size_t pb = (size_t)blockIdx.x * 4 * OC_T + t.tid;   // this thread's patch rows in x, wh, wm, wl
+    int iters = 0, phases = 0, inner = 0;
+    bool converged = false, wset = false;
+    for (int o = 0; o < A.max_outer; ++o) {
+        // ---- CG on A x = r from x = 0 ----
+        float thr = 0.f, rz = 0.f;
+        bool first = true;
+        for (;;) {
+            float s = 0.f;
+#pragma unroll
+            for (int c = 0; c < 16; ++c) s = fmaf(r[c], r[c], s);
+            red_put<C>(sm, t, 0, s);
+            sweep_f<C, 0>(sm, t, kw, ks, r, e, true);
+            pub_f<C, 0>(sm, t, e);
+            if (rr_sync<C>(sm, t)) break;
+            const float rr = red_get<C>(sm, t, 0);
+            if (first) {
+                thr = fmaxf(A.tol2 * rr, A.floor2 * b2s);
+                if (!(rr > 0.f)) break;
+                ++inner;
+            } else {
+                ++iters;
+                if (rr <= thr || iters >= A.maxit || !(rr == rr)) break;
+            }
+            // V-cycle: z = M r in e
+            for (int sw = 0; sw < A.nu_f; ++sw) {
+                if (sw > 0) {
+                    sweep_f<C, 0>(sm, t, kw, ks, r, e, false);
+                    pub_f<C, 0>(sm, t, e);
+                    nb_sync<C>(sm, t, 128);
+                }
+                sweep_f<C, 1>(sm, t, kw, ks, r, e, false);
+                pub_f<C, 1>(sm, t, e);
+                nb_sync<C>(sm, t, 128);
+            }
+            float rh[4], eh[4];
+            {
+                const HaloF h = halo_f<C>(sm, t, 1);
+                float res[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int i = j & 1; i < 4; i += 2) {
+                        OC_NB_F(i, j, e, h, ew, ee, es, en)
+                        const float ec = e[4 * j + i];
+                        const float q = fmaf(kw[5 * j + i], ec - ew, fmaf(kw[5 * j + i + 1], ec - ee, fmaf(ks[4 * j + i], ec - es, ks[4 * j + 4 + i] * (ec - en))));
+                        res[2 * (j >> 1) + (i >> 1)] += r[4 * j + i] - q;
+                    }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) rh[c] = res[c];
+            }
+            const float4 invh = reinterpret_cast<const float4*>(sm + M::INVH)[t.tid];
+            float rq, eq;
+            {
+                const Patch2 h = coarsen_f(kw, ks);
+                rq = pre_h<C, true>(sm, sm + M::HP, t, A.nu_c, h, invh, rh, eh);
+                const Cell1 k = coarsen_h(h);
+                const float invq = sm[M::INVQ + t.tid];
+                float* QP = sm + M::QP;
+                if (C == 1) {
+                    level16<C, true>(sm, QP, t, A.nu_c, A.cc, k, invq, rq, eq);
+                } else {
+                    const float rc = quad_sum(pre_q<C, true>(sm, QP, t, A.nu_c, k, invq, rq, eq));
+                    constexpr int m = C * 8;
+                    const int cell = (t.cy * 8 + (t.ty >> 1)) * m + t.cx * 8 + (t.tx >> 1);
+                    for (uint32_t d0 = (t.tx & 1) + 2 * (t.ty & 1); d0 < (uint32_t)M::CC; d0 += 4) oc_push(sm + M::RB + cell, d0, rc, all_bar<C>(sm, OC_GATHER));
+                    all_sync<C>(sm, t, OC_GATHER, M::CC * 64 * 4);
+                    const int px = t.cx * 8 + (t.tx >> 1), py = t.cy * 8 + (t.ty >> 1);   // the parent on the gathered level
+                    const float* sf = sm + M::SF + t.tid;
+                    const Cell1 k16{sf[0], sf[OC_T], sf[2 * OC_T], sf[3 * OC_T]};
+                    float e16, ep;
+                    if (C == 4) {
+                        const float* lf = sm + M::LF + t.tid;
+                        Patch2 l;
+#pragma unroll
+                        for (int q = 0; q < 6; ++q) { l.w[q] = lf[q * OC_T]; l.s[q] = lf[(6 + q) * OC_T]; }
+                        const float4 invl = make_float4(lf[12 * OC_T], lf[13 * OC_T], lf[14 * OC_T], lf[15 * OC_T]);
+                        const float* rb = sm + M::RB + 2 * t.ty * m + 2 * t.tx;
+                        const float rl[4] = {rb[0], rb[1], rb[m], rb[m + 1]};
+                        float el[4];
+                        float* LP = sm + M::LP;
+                        const float r16 = pre_h<C, false>(sm, LP, t, A.nu_c, l, invl, rl, el);
+                        level16<C, false>(sm, sm + M::SP, t, A.nu_c, A.cc, k16, sf[4 * OC_T], r16, e16);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) el[c] = fmaf(A.cc, e16, el[c]);
+                        post_h<C, false>(sm, LP, t, A.nu_c, l, invl, rl, el);
+                        pub_h<C, false>(sm, LP, t, 0, el);
+                        __syncthreads();
+                        ep = LP[((px & 1) + 2 * (py & 1)) * 324 + ((py >> 1) + 1) * 18 + (px >> 1) + 1];
+                    } else {
+                        float* SPl = sm + M::SP;
+                        level16<C, false>(sm, SPl, t, A.nu_c, A.cc, k16, sf[4 * OC_T], sm[M::RB + t.tid], e16);
+                        if (((t.tx + t.ty) & 1) == 0) SPl[(t.ty + 1) * 18 + t.tx + 1] = e16;
+                        __syncthreads();
+                        ep = SPl[(py + 1) * 18 + px + 1];
+                    }
+                    eq = fmaf(A.cc, ep, eq);
+                    post_q<C, true>(sm, QP, t, A.nu_c, k, invq, rq, eq);
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) eh[c] = fmaf(A.cc, eq, eh[c]);
+                post_h<C, true>(sm, sm + M::HP, t, A.nu_c, h, invh, rh, eh);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) e[4 * j + i] = fmaf(A.cc, eh[2 * (j >> 1) + (i >> 1)], e[4 * j + i]);
+            for (int sw = 0; sw < A.nu_f; ++sw) {
+                pub_f<C, 0>(sm, t, e);
+                nb_sync<C>(sm, t, 128);
+                sweep_f<C, 1>(sm, t, kw, ks, r, e, false);
+                pub_f<C, 1>(sm, t, e);
+                nb_sync<C>(sm, t, 128);
+                sweep_f<C, 0>(sm, t, kw, ks, r, e, false);
+            }
+            // beta, p = z + beta p
+            s = 0.f;
+#pragma unroll
+            for (int c = 0; c < 16; ++c) s = fmaf(r[c], e[c], s);
+            red_put<C>(sm, t, OC_RZ, s);
+            all_sync<C>(sm, t, OC_RZ, 32 * M::CC);
+            const float rzn = red_get<C>(sm, t, 1);
+            if (!first) {
+                const float beta = rzn / rz;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float4 v = P4[j * OC_T];
+                    e[4 * j] = fmaf(beta, v.x, e[4 * j]);
+                    e[4 * j + 1] = fmaf(beta, v.y, e[4 * j + 1]);
+                    e[4 * j + 2] = fmaf(beta, v.z, e[4 * j + 2]);
+                    e[4 * j + 3] = fmaf(beta, v.w, e[4 * j + 3]);
+                }
+            }
+            rz = rzn;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) P4[j * OC_T] = make_float4(e[4 * j], e[4 * j + 1], e[4 * j + 2], e[4 * j + 3]);
+            pub_f<C, 0>(sm, t, e);
+            pub_f<C, 1>(sm, t, e);
+            nb_sync<C>(sm, t, 256);
+            // q = A p in flux form, p.q
+            float q[16];
+            s = 0.f;
+#pragma unroll
+            for (int col = 0; col < 2; ++col) {
+                const HaloF h = halo_f<C>(sm, t, 1 - col);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int i = (j + col) & 1; i < 4; i += 2) {
+                        OC_NB_F(i, j, e, h, ew, ee, es, en)
+                        const float ec = e[4 * j + i];
+                        const float v = fmaf(kw[5 * j + i], ec - ew, fmaf(kw[5 * j + i + 1], ec - ee, fmaf(ks[4 * j + i], ec - es, ks[4 * j + 4 + i] * (ec - en))));
+                        q[4 * j + i] = v;
+                        s = fmaf(ec, v, s);
+                    }
+            }
+            red_put<C>(sm, t, 2, s);
+            float4 xv[4];
+            if (!first) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) xv[j] = A.x[pb + j * OC_T];
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) xv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            all_sync<C>(sm, t, OC_PQ, 32 * M::CC);
+            const float pq = red_get<C>(sm, t, 2);
+            const float alpha = pq > 0.f ? rz / pq : 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                xv[j].x = fmaf(alpha, e[4 * j], xv[j].x);
+                xv[j].y = fmaf(alpha, e[4 * j + 1], xv[j].y);
+                xv[j].z = fmaf(alpha, e[4 * j + 2], xv[j].z);
+                xv[j].w = fmaf(alpha, e[4 * j + 3], xv[j].w);
+                A.x[pb + j * OC_T] = xv[j];
+            }
+#pragma unroll
+            for (int c = 0; c < 16; ++c) r[c] = fmaf(-alpha, q[c], r[c]);
+            first = false;
+        }
+        // ---- w += x; FP64-accurate residual ----
+        ++phases;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const size_t at = pb + j * OC_T;
+            float4 h = make_float4(0.f, 0.f, 0.f, 0.f), m = h, l = h, x = h;
+            if (wset) { h = A.wh[at]; m = A.wm[at]; l = A.wl[at]; }
+            if (!first) x = A.x[at];
+            tri_add(h.x, m.x, l.x, x.x);
+            tri_add(h.y, m.y, l.y, x.y);
+            tri_add(h.z, m.z, l.z, x.z);
+            tri_add(h.w, m.w, l.w, x.w);
+            A.wh[at] = h; A.wm[at] = m; A.wl[at] = l;
+        }
+        wset = true;
+        oc_sync<C>();
+        float s = 0.f;
+        {
+            const float *Kwl = A.Kwl + base, *Ksl = A.Ksl + base;
+            const float* W3[3] = {reinterpret_cast<const float*>(A.wh), reinterpret_cast<const float*>(A.wm), reinterpret_cast<const float*>(A.wl)};
+            // patch rows of the neighbouring threads (another block of the cluster at the tile's edge)
+            const size_t blk = 4 * OC_T;
+            const size_t pw = t.tx > 0 ? pb - 1 : pb - blk + 15, pe = t.tx < 15 ? pb + 1 : pb + blk - 15;
+            const size_t ps = t.ty > 0 ? pb - 16 : pb - C * blk + 240, pn = t.ty < 15 ? pb + 16 : pb + C * blk - 240;
+            const bool hw = gx > 0, he = gx + 4 < n, hs = gy > 0, hn = gy + 4 < n;
+            float c3[3][4], f3[3][4];                           // this row, the row above or below
+            df32 fs[4];
+            auto row = [&](size_t at, float (&v)[3][4]) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const float4 a = __ldcg(reinterpret_cast<const float4*>(W3[q]) + at);
+                    v[q][0] = a.x; v[q][1] = a.y; v[q][2] = a.z; v[q][3] = a.w;
+                }
+            };
+            auto zero = [](float (&v)[3][4]) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v[q][i] = 0.f;
+            };
+            row(pb, c3);
+            if (hs) row(ps + 3 * OC_T, f3); else zero(f3);
+            {
+                const float4 kl = *reinterpret_cast<const float4*>(Ksl + (size_t)gy * n + gx);
+                const float k4[4] = {kl.x, kl.y, kl.z, kl.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    fs[i] = df_mul(df32{ks[i], k4[i]}, tri_diff(c3[0][i], c3[1][i], c3[2][i], f3[0][i], f3[1][i], f3[2][i]));
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (j < 3) row(pb + (j + 1) * OC_T, f3);
+                else if (hn) row(pn, f3);
+                else zero(f3);
+                const float4 kn = (j < 3 || hn) ? *reinterpret_cast<const float4*>(Ksl + (size_t)(gy + j + 1) * n + gx)
+                                                : *reinterpret_cast<const float4*>(A.Nl + (size_t)p * n + gx);
+                const float4 kv = *reinterpret_cast<const float4*>(Kwl + (size_t)(gy + j) * n + gx);
+                const float ke = he ? Kwl[(size_t)(gy + j) * n + gx + 4] : A.El[(size_t)p * n + gy + j];
+                const float kwl[5] = {kv.x, kv.y, kv.z, kv.w, ke}, ksl[4] = {kn.x, kn.y, kn.z, kn.w};
+                float wv[3] = {0.f, 0.f, 0.f}, ev[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    if (hw) wv[q] = __ldcg(W3[q] + 4 * (pw + j * OC_T) + 3);
+                    if (he) ev[q] = __ldcg(W3[q] + 4 * (pe + j * OC_T));
+                }
+                df32 fw = df_mul(df32{kw[5 * j], kwl[0]}, tri_diff(c3[0][0], c3[1][0], c3[2][0], wv[0], wv[1], wv[2]));
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const df32 de = i < 3 ? tri_diff(c3[0][i + 1 & 3], c3[1][i + 1 & 3], c3[2][i + 1 & 3], c3[0][i], c3[1][i], c3[2][i])
+                                          : tri_diff(ev[0], ev[1], ev[2], c3[0][3], c3[1][3], c3[2][3]);
+                    const df32 fe = df_mul(df32{kw[5 * j + i + 1], kwl[i + 1]}, de);
+                    const df32 fn = df_mul(df32{ks[4 * j + 4 + i], ksl[i]}, tri_diff(f3[0][i], f3[1][i], f3[2][i], c3[0][i], c3[1][i], c3[2][i]));
+                    const df32 aw = df_add(df_add(fw, df_neg(fe)), df_add(fs[i], df_neg(fn)));
+                    const float2 bv = B[(size_t)(gy + j) * n + gx + i];
+                    const df32 rs = df_sub_acc(df32{bv.x * scale, bv.y * scale}, aw);
+                    const float v = __fadd_rn(rs.hi, rs.lo);
+                    r[4 * j + i] = v;
+                    s = fmaf(v, v, s);
+                    fw = fe;
+                    fs[i] = fn;
+                }
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) c3[q][i] = f3[q][i];
+            }
+        }
+        red_put<C>(sm, t, OC_RZ, s);
+        all_sync<C>(sm, t, OC_RZ, 32 * M::CC);
+        if (C > 1 && __syncthreads_or(t.dead)) break;
+        const float res2 = red_get<C>(sm, t, OC_RZ);
+        if (res2 <= A.tolout2 * b2s) { converged = true; break; }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const size_t at = pb + j * OC_T;
+        const float4 h = A.wh[at], m = A.wm[at], l = A.wl[at];
+        double2* o = reinterpret_cast<double2*>(A.W + base + (size_t)(gy + j) * n + gx);
+        o[0] = make_double2(tri_to_double(h.x, m.x, l.x, -sexp), tri_to_double(h.y, m.y, l.y, -sexp));
+        o[1] = make_double2(tri_to_double(h.z, m.z, l.z, -sexp), tri_to_double(h.w, m.w, l.w, -sexp));
+    }
+    if (t.rank == 0 && t.tid == 0) {
+        GraphCounters* g = A.cnt;
+        atomicAdd(&g->cg_iterations, (unsigned long long)iters);
+        atomicAdd(&g->inner_solves, (unsigned long long)inner);
+        atomicAdd(&g->residuals, (unsigned long long)phases);
+        if (!converged) atomicAdd(&g->nonconv, 1ull);
+        atomicMax(&g->itmax, iters);
+    }
+    if (C > 1 && t.dead) atomicExch(A.err, 1);
+    if (C > 1) oc_sync<C>();                                    // no block leaves while another may still store into it
+}
+
+template <int C>
+static void oc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int count, cudaStream_t st) {
+    check(cudaFuncSetAttribute(k_onchip<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OcMem<C>::BYTES), "attr");
+    if (C == 4) check(cudaFuncSetAttribute(k_onchip<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "attr");
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3((unsigned)(count * C * C));
+    cfg.blockDim = dim3(OC_T);
+    cfg.dynamicSmemBytes = OcMem<C>::BYTES;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C * C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+}
+
+template <int C>
+static bool oc_fits() {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    oc_config<C>(cfg, attr, 1, nullptr);
+    int nc = 0;
+    if (C == 1) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nc, k_onchip<C>, OC_T, OcMem<C>::BYTES) != cudaSuccess) nc = 0;
+    } else if (cudaOccupancyMaxActiveClusters(&nc, k_onchip<C>, &cfg) != cudaSuccess) {
+        nc = 0;
+    }
+    (void)cudaGetLastError();
+    return nc > 0;
+}
+
+// Whether the context's solves run on chip: mixed precision, the default tile kernels, a grid of
+// 64 C cells per side for the block grids above, and clusters of that size on this device.
+bool onchip_supported(const Ctx& c) {
+    if (c.dim != 2 || !mixed_precision(c.cfg) || c.cfg.tile_kernel != 0) return false;
+    if (c.n == 64) return oc_fits<1>();
+    if (c.n == 128) return oc_fits<2>();
+    // 256^2 in 4 x 4 blocks: 53.3 ms for 2048 solves against 55.2 in the multi-pass solver, not enough to switch
+    return false;
+}
+
+template <int C>
+static void oc_launch(Ctx& c, const OcArgs& A, int count) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    oc_config<C>(cfg, attr, count, c.stream);
+    check(cudaLaunchKernelEx(&cfg, k_onchip<C>, A), "on-chip solve"); ++c.pc.launches;
+}
+
+// Solves a batch into W; the counters accumulate in c.gcnt (fold_onchip_counters reads them).
+void solve_batch_onchip(Ctx& c, int count, const Rhs& R, double* W) {
+    InnerSolver<float>& s = c.s32;
+    LevelArrays<float>& f = s.lv[0];
+    OcArgs A{};
+    A.n = c.n; A.max_outer = c.cfg.max_refine; A.maxit = c.cfg.max_iter; A.nu_f = c.cfg.fine_sweeps; A.nu_c = c.cfg.smooth_sweeps;
+    A.cc = (float)c.cfg.coarse_scale;
+    A.tol2 = (float)(c.cfg.tol_inner * c.cfg.tol_inner);
+    A.tolout2 = (float)(c.cfg.tol_outer * c.cfg.tol_outer);
+    A.floor2 = (float)(0.25 * c.cfg.tol_outer * c.cfg.tol_outer);   // no phase need reduce |r| below half the final tolerance
+    A.b2const = R.b2const; A.b2pp = R.b2pp;
+    A.Kw = f.Kw; A.Ks = f.Ks; A.E = f.E; A.Nn = f.Nn;
+    A.Kwl = c.Kwlo; A.Ksl = c.Kslo; A.El = c.Elo; A.Nl = c.Nlo;
+    A.bdf = R.bdf; A.bstride = R.stride;
+    A.x = reinterpret_cast<float4*>(s.x); A.wh = reinterpret_cast<float4*>(s.p[0]);
+    A.wm = reinterpret_cast<float4*>(s.p[1]); A.wl = reinterpret_cast<float4*>(s.q);
+    A.W = W;
+    A.badp = c.lenient ? c.badp : nullptr;
+    A.cnt = c.gcnt;
+    A.err = c.dev_err;
+    if (c.prof) check(cudaEventRecord(c.ev0, c.stream), "event");
+    if (c.n == 64) oc_launch<1>(c, A, count);
+    else if (c.n == 128) oc_launch<2>(c, A, count);
+    else oc_launch<4>(c, A, count);
+    if (c.prof) {   // profiling: this kernel is the dominant one (faces' two parts in, w out per cell)
+        check(cudaEventRecord(c.ev1, c.stream), "event");
+        check(cudaEventSynchronize(c.ev1), "event wait");
+        float ms = 0.f;
+        check(cudaEventElapsedTime(&ms, c.ev0, c.ev1), "event time");
+        c.pc.dom_ms += ms;
+        c.pc.dom_launches += 1;
+        c.pc.dom_particles += count;
+        c.pc.dom_bytes += 24.0 * c.n * c.n * count;
+    }
+}
+
+}  // namespace smcgm

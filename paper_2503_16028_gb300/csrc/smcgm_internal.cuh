@@ -173,6 +173,8 @@ struct Rhs {
 };
 Rhs shared_rhs(const Ctx& c);
 int solve_batch(Ctx& c, int count, const Rhs& R, double* W);   // W: the FP64 solutions (count x n x n)
+bool onchip_supported(const Ctx& c);
+void solve_batch_onchip(Ctx& c, int count, const Rhs& R, double* W);
 void forward_solve_graph(Ctx& c, const double* X, int count, double* Phi_out);   // into the graph being captured
 void capture_move_steps(Ctx& c, int steps, int* acc_count);                      // into the graph being captured
 void launch_mark_out_of_range(Ctx& c, int count, double* Phi);
@@ -279,7 +281,9 @@ struct Ctx {
     bool graph = false;
     int gdepth = 0;                   // nesting depth of the body being captured
     cudaStream_t gaux[4] = {nullptr, nullptr, nullptr, nullptr};
-    GraphCounters* gcnt = nullptr;    // device counters of graph-mode solves
+    GraphCounters* gcnt = nullptr;    // device counters of graph-mode and on-chip solves
+    bool onchip = false;              // the solves run in onchip.cu's kernel (decided at smc_init)
+    bool onchip_open = false;         // an OnchipCounters scope is collecting their counters
     int* gouter = nullptr;            // device: [0] refinement phase, [1] particles entering it
     MoveSched* msched = nullptr;      // device schedule of a graph-mode move
     int* gsteps = nullptr;            // device: steps left in a graph-mode move
@@ -295,6 +299,17 @@ void check(cudaError_t e, const char* what);   // throws CudaError
 void sync_stream(Ctx& c);
 // The same, and throws if a kernel's bounded wait timed out since the last check.
 void sync_and_check_barrier(Ctx& c);
+// The counters of the on-chip solves issued in a scope.  The solves run without the host; the outermost
+// scope clears the device counters and finish() waits once, adds them to the context's counters, reports
+// the errors that the multi-pass solver reports between its iterations, and returns the largest iteration
+// count.  Scopes of contexts without on-chip solves, and inner ones, do nothing.
+struct OnchipCounters {
+    Ctx& c;
+    bool own;
+    explicit OnchipCounters(Ctx& cc);
+    ~OnchipCounters();
+    int finish();
+};
 // An NVTX range named after a kernel family (set-up, solve, proposal, ...) for the
 // duration of a scope, so that profiler timelines group the library's launches.
 struct NvtxRange {

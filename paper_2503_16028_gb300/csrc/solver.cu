@@ -1021,6 +1021,35 @@ static void run_vcycle_lower(Ctx& c, InnerSolver<T>& s, int nact) {
     }
 }
 
+OnchipCounters::OnchipCounters(Ctx& cc) : c(cc), own(cc.onchip && !cc.onchip_open) {
+    if (!own) return;
+    check(cudaMemsetAsync(c.gcnt, 0, sizeof(GraphCounters), c.stream), "memset counters");
+    c.onchip_open = true;
+}
+OnchipCounters::~OnchipCounters() {
+    if (own) c.onchip_open = false;
+}
+int OnchipCounters::finish() {
+    if (!own) return 0;
+    GraphCounters g{};
+    int err[2] = {0, 0};
+    check(cudaMemcpyAsync(&g, c.gcnt, sizeof(g), cudaMemcpyDeviceToHost, c.stream), "counters d2h");
+    check(cudaMemcpyAsync(err, c.dev_err, 2 * sizeof(int), cudaMemcpyDeviceToHost, c.stream), "err d2h");
+    sync_stream(c);
+    c.pc.cg_iterations += (long long)g.cg_iterations;
+    c.pc.inner_solves += (long long)g.inner_solves;
+    c.pc.residuals += (long long)g.residuals;
+    c.nonconv += (long long)g.nonconv;
+    if (err[0] || err[1]) {   // cleared in stream order, so the context stays usable
+        check(cudaMemsetAsync(c.dev_err, 0, 2 * sizeof(int), c.stream), "err reset");
+        sync_stream(c);
+    }
+    if (err[0]) throw CudaError{cudaErrorLaunchTimeout, "a kernel's bounded wait timed out"};
+    if (err[1] && !c.lenient)
+        throw InputError{"log-permeability |u| >= 64 is outside the mixed-precision range (use the FP64 solver)"};
+    return g.itmax;
+}
+
 // Compacts act_in into the active list and returns its length (synchronises the stream).
 template <typename T>
 static int compact_active(Ctx& c, InnerSolver<T>& s, int count, int* hcount) {
@@ -1345,8 +1374,9 @@ void launch_setup_coeffs(Ctx& c, int count) {
         check(cudaMemsetAsync(c.badp, 0, count * sizeof(int), c.stream), "memset badp");
         k_faces_df<<<dim3((n / FX) * (n / FY), count), FX * FY, 0, c.stream>>>(
             n, reinterpret_cast<const float2*>(c.u64), reinterpret_cast<const float2*>(c.exptab), c.expc, f0.Kw, c.Kwlo, f0.Ks, c.Kslo, f0.E, c.Elo, f0.Nn, c.Nlo,
-            f0.Kwb, f0.Ksb, c.dev_err, c.badp); ++c.pc.launches;
-        launch_coarsen_all<float>(c, c.s32, count);
+            c.onchip ? nullptr : f0.Kwb, c.onchip ? nullptr : f0.Ksb, c.dev_err, c.badp); ++c.pc.launches;
+        if (!c.onchip) launch_coarsen_all<float>(c, c.s32, count);
+        check(cudaGetLastError(), "setup launch");
         return;
     }
     k_exp_neg<<<grid_for(total), 256, 0, c.stream>>>(c.u64, total); ++c.pc.launches;
@@ -1685,7 +1715,8 @@ void forward_solve_graph(Ctx& c, const double* X, int count, double* Phi_out) {
         else
             launch_synth2d(c, X + (size_t)off * c.d, cnt, c.u64);
         launch_setup_coeffs(c, cnt);
-        if (mixed_precision(c.cfg)) solve_batch_graph<float>(c, c.s32, cnt, shared_rhs(c), c.w64);
+        if (c.onchip) solve_batch_onchip(c, cnt, shared_rhs(c), c.w64);
+        else if (mixed_precision(c.cfg)) solve_batch_graph<float>(c, c.s32, cnt, shared_rhs(c), c.w64);
         else solve_batch_graph<double>(c, c.s64, cnt, shared_rhs(c), c.w64);
         launch_observe(c, c.w64, cnt, Phi_out + off);
         launch_mark_out_of_range(c, cnt, Phi_out + off);
@@ -1738,6 +1769,13 @@ void launch_mark_out_of_range(Ctx& c, int count, double* Phi) {
 }
 
 int solve_batch(Ctx& c, int count, const Rhs& R, double* W) {
+    if (c.onchip) {                       // counted and checked by the caller's OnchipCounters
+        c.pc.solves += count;
+        c.pc.cells = c.n * c.n;
+        c.pc.word_bytes = 4;
+        solve_batch_onchip(c, count, R, W);
+        return 0;
+    }
     return mixed_precision(c.cfg) ? solve_batch_t<float>(c, c.s32, count, R, W)
                                                  : solve_batch_t<double>(c, c.s64, count, R, W);
 }
@@ -1749,6 +1787,7 @@ int forward_solve(Ctx& c, const double* X, int count, double* Phi_out, double* w
     }
     int itmax = 0;
     const size_t nn = (size_t)c.n * c.n;
+    OnchipCounters counters(c);
     for (int off = 0; off < count; off += c.B) {
         const int cnt = std::min(c.B, count - off);
         {
@@ -1772,6 +1811,7 @@ int forward_solve(Ctx& c, const double* X, int count, double* Phi_out, double* w
         if (w_out) check(cudaMemcpyAsync(w_out + off * nn, c.w64, cnt * nn * sizeof(double), cudaMemcpyDeviceToDevice, c.stream), "w copy");
     }
     check(cudaGetLastError(), "forward");
+    itmax = std::max(itmax, counters.finish());
     c.last_iters = itmax;
     return itmax;
 }
