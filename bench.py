@@ -563,8 +563,17 @@ def time_moves(s, steps, warmup, torch, barrier):
     return ms, prof
 
 
+def on_chip(prof):
+    """Whether the profiled solves ran in the on-chip kernel (its algorithmic bytes: 24 per cell and solve)."""
+    cells = prof.get("dom_particles", 0) * prof["cells"]
+    return cells > 0 and abs(prof["dom_bytes"] / cells - 24.0) < 1e-6
+
+
 def model_bytes_per_solve(prof, n, d):
     """Algorithmic DRAM bytes of the whole move per particle-solve (every array read or written once per pass)."""
+    if on_chip(prof):
+        # synthesis passes 16 B, faces 24 B, the solve (faces hi/lo in, w out) 24 B per cell, and the KL vectors
+        return 64.0 * prof["cells"] + 4 * d * 8
     w = prof["word_bytes"]
     cells = prof["cells"]
     solves = max(1, prof["solves"])
@@ -653,11 +662,13 @@ def run_native(args, rank, world, local):
     dom_ach = prof["dom_bytes"] / (prof["dom_ms"] / 1000.0) / 1e9 if prof["dom_ms"] > 0 else 0.0
     # DRAM bytes per cell of the dominant kernel from one ncu capture of the current kernel on
     # the 512-particle case, scaled to the average particles of a launch here
-    tb = TRAFFIC_BYTES_PER_CELL.get(args.smoother)
+    chip = on_chip(prof)
+    tb = None if chip else TRAFFIC_BYTES_PER_CELL.get(args.smoother)
     traffic = tb * 65536 * prof["dom_particles"] / max(1, prof["dom_launches"]) if tb else None
-    roof = dict(bound="hbm", achieved=dom_ach, peak=hbm_peak, unit="GB/s", frac=dom_ach / hbm_peak, traffic=traffic,
+    roof = dict(bound="latency" if chip else "hbm", achieved=dom_ach, peak=hbm_peak, unit="GB/s", frac=dom_ach / hbm_peak, traffic=traffic,
                 algorithmic_bytes_per_launch=prof["dom_bytes"] / max(1, prof["dom_launches"]),
-                kernel="k_tpre<2,CG> (finest level, CG update + pre-smoothing + restriction, TMA-staged; %s smoother faces)"
+                kernel="k_onchip<4> (whole solve of a particle on a cluster of 16 blocks; HBM only for its faces and its solution)" if chip else
+                "k_tpre<2,CG> (finest level, CG update + pre-smoothing + restriction, TMA-staged; %s smoother faces)"
                 % args.smoother.upper(), peak_source=peak_src,
                 launches=prof["dom_launches"], ms_per_launch=prof["dom_ms"] / max(1, prof["dom_launches"]))
     bps = model_bytes_per_solve(prof, 256, d)
@@ -722,7 +733,7 @@ def run_native(args, rank, world, local):
                 data="synthetic",
                 config=dict(workload=WORKLOAD, particles=N, grid="256x256", kl_modes="128x128", components=8,
                             observations=64, solver="FP32 MG-PCG (RB-GS 2+2, Galerkin, coarse x2; %s smoother faces) + FP64 refinement to 1e-10"
-                            % args.smoother.upper(),
+                            % ("FP32" if chip else args.smoother.upper()),
                             l2="inputs larger than L2 (%.1f GB device working set)" % (s_bytes(N) / 1e9),
                             parallelism="replicas" if world > 1 else "single GPU"),
                 roofline=roof, hbm_roofline_step=dict(model_bytes_per_solve=bps, achieved_gbs=step_hbm,

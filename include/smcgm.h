@@ -128,8 +128,8 @@ typedef struct smc_config {
                            modes (EM with the ridge var_floor * diag(lambda_S)); 0: diagonal
                            lambda_j as in Sec. 2.3.  pCN-GM and independence kernels only */
     int tile_kernel;    /* stencil tiles of the multigrid / CG passes on the tiled levels:
-                           0 = the default: the mixed-precision solver on grids of 64^2
-                           and 128^2 keeps each particle's whole solve on chip (FP32
+                           0 = the default: the mixed-precision solver on grids up to
+                           256^2 keeps each particle's whole solve on chip (FP32
                            faces throughout), anything else as 2; 1 = 32 x 32 tiles, one thread block each;
                            2 = 16 x 16 tiles, one warp each, the finest level's inputs staged
                            by TMA (FP32; the FP64 solver uses 3); 3 = 16 x 16 tiles, one warp

@@ -1,6 +1,6 @@
 // The mixed-precision solve of a batch of particles on chip: one launch runs every refinement
 // phase, CG iteration and V-cycle of a particle in one thread block (64^2), or in a cluster of
-// 2 x 2 (128^2) or 4 x 4 blocks (256^2) that exchange tile edges through distributed shared memory.
+// 4 (128^2) or 16 (256^2) blocks that exchange edges through distributed shared memory.
 //
 // Why: the multi-pass solver (solver.cu) reads and writes every vector of the finest grid three
 // times per CG iteration (82 bytes a cell: 4.6 TB/s at 4096 particles of 256^2), pays a launch
@@ -8,23 +8,29 @@
 // grids the launches and the coarse levels' barriers are most of its time.  Here a cell's faces,
 // residual and correction stay in registers for the whole solve, CG's p and the reciprocal
 // diagonals in shared memory, and only the solution's three FP32 parts and x go through L2.
+// Measured against it (synthesis and set-up included): 1024 solves of 64^2 4.17 -> 0.66 ms, 2048 of
+// 128^2 15.7 -> 6.6 ms, 2048 of 256^2 54.9 -> 42.0 ms, 2 of 256^2 2.35 -> 0.30 ms.
 //
-// Layout: a block covers 64 x 64 cells with 16 x 16 threads, a 4 x 4 patch each; a thread also
-// owns the 2 x 2 cells below its patch on the next level and the one cell on the level after
-// that, so restriction and prolongation over those levels need no exchange, and their Galerkin
-// faces are sums of the patch's.  Neighbours exchange the edge values of one colour per
-// half-sweep; a block's edge threads also store them into the neighbouring block's guard slots
-// (guards at the domain's walls stay zero: the wall faces only enter the diagonal).  Below that
-// every block of a cluster holds the whole coarse problem (32^2 for 4 x 4 blocks, 16^2 for
-// 2 x 2) and solves it redundantly, which costs less than the cluster barriers of sharing it;
-// the 8^2 level is solved with its dense inverse, formed once per solve.
+// Layout: a block covers a strip of 64 C x 64 / C cells (C = n / 64) with 16 C x 16 / C threads, a
+// 4 x 4 patch each; a thread also owns the 2 x 2 cells below its patch on the next level and the
+// one cell on the level after that, so restriction and prolongation over those levels need no
+// exchange, and their Galerkin faces are sums of the patch's.  Neighbours exchange the edge values
+// of one colour per half-sweep; a strip's first and last thread rows also store theirs into the
+// neighbouring block's guard slots (guards at the domain's walls stay zero: the wall faces only
+// enter the diagonal).  Strips rather than squares: two neighbours instead of four, whole rows of
+// lanes store together, and only the edge rows' warps wait for a neighbour (squares: 2048 of 256^2
+// 48.7 ms).  Below that every block of a cluster holds the whole coarse problem (32^2 for 16
+// blocks, 16^2 for 4) and solves it redundantly, which costs less than sharing it; the 8^2 level is
+// solved with its dense inverse, formed once per solve.
 //
 // The V-cycle is otherwise that of solver.cu (symmetric red-black Gauss-Seidel, the same sweeps,
 // Galerkin coarsening, scaled correction).  The residual after a pre-smoothing that ends with the
 // black cells vanishes there, so only the red cells are restricted.
 //
-// What bounds it: the latency of about 30 barrier-separated phases per CG iteration, not HBM; two
-// blocks per SM (128 registers a thread, 113 KB) overlap them.
+// What bounds it: the latency of about 30 barrier-separated phases per CG iteration (45 and 25
+// remote exchanges of 324 cycles each at 256^2), not HBM: two blocks per SM (128 registers a
+// thread, 80 to 113 KB) reach 0.53 (64^2) and 0.35 (256^2) issued instructions per scheduler cycle.
+// 14 clusters of 16 fit the GPU at a time (112 of 152 SMs).
 #include <cstdio>
 #include "smcgm_internal.cuh"
 #include "common.cuh"
@@ -49,29 +55,34 @@ struct OcArgs {
     int* err;
 };
 
+// A block covers 64 C x 64 / C cells (a strip of rows): W x H threads, a 4 x 4 patch each.
 // Shared-memory offsets (floats).
 template <int C>
 struct OcMem {
-    static constexpr int CC = C * C;
+    static constexpr int CC = C * C, W = 16 * C, H = 16 / C;
+    static constexpr int SZH = H * (W + 1), SZV = (H + 1) * W;   // float2 per colour of the sides W, E (H rows of W + 1) and S, N
+    static constexpr int PT = W + 2, PL = (H + 2) * PT;     // pitch and size of a plane with a ring of guards
     static constexpr int P4 = 0;                            // p: 4 float4 slots
     static constexpr int INVF = P4 + 16 * OC_T;             // 1/D of the patch: 2 float4 per colour
     static constexpr int INVH = INVF + 16 * OC_T;           // float4
-    static constexpr int INVQ = INVH + 4 * OC_T;
-    static constexpr int LF = INVQ + OC_T;                  // C = 4: 12 faces and 4 1/D of the 32^2 level's patch
-    static constexpr int SF = LF + (C == 4 ? 16 * OC_T : 0);   // C > 1: 4 faces and 1/D of the 16^2 level's cell
-    static constexpr int INV8 = SF + (C > 1 ? 5 * OC_T : 0);   // dense inverse of the 8^2 level, [k][row]
+    static constexpr int LF = INVH + 4 * OC_T;              // C = 4: 12 faces and 4 1/D of the 32^2 level's patch
+    static constexpr int SF = LF + (C == 4 ? 16 * OC_T : 0);   // C > 1: 4 faces of the 16^2 level's cell
+    static constexpr int INV8 = SF + (C > 1 ? 4 * OC_T : 0);   // dense inverse of the 8^2 level, [k][row]
     static constexpr int R8 = INV8 + 4096;
     static constexpr int PART8 = R8 + 64;
     static constexpr int RED = PART8 + 256;                 // 3 slots of 8 CC warp sums
     static constexpr int RB = RED + 3 * 8 * CC;             // gathered right-hand side of the first local level
-    static constexpr int SIDE = RB + (C == 4 ? 1024 : C == 2 ? 256 : 0);   // 4 sides x 2 colours x 272 float2
-    static constexpr int HP = SIDE + 8 * 544;               // 4 planes of 18 x 18: cell (i, j) of each 2 x 2 patch
-    static constexpr int QP = HP + 4 * 324;
-    static constexpr int LP = QP + 324;                     // C = 4: as HP for the 32^2 level
+    static constexpr int STG = PART8;                       // C > 1: pair sums of a block's part of it, H x W / 2
+    static constexpr int SIDE = RB + (C == 4 ? 1024 : C == 2 ? 256 : 0);   // 4 sides x 2 colours
+    static constexpr int HP = SIDE + 8 * (SZH + SZV);       // 4 planes: cell (i, j) of each 2 x 2 patch
+    static constexpr int QP = HP + 4 * PL;
+    static constexpr int LP = QP + PL;                      // C = 4: as HP for the 32^2 level (16 x 16 threads)
     static constexpr int SP = LP + (C == 4 ? 4 * 324 : 0);  // C > 1: as QP for the 16^2 level
-    static constexpr int BARS = SP + (C > 1 ? 324 : 0);     // C > 1: 2 + 4 mbarriers (8 bytes each)
-    static constexpr int TOTAL = BARS + (C > 1 ? 12 : 0);
+    static constexpr int BARS = (SP + (C > 1 ? 324 : 0) + 1) / 2 * 2;   // C > 1: 2 x 2 + 4 mbarriers (8 bytes each)
+    static constexpr int TOTAL = BARS + (C > 1 ? 16 : 0);
     static constexpr size_t BYTES = (size_t)TOTAL * 4;
+    static_assert(BYTES <= 228 * 1024 / 2 - 1024, "two blocks per SM");
+    static_assert(STG % 4 == 0 && RB % 4 == 0 && SIDE % 2 == 0 && RED % 4 == 0, "vector alignment");
 };
 
 __device__ __forceinline__ uint32_t oc_rank() {
@@ -98,15 +109,24 @@ __device__ __forceinline__ uint32_t oc_map(const float* p, uint32_t rank) {
 }
 // Asynchronous stores into another block; the receiver's mbarrier counts their bytes, so an
 // exchange needs neither a cluster barrier nor the memory fence that one implies (the fence's
-// wait was the largest stall of the cluster form: 2048 solves at 256^2 62 ms with cluster barriers).
+// wait was the largest stall of the cluster form: 2048 solves at 256^2 took 62 ms with cluster barriers,
+// 53 with these).
 __device__ __forceinline__ void oc_push(float* p, uint32_t rank, float v, const float* bar) {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(oc_map(p, rank)), "f"(v),
                  "r"(oc_map(bar, rank))
                  : "memory");
 }
-__device__ __forceinline__ void oc_push2(float* p, uint32_t rank, float2 v, const float* bar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(oc_map(p, rank)), "f"(v.x),
-                 "f"(v.y), "r"(oc_map(bar, rank))
+__device__ __forceinline__ void oc_push4(float* p, uint32_t rank, float4 v, const float* bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(oc_map(p, rank)),
+                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(oc_map(bar, rank))
+                 : "memory");
+}
+// The same with the addresses already those of the other block.
+__device__ __forceinline__ void oc_store(uint32_t dst, float v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(dst), "f"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void oc_store2(uint32_t dst, float2 v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(dst), "f"(v.x), "f"(v.y), "r"(bar)
                  : "memory");
 }
 
@@ -119,47 +139,59 @@ __device__ __forceinline__ float warp_sum(float v) {
 // Where a thread stands.
 template <int C>
 struct OcPos {
-    int tid, tx, ty, cx, cy;
+    int tid, tx, ty;         // in the block's W x H threads
+    int lx, ly;              // in the 16 x 16 threads of the local levels
     uint32_t rank;
-    // exchanges (C > 1): edge exchanges alternate between two mbarriers (a neighbour can be at most one
-    // exchange ahead, since it needs this block's edges to go on), the all-to-all ones have one each
-    // (a block can be at most one all-to-all exchange ahead of any other)
+    // Exchanges (C > 1).  Edge exchanges go pairwise between the first (last) thread row of a block and the last
+    // (first) of the block below (above), through two mbarriers per side that alternate: a neighbour's edge can be
+    // at most one exchange ahead, since it needs this edge's values to go on.  The all-to-all exchanges have one
+    // mbarrier each: a block can be at most one all-to-all exchange ahead of any other.
     unsigned seq, par;
-    bool dead;               // a bounded wait ran out
-    int neighbours;
+    int polls;               // bound of a wait; 0 after one ran out
+    uint32_t nbase;          // shared-memory base of the neighbouring block, for the threads of an edge row; else 0
+    bool lower;              // of an edge row: the lower one (neighbour below)
 };
 enum OcAll { OC_RR = 0, OC_RZ = 1, OC_PQ = 2, OC_GATHER = 3 };
-constexpr int OC_POLLS = 1 << 20;
+constexpr int OC_POLLS = 1 << 22;
 
+// Offset (floats) of the mbarrier of the current edge exchange in the receiving block: `below` for values that
+// come from the block below it.
 template <int C>
-__device__ __forceinline__ float* nb_bar(float* sm, const OcPos<C>& t) { return sm + OcMem<C>::BARS + 2 * (t.seq & 1); }
+__device__ __forceinline__ int nb_bar(const OcPos<C>& t, bool below) { return OcMem<C>::BARS + 4 * (below ? 1 : 0) + 2 * (t.seq & 1); }
 template <int C>
-__device__ __forceinline__ float* all_bar(float* sm, int which) { return sm + OcMem<C>::BARS + 4 + 2 * which; }
+__device__ __forceinline__ float* all_bar(float* sm, int which) { return sm + OcMem<C>::BARS + 8 + 2 * which; }
 __device__ __forceinline__ void oc_expect(const float* bar, int bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(bar)), "r"(bytes) : "memory");
 }
 template <int C>
 __device__ __forceinline__ void oc_wait(OcPos<C>& t, const float* bar, unsigned parity) {
-    if (t.dead) return;
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(bar);
     uint32_t ok = 0;
-    for (int k = 0; k < OC_POLLS && !ok; ++k)
-        asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}"
+#pragma unroll 1
+    for (int k = 0; k < t.polls && !ok; ++k)
+        asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}"
                      : "=r"(ok)
                      : "r"(a), "r"(parity)
                      : "memory");
-    if (!ok) t.dead = true;
+    if (!ok) t.polls = 0;
 }
-// After the pushes of an edge exchange (`bytes` from each neighbour): the block's own stores and the
-// neighbours' are visible.
+// The edge rows' part of an exchange: waits for the neighbour's values (`bytes` for the whole row).
 template <int C>
-__device__ __forceinline__ void nb_sync(float* sm, OcPos<C>& t, int bytes) {
-    if (C > 1 && t.tid == 0) oc_expect(nb_bar(sm, t), bytes * t.neighbours);
-    __syncthreads();
+__device__ __forceinline__ void nb_wait(float* sm, OcPos<C>& t, int bytes) {
     if (C > 1) {
-        oc_wait<C>(t, nb_bar(sm, t), (t.seq >> 1) & 1);
+        if (t.nbase) {
+            const float* bar = sm + nb_bar(t, t.lower);
+            if (t.tx == 0) oc_expect(bar, bytes);
+            oc_wait<C>(t, bar, (t.seq >> 1) & 1);
+        }
         ++t.seq;
     }
+}
+// After the stores of an edge exchange: the block's own are visible, and to the edge rows the neighbours'.
+template <int C>
+__device__ __forceinline__ void nb_sync(float* sm, OcPos<C>& t, int bytes) {
+    __syncthreads();
+    nb_wait<C>(sm, t, bytes);
 }
 // The same for an all-to-all exchange (`bytes` from all blocks together).
 template <int C>
@@ -171,7 +203,6 @@ __device__ __forceinline__ void all_sync(float* sm, OcPos<C>& t, int which, int 
         t.par ^= 1u << which;
     }
 }
-
 // The exchange that starts an iteration: |r|^2 and the first red edges.  True if a wait ran out in any thread
 // of the block, which then leaves the loops alike (threads must not decide on sums that others did not see).
 template <int C>
@@ -180,15 +211,11 @@ __device__ __forceinline__ bool rr_sync(float* sm, OcPos<C>& t) {
         __syncthreads();
         return false;
     }
-    if (t.tid == 0) {
-        oc_expect(nb_bar(sm, t), 128 * t.neighbours);
-        oc_expect(all_bar<C>(sm, OC_RR), 32 * OcMem<C>::CC);
-    }
-    oc_wait<C>(t, nb_bar(sm, t), (t.seq >> 1) & 1);
+    if (t.tid == 0) oc_expect(all_bar<C>(sm, OC_RR), 32 * OcMem<C>::CC);
+    nb_wait<C>(sm, t, 8 * OcMem<C>::W);
     oc_wait<C>(t, all_bar<C>(sm, OC_RR), (t.par >> OC_RR) & 1);
-    ++t.seq;
     t.par ^= 1u << OC_RR;
-    return __syncthreads_or(t.dead);
+    return __syncthreads_or(t.polls == 0);
 }
 
 // ---- sums over the particle's cells: every thread of every block ends with the same bits ----
@@ -224,41 +251,39 @@ __device__ __forceinline__ float red_get(const float* sm, const OcPos<C>& t, int
 }
 
 // ---- the finest level: a 4 x 4 patch, e[4 j + i] of cell (i, j); red: i + j even ----
-// Sides of colour col: W, E (rows of 17), S, N (17 rows of 16); the pair holds the side's two cells of
-// that colour in ascending order.
+// Sides of colour col: 0 W, 1 E (rows of W + 1), 2 S, 3 N (H + 1 rows of W); the pair holds the side's two
+// cells of that colour in ascending order.
 template <int C>
 __device__ __forceinline__ float2* side(float* sm, int s, int col) {
-    return reinterpret_cast<float2*>(sm + OcMem<C>::SIDE) + (s * 2 + col) * 272;
+    using M = OcMem<C>;
+    return reinterpret_cast<float2*>(sm + M::SIDE) + (s < 2 ? (s * 2 + col) * M::SZH : 4 * M::SZH + ((s - 2) * 2 + col) * M::SZV);
 }
 
 template <int C, int COL>
 __device__ __forceinline__ void pub_f(float* sm, const OcPos<C>& t, const float (&e)[16]) {
-    const float2 w = COL == 0 ? make_float2(e[0], e[8]) : make_float2(e[4], e[12]);
-    const float2 ea = COL == 0 ? make_float2(e[7], e[15]) : make_float2(e[3], e[11]);
+    using M = OcMem<C>;
     const float2 s = COL == 0 ? make_float2(e[0], e[2]) : make_float2(e[1], e[3]);
     const float2 n = COL == 0 ? make_float2(e[13], e[15]) : make_float2(e[12], e[14]);
-    float2 *W = side<C>(sm, 0, COL), *E = side<C>(sm, 1, COL), *S = side<C>(sm, 2, COL), *N = side<C>(sm, 3, COL);
-    W[t.ty * 17 + t.tx] = w;
-    E[t.ty * 17 + t.tx + 1] = ea;
-    S[t.ty * 16 + t.tx] = s;
-    N[(t.ty + 1) * 16 + t.tx] = n;
-    if (C > 1) {
-        const float* bar = nb_bar(sm, t);
-        if (t.tx == 0 && t.cx > 0) oc_push2(reinterpret_cast<float*>(W + t.ty * 17 + 16), t.rank - 1, w, bar);
-        if (t.tx == 15 && t.cx < C - 1) oc_push2(reinterpret_cast<float*>(E + t.ty * 17), t.rank + 1, ea, bar);
-        if (t.ty == 0 && t.cy > 0) oc_push2(reinterpret_cast<float*>(S + 16 * 16 + t.tx), t.rank - C, s, bar);
-        if (t.ty == 15 && t.cy < C - 1) oc_push2(reinterpret_cast<float*>(N + t.tx), t.rank + C, n, bar);
+    if (C > 1 && t.nbase) {
+        // to the neighbour's guard row: its north side's row 0 from below it, its south side's row H from above
+        const int at = 4 * M::SZH + (t.lower ? COL * M::SZV + M::H * M::W : (2 + COL) * M::SZV);
+        oc_store2(t.nbase + 4 * M::SIDE + 8 * (at + t.tx), t.lower ? s : n, t.nbase + 4 * nb_bar(t, !t.lower));
     }
+    side<C>(sm, 0, COL)[t.ty * (M::W + 1) + t.tx] = COL == 0 ? make_float2(e[0], e[8]) : make_float2(e[4], e[12]);
+    side<C>(sm, 1, COL)[t.ty * (M::W + 1) + t.tx + 1] = COL == 0 ? make_float2(e[7], e[15]) : make_float2(e[3], e[11]);
+    side<C>(sm, 2, COL)[t.ty * M::W + t.tx] = s;
+    side<C>(sm, 3, COL)[(t.ty + 1) * M::W + t.tx] = n;
 }
 
 struct HaloF { float2 w, e, s, n; };
 template <int C>
 __device__ __forceinline__ HaloF halo_f(float* sm, const OcPos<C>& t, int col) {   // the neighbours' cells of colour col
     HaloF h;
-    h.w = side<C>(sm, 1, col)[t.ty * 17 + t.tx];
-    h.e = side<C>(sm, 0, col)[t.ty * 17 + t.tx + 1];
-    h.s = side<C>(sm, 3, col)[t.ty * 16 + t.tx];
-    h.n = side<C>(sm, 2, col)[(t.ty + 1) * 16 + t.tx];
+    using M = OcMem<C>;
+    h.w = side<C>(sm, 1, col)[t.ty * (M::W + 1) + t.tx];
+    h.e = side<C>(sm, 0, col)[t.ty * (M::W + 1) + t.tx + 1];
+    h.s = side<C>(sm, 3, col)[t.ty * M::W + t.tx];
+    h.n = side<C>(sm, 2, col)[(t.ty + 1) * M::W + t.tx];
     return h;
 }
 __device__ __forceinline__ float pick(float2 v, int k) { return k ? v.y : v.x; }
@@ -302,31 +327,35 @@ __device__ __forceinline__ void sweep_f(float* sm, const OcPos<C>& t, const floa
 
 // ---- a level with a 2 x 2 patch per thread: cells 0 (0,0), 1 (1,0), 2 (0,1), 3 (1,1); red: 0 and 3 ----
 struct Patch2 { float w[6], s[6]; };   // west faces [j][0..2], south faces [0..2][i]
+// A thread's entry, pitch and plane size: the block's own planes (SHARED) or those of a local level.
+template <int C, bool SHARED> struct OcPl {
+    static constexpr int PT = SHARED ? OcMem<C>::PT : 18, PL = SHARED ? OcMem<C>::PL : 324;
+    static __device__ __forceinline__ int at(const OcPos<C>& t) { return SHARED ? (t.ty + 1) * PT + t.tx + 1 : (t.ly + 1) * PT + t.lx + 1; }
+};
 template <int C, bool SHARED>
-__device__ __forceinline__ void pub_h(float* sm, float* pl, const OcPos<C>& t, int col, const float (&e)[4]) {
-    const int at = (t.ty + 1) * 18 + t.tx + 1;
-    const int a = col ? 1 : 0, b = col ? 2 : 3;
-    pl[a * 324 + at] = e[col ? 1 : 0];
-    pl[b * 324 + at] = e[col ? 2 : 3];
-    if (SHARED && C > 1) {
-        const float* bar = nb_bar(sm, t);
-        if (t.tx == 0 && t.cx > 0) oc_push(pl + (col ? 2 : 0) * 324 + (t.ty + 1) * 18 + 17, t.rank - 1, col ? e[2] : e[0], bar);
-        if (t.tx == 15 && t.cx < C - 1) oc_push(pl + (col ? 1 : 3) * 324 + (t.ty + 1) * 18, t.rank + 1, col ? e[1] : e[3], bar);
-        if (t.ty == 0 && t.cy > 0) oc_push(pl + (col ? 1 : 0) * 324 + 17 * 18 + t.tx + 1, t.rank - C, col ? e[1] : e[0], bar);
-        if (t.ty == 15 && t.cy < C - 1) oc_push(pl + (col ? 2 : 3) * 324 + t.tx + 1, t.rank + C, col ? e[2] : e[3], bar);
+__device__ __forceinline__ void pub_h(float* pl, const OcPos<C>& t, int col, const float (&e)[4]) {
+    using O = OcPl<C, SHARED>;
+    if (SHARED && C > 1 && t.nbase) {   // cells 0, 1 (2, 3) to the block below (above), into its guard row
+        using M = OcMem<C>;
+        const int plane = t.lower ? (col ? 1 : 0) : (col ? 2 : 3);
+        oc_store(t.nbase + 4 * (M::HP + plane * M::PL + (t.lower ? (M::H + 1) * M::PT : 0) + t.tx + 1),
+                 t.lower ? (col ? e[1] : e[0]) : (col ? e[2] : e[3]), t.nbase + 4 * nb_bar(t, !t.lower));
     }
+    const int at = O::at(t);
+    pl[(col ? 1 : 0) * O::PL + at] = e[col ? 1 : 0];
+    pl[(col ? 2 : 3) * O::PL + at] = e[col ? 2 : 3];
 }
 // Sum of k e over the four neighbours of the two cells of a colour (0: cells 0 and 3, 1: cells 1 and 2).
-template <int C>
+template <int C, bool SHARED>
 __device__ __forceinline__ void nb_h(const float* pl, const OcPos<C>& t, int col, const Patch2& k, const float (&e)[4], float& a, float& b) {
-    const int at = (t.ty + 1) * 18 + t.tx + 1;
-    const float *p0 = pl + at, *p1 = p0 + 324, *p2 = p1 + 324, *p3 = p2 + 324;
+    using O = OcPl<C, SHARED>;
+    const float *p0 = pl + O::at(t), *p1 = p0 + O::PL, *p2 = p1 + O::PL, *p3 = p2 + O::PL;
     if (col == 0) {
-        a = fmaf(k.w[0], p1[-1], fmaf(k.s[0], p2[-18], fmaf(k.w[1], e[1], k.s[2] * e[2])));
-        b = fmaf(k.w[5], p2[1], fmaf(k.s[5], p1[18], fmaf(k.w[4], e[2], k.s[3] * e[1])));
+        a = fmaf(k.w[0], p1[-1], fmaf(k.s[0], p2[-O::PT], fmaf(k.w[1], e[1], k.s[2] * e[2])));
+        b = fmaf(k.w[5], p2[1], fmaf(k.s[5], p1[O::PT], fmaf(k.w[4], e[2], k.s[3] * e[1])));
     } else {
-        a = fmaf(k.w[2], p0[1], fmaf(k.s[1], p3[-18], fmaf(k.w[1], e[0], k.s[3] * e[3])));
-        b = fmaf(k.w[3], p3[-1], fmaf(k.s[4], p0[18], fmaf(k.w[4], e[3], k.s[2] * e[0])));
+        a = fmaf(k.w[2], p0[1], fmaf(k.s[1], p3[-O::PT], fmaf(k.w[1], e[0], k.s[3] * e[3])));
+        b = fmaf(k.w[3], p3[-1], fmaf(k.s[4], p0[O::PT], fmaf(k.w[4], e[3], k.s[2] * e[0])));
     }
 }
 __device__ __forceinline__ void diag_h(const Patch2& k, float (&d)[4]) {
@@ -340,24 +369,25 @@ __device__ __forceinline__ void diag_h(const Patch2& k, float (&d)[4]) {
 template <int C, bool SHARED>
 __device__ __forceinline__ float pre_h(float* sm, float* pl, OcPos<C>& t, int nu, const Patch2& k, const float4 inv, const float (&r)[4], float (&e)[4]) {
     float a, b;
+#pragma unroll 1
     for (int sw = 0; sw < nu; ++sw) {
         if (sw == 0) {
             e[0] = r[0] * inv.x;
             e[3] = r[3] * inv.w;
         } else {
-            nb_h<C>(pl, t, 0, k, e, a, b);
+            nb_h<C, SHARED>(pl, t, 0, k, e, a, b);
             e[0] = (r[0] + a) * inv.x;
             e[3] = (r[3] + b) * inv.w;
         }
-        pub_h<C, SHARED>(sm, pl, t, 0, e);
-        if (SHARED) nb_sync<C>(sm, t, 64); else __syncthreads();
-        nb_h<C>(pl, t, 1, k, e, a, b);
+        pub_h<C, SHARED>(pl, t, 0, e);
+        if (SHARED) nb_sync<C>(sm, t, 4 * OcMem<C>::W); else __syncthreads();
+        nb_h<C, SHARED>(pl, t, 1, k, e, a, b);
         e[1] = (r[1] + a) * inv.y;
         e[2] = (r[2] + b) * inv.z;
-        pub_h<C, SHARED>(sm, pl, t, 1, e);
-        if (SHARED) nb_sync<C>(sm, t, 64); else __syncthreads();
+        pub_h<C, SHARED>(pl, t, 1, e);
+        if (SHARED) nb_sync<C>(sm, t, 4 * OcMem<C>::W); else __syncthreads();
     }
-    nb_h<C>(pl, t, 0, k, e, a, b);
+    nb_h<C, SHARED>(pl, t, 0, k, e, a, b);
     float d[4];
     diag_h(k, d);
     return (r[0] + fmaf(-d[0], e[0], a)) + (r[3] + fmaf(-d[3], e[3], b));
@@ -366,15 +396,16 @@ __device__ __forceinline__ float pre_h(float* sm, float* pl, OcPos<C>& t, int nu
 template <int C, bool SHARED>
 __device__ __forceinline__ void post_h(float* sm, float* pl, OcPos<C>& t, int nu, const Patch2& k, const float4 inv, const float (&r)[4], float (&e)[4]) {
     float a, b;
+#pragma unroll 1
     for (int sw = 0; sw < nu; ++sw) {
-        pub_h<C, SHARED>(sm, pl, t, 0, e);
-        if (SHARED) nb_sync<C>(sm, t, 64); else __syncthreads();
-        nb_h<C>(pl, t, 1, k, e, a, b);
+        pub_h<C, SHARED>(pl, t, 0, e);
+        if (SHARED) nb_sync<C>(sm, t, 4 * OcMem<C>::W); else __syncthreads();
+        nb_h<C, SHARED>(pl, t, 1, k, e, a, b);
         e[1] = (r[1] + a) * inv.y;
         e[2] = (r[2] + b) * inv.z;
-        pub_h<C, SHARED>(sm, pl, t, 1, e);
-        if (SHARED) nb_sync<C>(sm, t, 64); else __syncthreads();
-        nb_h<C>(pl, t, 0, k, e, a, b);
+        pub_h<C, SHARED>(pl, t, 1, e);
+        if (SHARED) nb_sync<C>(sm, t, 4 * OcMem<C>::W); else __syncthreads();
+        nb_h<C, SHARED>(pl, t, 0, k, e, a, b);
         e[0] = (r[0] + a) * inv.x;
         e[3] = (r[3] + b) * inv.w;
     }
@@ -383,50 +414,53 @@ __device__ __forceinline__ void post_h(float* sm, float* pl, OcPos<C>& t, int nu
 // ---- a level with one cell per thread; red: tx + ty even ----
 struct Cell1 { float w, e, s, n; };
 template <int C, bool SHARED>
-__device__ __forceinline__ void pub_q(float* sm, float* pl, const OcPos<C>& t, float e) {
-    pl[(t.ty + 1) * 18 + t.tx + 1] = e;
-    if (SHARED && C > 1) {
-        const float* bar = nb_bar(sm, t);
-        if (t.tx == 0 && t.cx > 0) oc_push(pl + (t.ty + 1) * 18 + 17, t.rank - 1, e, bar);
-        if (t.tx == 15 && t.cx < C - 1) oc_push(pl + (t.ty + 1) * 18, t.rank + 1, e, bar);
-        if (t.ty == 0 && t.cy > 0) oc_push(pl + 17 * 18 + t.tx + 1, t.rank - C, e, bar);
-        if (t.ty == 15 && t.cy < C - 1) oc_push(pl + t.tx + 1, t.rank + C, e, bar);
+__device__ __forceinline__ void pub_q(float* pl, const OcPos<C>& t, float e) {
+    if (SHARED && C > 1 && t.nbase) {
+        using M = OcMem<C>;
+        oc_store(t.nbase + 4 * (M::QP + (t.lower ? (M::H + 1) * M::PT : 0) + t.tx + 1), e, t.nbase + 4 * nb_bar(t, !t.lower));
     }
+    pl[OcPl<C, SHARED>::at(t)] = e;
 }
-__device__ __forceinline__ float nb_q(const float* pl, int tx, int ty, const Cell1& k) {
-    const float* p = pl + (ty + 1) * 18 + tx + 1;
-    return fmaf(k.w, p[-1], fmaf(k.e, p[1], fmaf(k.s, p[-18], k.n * p[18])));
+template <int C, bool SHARED>
+__device__ __forceinline__ float nb_q(const float* pl, const OcPos<C>& t, const Cell1& k) {
+    using O = OcPl<C, SHARED>;
+    const float* p = pl + O::at(t);
+    return fmaf(k.w, p[-1], fmaf(k.e, p[1], fmaf(k.s, p[-O::PT], k.n * p[O::PT])));
 }
+template <int C, bool SHARED>
+__device__ __forceinline__ bool red_q(const OcPos<C>& t) { return ((SHARED ? t.tx + t.ty : t.lx + t.ly) & 1) == 0; }
 // Pre-smoothing from e = 0; returns the residual of a red cell, 0 for a black one.
 template <int C, bool SHARED>
 __device__ __forceinline__ float pre_q(float* sm, float* pl, OcPos<C>& t, int nu, const Cell1& k, float inv, float r, float& e) {
-    const bool red = ((t.tx + t.ty) & 1) == 0;
+    const bool red = red_q<C, SHARED>(t);
+#pragma unroll 1
     for (int sw = 0; sw < nu; ++sw) {
         if (red) {
-            e = (sw == 0 ? r : r + nb_q(pl, t.tx, t.ty, k)) * inv;
-            pub_q<C, SHARED>(sm, pl, t, e);
+            e = (sw == 0 ? r : r + nb_q<C, SHARED>(pl, t, k)) * inv;
+            pub_q<C, SHARED>(pl, t, e);
         }
-        if (SHARED) nb_sync<C>(sm, t, 32); else __syncthreads();
+        if (SHARED) nb_sync<C>(sm, t, 2 * OcMem<C>::W); else __syncthreads();
         if (!red) {
-            e = (r + nb_q(pl, t.tx, t.ty, k)) * inv;
-            pub_q<C, SHARED>(sm, pl, t, e);
+            e = (r + nb_q<C, SHARED>(pl, t, k)) * inv;
+            pub_q<C, SHARED>(pl, t, e);
         }
-        if (SHARED) nb_sync<C>(sm, t, 32); else __syncthreads();
+        if (SHARED) nb_sync<C>(sm, t, 2 * OcMem<C>::W); else __syncthreads();
     }
-    return red ? r + fmaf(-((k.w + k.e) + (k.s + k.n)), e, nb_q(pl, t.tx, t.ty, k)) : 0.f;
+    return red ? r + fmaf(-((k.w + k.e) + (k.s + k.n)), e, nb_q<C, SHARED>(pl, t, k)) : 0.f;
 }
 template <int C, bool SHARED>
 __device__ __forceinline__ void post_q(float* sm, float* pl, OcPos<C>& t, int nu, const Cell1& k, float inv, float r, float& e) {
-    const bool red = ((t.tx + t.ty) & 1) == 0;
+    const bool red = red_q<C, SHARED>(t);
+#pragma unroll 1
     for (int sw = 0; sw < nu; ++sw) {
-        if (red) pub_q<C, SHARED>(sm, pl, t, e);
-        if (SHARED) nb_sync<C>(sm, t, 32); else __syncthreads();
+        if (red) pub_q<C, SHARED>(pl, t, e);
+        if (SHARED) nb_sync<C>(sm, t, 2 * OcMem<C>::W); else __syncthreads();
         if (!red) {
-            e = (r + nb_q(pl, t.tx, t.ty, k)) * inv;
-            pub_q<C, SHARED>(sm, pl, t, e);
+            e = (r + nb_q<C, SHARED>(pl, t, k)) * inv;
+            pub_q<C, SHARED>(pl, t, e);
         }
-        if (SHARED) nb_sync<C>(sm, t, 32); else __syncthreads();
-        if (red) e = (r + nb_q(pl, t.tx, t.ty, k)) * inv;
+        if (SHARED) nb_sync<C>(sm, t, 2 * OcMem<C>::W); else __syncthreads();
+        if (red) e = (r + nb_q<C, SHARED>(pl, t, k)) * inv;
     }
 }
 
@@ -453,8 +487,8 @@ __device__ __forceinline__ void build_inv8(float* sm, const OcPos<C>& t, const C
     using M = OcMem<C>;
     float* M8 = sm + M::INV8;
     float* fa = M8;                                         // 4 x 64 faces first
-    if (((t.tx | t.ty) & 1) == 0) {
-        const int c = (t.ty >> 1) * 8 + (t.tx >> 1);
+    if (((t.lx | t.ly) & 1) == 0) {
+        const int c = (t.ly >> 1) * 8 + (t.lx >> 1);
         fa[c] = k8.w; fa[64 + c] = k8.e; fa[128 + c] = k8.s; fa[192 + c] = k8.n;
     }
     __syncthreads();
@@ -477,6 +511,7 @@ __device__ __forceinline__ void build_inv8(float* sm, const OcPos<C>& t, const C
     }
     __syncthreads();
     float* buf = M8;                                        // two buffers of (row 64, column 64)
+#pragma unroll 1
     for (int q0 = 0; q0 < 4; ++q0) {
 #pragma unroll
         for (int kk = 0; kk < 16; ++kk) {
@@ -514,7 +549,7 @@ template <int C, bool SHARED>
 __device__ __forceinline__ void level16(float* sm, float* pl, OcPos<C>& t, int nu, float cc, const Cell1& k, float inv, float r, float& e) {
     using M = OcMem<C>;
     const float res = quad_sum(pre_q<C, SHARED>(sm, pl, t, nu, k, inv, r, e));
-    if (((t.tx | t.ty) & 1) == 0) sm[M::R8 + (t.ty >> 1) * 8 + (t.tx >> 1)] = res;
+    if (((t.lx | t.ly) & 1) == 0) sm[M::R8 + (t.ly >> 1) * 8 + (t.lx >> 1)] = res;
     __syncthreads();
     {
         const int row = t.tid & 63, q = t.tid >> 6;
@@ -532,7 +567,7 @@ __device__ __forceinline__ void level16(float* sm, float* pl, OcPos<C>& t, int n
         sm[M::PART8 + 64 * q + row] = a + b;
     }
     __syncthreads();
-    const float* p8 = sm + M::PART8 + (t.ty >> 1) * 8 + (t.tx >> 1);
+    const float* p8 = sm + M::PART8 + (t.ly >> 1) * 8 + (t.lx >> 1);
     e = fmaf(cc, (p8[0] + p8[64]) + (p8[128] + p8[192]), e);
     post_q<C, SHARED>(sm, pl, t, nu, k, inv, r, e);
 }
@@ -563,22 +598,35 @@ __device__ __forceinline__ void tri_add(float& h, float& m, float& l, float x) {
     fast_two_sum(s, u, h, u2);
     fast_two_sum(u2, l2, m, l);
 }
-// a - b as df32 (exact to ~2^-47 of the difference of neighbouring values).
-__device__ __forceinline__ df32 tri_diff(float ah, float am, float al, float bh, float bm, float bl) {
+// The flux k (a - b) of a face as p + e: the difference to ~2^-70 |a| (hi rounded, lo the rest), p the
+// rounded product of the high parts, e its error and the products with the low parts.
+__device__ __forceinline__ df32 tri_flux(float kh, float kl, float ah, float am, float al, float bh, float bm, float bl) {
     float s, e, s2, e2, u, u2;
     two_sum(ah, -bh, s, e);
     two_sum(am, -bm, s2, e2);
     two_sum(s, s2, u, u2);
     const float low = __fadd_rn(__fadd_rn(u2, e), __fadd_rn(e2, __fsub_rn(al, bl)));
     df32 r;
-    fast_two_sum(u, low, r.hi, r.lo);
+    r.hi = __fmul_rn(kh, u);
+    r.lo = fmaf(kh, low, fmaf(kl, u, fmaf(kh, u, -r.hi)));
     return r;
+}
+// acc += f (TwoSum of the high parts, the rest in plain FP32: a compensated sum, error ~2^-47 of the terms).
+__device__ __forceinline__ void acc_add(df32& acc, float hi, float lo) {
+    float s, e;
+    two_sum(acc.hi, hi, s, e);
+    acc.hi = s;
+    acc.lo = __fadd_rn(acc.lo, __fadd_rn(e, lo));
+}
+// Parts outside the range of the integer form below (zeros, mostly).
+__device__ __noinline__ double tri_to_double_slow(float h, float m, float l, int add) {
+    return ((double)h + ((double)m + (double)l)) * exp2((double)add);
 }
 // (h + m + l) 2^add, rounded to FP64 with one integer conversion.
 __device__ __forceinline__ double tri_to_double(float h, float m, float l, int add) {
     const int bh = __float_as_int(h), bm = __float_as_int(m), bl = __float_as_int(l);
     const int eh = (bh >> 23) & 255, em = (bm >> 23) & 255, el = (bl >> 23) & 255;
-    if (eh < 64 || eh > 250) return ((double)h + ((double)m + (double)l)) * exp2((double)add);
+    if (eh < 64 || eh > 250) return tri_to_double_slow(h, m, l, add);
     auto mant = [](int b, int e) -> long long {
         const int v = e ? (b & 0x7fffff) | 0x800000 : 0;
         return (long long)(b < 0 ? -v : v);
@@ -602,12 +650,18 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     const int n = 64 * C;
     const int p = blockIdx.x / M::CC;
     OcPos<C> t;
-    t.tid = threadIdx.x; t.tx = t.tid & 15; t.ty = t.tid >> 4;
+    t.tid = threadIdx.x;
+    t.tx = t.tid % M::W; t.ty = t.tid / M::W;
+    t.lx = t.tid & 15; t.ly = t.tid >> 4;
     t.rank = C == 1 ? 0u : oc_rank();
-    t.cx = (int)t.rank % C; t.cy = (int)t.rank / C;
-    t.seq = 0; t.par = 0; t.dead = false;
-    t.neighbours = (t.cx > 0) + (t.cx < C - 1) + (t.cy > 0) + (t.cy < C - 1);
-    const int gx = 64 * t.cx + 4 * t.tx, gy = 64 * t.cy + 4 * t.ty;
+    t.seq = 0; t.par = 0; t.polls = OC_POLLS;
+    t.nbase = 0;
+    t.lower = t.ty == 0;
+    if (C > 1) {
+        if (t.ty == 0 && t.rank > 0) t.nbase = oc_map(sm, t.rank - 1);
+        if (t.ty == M::H - 1 && t.rank < M::CC - 1) t.nbase = oc_map(sm, t.rank + 1);
+    }
+    const int gx = 4 * t.tx, gy = 4 * ((int)t.rank * M::H + t.ty);
     const size_t base = (size_t)p * n * n;
     const double b2 = A.b2pp ? A.b2pp[p] : A.b2const;
     if (!(b2 > 0.0) || (A.badp && A.badp[p])) {             // not solved: w = 0 (the whole cluster alike)
@@ -626,7 +680,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     // guards and planes
     for (int i = M::SIDE + t.tid; i < M::BARS; i += OC_T) sm[i] = 0.f;
     if (C > 1 && t.tid == 0) {
-        for (int k = 0; k < 6; ++k)
+        for (int k = 0; k < 8; ++k)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(sm + M::BARS + 2 * k)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -668,31 +722,32 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
         diag_h(h, d);
         reinterpret_cast<float4*>(sm + M::INVH)[t.tid] = make_float4(1.f / d[0], 1.f / d[1], 1.f / d[2], 1.f / d[3]);
         const Cell1 k = coarsen_h(h);
-        sm[M::INVQ + t.tid] = 1.f / ((k.w + k.e) + (k.s + k.n));
-        const Cell1 kc = coarse_faces(k, t.tx, t.ty);
         oc_sync<C>();                                       // every block of the cluster runs: its shared memory may be written
         if (C == 1) {
-            build_inv8<C>(sm, t, kc);
+            build_inv8<C>(sm, t, coarse_faces(k, t.lx, t.ly));
         } else {
-            // gather the next level's faces in every block (through the inverse's storage)
-            constexpr int m = C * 8;
+            // gather the next level's faces in every block (through the inverse's storage): the block's part is formed
+            // where p will be, 4 values of H / 2 x W / 2 cells
+            constexpr int m = C * 8, part = (M::H / 2) * (M::W / 2), all = m * m;
+            float* st = sm + M::P4;
+            const float2 ws = make_float2(__shfl_xor_sync(0xffffffffu, k.s, 1) + k.s, __shfl_xor_sync(0xffffffffu, k.n, 1) + k.n);
+            st[t.tid] = k.w; st[OC_T + t.tid] = k.e; st[2 * OC_T + t.tid] = ws.x; st[3 * OC_T + t.tid] = ws.y;
+            __syncthreads();
             float* fb = sm + M::INV8;
-            const int cell = (t.cy * 8 + (t.ty >> 1)) * m + t.cx * 8 + (t.tx >> 1);
-            for (uint32_t d0 = (t.tx & 1) + 2 * (t.ty & 1); d0 < (uint32_t)M::CC; d0 += 4) {
-                const float* bar = all_bar<C>(sm, OC_GATHER);
-                oc_push(fb + cell, d0, kc.w, bar);
-                oc_push(fb + m * m + cell, d0, kc.e, bar);
-                oc_push(fb + 2 * m * m + cell, d0, kc.s, bar);
-                oc_push(fb + 3 * m * m + cell, d0, kc.n, bar);
+            for (int i = t.tid; i < 4 * part; i += OC_T) {
+                const int f = i / part, c = i % part, I = c % (M::W / 2), J = c / (M::W / 2);
+                const float* q = st + f * OC_T + 2 * J * M::W + 2 * I;
+                const float v = f == 0 ? q[0] + q[M::W] : f == 1 ? q[1] + q[M::W + 1] : f == 2 ? q[0] : q[M::W];
+                for (int d0 = 0; d0 < M::CC; ++d0) oc_push(fb + f * all + (int)t.rank * part + c, (uint32_t)d0, v, all_bar<C>(sm, OC_GATHER));
             }
-            all_sync<C>(sm, t, OC_GATHER, M::CC * 64 * 16);
+            all_sync<C>(sm, t, OC_GATHER, all * 16);
             Cell1 k16;
             if (C == 4) {
                 float* lf = sm + M::LF + t.tid;
                 Patch2 l;
 #pragma unroll
                 for (int J = 0; J < 2; ++J) {
-                    const int c = (2 * t.ty + J) * m + 2 * t.tx;
+                    const int c = (2 * t.ly + J) * m + 2 * t.lx;
                     l.w[3 * J] = fb[c]; l.w[3 * J + 1] = fb[c + 1]; l.w[3 * J + 2] = fb[m * m + c + 1];
                     l.s[2 * J] = fb[2 * m * m + c]; l.s[2 * J + 1] = fb[2 * m * m + c + 1];
                     if (J == 1) { l.s[4] = fb[3 * m * m + c]; l.s[5] = fb[3 * m * m + c + 1]; }
@@ -708,8 +763,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             }
             float* sf = sm + M::SF + t.tid;
             sf[0] = k16.w; sf[OC_T] = k16.e; sf[2 * OC_T] = k16.s; sf[3 * OC_T] = k16.n;
-            sf[4 * OC_T] = 1.f / ((k16.w + k16.e) + (k16.s + k16.n));
-            const Cell1 k8 = coarse_faces(k16, t.tx, t.ty);
+            const Cell1 k8 = coarse_faces(k16, t.lx, t.ly);
             __syncthreads();
             build_inv8<C>(sm, t, k8);
         }
@@ -727,6 +781,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     const size_t pb = (size_t)blockIdx.x * 4 * OC_T + t.tid;   // this thread's patch rows in x, wh, wm, wl
     int iters = 0, phases = 0, inner = 0;
     bool converged = false, wset = false;
+#pragma unroll 1
     for (int o = 0; o < A.max_outer; ++o) {
         // ---- CG on A x = r from x = 0 ----
         float thr = 0.f, rz = 0.f;
@@ -749,15 +804,16 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                 if (rr <= thr || iters >= A.maxit || !(rr == rr)) break;
             }
             // V-cycle: z = M r in e
+#pragma unroll 1
             for (int sw = 0; sw < A.nu_f; ++sw) {
                 if (sw > 0) {
                     sweep_f<C, 0>(sm, t, kw, ks, r, e, false);
                     pub_f<C, 0>(sm, t, e);
-                    nb_sync<C>(sm, t, 128);
+                    nb_sync<C>(sm, t, 8 * M::W);
                 }
                 sweep_f<C, 1>(sm, t, kw, ks, r, e, false);
                 pub_f<C, 1>(sm, t, e);
-                nb_sync<C>(sm, t, 128);
+                nb_sync<C>(sm, t, 8 * M::W);
             }
             float rh[4], eh[4];
             {
@@ -781,19 +837,29 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                 const Patch2 h = coarsen_f(kw, ks);
                 rq = pre_h<C, true>(sm, sm + M::HP, t, A.nu_c, h, invh, rh, eh);
                 const Cell1 k = coarsen_h(h);
-                const float invq = sm[M::INVQ + t.tid];
+                const float invq = 1.f / ((k.w + k.e) + (k.s + k.n));
                 float* QP = sm + M::QP;
                 if (C == 1) {
                     level16<C, true>(sm, QP, t, A.nu_c, A.cc, k, invq, rq, eq);
                 } else {
-                    const float rc = quad_sum(pre_q<C, true>(sm, QP, t, A.nu_c, k, invq, rq, eq));
-                    constexpr int m = C * 8;
-                    const int cell = (t.cy * 8 + (t.ty >> 1)) * m + t.cx * 8 + (t.tx >> 1);
-                    for (uint32_t d0 = (t.tx & 1) + 2 * (t.ty & 1); d0 < (uint32_t)M::CC; d0 += 4) oc_push(sm + M::RB + cell, d0, rc, all_bar<C>(sm, OC_GATHER));
-                    all_sync<C>(sm, t, OC_GATHER, M::CC * 64 * 4);
-                    const int px = t.cx * 8 + (t.tx >> 1), py = t.cy * 8 + (t.ty >> 1);   // the parent on the gathered level
+                    // the coarse right-hand side: pair sums per thread row, then four values per thread to one block each
+                    float rc = pre_q<C, true>(sm, QP, t, A.nu_c, k, invq, rq, eq);
+                    rc += __shfl_xor_sync(0xffffffffu, rc, 1);
+                    if ((t.tx & 1) == 0) sm[M::STG + t.ty * (M::W / 2) + (t.tx >> 1)] = rc;
+                    __syncthreads();
+                    constexpr int m = C * 8, part = (M::H / 2) * (M::W / 2);
+                    if (t.tid < M::CC * part / 4) {
+                        const int c = 4 * (t.tid % (part / 4)), J = c / (M::W / 2), I = c % (M::W / 2);
+                        const float4 u = *reinterpret_cast<const float4*>(sm + M::STG + 2 * J * (M::W / 2) + I);
+                        const float4 v = *reinterpret_cast<const float4*>(sm + M::STG + (2 * J + 1) * (M::W / 2) + I);
+                        oc_push4(sm + M::RB + (int)t.rank * part + c, (uint32_t)(t.tid / (part / 4)),
+                                 make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w), all_bar<C>(sm, OC_GATHER));
+                    }
+                    all_sync<C>(sm, t, OC_GATHER, m * m * 4);
+                    const int px = t.tx >> 1, py = (int)t.rank * (M::H / 2) + (t.ty >> 1);   // the parent on the gathered level
                     const float* sf = sm + M::SF + t.tid;
                     const Cell1 k16{sf[0], sf[OC_T], sf[2 * OC_T], sf[3 * OC_T]};
+                    const float inv16 = 1.f / ((k16.w + k16.e) + (k16.s + k16.n));
                     float e16, ep;
                     if (C == 4) {
                         const float* lf = sm + M::LF + t.tid;
@@ -801,22 +867,22 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
 #pragma unroll
                         for (int q = 0; q < 6; ++q) { l.w[q] = lf[q * OC_T]; l.s[q] = lf[(6 + q) * OC_T]; }
                         const float4 invl = make_float4(lf[12 * OC_T], lf[13 * OC_T], lf[14 * OC_T], lf[15 * OC_T]);
-                        const float* rb = sm + M::RB + 2 * t.ty * m + 2 * t.tx;
+                        const float* rb = sm + M::RB + 2 * t.ly * m + 2 * t.lx;
                         const float rl[4] = {rb[0], rb[1], rb[m], rb[m + 1]};
                         float el[4];
                         float* LP = sm + M::LP;
                         const float r16 = pre_h<C, false>(sm, LP, t, A.nu_c, l, invl, rl, el);
-                        level16<C, false>(sm, sm + M::SP, t, A.nu_c, A.cc, k16, sf[4 * OC_T], r16, e16);
+                        level16<C, false>(sm, sm + M::SP, t, A.nu_c, A.cc, k16, inv16, r16, e16);
 #pragma unroll
                         for (int c = 0; c < 4; ++c) el[c] = fmaf(A.cc, e16, el[c]);
                         post_h<C, false>(sm, LP, t, A.nu_c, l, invl, rl, el);
-                        pub_h<C, false>(sm, LP, t, 0, el);
+                        pub_h<C, false>(LP, t, 0, el);
                         __syncthreads();
                         ep = LP[((px & 1) + 2 * (py & 1)) * 324 + ((py >> 1) + 1) * 18 + (px >> 1) + 1];
                     } else {
                         float* SPl = sm + M::SP;
-                        level16<C, false>(sm, SPl, t, A.nu_c, A.cc, k16, sf[4 * OC_T], sm[M::RB + t.tid], e16);
-                        if (((t.tx + t.ty) & 1) == 0) SPl[(t.ty + 1) * 18 + t.tx + 1] = e16;
+                        level16<C, false>(sm, SPl, t, A.nu_c, A.cc, k16, inv16, sm[M::RB + t.tid], e16);
+                        if (((t.lx + t.ly) & 1) == 0) SPl[(t.ly + 1) * 18 + t.lx + 1] = e16;
                         __syncthreads();
                         ep = SPl[(py + 1) * 18 + px + 1];
                     }
@@ -831,12 +897,13 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             for (int j = 0; j < 4; ++j)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) e[4 * j + i] = fmaf(A.cc, eh[2 * (j >> 1) + (i >> 1)], e[4 * j + i]);
+#pragma unroll 1
             for (int sw = 0; sw < A.nu_f; ++sw) {
                 pub_f<C, 0>(sm, t, e);
-                nb_sync<C>(sm, t, 128);
+                nb_sync<C>(sm, t, 8 * M::W);
                 sweep_f<C, 1>(sm, t, kw, ks, r, e, false);
                 pub_f<C, 1>(sm, t, e);
-                nb_sync<C>(sm, t, 128);
+                nb_sync<C>(sm, t, 8 * M::W);
                 sweep_f<C, 0>(sm, t, kw, ks, r, e, false);
             }
             // beta, p = z + beta p
@@ -862,7 +929,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             for (int j = 0; j < 4; ++j) P4[j * OC_T] = make_float4(e[4 * j], e[4 * j + 1], e[4 * j + 2], e[4 * j + 3]);
             pub_f<C, 0>(sm, t, e);
             pub_f<C, 1>(sm, t, e);
-            nb_sync<C>(sm, t, 256);
+            nb_sync<C>(sm, t, 16 * M::W);
             // q = A p in flux form, p.q
             float q[16];
             s = 0.f;
@@ -926,8 +993,9 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             const float* W3[3] = {reinterpret_cast<const float*>(A.wh), reinterpret_cast<const float*>(A.wm), reinterpret_cast<const float*>(A.wl)};
             // patch rows of the neighbouring threads (another block of the cluster at the tile's edge)
             const size_t blk = 4 * OC_T;
-            const size_t pw = t.tx > 0 ? pb - 1 : pb - blk + 15, pe = t.tx < 15 ? pb + 1 : pb + blk - 15;
-            const size_t ps = t.ty > 0 ? pb - 16 : pb - C * blk + 240, pn = t.ty < 15 ? pb + 16 : pb + C * blk - 240;
+            const size_t pw = pb - 1, pe = pb + 1;
+            const size_t ps = t.ty > 0 ? pb - M::W : pb - blk + (M::H - 1) * M::W;
+            const size_t pn = t.ty < M::H - 1 ? pb + M::W : pb + blk - (M::H - 1) * M::W;
             const bool hw = gx > 0, he = gx + 4 < n, hs = gy > 0, hn = gy + 4 < n;
             float c3[3][4], f3[3][4];                           // this row, the row above or below
             df32 fs[4];
@@ -951,7 +1019,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                 const float k4[4] = {kl.x, kl.y, kl.z, kl.w};
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    fs[i] = df_mul(df32{ks[i], k4[i]}, tri_diff(c3[0][i], c3[1][i], c3[2][i], f3[0][i], f3[1][i], f3[2][i]));
+                    fs[i] = tri_flux(ks[i], k4[i], c3[0][i], c3[1][i], c3[2][i], f3[0][i], f3[1][i], f3[2][i]);
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -969,16 +1037,19 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                     if (hw) wv[q] = __ldcg(W3[q] + 4 * (pw + j * OC_T) + 3);
                     if (he) ev[q] = __ldcg(W3[q] + 4 * (pe + j * OC_T));
                 }
-                df32 fw = df_mul(df32{kw[5 * j], kwl[0]}, tri_diff(c3[0][0], c3[1][0], c3[2][0], wv[0], wv[1], wv[2]));
+                df32 fw = tri_flux(kw[5 * j], kwl[0], c3[0][0], c3[1][0], c3[2][0], wv[0], wv[1], wv[2]);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const df32 de = i < 3 ? tri_diff(c3[0][i + 1 & 3], c3[1][i + 1 & 3], c3[2][i + 1 & 3], c3[0][i], c3[1][i], c3[2][i])
-                                          : tri_diff(ev[0], ev[1], ev[2], c3[0][3], c3[1][3], c3[2][3]);
-                    const df32 fe = df_mul(df32{kw[5 * j + i + 1], kwl[i + 1]}, de);
-                    const df32 fn = df_mul(df32{ks[4 * j + 4 + i], ksl[i]}, tri_diff(f3[0][i], f3[1][i], f3[2][i], c3[0][i], c3[1][i], c3[2][i]));
-                    const df32 aw = df_add(df_add(fw, df_neg(fe)), df_add(fs[i], df_neg(fn)));
+                    const int i1 = (i + 1) & 3;
+                    const df32 fe = i < 3 ? tri_flux(kw[5 * j + i + 1], kwl[i + 1], c3[0][i1], c3[1][i1], c3[2][i1], c3[0][i], c3[1][i], c3[2][i])
+                                          : tri_flux(kw[5 * j + 4], kwl[4], ev[0], ev[1], ev[2], c3[0][3], c3[1][3], c3[2][3]);
+                    const df32 fn = tri_flux(ks[4 * j + 4 + i], ksl[i], f3[0][i], f3[1][i], f3[2][i], c3[0][i], c3[1][i], c3[2][i]);
                     const float2 bv = B[(size_t)(gy + j) * n + gx + i];
-                    const df32 rs = df_sub_acc(df32{bv.x * scale, bv.y * scale}, aw);
+                    df32 rs{bv.x * scale, bv.y * scale};
+                    acc_add(rs, -fw.hi, -fw.lo);
+                    acc_add(rs, fe.hi, fe.lo);
+                    acc_add(rs, -fs[i].hi, -fs[i].lo);
+                    acc_add(rs, fn.hi, fn.lo);
                     const float v = __fadd_rn(rs.hi, rs.lo);
                     r[4 * j + i] = v;
                     s = fmaf(v, v, s);
@@ -993,11 +1064,11 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
         }
         red_put<C>(sm, t, OC_RZ, s);
         all_sync<C>(sm, t, OC_RZ, 32 * M::CC);
-        if (C > 1 && __syncthreads_or(t.dead)) break;
+        if (C > 1 && __syncthreads_or(t.polls == 0)) break;
         const float res2 = red_get<C>(sm, t, OC_RZ);
         if (res2 <= A.tolout2 * b2s) { converged = true; break; }
     }
-#pragma unroll
+#pragma unroll 1
     for (int j = 0; j < 4; ++j) {
         const size_t at = pb + j * OC_T;
         const float4 h = A.wh[at], m = A.wm[at], l = A.wl[at];
@@ -1013,7 +1084,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
         if (!converged) atomicAdd(&g->nonconv, 1ull);
         atomicMax(&g->itmax, iters);
     }
-    if (C > 1 && t.dead) atomicExch(A.err, 1);
+    if (C > 1 && t.polls == 0) atomicExch(A.err, 1);
     if (C > 1) oc_sync<C>();                                    // no block leaves while another may still store into it
 }
 
@@ -1049,13 +1120,14 @@ static bool oc_fits() {
     return nc > 0;
 }
 
-// Whether the context's solves run on chip: mixed precision, the default tile kernels, a grid of
-// 64 C cells per side for the block grids above, and clusters of that size on this device.
+// Whether the context's solves run on chip: mixed precision, the default tile kernels, a grid of 64,
+// 128 or 256 cells per side (a 512^2 strip would not fit a cluster of 16; at each of the three this is
+// the faster solver from 2 particles to thousands), and clusters of that size on this device.
 bool onchip_supported(const Ctx& c) {
     if (c.dim != 2 || !mixed_precision(c.cfg) || c.cfg.tile_kernel != 0) return false;
     if (c.n == 64) return oc_fits<1>();
     if (c.n == 128) return oc_fits<2>();
-    // 256^2 in 4 x 4 blocks: 53.3 ms for 2048 solves against 55.2 in the multi-pass solver, not enough to switch
+    if (c.n == 256) return oc_fits<4>();
     return false;
 }
 
