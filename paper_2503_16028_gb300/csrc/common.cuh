@@ -71,12 +71,17 @@ __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;" :
 // GRID_SPINS polls the block sets *err and returns false, and the caller returns.  What
 // other blocks wrote before the barrier must be read with __ldcg (their L2 copies).
 constexpr unsigned GRID_SPINS = 1u << 23;
-__device__ inline bool grid_barrier(unsigned* count, unsigned target, int* err) {
-    __shared__ int ok;
+// The two halves of the barrier: work that needs no other block's results goes between them.
+__device__ inline void grid_arrive(unsigned* count) {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(count, 1u);
+    }
+}
+__device__ inline bool grid_wait(unsigned* count, unsigned target, int* err) {
+    __shared__ int ok;
+    if (threadIdx.x == 0) {
         unsigned seen = 0, spins = 0;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
@@ -87,6 +92,10 @@ __device__ inline bool grid_barrier(unsigned* count, unsigned target, int* err) 
     }
     __syncthreads();
     return ok != 0;
+}
+__device__ inline bool grid_barrier(unsigned* count, unsigned target, int* err) {
+    grid_arrive(count);
+    return grid_wait(count, target, err);
 }
 
 }  // namespace smcgm

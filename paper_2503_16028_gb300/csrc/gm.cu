@@ -70,26 +70,27 @@ __global__ void k_em_init(int N, int K, int r, EmPicks init, const double* __res
 // The pivot moves with the fit, so the subtraction loses nothing once the means settle
 // (|m - c|^2 << lambda), and a component's next iteration starts from the new mean.
 // A collapsed component (N_j < 2) is found by every block alike (same sums, same order).
-// Measured (r = 64, 50 iterations, ncu): N = 1024, K = 4 9.0 -> 1.20 ms, N = 256, K = 2 7.2 -> 1.02 ms
-// (what is left is the chain of FP64 latencies through an iteration, 20 us).
+// Measured (r = 64, 50 iterations, ncu): N = 1024, K = 4 9.0 -> 1.10 ms, N = 256, K = 2 7.2 -> 0.95 ms
+// (what is left is the chain of FP64 latencies through an iteration, 19 us: the FP64 pipe is 6 % busy).
 // ------------------------------------------------------------------------
 constexpr int EM_THREADS = 256;
 constexpr int EM_BLOCKS = 152;      // most blocks of the launch (rows of `part`)
 constexpr int EM_MINP = 8;          // least particles per block: fewer blocks make cheaper barriers
+constexpr int EM_SPLIT = 4;         // most groups of threads sharing the M-step sums' particles
 
 __host__ __device__ inline int em_pad(int r) { return ((r + 11) / 16) * 16 + 4; }   // >= r, 4 mod 16: rows of 4 s fall on other banks
 static size_t em_smem(int K, int r, int per, bool xs_in_smem) {
-    return sizeof(double) * ((size_t)2 * K * em_pad(r) + 2 * (size_t)K * per + 3 * (size_t)K + 40 +
+    return sizeof(double) * ((size_t)2 * K * em_pad(r) + 2 * (size_t)K * per + 3 * (size_t)K + 40 + 2 * EM_THREADS +
                              (xs_in_smem ? (size_t)per * em_pad(r) : 0));
 }
-size_t em_partial_doubles(int K, int r) { return (size_t)EM_BLOCKS * (2 * (size_t)K * r + K + 2) + 2 * (size_t)K * r; }
+size_t em_partial_doubles(int K, int r) { return 2 * (size_t)EM_BLOCKS * (2 * (size_t)K * r + K + 2) + (size_t)K * r; }
 
 struct EmArgs {
-    int N, K, r, iters;
+    int N, K, r, iters, lg_lanes;   // lanes per (particle, component) in the E-step: 2^lg_lanes
     double floor_frac;
     const double *xsT, *pooled, *lamS;
     double *w, *m, *lam;          // in: the initial mixture; out: the fitted one
-    double *part;                 // gridDim rows of (S1, S2: K r; N_j: K; min of gmax, its particle), then si, lg: K r each
+    double *part;                 // two buffers of gridDim rows (S1, S2: K r; N_j: K; min of gmax, its particle), then 1 / (2 lambda): K r
     double *loglik;
     unsigned* bar;
     int* err;
@@ -109,9 +110,10 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
     double* nj = cst + K;
     double* sw = nj + K;                   // weights
     double* red = sw + K;                  // 40
-    double* xs = red + 40;                 // [per][rp]
-    double* g_si = A.part + (size_t)G * row;
-    double* g_lg = g_si + Kr;
+    double* spl = red + 40;                // 2 EM_THREADS: the M-step sums of the second and later thread groups
+    double* xs = spl + 2 * EM_THREADS;     // [per][rp]
+    double* g_si = A.part + 2 * (size_t)G * row;
+    const int lanes = 1 << A.lg_lanes, split = max(1, min(EM_SPLIT, EM_THREADS / Kr));
     auto X = [&](int p, int s) -> double { return XS ? xs[(size_t)p * rp + s] : A.xsT[(size_t)s * N + n0 + p]; };
     if (XS)
         for (int t = tid; t < np * r; t += EM_THREADS) {
@@ -135,26 +137,25 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
         for (int j = tid; j < K; j += EM_THREADS) cst[j] = log(sw[j]) + red[32];
         __syncthreads();
     }
-    __shared__ double rs[2][8][8];
     unsigned arrivals = 0;
     for (int it = 0;; ++it) {
-        // log densities: four lanes per (particle, component)
+        // log densities: 2^lg_lanes lanes per (particle, component)
         const int items = np * K;
-        for (int base = 0; base < items * 4; base += EM_THREADS) {
-            const int item = (base + tid) >> 2, l4 = tid & 3;
+        for (int base = 0; base < items << A.lg_lanes; base += EM_THREADS) {
+            const int item = (base + tid) >> A.lg_lanes, ln = tid & (lanes - 1);
             const bool on = item < items;
             const int p = on ? item / K : 0, j = on ? item % K : 0;
             double acc = 0.0;
             if (on) {
                 const double *mj = sm + (size_t)j * rp, *ij = si + (size_t)j * rp;
-                for (int s = l4; s < r; s += 4) {
+#pragma unroll 4
+                for (int s = ln; s < r; s += lanes) {
                     const double e = X(p, s) - mj[s];
                     acc -= e * e * ij[s];
                 }
             }
-            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-            acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-            if (on && l4 == 0) lp[(size_t)j * per + p] = acc + cst[j];
+            for (int o = lanes >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (on && ln == 0) lp[(size_t)j * per + p] = acc + cst[j];
         }
         __syncthreads();
         for (int t = tid; t < items; t += EM_THREADS) {
@@ -173,11 +174,12 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
                 a += mx + log(sum);
             }
             a = block_sum(a, red);
-            if (tid == 0) A.part[(size_t)b * row] = a;
+            double* fin = A.part + (size_t)(it & 1) * G * row;
+            if (tid == 0) fin[(size_t)b * row] = a;
             if (!grid_barrier(A.bar, arrivals += G, A.err)) return;
             if (b == 0) {
                 a = 0.0;
-                for (int k = tid; k < G; k += EM_THREADS) a += __ldcg(&A.part[(size_t)k * row]);
+                for (int k = tid; k < G; k += EM_THREADS) a += __ldcg(&fin[(size_t)k * row]);
                 a = block_sum(a, red);
                 if (tid == 0) *A.loglik = a;
                 for (int j = tid; j < K; j += EM_THREADS) A.w[j] = sw[j];
@@ -186,31 +188,49 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
         }
         double gmin = 1.0 / 0.0;           // least max_j g of the block's particles, lowest index on ties
         int imin = N;
-        for (int p = tid; p < np; p += EM_THREADS) {
-            double mx = -1.0 / 0.0, sum = 0.0;
-            for (int q = 0; q < K; ++q) mx = fmax(mx, lp[(size_t)q * per + p]);
-            for (int q = 0; q < K; ++q) sum += ex[(size_t)q * per + p];
-            ex[p] = mx + log(sum);         // row 0: read above by this thread alone
-        }
-        __syncthreads();
-        for (int t = tid; t < items; t += EM_THREADS) {
+        for (int t = tid; t < items; t += EM_THREADS) {   // responsibilities
             const int j = t / np, p = t % np;
-            lp[(size_t)j * per + p] = exp(lp[(size_t)j * per + p] - ex[p]);
+            double sum = 0.0;
+            for (int q = 0; q < K; ++q) sum += ex[(size_t)q * per + p];
+            lp[(size_t)j * per + p] = ex[(size_t)j * per + p] / sum;
         }
         __syncthreads();
-        double* out = A.part + (size_t)b * row;
-        for (int t = tid; t < Kr; t += EM_THREADS) {
-            const int j = t / r, s = t % r;
-            const double c = sm[(size_t)j * rp + s];
-            const double* g = lp + (size_t)j * per;
+        double* part = A.part + (size_t)(it & 1) * G * row;   // the other buffer may still be read
+        double* out = part + (size_t)b * row;
+        if (split > 1) {                   // few pairs: groups of Kr threads share the particles
+            const int h = tid / Kr, q = tid % Kr, j = q / r, s = q % r;
             double s1 = 0.0, s2 = 0.0;
-            for (int p = 0; p < np; ++p) {
-                const double e = X(p, s) - c, ge = g[p] * e;
-                s1 += ge;
-                s2 = fma(ge, e, s2);
+            if (h < split) {
+                const double c = sm[(size_t)j * rp + s];
+                const double* g = lp + (size_t)j * per;
+                for (int p = h; p < np; p += split) {
+                    const double e = X(p, s) - c, ge = g[p] * e;
+                    s1 += ge;
+                    s2 = fma(ge, e, s2);
+                }
+                spl[tid] = s1;
+                spl[EM_THREADS + tid] = s2;
             }
-            out[t] = s1;
-            out[Kr + t] = s2;
+            __syncthreads();
+            if (h == 0) {
+                for (int k = 1; k < split; ++k) { s1 += spl[k * Kr + q]; s2 += spl[EM_THREADS + k * Kr + q]; }
+                out[q] = s1;
+                out[Kr + q] = s2;
+            }
+        } else {
+            for (int t = tid; t < Kr; t += EM_THREADS) {
+                const int j = t / r, s = t % r;
+                const double c = sm[(size_t)j * rp + s];
+                const double* g = lp + (size_t)j * per;
+                double s1 = 0.0, s2 = 0.0;
+                for (int p = 0; p < np; ++p) {
+                    const double e = X(p, s) - c, ge = g[p] * e;
+                    s1 += ge;
+                    s2 = fma(ge, e, s2);
+                }
+                out[t] = s1;
+                out[Kr + t] = s2;
+            }
         }
         for (int j = tid >> 5; j < K; j += EM_THREADS / 32) {
             double a = 0.0;
@@ -234,82 +254,94 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
             if (tid == 0) { out[2 * Kr + K] = gmin; out[2 * Kr + K + 1] = (double)imin; }
         }
         if (!grid_barrier(A.bar, arrivals += G, A.err)) return;
-        // N_j and the weights (every block alike)
-        for (int j = tid >> 5; j < K; j += EM_THREADS / 32) {
+        // this block's slice of the pairs, a warp per pair (and N_j alike in every warp that needs it)
+        const int lo = (int)((size_t)Kr * b / G), hi = (int)((size_t)Kr * (b + 1) / G), lane = tid & 31, wid = tid >> 5;
+        auto nj_of = [&](int j) {
             double a = 0.0;
-            for (int k = tid & 31; k < G; k += 32) a += __ldcg(&A.part[(size_t)k * row + 2 * Kr + j]);
+            for (int k = lane; k < G; k += 32) a += __ldcg(&part[(size_t)k * row + 2 * Kr + j]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if ((tid & 31) == 0) nj[j] = a;
-        }
-        __syncthreads();
-        bool low = false;
-        for (int j = 0; j < K; ++j) low |= nj[j] < 2.0;
-        int star = 0;
-        if (low) {                          // rare: the particle with the lowest max_j g
-            double bg = 1.0 / 0.0;
-            double bi = (double)N;
-            for (int k = 0; k < G; ++k) {
-                const double vg = __ldcg(&A.part[(size_t)k * row + 2 * Kr + K]), vi = __ldcg(&A.part[(size_t)k * row + 2 * Kr + K + 1]);
-                if (vg < bg || (vg == bg && vi < bi)) { bg = vg; bi = vi; }
+            return a;
+        };
+        for (int q = lo + wid; q < hi; q += EM_THREADS / 32) {
+            const int j = q / r, s = q % r;
+            double s1 = 0.0, s2 = 0.0, n = 0.0;
+            for (int k = lane; k < G; k += 32) {
+                const double* pr = part + (size_t)k * row;
+                s1 += __ldcg(&pr[q]);
+                s2 += __ldcg(&pr[Kr + q]);
+                n += __ldcg(&pr[2 * Kr + j]);
             }
-            star = (int)bi;
-        }
-        if (tid == 0) {
-            double tot = 0.0;
-            for (int j = 0; j < K; ++j) { sw[j] = nj[j] < 2.0 ? 1.0 / N : nj[j] / N; tot += sw[j]; }
-            for (int j = 0; j < K; ++j) sw[j] = sw[j] / tot;
-        }
-        // this block's slice of the pairs: 8 pairs at a time, 32 threads adding a pair's rows
-        const int lo = (int)((size_t)Kr * b / G), hi = (int)((size_t)Kr * (b + 1) / G);
-        for (int q0 = lo; q0 < hi; q0 += 8) {
-            const int q = q0 + (tid & 7), bl = tid >> 3;
-            double s1 = 0.0, s2 = 0.0;
-            if (q < hi)
-                for (int k = bl; k < G; k += 32) {
-                    s1 += __ldcg(&A.part[(size_t)k * row + q]);
-                    s2 += __ldcg(&A.part[(size_t)k * row + Kr + q]);
-                }
 #pragma unroll
-            for (int o = 16; o >= 8; o >>= 1) {
+            for (int o = 16; o > 0; o >>= 1) {
                 s1 += __shfl_xor_sync(0xffffffffu, s1, o);
                 s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+                n += __shfl_xor_sync(0xffffffffu, n, o);
             }
-            __syncthreads();
-            if ((tid & 31) < 8) { rs[0][tid >> 5][tid & 7] = s1; rs[1][tid >> 5][tid & 7] = s2; }
-            __syncthreads();
-            if (tid < 8 && q < hi) {
-                s1 = 0.0; s2 = 0.0;
-                for (int k = 0; k < 8; ++k) { s1 += rs[0][k][tid]; s2 += rs[1][k][tid]; }
-                const int j = q / r, s = q % r;
-                double mv, lv;
-                if (nj[j] < 2.0) {
-                    mv = A.xsT[(size_t)s * N + star];
-                    lv = A.pooled[s];
-                } else {
-                    const double dm = s1 / nj[j];
-                    mv = sm[(size_t)j * rp + s] + dm;
-                    lv = fmax(s2 / nj[j] - dm * dm, A.floor_frac * A.lamS[s]);
+            double mv, lv;
+            if (n < 2.0) {                  // rare: re-seeded at the particle with the lowest max_j g
+                double bg = 1.0 / 0.0, bi = (double)N;
+                for (int k = 0; k < G; ++k) {
+                    const double vg = __ldcg(&part[(size_t)k * row + 2 * Kr + K]), vi = __ldcg(&part[(size_t)k * row + 2 * Kr + K + 1]);
+                    if (vg < bg || (vg == bg && vi < bi)) { bg = vg; bi = vi; }
                 }
+                mv = A.xsT[(size_t)s * N + (int)bi];
+                lv = A.pooled[s];
+            } else {
+                const double dm = s1 / n;
+                mv = sm[(size_t)j * rp + s] + dm;
+                lv = fmax(s2 / n - dm * dm, A.floor_frac * A.lamS[s]);
+            }
+            if (lane == 0) {
                 A.m[q] = mv;
                 A.lam[q] = lv;
                 g_si[q] = 1.0 / (2.0 * lv);
-                g_lg[q] = -0.5 * log(2.0 * M_PI * lv);
             }
         }
-        if (!grid_barrier(A.bar, arrivals += G, A.err)) return;
+        // while the other blocks arrive: N_j, the weights and their logarithms (every block alike)
+        grid_arrive(A.bar);
+        for (int j = wid; j < K; j += EM_THREADS / 32) {
+            const double a = nj_of(j);
+            if (lane == 0) nj[j] = a;
+        }
+        __syncthreads();
+        if (tid < K) {
+            double tot = 0.0;
+            for (int j = 0; j < K; ++j) tot += nj[j] < 2.0 ? 1.0 / N : nj[j] / N;
+            const double w = (nj[tid] < 2.0 ? 1.0 / N : nj[tid] / N) / tot;
+            sw[tid] = w;
+            cst[tid] = log(w) - 0.5 * r * log(2.0 * M_PI);
+        }
+        if (!grid_wait(A.bar, arrivals += G, A.err)) return;
         for (int t = tid; t < Kr; t += EM_THREADS) {
             const int j = t / r, s = t % r;
             sm[(size_t)j * rp + s] = __ldcg(&A.m[t]);
             si[(size_t)j * rp + s] = __ldcg(&g_si[t]);
         }
-        for (int j = tid >> 5; j < K; j += EM_THREADS / 32) {
-            double a = 0.0;
-            for (int s = tid & 31; s < r; s += 32) a += __ldcg(&g_lg[(size_t)j * r + s]);
+        // sum_s log lambda_js as one logarithm per component: the product of the mantissas (in [1, 2), at most 256 of
+        // them: no overflow) and the sum of the exponents
+        for (int j = wid; j < K; j += EM_THREADS / 32) {
+            double prod = 1.0;
+            int ex2 = 0;
+            for (int s = lane; s < r; s += 32) {
+                const double v = __ldcg(&A.lam[(size_t)j * r + s]);
+                const int hi2 = __double2hiint(v), e = (hi2 >> 20) & 0x7ff;
+                if (e > 0 && e < 0x7ff) {
+                    prod *= __hiloint2double((hi2 & 0x800fffff) | 0x3ff00000, __double2loint(v));
+                    ex2 += e - 1023;
+                } else {
+                    prod *= v;               // zero, denormal, infinity, NaN
+                }
+            }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if ((tid & 31) == 0) cst[j] = log(sw[j]) + a;
+            for (int o = 16; o > 0; o >>= 1) {
+                prod *= __shfl_xor_sync(0xffffffffu, prod, o);
+                ex2 += __shfl_xor_sync(0xffffffffu, ex2, o);
+            }
+            if (lane == 0) { spl[j] = prod; spl[MAXK + j] = (double)ex2; }
         }
+        __syncthreads();
+        if (tid < K) cst[tid] -= 0.5 * (log(spl[tid]) + M_LN2 * spl[MAXK + tid]);
         __syncthreads();
     }
 }
@@ -336,9 +368,9 @@ __global__ void k_sum(int N, const double* __restrict__ a, double* __restrict__ 
 // An iteration is k_chol, k_estep_full, k_resp, k_cov_acc, k_cov_finish.  The E-step and the
 // contraction are N K r^2 / 2 FP64 multiply-adds each (108 us at N = 4096, K = 8, r = 64 on the
 // FP64 pipes), everything else should stay small beside them.  Measured per 50-iteration fit
-// there: 70.2 -> 22.3 ms (one block per particle reading rows of L^-1 uncoalesced 631 -> 149 us,
-// the factor with its column sums in global memory 416 -> 79 us, the contraction on 32 x 32
-// tiles 292 -> 173 us).
+// there: 70.2 -> 22 ms (one block per particle reading rows of L^-1 uncoalesced 631 -> 150 us, FP64
+// pipe 76 % busy; the factor with its column sums in global memory 416 -> 79 us; the contraction on
+// 32 x 32 tiles 292 -> 173 us, FP64 pipe 87 %).
 // ------------------------------------------------------------------------
 
 // Rows in blocks of four: block I holds L[4I + q][k] at 8 I (I + 1) + 4 k + q, k < 4 I + 4, with
@@ -355,36 +387,66 @@ size_t cov_lb_doubles(int K, int r) { return (size_t)K * lb_size(r) + K; }
 // as 1 so the rest stays finite.  cst_j = log w_j - r/2 log(2 pi) - log det L_j when w is given.
 // Bound by the FP64 pipe of one SM (r^3 / 6 multiply-adds, 11 us at r = 64) and 2 r barriers.
 constexpr int CHOL_SMEM_R = 160;
+
+// 1 / d for a positive normal d to ~1 ulp: the hardware's approximate FP64 reciprocal (full exponent range) and two
+// Newton steps, half the latency of a rounded division.
+__device__ __forceinline__ double rcp_newton(double d) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    y = fma(y, fma(-d, y, 1.0), y);
+    return fma(y, fma(-d, y, 1.0), y);
+}
+template <bool SMEM>
 __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ cov, const double* __restrict__ w, double* __restrict__ L,
                                               double* __restrict__ Lb, double* __restrict__ logdet, double* __restrict__ cst,
                                               int* __restrict__ bad) {
     extern __shared__ __align__(16) double chsm[];
-    __shared__ double T[MAXR], rs[MAXR], red[32];
+    __shared__ double T[MAXR], rs[MAXR], red[32], s_rinv;
     const int j = blockIdx.x, tid = threadIdx.x;
     const size_t rr = (size_t)r * r;
     const double* A = cov + j * rr;
     double* Lj = L + j * rr;
-    const bool in_smem = r <= CHOL_SMEM_R;
-    double* Wk = in_smem ? chsm : Lj;
-    const int ws = in_smem ? r + 1 : r;
+    double* Wk = SMEM ? chsm : Lj;
+    const int ws = SMEM ? r + 1 : r;
     for (int e = tid; e < (int)rr; e += 256) {
         const int i = e / r, c = e % r;
-        if (c <= i) Wk[(size_t)i * ws + c] = A[e];
+        if (c <= i) Wk[i * ws + c] = A[e];
     }
     __syncthreads();
     const int tx = tid & 15, ty = tid >> 4;
-    for (int k = 0; k < r; ++k) {
-        double d = Wk[(size_t)k * ws + k];
+    // the pivot's reciprocal is formed by the thread that finishes it, while the others update
+    auto pivot = [&](double d, int k) {
         if (!(d > 0.0)) {
             d = 1.0;
-            if (tid == 0) atomicExch(bad, 1);
+            atomicExch(bad, 1);
         }
-        if (k + 1 + tid < r) T[k + 1 + tid] = Wk[(size_t)(k + 1 + tid) * ws + k] / d;   // r <= 256 = the threads
-        if (tid == 0) rs[k] = d;
+        rs[k] = d;
+        s_rinv = rcp_newton(d);
+    };
+    if (tid == 0) pivot(Wk[0], 0);
+    __syncthreads();
+    for (int k = 0; k < r; ++k) {
+        if (k + 1 + tid < r) T[k + 1 + tid] = Wk[(k + 1 + tid) * ws + k] * s_rinv;   // r <= 256 = the threads
         __syncthreads();
-        for (int i = k + 1 + ty; i < r; i += 16) {
-            const double wi = Wk[(size_t)i * ws + k];
-            for (int c = k + 1 + tx; c <= i; c += 16) Wk[(size_t)i * ws + c] -= wi * T[c];
+        if (tid == 0 && k + 1 < r) {                      // the next pivot first
+            const double v = fma(-Wk[(k + 1) * ws + k], T[k + 1], Wk[(k + 1) * ws + k + 1]);
+            Wk[(k + 1) * ws + k + 1] = v;
+            pivot(v, k + 1);
+        }
+        // rows from the longest down, four of a thread's elements at a time
+        for (int c0 = k + 1 + tx; c0 < r; c0 += 16) {
+            const double tc = T[c0];
+            int i = c0 + ((ty - c0) & 15);                // the first row >= c0 of this thread's rows (ty mod 16)
+            for (; i + 48 < r; i += 64) {
+                double w[4], v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) { w[q] = Wk[(i + 16 * q) * ws + k]; v[q] = Wk[(i + 16 * q) * ws + c0]; }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (q > 0 || i != k + 1) Wk[(i + 16 * q) * ws + c0] = fma(-w[q], tc, v[q]);
+            }
+            for (; i < r; i += 16)
+                if (i != k + 1) Wk[i * ws + c0] = fma(-Wk[i * ws + k], tc, Wk[i * ws + c0]);
         }
         __syncthreads();
     }
@@ -408,7 +470,7 @@ __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ 
         if (c > (i | 3)) continue;
         double v = 0.0;
         if (c == i) v = i < r ? rs[i] : 1.0;
-        else if (c < i && i < r) v = Wk[(size_t)i * ws + c] * rs[c];
+        else if (c < i && i < r) v = Wk[i * ws + c] * rs[c];
         Lbj[8 * (i >> 2) * ((i >> 2) + 1) + 4 * c + (i & 3)] = v;
     }
     __syncthreads();
@@ -416,7 +478,7 @@ __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ 
         const int i = e / r, c = e % r;
         double v = 0.0;
         if (c == i) v = T[i];
-        else if (c < i) v = Wk[(size_t)i * ws + c] * rs[c];
+        else if (c < i) v = Wk[i * ws + c] * rs[c];
         Lj[e] = v;                            // in place when the work array is L_j itself
     }
 }
@@ -600,34 +662,42 @@ __global__ void __launch_bounds__(256) k_cov_finish(int N, int K, int r, int nch
                                                     const double* __restrict__ xsT, const double* __restrict__ pooled,
                                                     const double* __restrict__ lamS, double floor_frac, double* __restrict__ w,
                                                     double* __restrict__ m, double* __restrict__ lam, double* __restrict__ cov) {
+    // four threads per element (and per mode, component) share the chunks
     __shared__ double dm[MAXR], s_nj[MAXK], s_v[256];
     __shared__ int s_i[256];
-    const int j = blockIdx.y, tid = threadIdx.x, T = cov_tiles(r);
+    const int j = blockIdx.y, tid = threadIdx.x, T = cov_tiles(r), cg = tid >> 6, el = tid & 63;
     const size_t row = cov_row(r);
     const double* pj = part + (size_t)j * nch * row;
-    if (tid < K) {
+    auto chunk_sum = [&](const double* p0, bool on) {       // the sum over the chunks of p0[c * row], in the first 64 threads
         double a = 0.0;
-        for (int c = 0; c < nch; ++c) a += part[((size_t)tid * nch + c) * row + (size_t)T * 16 + r];
-        s_nj[tid] = a;
+        if (on)
+#pragma unroll 5
+            for (int c = cg; c < nch; c += 4) a += p0[c * row];
+        __syncthreads();
+        s_v[tid] = a;
+        __syncthreads();
+        return (s_v[el] + s_v[64 + el]) + (s_v[128 + el] + s_v[192 + el]);
+    };
+    {
+        const double a = chunk_sum(part + (size_t)min(el, K - 1) * nch * row + (size_t)T * 16 + r, el < K);
+        if (tid < K) s_nj[tid] = a;
+        __syncthreads();
     }
-    double sum1 = 0.0;
-    if (tid < r)
-        for (int c = 0; c < nch; ++c) sum1 += pj[c * row + (size_t)T * 16 + tid];
-    __syncthreads();
     const double nj = s_nj[j];
     const bool low = nj < 2.0;
-    if (tid < r) dm[tid] = sum1 / nj;
-    __syncthreads();
-    const size_t e = (size_t)blockIdx.x * 256 + tid;
-    if (e < (size_t)T * 16) {
+    for (int m0 = 0; m0 < r; m0 += 64) {
+        const double a = chunk_sum(pj + (size_t)T * 16 + m0 + el, m0 + el < r);
+        if (tid < 64 && m0 + tid < r) dm[m0 + tid] = a / nj;
+    }
+    const size_t e = (size_t)blockIdx.x * 64 + el;
+    const double s = chunk_sum(pj + e, e < (size_t)T * 16);
+    if (tid < 64 && e < (size_t)T * 16) {
         const int t = (int)(e >> 4), q = (int)(e & 15);
         int ta = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
         while (ta * (ta + 1) / 2 > t) --ta;
         while ((ta + 1) * (ta + 2) / 2 <= t) ++ta;
         const int a = 4 * ta + (q >> 2), b = 4 * (t - ta * (ta + 1) / 2) + (q & 3);
         if (a < r && b <= a) {
-            double s = 0.0;
-            for (int c = 0; c < nch; ++c) s += pj[c * row + e];
             double v = s / nj - dm[a] * dm[b] + (a == b ? floor_frac * lamS[a] : 0.0);
             if (low) v = a == b ? pooled[a] : 0.0;
             cov[((size_t)j * r + a) * r + b] = v;
@@ -636,6 +706,7 @@ __global__ void __launch_bounds__(256) k_cov_finish(int N, int K, int r, int nch
         }
     }
     if (blockIdx.x != 0) return;
+    __syncthreads();
     if (low) {
         double best = 1.0 / 0.0;
         int bi = N;
@@ -671,10 +742,14 @@ static int* factor_flag(Ctx& c) { return c.icount + 40; }
 
 // L_j, log det L_j and the blocked rows of every C_j; with w also the E-step's constants.
 static void launch_chol(Ctx& c, bool estep_constants) {
-    const size_t sm = c.r <= CHOL_SMEM_R ? sizeof(double) * (size_t)c.r * (c.r + 1) : 0;
-    check(cudaFuncSetAttribute(k_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * CHOL_SMEM_R * (CHOL_SMEM_R + 1))), "attr");
-    k_chol<<<c.K, 256, sm, c.stream>>>(c.r, c.gcov, c.gw, c.gL, c.gLb, c.glogdet,
-                                       estep_constants ? c.gLb + (size_t)c.K * lb_size(c.r) : nullptr, factor_flag(c)); ++c.pc.launches;
+    double* cst = estep_constants ? c.gLb + (size_t)c.K * lb_size(c.r) : nullptr;
+    if (c.r <= CHOL_SMEM_R) {
+        check(cudaFuncSetAttribute(k_chol<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * CHOL_SMEM_R * (CHOL_SMEM_R + 1))), "attr");
+        k_chol<true><<<c.K, 256, sizeof(double) * (size_t)c.r * (c.r + 1), c.stream>>>(c.r, c.gcov, c.gw, c.gL, c.gLb, c.glogdet, cst, factor_flag(c));
+    } else {
+        k_chol<false><<<c.K, 256, 0, c.stream>>>(c.r, c.gcov, c.gw, c.gL, c.gLb, c.glogdet, cst, factor_flag(c));
+    }
+    ++c.pc.launches;
     check(cudaGetLastError(), "factor launch");
 }
 
@@ -726,7 +801,7 @@ static void em_full(Ctx& c, const double* lamS, double* ll) {
         launch_chol(c, true);
         estep();
         k_cov_acc<<<dim3(tg, K, nch), 256, csm, c.stream>>>(N, r, c.xsT, c.resp, c.gmu, c.covpart);
-        k_cov_finish<<<dim3((cov_tiles(r) * 16 + 255) / 256, K), 256, 0, c.stream>>>(N, K, r, nch, c.covpart, c.gmax, c.xsT, c.pooled, lamS,
+        k_cov_finish<<<dim3((cov_tiles(r) * 16 + 63) / 64, K), 256, 0, c.stream>>>(N, K, r, nch, c.covpart, c.gmax, c.xsT, c.pooled, lamS,
                                                                                    c.cfg.var_floor, c.gw, c.gmu, c.glam, c.gcov);
         c.pc.launches += 2;
     }
@@ -741,11 +816,12 @@ static void em_full(Ctx& c, const double* lamS, double* ll) {
 static void em_diag(Ctx& c, const double* lamS, double* ll) {
     const int N = c.N, K = c.K, r = c.r;
     EmArgs A{};
-    A.N = N; A.K = K; A.r = r; A.iters = c.cfg.em_iters; A.floor_frac = c.cfg.var_floor;
+    A.N = N; A.K = K; A.r = r; A.iters = c.cfg.em_iters; A.lg_lanes = 2; A.floor_frac = c.cfg.var_floor;
     A.xsT = c.xsT; A.pooled = c.pooled; A.lamS = lamS; A.w = c.gw; A.m = c.gmu; A.lam = c.glam;
     A.part = c.empart; A.loglik = ll; A.bar = reinterpret_cast<unsigned*>(c.icount + 44); A.err = c.dev_err;
     const int G = std::max(1, std::min({EM_BLOCKS, c.sm_count, (N + EM_MINP - 1) / EM_MINP}));
     const int per = (N + G - 1) / G;
+    while (A.lg_lanes < 5 && (per * K << A.lg_lanes) < EM_THREADS) ++A.lg_lanes;   // the chain of FP64 latencies is what bounds small fits
     constexpr size_t LIMIT = 200 * 1024;
     const bool xs = em_smem(K, r, per, true) <= LIMIT;
     const size_t sm = em_smem(K, r, per, xs);

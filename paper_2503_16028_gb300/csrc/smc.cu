@@ -22,46 +22,48 @@ namespace smcgm {
 // cost is FP64 exponentials (some 30 FP64 operations each, and one SM's FP64 pipe does two lanes a
 // cycle), so one block took 2.0 ms for the 66 x 4096 exponentials of a tempering step and 3.5 ms
 // for 8192 particles, however fast its reductions, and resampling 8192 another 206 us.  Reweighting
-// and resampling 8192 particles of 1024 modes, as called: 3.85 -> 0.44 ms.
+// and resampling 8192 particles of 1024 modes, as called: 3.85 -> 0.41 ms.
 constexpr int SMC_BLOCKS = 152;
 constexpr int SMC_THREADS = 256;
-constexpr int TEMPER_MINP = 32;    // particles per block and round: 32 x 8 candidates, one exponential per thread
+constexpr int TEMPER_LEVELS = 4, TEMPER_C = 1 << TEMPER_LEVELS;   // decisions per round; candidates: one less, and 1 - t
+constexpr int TEMPER_MINP = SMC_THREADS / TEMPER_C;   // least particles per block: one exponential per thread and round
 
 static int smc_grid(int N, int per_block, int sms) {
     return std::max(1, std::min({SMC_BLOCKS, sms, (N + per_block - 1) / per_block}));
 }
-size_t smc_partial_doubles() { return 2 * SMC_BLOCKS * 16 + 2 * SMC_BLOCKS; }
+size_t smc_partial_doubles() { return 2 * SMC_BLOCKS * 2 * TEMPER_C + 2 * SMC_BLOCKS; }
 
-// Value v (of 16) of all blocks' partials, added in a fixed order; every thread of every block
-// gets the same 16 sums in `tot`.
-__device__ inline void sum_partials16(const double* part, int G, double* scr, double* tot) {
-    const int v = threadIdx.x & 15, ch = threadIdx.x >> 4;
+// Value v (of 2 TEMPER_C) of all blocks' partials, added in a fixed order; every thread of every block
+// gets the same sums in `tot`.
+__device__ inline void sum_partials(const double* part, int G, double* scr, double* tot) {
+    constexpr int V = 2 * TEMPER_C, CH = SMC_THREADS / V;
+    const int v = threadIdx.x % V, ch = threadIdx.x / V;
     double a = 0.0;
-    for (int g = ch; g < G; g += SMC_THREADS / 16) a += __ldcg(&part[(size_t)g * 16 + v]);
-    a += __shfl_xor_sync(0xffffffffu, a, 16);
+#pragma unroll 4
+    for (int g = ch; g < G; g += CH) a += __ldcg(&part[(size_t)g * V + v]);
     __syncthreads();
-    if ((threadIdx.x & 16) == 0) scr[(threadIdx.x >> 5) * 16 + v] = a;
+    scr[threadIdx.x] = a;
     __syncthreads();
-    if (threadIdx.x < 16) {
+    if (threadIdx.x < V) {
         a = 0.0;
-        for (int k = 0; k < SMC_THREADS / 32; ++k) a += scr[k * 16 + threadIdx.x];
+        for (int k = 0; k < CH; ++k) a += scr[k * V + threadIdx.x];
         tot[threadIdx.x] = a;
     }
     __syncthreads();
 }
 
-// Tempering.  The 64 bisection decisions are taken three at a time: a round evaluates the ESS at
-// the seven points that the next three halvings can visit (the same midpoints, formed the same
-// way) and then walks down, so 22 rounds of one barrier replace 64; the eighth lane of the first
-// round evaluates h = 1 - t.  More points per round cost more exponentials than the barriers saved.
+// Tempering.  The 64 bisection decisions are taken four at a time: a round evaluates the ESS at
+// the fifteen points that the next four halvings can visit (the same midpoints, formed the same
+// way) and then walks down, so 16 rounds of one barrier replace 64; the sixteenth lane of the first
+// round evaluates h = 1 - t.
 // out: [0] h, [1] ESS(h), [2] log Z increment, [3] new t
 __global__ void __launch_bounds__(SMC_THREADS) k_temper(int N, const double* __restrict__ phi, double t, double target,
                                                         double* __restrict__ logw, double* __restrict__ out, double* part, unsigned* bar,
                                                         int* err) {
-    __shared__ double red[32], scr[SMC_THREADS / 32 * 16], tot[16], cand[8];
+    __shared__ double red[32], scr[SMC_THREADS], tot[2 * TEMPER_C], cand[TEMPER_C + 1], ess[TEMPER_C];
     const int G = gridDim.x, tid = threadIdx.x;
     const int per = (N + G - 1) / G, n0 = min(N, (int)blockIdx.x * per), n1 = min(N, n0 + per);
-    double* pmin = part + 2 * SMC_BLOCKS * 16;
+    double* pmin = part + 2 * SMC_BLOCKS * 2 * TEMPER_C;
     unsigned arrivals = 0;
     double mn = 1.0 / 0.0;
     for (int i = n0 + tid; i < n1; i += SMC_THREADS) mn = fmin(mn, phi[i]);
@@ -76,55 +78,48 @@ __global__ void __launch_bounds__(SMC_THREADS) k_temper(int N, const double* __r
     const double phimin = tot[0];
     const double rest = 1.0 - t;
     double lo = 0.0, hi = rest, ess_lo = (double)N, h;
-    int done = 0;
     for (int round = 0;; ++round) {
-        const double c4 = 0.5 * (lo + hi), c2 = 0.5 * (lo + c4), c6 = 0.5 * (c4 + hi);
+        // cand[m], m = 1 .. 15: the midpoint of cand[m - s] and cand[m + s], s the lowest set bit of m (cand[0] = lo,
+        // cand[16] = hi), level by level as the halvings would form them; slot 0 then holds 1 - t
         __syncthreads();
         if (tid == 0) {
-            cand[0] = 0.5 * (lo + c2); cand[1] = c2; cand[2] = 0.5 * (c2 + c4); cand[3] = c4;
-            cand[4] = 0.5 * (c4 + c6); cand[5] = c6; cand[6] = 0.5 * (c6 + hi); cand[7] = rest;
+            cand[0] = lo;
+            cand[TEMPER_C] = hi;
+            for (int st = TEMPER_C / 2; st >= 1; st >>= 1)
+                for (int m = st; m < TEMPER_C; m += 2 * st) cand[m] = 0.5 * (cand[m - st] + cand[m + st]);
+            cand[0] = rest;
         }
         __syncthreads();
-        const int k = tid & 7;
-        const bool on = round == 0 || (done + 3 <= 64 ? k < 7 : k == 3);
+        const int k = tid % TEMPER_C;
         const double hk = cand[k];
         double s1 = 0.0, s2 = 0.0;
-        if (on)
-            for (int i = n0 + (tid >> 3); i < n1; i += SMC_THREADS / 8) {
+        if (round == 0 || k > 0)
+            for (int i = n0 + tid / TEMPER_C; i < n1; i += SMC_THREADS / TEMPER_C) {
                 const double e = exp(-hk * (phi[i] - phimin));
                 s1 += e;
                 s2 += e * e;
             }
-#pragma unroll
-        for (int o = 16; o >= 8; o >>= 1) {
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        }
-        if ((tid & 31) < 8) { scr[(tid >> 5) * 16 + k] = s1; scr[(tid >> 5) * 16 + 8 + k] = s2; }
+        s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, 16);
+        if ((tid & 31) < TEMPER_C) { scr[(tid >> 5) * 2 * TEMPER_C + k] = s1; scr[(tid >> 5) * 2 * TEMPER_C + TEMPER_C + k] = s2; }
         __syncthreads();
-        double* pr = part + (size_t)(round & 1) * SMC_BLOCKS * 16;   // the other half is still being read
-        if (tid < 16) {
+        double* pr = part + (size_t)(round & 1) * SMC_BLOCKS * 2 * TEMPER_C;   // the other half is still being read
+        if (tid < 2 * TEMPER_C) {
             double a = 0.0;
-            for (int w = 0; w < SMC_THREADS / 32; ++w) a += scr[w * 16 + tid];
-            pr[(size_t)blockIdx.x * 16 + tid] = a;
+            for (int w = 0; w < SMC_THREADS / 32; ++w) a += scr[w * 2 * TEMPER_C + tid];
+            pr[(size_t)blockIdx.x * 2 * TEMPER_C + tid] = a;
         }
         if (!grid_barrier(bar, arrivals += G, err)) return;
-        sum_partials16(pr, G, scr, tot);
-        auto ess = [&](int q) { return tot[q] * tot[q] / tot[8 + q]; };
-        if (round == 0) {
-            const double e = ess(7);
-            if (e >= target) { h = rest; ess_lo = e; break; }
+        sum_partials(pr, G, scr, tot);
+        if (tid < TEMPER_C) ess[tid] = tot[tid] * tot[tid] / tot[TEMPER_C + tid];
+        __syncthreads();
+        if (round == 0 && ess[0] >= target) { h = rest; ess_lo = ess[0]; break; }
+        int at = TEMPER_C / 2;                   // walk down: the middle, a quarter point, ...
+        for (int st = TEMPER_C / 4, l = 0; l < TEMPER_LEVELS; ++l, st >>= 1) {
+            if (ess[at] >= target) { lo = cand[at]; ess_lo = ess[at]; at += st; }
+            else { hi = cand[at]; at -= st; }
         }
-        int at = 3, step = 2;                   // walk down: c4, then c2 or c6, then the quarter points
-        const int levels = min(3, 64 - done);
-        for (int l = 0; l < levels; ++l) {
-            const double e = ess(at);
-            if (e >= target) { lo = cand[at]; ess_lo = e; at += step; }
-            else { hi = cand[at]; at -= step; }
-            step >>= 1;
-        }
-        done += levels;
-        if (done == 64) { h = lo; break; }
+        if (round == 64 / TEMPER_LEVELS - 1) { h = lo; break; }
     }
     // log weights -h Phi, their LSE (the largest is -h min Phi), normalised weights; log Z increment = LSE - log N
     const double mx = -h * phimin;
