@@ -103,6 +103,7 @@ struct LevelArrays {
     T* r = nullptr;   // right-hand side at this level (levels >= 1)
     T* e = nullptr;   // pre-smoothed correction
     T* e2 = nullptr;  // post-smoothed correction (levels >= 1)
+    T* inv = nullptr; // 1/D of every cell (the FP64 solver)
     // SMC_P_BF16SMOOTH_REFINE: BF16 copies of Kw and Ks for the smoother (tiled levels)
     __nv_bfloat16* Kwb = nullptr;
     __nv_bfloat16* Ksb = nullptr;

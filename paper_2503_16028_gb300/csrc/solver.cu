@@ -165,6 +165,19 @@ __global__ void k_coarsen(int m, int count, const T* __restrict__ Kw, const T* _
     }
 }
 
+// 1/D of every cell of a level (the FP64 solver's smoothing passes read it).
+template <typename T>
+__global__ void k_inv_diag(int n, size_t total, const T* __restrict__ Kw, const T* __restrict__ Ks, const T* __restrict__ E,
+                           const T* __restrict__ Nn, T* __restrict__ inv) {
+    const size_t nn = (size_t)n * n, stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += stride) {
+        const size_t p = t / nn;
+        const int c = (int)(t - p * nn), i = c % n, j = c / n;
+        const T e = i + 1 < n ? Kw[t + 1] : E[p * n + j], nb = j + 1 < n ? Ks[t + n] : Nn[p * n + i];
+        inv[t] = recip_nr(Kw[t] + e + Ks[t] + nb);
+    }
+}
+
 // ------------------------------------------------------------------------
 // Tiled smoothing kernels.  A block covers a TILE x TILE tile of one particle
 // plus a halo of H cells, a region of R x R cells (R = TILE + 2H).  Thread t
@@ -459,6 +472,7 @@ namespace smcgm {
 template <typename T>
 struct CoarseLevelPtrs {
     const T* Kw[12]; const T* Ks[12]; const T* E[12]; const T* Nn[12];
+    const T* inv[12];   // 1/D (FP64; null: formed here)
     const T* rtop; T* etop;
     int ntop, nlev;   // nlev levels: ntop, ntop/2, ..., 1
     const int* nact;  // device count of active particles (a launch sized before it was known), or null
@@ -522,6 +536,7 @@ __global__ void __launch_bounds__(COARSE_THREADS, 7) k_coarse(CoarseLevelPtrs<T>
         for (int i = threadIdx.x; i < nn; i += blockDim.x) {
             cp_async_elem(kw[l] + i, gkw + i);
             cp_async_elem(ks[l] + i, gks + i);
+            if (sizeof(T) == 8) cp_async_elem(e[l] + nn + i, P.inv[l] + (size_t)pb * nn + i);
         }
         for (int i = threadIdx.x; i < nl; i += blockDim.x) {
             cp_async_elem(E[l] + i, P.E[l] + (size_t)pb * nl + i);
@@ -536,14 +551,16 @@ __global__ void __launch_bounds__(COARSE_THREADS, 7) k_coarse(CoarseLevelPtrs<T>
     }
     cp_async_wait_all();   // every copy of this thread is in shared memory
     __syncthreads();
-    // 1/D of every cell of every level, once (the half-sweeps multiply by it)
-    nl = P.ntop;
-    for (int l = 0; l < P.nlev; ++l) {
-        for (int c = threadIdx.x; c < nl * nl; c += blockDim.x)
-            e[l][nl * nl + c] = T(1) / cdiag(kw[l], ks[l], E[l], Nn[l], nl, c % nl, c / nl);
-        nl >>= 1;
+    // 1/D of every cell of every level, once (the half-sweeps multiply by it); FP64 has it from the set-up
+    if (sizeof(T) == 4) {
+        nl = P.ntop;
+        for (int l = 0; l < P.nlev; ++l) {
+            for (int c = threadIdx.x; c < nl * nl; c += blockDim.x)
+                e[l][nl * nl + c] = T(1) / cdiag(kw[l], ks[l], E[l], Nn[l], nl, c % nl, c / nl);
+            nl >>= 1;
+        }
+        __syncthreads();
     }
-    __syncthreads();
     // down
     nl = P.ntop;
     for (int l = 0; l < P.nlev - 1; ++l) {
@@ -560,11 +577,10 @@ __global__ void __launch_bounds__(COARSE_THREADS, 7) k_coarse(CoarseLevelPtrs<T>
         for (int k = threadIdx.x; k < m * m; k += blockDim.x) {
             const int I = k % m, J = k / m;
             T s = T(0);
-            for (int dj = 0; dj < 2; ++dj)
-                for (int di = 0; di < 2; ++di) {
-                    const int i = 2 * I + di, j = 2 * J + dj, c = j * nl + i;
-                    s += r[l][c] - (cdiag(kw[l], ks[l], E[l], Nn[l], nl, i, j) * e[l][c] - cnbr(kw[l], ks[l], e[l], nl, i, j));
-                }
+            for (int d = 0; d < 2; ++d) {          // the red cells; the last half-sweep left the black ones' residual at zero
+                const int i = 2 * I + d, j = 2 * J + d, c = j * nl + i;
+                s += r[l][c] - (cdiag(kw[l], ks[l], E[l], Nn[l], nl, i, j) * e[l][c] - cnbr(kw[l], ks[l], e[l], nl, i, j));
+            }
             r[l + 1][k] = s;
         }
         __syncthreads();
@@ -1082,7 +1098,7 @@ static void launch_wpre(Ctx& c, InnerSolver<T>& s, int level, int nact, const T*
     A.a.nact = c.graph ? s.nact : nullptr;
     A.Kw = L.Kw; A.Ks = L.Ks; A.E = L.E; A.Nn = L.Nn; A.rin = rin; A.q = s.q; A.p = p;
     A.rout = rout; A.e_out = L.e; A.rc = s.lv[level + 1].r; A.x = s.x; A.alpha = c.sc.alpha; A.part_rr = c.part.rr;
-    A.cg = cg; A.want_rr = want_rr; A.Kwb = L.Kwb; A.Ksb = L.Ksb;
+    A.cg = cg; A.want_rr = want_rr; A.Kwb = L.Kwb; A.Ksb = L.Ksb; A.inv = L.inv;
     const int grid = (A.a.total + WPB - 1) / WPB;
     if constexpr (sizeof(T) == 4) {
         if (L.Kwb) {   // the BF16 smoother faces
@@ -1115,7 +1131,7 @@ static void launch_wpost(Ctx& c, InnerSolver<T>& s, int level, int nact, const T
     A.a.n = L.n; A.a.ntiles = wtiles(L.n); A.a.lg_tpr = lg_tiles_per_row(L.n); A.a.total = nact * A.a.ntiles; A.a.list = s.list;
     A.a.nact = c.graph ? s.nact : nullptr;
     A.Kw = L.Kw; A.Ks = L.Ks; A.E = L.E; A.Nn = L.Nn; A.r = r; A.e_in = L.e; A.ec = s.lv[level + 1].e2;
-    A.cc = (T)c.cfg.coarse_scale; A.e_out = eout; A.part_rz = c.part.rz; A.cg = cg; A.Kwb = L.Kwb; A.Ksb = L.Ksb;
+    A.cc = (T)c.cfg.coarse_scale; A.e_out = eout; A.part_rz = c.part.rz; A.cg = cg; A.Kwb = L.Kwb; A.Ksb = L.Ksb; A.inv = L.inv;
     const int grid = (A.a.total + WPB - 1) / WPB;
     if constexpr (sizeof(T) == 4) {
         if (L.Kwb) {   // the BF16 smoother faces
@@ -1146,6 +1162,7 @@ static void launch_coarse(Ctx& c, InnerSolver<T>& s, int nact) {
     P.nlev = s.nlev - top;
     for (int l = 0; l < P.nlev; ++l) {
         P.Kw[l] = s.lv[top + l].Kw; P.Ks[l] = s.lv[top + l].Ks; P.E[l] = s.lv[top + l].E; P.Nn[l] = s.lv[top + l].Nn;
+        P.inv[l] = s.lv[top + l].inv;
     }
     P.rtop = s.lv[top].r;
     P.etop = s.lv[top].e2;
@@ -1361,6 +1378,12 @@ void launch_coarsen_all(Ctx& c, InnerSolver<T>& s, int count) {
         k_coarsen<T><<<grid_for(total), 256, 0, c.stream>>>(Bc.n, count, A.Kw, A.Ks, A.E, A.Nn, Bc.Kw, Bc.Ks, Bc.E, Bc.Nn,
                                                             Bc.Kwb, Bc.Ksb); ++c.pc.launches;
     }
+    if constexpr (sizeof(T) == 8)
+        for (int l = 0; l < s.nlev; ++l) {
+            LevelArrays<T>& A = s.lv[l];
+            const size_t total = (size_t)A.n * A.n * count;
+            k_inv_diag<T><<<grid_for(total), 256, 0, c.stream>>>(A.n, total, A.Kw, A.Ks, A.E, A.Nn, A.inv); ++c.pc.launches;
+        }
 }
 template void launch_coarsen_all<float>(Ctx&, InnerSolver<float>&, int);
 template void launch_coarsen_all<double>(Ctx&, InnerSolver<double>&, int);

@@ -201,14 +201,24 @@ template <> __device__ inline float smoother_rcp<float>(float d) {
 }
 template <> __device__ inline double smoother_rcp<double>(double d) { return recip_nr(d); }
 
+// The FP64 solver reads 1/D from the level's array (formed once per solve): forming it takes ten FP64
+// operations per cell and pass, region cells included, against ten for everything else that the
+// finest pre-smoothing pass does (GB300's FP64 pipe: two lanes per SM and cycle).  FP32 forms it from
+// the faces it holds: three additions and one MUFU are cheaper than another 4 bytes per cell.  With the
+// restriction of the red residuals alone: finest pre-smoothing of 256 particles of 256^2 975 -> 459 us,
+// post-smoothing 666 -> 382 us, the levels below 255 and 230 -> 141 and 139 us.
+template <typename T> constexpr bool stored_inv() { return sizeof(T) == 8; }
+
 template <typename T>
 __device__ inline void faces_from_raw(WQuad<T>& Q, const WRaw<T>& R) {
     Q.w[0] = R.a0; Q.e[0] = R.a1; Q.w[1] = R.a1; Q.e[1] = R.ea;
     Q.w[2] = R.b0; Q.e[2] = R.b1; Q.w[3] = R.b1; Q.e[3] = R.eb;
     Q.s[0] = R.s0; Q.n[0] = R.m0; Q.s[1] = R.s1; Q.n[1] = R.m1;
     Q.s[2] = R.m0; Q.n[2] = R.t0; Q.s[3] = R.m1; Q.n[3] = R.t1;
+    if constexpr (!stored_inv<T>()) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) Q.inv[k] = smoother_rcp(Q.w[k] + Q.e[k] + Q.s[k] + Q.n[k]);
+        for (int k = 0; k < 4; ++k) Q.inv[k] = smoother_rcp(Q.w[k] + Q.e[k] + Q.s[k] + Q.n[k]);
+    }
 }
 
 // Offset, from the quad base b = (qy + 1) QS + qx + 1, of cell k of the quad
@@ -261,6 +271,7 @@ struct WPreArgs {
     double* part_rr;
     int cg, want_rr;
     const __nv_bfloat16 *Kwb, *Ksb;   // BF16 smoother faces (kernels instantiated for them)
+    const T* inv;                     // 1/D of the level's cells (stored_inv)
 };
 
 template <typename T>
@@ -272,6 +283,7 @@ struct WPostArgs {
     double* part_rz;
     int cg;
     const __nv_bfloat16 *Kwb, *Ksb;
+    const T* inv;
 };
 
 // Inputs of one work item read straight from global memory.  (x0, y0) is the
@@ -283,7 +295,13 @@ struct GlobalSrc {
     const F *kw, *ks;
     const T *Ep, *Np, *a, *b, *x, *p;   // a: r, b: q (pre) or e_in (post)
     int n;
+    const T* iv;                        // 1/D (stored_inv)
     __device__ void faces(WRaw<T>& R, int gx, int gy) const { load_faces_raw(R, kw, ks, Ep, Np, n, gx, gy); }
+    __device__ void vi(T* v, int gx, int gy) const {
+        const int gi = gy * n + gx;
+        ld2(iv + gi, v[0], v[1]);
+        ld2(iv + gi + n, v[2], v[3]);
+    }
     __device__ void va(T* v, int gx, int gy) const {
         const int gi = gy * n + gx;
         ld2(a + gi, v[0], v[1]);
@@ -358,6 +376,7 @@ __device__ inline void wpre_item(const WPreArgs<T>& A, const Src& S, T* se, int 
         gq[sl] = gy * n + gx;
         if (live[sl]) {
             S.faces(Rw[sl], gx, gy);
+            if constexpr (stored_inv<T>()) S.vi(Q[sl].inv, gx, gy);
             S.va(rq[sl], gx, gy);
             if (CG) {
                 if constexpr (early) {
@@ -394,7 +413,8 @@ __device__ inline void wpre_item(const WPreArgs<T>& A, const Src& S, T* se, int 
                 if (gx >= 0 && gx < n && gy >= 0 && gy < n) {
                     T rv, qv, fw, fe, fs, fn;
                     S.cell(gx, gy, CG, rv, qv, fw, fe, fs, fn);
-                    val = (CG ? rv - al * qv : rv) * smoother_rcp(fw + fe + fs + fn);
+                    if constexpr (stored_inv<T>()) val = (CG ? rv - al * qv : rv) * S.iv[gy * n + gx];
+                    else val = (CG ? rv - al * qv : rv) * smoother_rcp(fw + fe + fs + fn);
                 }
             }
             const int c = (qy + 1) * G::QS + qx + 1;
@@ -447,15 +467,18 @@ __device__ inline void wpre_item(const WPreArgs<T>& A, const Src& S, T* se, int 
         const int gi = gq[sl];
         const int qi = lane + G::LANES * sl;
         const int gx = tx * WT + 2 * (qi % G::IQ), gy = ty * WT + 2 * (qi / G::IQ);
+        // the last half-sweep left the black cells' residual at zero, so the restriction sums the red ones';
+        // after a single sweep from zero theirs is sum k e over the neighbours (D e = r there)
         T rsum = T(0), ev[4];
+        const int b = c0[sl];
+        const WQuad<T>& q = Q[sl];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int b = c0[sl];
-            const WQuad<T>& q = Q[sl];
-            ev[k] = se[b + qoff<G>(k, 4)];
-            rsum += q.r[k] - ((q.w[k] + q.e[k] + q.s[k] + q.n[k]) * ev[k] -
-                              (q.w[k] * se[b + qoff<G>(k, 0)] + q.e[k] * se[b + qoff<G>(k, 1)] +
-                               q.s[k] * se[b + qoff<G>(k, 2)] + q.n[k] * se[b + qoff<G>(k, 3)]));
+        for (int k = 0; k < 4; ++k) ev[k] = se[b + qoff<G>(k, 4)];
+#pragma unroll
+        for (int k = 0; k < 4; k += 3) {
+            const T nb = q.w[k] * se[b + qoff<G>(k, 0)] + q.e[k] * se[b + qoff<G>(k, 1)] + q.s[k] * se[b + qoff<G>(k, 2)] +
+                         q.n[k] * se[b + qoff<G>(k, 3)];
+            rsum += NU == 1 ? nb : q.r[k] - ((q.w[k] + q.e[k] + q.s[k] + q.n[k]) * ev[k] - nb);
         }
         st2(A.e_out + base + gi, ev[0], ev[1]);
         st2(A.e_out + base + gi + n, ev[2], ev[3]);
@@ -497,6 +520,7 @@ __device__ inline void wpost_item(const WPostArgs<T>& A, const Src& S, T* se, in
         gq[sl] = gy * n + gx;
         if (live[sl]) {
             S.faces(Rw[sl], gx, gy);
+            if constexpr (stored_inv<T>()) S.vi(Q[sl].inv, gx, gy);
             S.va(Q[sl].r, gx, gy);
             S.vb(ev[sl], gx, gy);
             ev[sl][4] = S.parent(m, gx, gy);
@@ -602,7 +626,7 @@ __global__ void __launch_bounds__(32 * WPB, WI == 2 ? (sizeof(T) == 4 ? 6 : 3) :
     const size_t base = (size_t)p * n * n;
     const auto fc = smoother_faces<T, BF>(A, base);
     GlobalSrc<T, F> S{fc.kw, fc.ks, A.E + (size_t)p * n, A.Nn + (size_t)p * n, A.rin + base, A.q + base,
-                      A.x + base, A.p + base, n};
+                      A.x + base, A.p + base, n, A.inv + base};
     zero_border<T, G>(sme[slot], lane);
     wpre_item<T, H, CG, GlobalSrc<T, F>, NoHook, WI>(A, S, sme[slot], lane, p, tile, tx, ty);
 }
@@ -623,7 +647,7 @@ __global__ void __launch_bounds__(32 * WPB, WI == 2 ? (sizeof(T) == 4 ? 6 : 3) :
     const size_t base = (size_t)p * n * n;
     const auto fc = smoother_faces<T, BF>(A, base);
     GlobalSrc<T, F> S{fc.kw, fc.ks, A.E + (size_t)p * n, A.Nn + (size_t)p * n, A.r + base, A.e_in + base,
-                      A.ec + (size_t)p * m * m, nullptr, n};
+                      A.ec + (size_t)p * m * m, nullptr, n, A.inv + base};
     zero_border<T, G>(sme[slot], lane);
     wpost_item<T, H, CG, GlobalSrc<T, F>, NoHook, WI>(A, S, sme[slot], lane, p, tile, tx, ty);
 }
