@@ -70,12 +70,14 @@ __global__ void k_em_init(int N, int K, int r, EmPicks init, const double* __res
 // The pivot moves with the fit, so the subtraction loses nothing once the means settle
 // (|m - c|^2 << lambda), and a component's next iteration starts from the new mean.
 // A collapsed component (N_j < 2) is found by every block alike (same sums, same order).
-// Measured (r = 64, 50 iterations, ncu): N = 1024, K = 4 9.0 -> 1.10 ms, N = 256, K = 2 7.2 -> 0.95 ms
-// (what is left is the chain of FP64 latencies through an iteration, 19 us: the FP64 pipe is 6 % busy).
+// Measured (r = 64, 50 iterations, ncu): N = 1024, K = 4 9.0 -> 0.9 ms, N = 256, K = 2 7.2 -> 0.77 ms
+// (what is left is the chain of FP64 latencies through an iteration, 15 us: an exponential takes 1250
+// cycles, a logarithm 2200, a division 500; the FP64 pipe is 6 % busy).
 // ------------------------------------------------------------------------
 constexpr int EM_THREADS = 256;
 constexpr int EM_BLOCKS = 152;      // most blocks of the launch (rows of `part`)
 constexpr int EM_MINP = 8;          // least particles per block: fewer blocks make cheaper barriers
+constexpr int EM_ETHREADS = EM_THREADS - 32;   // threads of the E-step's densities; the last warp forms the constants meanwhile
 constexpr int EM_SPLIT = 4;         // most groups of threads sharing the M-step sums' particles
 
 __host__ __device__ inline int em_pad(int r) { return ((r + 11) / 16) * 16 + 4; }   // >= r, 4 mod 16: rows of 4 s fall on other banks
@@ -96,6 +98,14 @@ struct EmArgs {
     int* err;
 };
 
+// Division of a small index (< 2^16) by a divisor known per launch: the high word of a product.
+struct EmDiv {
+    int d;
+    unsigned m;
+    __device__ explicit EmDiv(int dd) : d(dd), m(dd > 1 ? 0xffffffffu / (unsigned)dd + 1u : 0u) {}
+    __device__ __forceinline__ int quot(int x) const { return d > 1 ? (int)__umulhi((unsigned)x, m) : x; }
+};
+
 template <bool XS>
 __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
     extern __shared__ __align__(16) double sh[];
@@ -113,6 +123,7 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
     double* spl = red + 40;                // 2 EM_THREADS: the M-step sums of the second and later thread groups
     double* xs = spl + 2 * EM_THREADS;     // [per][rp]
     double* g_si = A.part + 2 * (size_t)G * row;
+    const EmDiv by_np(max(1, np)), by_K(K), by_r(r);
     const int lanes = 1 << A.lg_lanes, split = max(1, min(EM_SPLIT, EM_THREADS / Kr));
     auto X = [&](int p, int s) -> double { return XS ? xs[(size_t)p * rp + s] : A.xsT[(size_t)s * N + n0 + p]; };
     if (XS)
@@ -121,7 +132,7 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
             xs[(size_t)p * rp + s] = A.xsT[(size_t)s * N + n0 + p];
         }
     for (int t = tid; t < Kr; t += EM_THREADS) {
-        const int j = t / r, s = t % r;
+        const int j = by_r.quot(t), s = t - j * r;
         const double l = A.lam[t];
         sm[(size_t)j * rp + s] = A.m[t];
         si[(size_t)j * rp + s] = 1.0 / (2.0 * l);
@@ -137,14 +148,19 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
         for (int j = tid; j < K; j += EM_THREADS) cst[j] = log(sw[j]) + red[32];
         __syncthreads();
     }
+    const double log_2pi = log(2.0 * M_PI);
     unsigned arrivals = 0;
     for (int it = 0;; ++it) {
         // log densities: 2^lg_lanes lanes per (particle, component)
         const int items = np * K;
-        for (int base = 0; base < items << A.lg_lanes; base += EM_THREADS) {
+        if (tid >= EM_ETHREADS && tid - EM_ETHREADS < K && it > 0) {   // the last warp: the constants, one logarithm each
+            const int j = tid - EM_ETHREADS;
+            cst[j] = 0.5 * (log(sw[j] * sw[j] / spl[j]) - M_LN2 * spl[MAXK + j]) - 0.5 * r * log_2pi;
+        }
+        for (int base = 0; tid < EM_ETHREADS && base < items << A.lg_lanes; base += EM_ETHREADS) {
             const int item = (base + tid) >> A.lg_lanes, ln = tid & (lanes - 1);
             const bool on = item < items;
-            const int p = on ? item / K : 0, j = on ? item % K : 0;
+            const int p = on ? by_K.quot(item) : 0, j = on ? item - p * K : 0;
             double acc = 0.0;
             if (on) {
                 const double *mj = sm + (size_t)j * rp, *ij = si + (size_t)j * rp;
@@ -155,21 +171,21 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
                 }
             }
             for (int o = lanes >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (on && ln == 0) lp[(size_t)j * per + p] = acc + cst[j];
+            if (on && ln == 0) lp[(size_t)j * per + p] = acc;
         }
         __syncthreads();
         for (int t = tid; t < items; t += EM_THREADS) {
-            const int j = t / np, p = t % np;
+            const int j = by_np.quot(t), p = t - j * np;
             double mx = -1.0 / 0.0;
-            for (int q = 0; q < K; ++q) mx = fmax(mx, lp[(size_t)q * per + p]);
-            ex[(size_t)j * per + p] = exp(lp[(size_t)j * per + p] - mx);
+            for (int q = 0; q < K; ++q) mx = fmax(mx, lp[(size_t)q * per + p] + cst[q]);
+            ex[(size_t)j * per + p] = exp(lp[(size_t)j * per + p] + cst[j] - mx);
         }
         __syncthreads();
         if (it == A.iters) {               // the final log-likelihood: sum over the particles of LSE_j
             double a = 0.0;
             for (int p = tid; p < np; p += EM_THREADS) {
                 double mx = -1.0 / 0.0, sum = 0.0;
-                for (int q = 0; q < K; ++q) mx = fmax(mx, lp[(size_t)q * per + p]);
+                for (int q = 0; q < K; ++q) mx = fmax(mx, lp[(size_t)q * per + p] + cst[q]);
                 for (int q = 0; q < K; ++q) sum += ex[(size_t)q * per + p];
                 a += mx + log(sum);
             }
@@ -189,7 +205,7 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
         double gmin = 1.0 / 0.0;           // least max_j g of the block's particles, lowest index on ties
         int imin = N;
         for (int t = tid; t < items; t += EM_THREADS) {   // responsibilities
-            const int j = t / np, p = t % np;
+            const int j = by_np.quot(t), p = t - j * np;
             double sum = 0.0;
             for (int q = 0; q < K; ++q) sum += ex[(size_t)q * per + p];
             lp[(size_t)j * per + p] = ex[(size_t)j * per + p] / sum;
@@ -198,7 +214,7 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
         double* part = A.part + (size_t)(it & 1) * G * row;   // the other buffer may still be read
         double* out = part + (size_t)b * row;
         if (split > 1) {                   // few pairs: groups of Kr threads share the particles
-            const int h = tid / Kr, q = tid % Kr, j = q / r, s = q % r;
+            const int h = tid / Kr, q = tid - h * Kr, j = by_r.quot(q), s = q - j * r;
             double s1 = 0.0, s2 = 0.0;
             if (h < split) {
                 const double c = sm[(size_t)j * rp + s];
@@ -219,7 +235,7 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
             }
         } else {
             for (int t = tid; t < Kr; t += EM_THREADS) {
-                const int j = t / r, s = t % r;
+                const int j = by_r.quot(t), s = t - j * r;
                 const double c = sm[(size_t)j * rp + s];
                 const double* g = lp + (size_t)j * per;
                 double s1 = 0.0, s2 = 0.0;
@@ -264,7 +280,7 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
             return a;
         };
         for (int q = lo + wid; q < hi; q += EM_THREADS / 32) {
-            const int j = q / r, s = q % r;
+            const int j = by_r.quot(q), s = q - j * r;
             double s1 = 0.0, s2 = 0.0, n = 0.0;
             for (int k = lane; k < G; k += 32) {
                 const double* pr = part + (size_t)k * row;
@@ -305,16 +321,14 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
             if (lane == 0) nj[j] = a;
         }
         __syncthreads();
-        if (tid < K) {
+        if (tid < K) {                       // w_j = N_j / N (1 / N for a re-seeded one), normalised: N cancels
             double tot = 0.0;
-            for (int j = 0; j < K; ++j) tot += nj[j] < 2.0 ? 1.0 / N : nj[j] / N;
-            const double w = (nj[tid] < 2.0 ? 1.0 / N : nj[tid] / N) / tot;
-            sw[tid] = w;
-            cst[tid] = log(w) - 0.5 * r * log(2.0 * M_PI);
+            for (int j = 0; j < K; ++j) tot += nj[j] < 2.0 ? 1.0 : nj[j];
+            sw[tid] = (nj[tid] < 2.0 ? 1.0 : nj[tid]) / tot;
         }
         if (!grid_wait(A.bar, arrivals += G, A.err)) return;
         for (int t = tid; t < Kr; t += EM_THREADS) {
-            const int j = t / r, s = t % r;
+            const int j = by_r.quot(t), s = t - j * r;
             sm[(size_t)j * rp + s] = __ldcg(&A.m[t]);
             si[(size_t)j * rp + s] = __ldcg(&g_si[t]);
         }
@@ -340,8 +354,6 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
             }
             if (lane == 0) { spl[j] = prod; spl[MAXK + j] = (double)ex2; }
         }
-        __syncthreads();
-        if (tid < K) cst[tid] -= 0.5 * (log(spl[tid]) + M_LN2 * spl[MAXK + tid]);
         __syncthreads();
     }
 }
@@ -821,7 +833,7 @@ static void em_diag(Ctx& c, const double* lamS, double* ll) {
     A.part = c.empart; A.loglik = ll; A.bar = reinterpret_cast<unsigned*>(c.icount + 44); A.err = c.dev_err;
     const int G = std::max(1, std::min({EM_BLOCKS, c.sm_count, (N + EM_MINP - 1) / EM_MINP}));
     const int per = (N + G - 1) / G;
-    while (A.lg_lanes < 5 && (per * K << A.lg_lanes) < EM_THREADS) ++A.lg_lanes;   // the chain of FP64 latencies is what bounds small fits
+    while (A.lg_lanes < 5 && (per * K << (A.lg_lanes + 1)) <= EM_ETHREADS) ++A.lg_lanes;   // the chain of FP64 latencies is what bounds small fits
     constexpr size_t LIMIT = 200 * 1024;
     const bool xs = em_smem(K, r, per, true) <= LIMIT;
     const size_t sm = em_smem(K, r, per, xs);
