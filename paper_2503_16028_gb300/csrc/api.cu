@@ -908,7 +908,7 @@ struct smc_batch {
     int steps = 0;
     cudaStream_t origin = nullptr;
     std::vector<cudaStream_t> streams;   // one capture stream per context
-    cudaStream_t aux[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaStream_t aux[2][4] = {};         // bodies of the conditional nodes, per priority class
     cudaEvent_t fork = nullptr;
     std::vector<cudaEvent_t> done;       // per context: its branch / its stream
     cudaGraph_t graph = nullptr;
@@ -920,7 +920,7 @@ static void batch_free(smc_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     for (cudaStream_t st : b->streams) if (st) cudaStreamDestroy(st);
-    for (cudaStream_t st : b->aux) if (st) cudaStreamDestroy(st);
+    for (auto& cls : b->aux) for (cudaStream_t st : cls) if (st) cudaStreamDestroy(st);
     if (b->origin) cudaStreamDestroy(b->origin);
     if (b->fork) cudaEventDestroy(b->fork);
     for (cudaEvent_t e : b->done) if (e) cudaEventDestroy(e);
@@ -958,11 +958,20 @@ smc_status smc_batch_create(smc_ctx* const* ctxs, int count, int steps, smc_batc
     int captured = -1;
     try {
         check(cudaStreamCreateWithFlags(&b->origin, cudaStreamNonBlocking), "stream");
-        for (auto& st : b->aux) check(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking), "stream");
+        // A branch whose solves run in passes is a chain of hundreds of short launches; each would queue behind the
+        // blocks of another branch's on-chip solve, which hold an SM for 0.1 to 0.3 ms and refill it at once.  So
+        // the chains' kernels get the higher priority (five problems of 64^2 to 512^2, two moves: 31.5 -> 30.6 ms).
+        int least = 0, greatest = 0;
+        check(cudaDeviceGetStreamPriorityRange(&least, &greatest), "priority range");
+        auto make_stream = [&](cudaStream_t* st, bool chain) {
+            check(cudaStreamCreateWithPriority(st, cudaStreamNonBlocking, chain ? greatest : least), "stream");
+        };
+        for (int cls = 0; cls < 2; ++cls)
+            for (auto& st : b->aux[cls]) make_stream(&st, cls == 1);
         b->streams.assign(count, nullptr);
         b->done.assign(count, nullptr);
         for (int i = 0; i < count; ++i) {
-            check(cudaStreamCreateWithFlags(&b->streams[i], cudaStreamNonBlocking), "stream");
+            make_stream(&b->streams[i], !ctxs[i]->c.onchip);
             check(cudaEventCreateWithFlags(&b->done[i], cudaEventDisableTiming), "event");
             check(cudaStreamSynchronize(ctxs[i]->c.stream), "sync");   // the context's own work is done
         }
@@ -977,7 +986,7 @@ smc_status smc_batch_create(smc_ctx* const* ctxs, int count, int steps, smc_batc
             const bool prof = c.prof;
             c.stream = b->streams[i];
             c.graph = true; c.lenient = true; c.prof = false; c.gdepth = 0;
-            for (int k = 0; k < 4; ++k) c.gaux[k] = b->aux[k];
+            for (int k = 0; k < 4; ++k) c.gaux[k] = b->aux[c.onchip ? 0 : 1][k];
             check(cudaStreamWaitEvent(c.stream, b->fork, 0), "fork wait");
             check(cudaMemsetAsync(c.icount, 0, sizeof(int), c.stream), "memset");
             check(cudaMemsetAsync(c.gcnt, 0, sizeof(GraphCounters), c.stream), "memset");
@@ -988,7 +997,7 @@ smc_status smc_batch_create(smc_ctx* const* ctxs, int count, int steps, smc_batc
             captured = -1;
         }
         check(cudaStreamEndCapture(b->origin, &b->graph), "end capture");
-        check(cudaGraphInstantiate(&b->exec, b->graph, 0), "instantiate");
+        check(cudaGraphInstantiate(&b->exec, b->graph, cudaGraphInstantiateFlagUseNodePriority), "instantiate");
     } catch (const CudaError& ce) {
         if (captured >= 0) {
             Ctx& c = ctxs[captured]->c;
