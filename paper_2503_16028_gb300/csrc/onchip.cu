@@ -35,6 +35,7 @@
 #include "smcgm_internal.cuh"
 #include "common.cuh"
 #include "df32.cuh"
+#include "onchip.cuh"
 
 namespace smcgm {
 
@@ -57,9 +58,9 @@ struct OcArgs {
 
 // A block covers 64 C x 64 / C cells (a strip of rows): W x H threads, a 4 x 4 patch each.
 // Shared-memory offsets (floats).
-template <int C>
+template <int C_>
 struct OcMem {
-    static constexpr int CC = C * C, W = 16 * C, H = 16 / C;
+    static constexpr int C = C_, CC = C * C, W = 16 * C, H = 16 / C;
     static constexpr int SZH = H * (W + 1), SZV = (H + 1) * W;   // float2 per colour of the sides W, E (H rows of W + 1) and S, N
     static constexpr int PT = W + 2, PL = (H + 2) * PT;     // pitch and size of a plane with a ring of guards
     static constexpr int P4 = 0;                            // p: 4 float4 slots
@@ -78,57 +79,13 @@ struct OcMem {
     static constexpr int QP = HP + 4 * PL;
     static constexpr int LP = QP + PL;                      // C = 4: as HP for the 32^2 level (16 x 16 threads)
     static constexpr int SP = LP + (C == 4 ? 4 * 324 : 0);  // C > 1: as QP for the 16^2 level
-    static constexpr int BARS = (SP + (C > 1 ? 324 : 0) + 1) / 2 * 2;   // C > 1: 2 x 2 + 4 mbarriers (8 bytes each)
-    static constexpr int TOTAL = BARS + (C > 1 ? 16 : 0);
+    static constexpr int ENDF = (SP + (C > 1 ? 324 : 0) + 1) / 2 * 2;   // C > 1: 2 x 2 + 4 mbarriers (8 bytes each)
+    static constexpr int BARS = 4 * ENDF;                   // bytes
+    static constexpr int TOTAL = ENDF + (C > 1 ? 16 : 0);
     static constexpr size_t BYTES = (size_t)TOTAL * 4;
     static_assert(BYTES <= 228 * 1024 / 2 - 1024, "two blocks per SM");
     static_assert(STG % 4 == 0 && RB % 4 == 0 && SIDE % 2 == 0 && RED % 4 == 0, "vector alignment");
 };
-
-__device__ __forceinline__ uint32_t oc_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// Barrier of the cluster (of the block when it is alone), ordering shared, distributed shared and
-// global memory among its threads.
-template <int C>
-__device__ __forceinline__ void oc_sync() {
-    if (C == 1) {
-        __syncthreads();
-    } else {
-        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    }
-}
-// The address of a shared-memory location of this block in block `rank` of the cluster.
-__device__ __forceinline__ uint32_t oc_map(const float* p, uint32_t rank) {
-    uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-// Asynchronous stores into another block; the receiver's mbarrier counts their bytes, so an
-// exchange needs neither a cluster barrier nor the memory fence that one implies (the fence's
-// wait was the largest stall of the cluster form: 2048 solves at 256^2 took 62 ms with cluster barriers,
-// 53 with these).
-__device__ __forceinline__ void oc_push(float* p, uint32_t rank, float v, const float* bar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(oc_map(p, rank)), "f"(v),
-                 "r"(oc_map(bar, rank))
-                 : "memory");
-}
-__device__ __forceinline__ void oc_push4(float* p, uint32_t rank, float4 v, const float* bar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(oc_map(p, rank)),
-                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(oc_map(bar, rank))
-                 : "memory");
-}
-// The same with the addresses already those of the other block.
-__device__ __forceinline__ void oc_store(uint32_t dst, float v, uint32_t bar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(dst), "f"(v), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void oc_store2(uint32_t dst, float2 v, uint32_t bar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(dst), "f"(v.x), "f"(v.y), "r"(bar)
-                 : "memory");
-}
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
@@ -136,91 +93,24 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Where a thread stands.
-template <int C>
-struct OcPos {
-    int tid, tx, ty;         // in the block's W x H threads
-    int lx, ly;              // in the 16 x 16 threads of the local levels
-    uint32_t rank;
-    // Exchanges (C > 1).  Edge exchanges go pairwise between the first (last) thread row of a block and the last
-    // (first) of the block below (above), through two mbarriers per side that alternate: a neighbour's edge can be
-    // at most one exchange ahead, since it needs this edge's values to go on.  The all-to-all exchanges have one
-    // mbarrier each: a block can be at most one all-to-all exchange ahead of any other.
-    unsigned seq, par;
-    int polls;               // bound of a wait; 0 after one ran out
-    uint32_t nbase;          // shared-memory base of the neighbouring block, for the threads of an edge row; else 0
-    bool lower;              // of an edge row: the lower one (neighbour below)
-};
-enum OcAll { OC_RR = 0, OC_RZ = 1, OC_PQ = 2, OC_GATHER = 3 };
-constexpr int OC_POLLS = 1 << 22;
-
-// Offset (floats) of the mbarrier of the current edge exchange in the receiving block: `below` for values that
-// come from the block below it.
-template <int C>
-__device__ __forceinline__ int nb_bar(const OcPos<C>& t, bool below) { return OcMem<C>::BARS + 4 * (below ? 1 : 0) + 2 * (t.seq & 1); }
-template <int C>
-__device__ __forceinline__ float* all_bar(float* sm, int which) { return sm + OcMem<C>::BARS + 8 + 2 * which; }
-__device__ __forceinline__ void oc_expect(const float* bar, int bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(bar)), "r"(bytes) : "memory");
-}
-template <int C>
-__device__ __forceinline__ void oc_wait(OcPos<C>& t, const float* bar, unsigned parity) {
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(bar);
-    uint32_t ok = 0;
-#pragma unroll 1
-    for (int k = 0; k < t.polls && !ok; ++k)
-        asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}"
-                     : "=r"(ok)
-                     : "r"(a), "r"(parity)
-                     : "memory");
-    if (!ok) t.polls = 0;
-}
-// The edge rows' part of an exchange: waits for the neighbour's values (`bytes` for the whole row).
-template <int C>
-__device__ __forceinline__ void nb_wait(float* sm, OcPos<C>& t, int bytes) {
-    if (C > 1) {
-        if (t.nbase) {
-            const float* bar = sm + nb_bar(t, t.lower);
-            if (t.tx == 0) oc_expect(bar, bytes);
-            oc_wait<C>(t, bar, (t.seq >> 1) & 1);
-        }
-        ++t.seq;
-    }
-}
-// After the stores of an edge exchange: the block's own are visible, and to the edge rows the neighbours'.
-template <int C>
-__device__ __forceinline__ void nb_sync(float* sm, OcPos<C>& t, int bytes) {
-    __syncthreads();
-    nb_wait<C>(sm, t, bytes);
-}
-// The same for an all-to-all exchange (`bytes` from all blocks together).
-template <int C>
-__device__ __forceinline__ void all_sync(float* sm, OcPos<C>& t, int which, int bytes) {
-    if (C > 1 && t.tid == 0) oc_expect(all_bar<C>(sm, which), bytes);
-    __syncthreads();
-    if (C > 1) {
-        oc_wait<C>(t, all_bar<C>(sm, which), (t.par >> which) & 1);
-        t.par ^= 1u << which;
-    }
-}
 // The exchange that starts an iteration: |r|^2 and the first red edges.  True if a wait ran out in any thread
 // of the block, which then leaves the loops alike (threads must not decide on sums that others did not see).
 template <int C>
-__device__ __forceinline__ bool rr_sync(float* sm, OcPos<C>& t) {
+__device__ __forceinline__ bool rr_sync(float* sm, OcPos<OcMem<C>>& t) {
     if (C == 1) {
         __syncthreads();
         return false;
     }
-    if (t.tid == 0) oc_expect(all_bar<C>(sm, OC_RR), 32 * OcMem<C>::CC);
-    nb_wait<C>(sm, t, 8 * OcMem<C>::W);
-    oc_wait<C>(t, all_bar<C>(sm, OC_RR), (t.par >> OC_RR) & 1);
+    if (t.tid == 0) oc_expect(all_bar<OcMem<C>>(sm, OC_RR), 32 * OcMem<C>::CC);
+    nb_wait(sm, t, 8 * OcMem<C>::W);
+    oc_wait(t, all_bar<OcMem<C>>(sm, OC_RR), (t.par >> OC_RR) & 1);
     t.par ^= 1u << OC_RR;
     return __syncthreads_or(t.polls == 0);
 }
 
 // ---- sums over the particle's cells: every thread of every block ends with the same bits ----
 template <int C>
-__device__ __forceinline__ void red_put(float* sm, const OcPos<C>& t, int slot, float v) {
+__device__ __forceinline__ void red_put(float* sm, const OcPos<OcMem<C>>& t, int slot, float v) {
     using M = OcMem<C>;
     v = warp_sum(v);
     const int lane = t.tid & 31, wid = t.tid >> 5;
@@ -228,11 +118,11 @@ __device__ __forceinline__ void red_put(float* sm, const OcPos<C>& t, int slot, 
     if (C == 1) {
         if (lane == 0) *dst = v;
     } else if (lane < M::CC) {
-        oc_push(dst, (uint32_t)lane, v, all_bar<C>(sm, slot));
+        oc_push(dst, (uint32_t)lane, v, all_bar<OcMem<C>>(sm, slot));
     }
 }
 template <int C>
-__device__ __forceinline__ float red_get(const float* sm, const OcPos<C>& t, int slot) {
+__device__ __forceinline__ float red_get(const float* sm, const OcPos<OcMem<C>>& t, int slot) {
     using M = OcMem<C>;
     const float* s = sm + M::RED + slot * 8 * M::CC;
     if (C == 1) {
@@ -260,14 +150,14 @@ __device__ __forceinline__ float2* side(float* sm, int s, int col) {
 }
 
 template <int C, int COL>
-__device__ __forceinline__ void pub_f(float* sm, const OcPos<C>& t, const float (&e)[16]) {
+__device__ __forceinline__ void pub_f(float* sm, const OcPos<OcMem<C>>& t, const float (&e)[16]) {
     using M = OcMem<C>;
     const float2 s = COL == 0 ? make_float2(e[0], e[2]) : make_float2(e[1], e[3]);
     const float2 n = COL == 0 ? make_float2(e[13], e[15]) : make_float2(e[12], e[14]);
     if (C > 1 && t.nbase) {
         // to the neighbour's guard row: its north side's row 0 from below it, its south side's row H from above
         const int at = 4 * M::SZH + (t.lower ? COL * M::SZV + M::H * M::W : (2 + COL) * M::SZV);
-        oc_store2(t.nbase + 4 * M::SIDE + 8 * (at + t.tx), t.lower ? s : n, t.nbase + 4 * nb_bar(t, !t.lower));
+        oc_store2(t.nbase + 4 * M::SIDE + 8 * (at + t.tx), t.lower ? s : n, t.nbase + nb_bar(t, !t.lower));
     }
     side<C>(sm, 0, COL)[t.ty * (M::W + 1) + t.tx] = COL == 0 ? make_float2(e[0], e[8]) : make_float2(e[4], e[12]);
     side<C>(sm, 1, COL)[t.ty * (M::W + 1) + t.tx + 1] = COL == 0 ? make_float2(e[7], e[15]) : make_float2(e[3], e[11]);
@@ -277,7 +167,7 @@ __device__ __forceinline__ void pub_f(float* sm, const OcPos<C>& t, const float 
 
 struct HaloF { float2 w, e, s, n; };
 template <int C>
-__device__ __forceinline__ HaloF halo_f(float* sm, const OcPos<C>& t, int col) {   // the neighbours' cells of colour col
+__device__ __forceinline__ HaloF halo_f(float* sm, const OcPos<OcMem<C>>& t, int col) {   // the neighbours' cells of colour col
     HaloF h;
     using M = OcMem<C>;
     h.w = side<C>(sm, 1, col)[t.ty * (M::W + 1) + t.tx];
@@ -296,14 +186,14 @@ __device__ __forceinline__ float pick(float2 v, int k) { return k ? v.y : v.x; }
     const float n_ = (j) < 3 ? e[4 * (j) + 4 + (i)] : pick(h.n, (i) >> 1);
 
 template <int C, int COL>
-__device__ __forceinline__ void inv_f(const float* sm, const OcPos<C>& t, float (&v)[8]) {
+__device__ __forceinline__ void inv_f(const float* sm, const OcPos<OcMem<C>>& t, float (&v)[8]) {
     const float4* p = reinterpret_cast<const float4*>(sm + OcMem<C>::INVF) + 2 * COL * OC_T + t.tid;
     const float4 a = p[0], b = p[OC_T];
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 
 template <int C, int COL>
-__device__ __forceinline__ void sweep_f(float* sm, const OcPos<C>& t, const float (&kw)[20], const float (&ks)[20], const float (&r)[16],
+__device__ __forceinline__ void sweep_f(float* sm, const OcPos<OcMem<C>>& t, const float (&kw)[20], const float (&ks)[20], const float (&r)[16],
                                         float (&e)[16], bool pointwise) {
     float inv[8];
     inv_f<C, COL>(sm, t, inv);
@@ -330,16 +220,16 @@ struct Patch2 { float w[6], s[6]; };   // west faces [j][0..2], south faces [0..
 // A thread's entry, pitch and plane size: the block's own planes (SHARED) or those of a local level.
 template <int C, bool SHARED> struct OcPl {
     static constexpr int PT = SHARED ? OcMem<C>::PT : 18, PL = SHARED ? OcMem<C>::PL : 324;
-    static __device__ __forceinline__ int at(const OcPos<C>& t) { return SHARED ? (t.ty + 1) * PT + t.tx + 1 : (t.ly + 1) * PT + t.lx + 1; }
+    static __device__ __forceinline__ int at(const OcPos<OcMem<C>>& t) { return SHARED ? (t.ty + 1) * PT + t.tx + 1 : (t.ly + 1) * PT + t.lx + 1; }
 };
 template <int C, bool SHARED>
-__device__ __forceinline__ void pub_h(float* pl, const OcPos<C>& t, int col, const float (&e)[4]) {
+__device__ __forceinline__ void pub_h(float* pl, const OcPos<OcMem<C>>& t, int col, const float (&e)[4]) {
     using O = OcPl<C, SHARED>;
     if (SHARED && C > 1 && t.nbase) {   // cells 0, 1 (2, 3) to the block below (above), into its guard row
         using M = OcMem<C>;
         const int plane = t.lower ? (col ? 1 : 0) : (col ? 2 : 3);
         oc_store(t.nbase + 4 * (M::HP + plane * M::PL + (t.lower ? (M::H + 1) * M::PT : 0) + t.tx + 1),
-                 t.lower ? (col ? e[1] : e[0]) : (col ? e[2] : e[3]), t.nbase + 4 * nb_bar(t, !t.lower));
+                 t.lower ? (col ? e[1] : e[0]) : (col ? e[2] : e[3]), t.nbase + nb_bar(t, !t.lower));
     }
     const int at = O::at(t);
     pl[(col ? 1 : 0) * O::PL + at] = e[col ? 1 : 0];
@@ -347,7 +237,7 @@ __device__ __forceinline__ void pub_h(float* pl, const OcPos<C>& t, int col, con
 }
 // Sum of k e over the four neighbours of the two cells of a colour (0: cells 0 and 3, 1: cells 1 and 2).
 template <int C, bool SHARED>
-__device__ __forceinline__ void nb_h(const float* pl, const OcPos<C>& t, int col, const Patch2& k, const float (&e)[4], float& a, float& b) {
+__device__ __forceinline__ void nb_h(const float* pl, const OcPos<OcMem<C>>& t, int col, const Patch2& k, const float (&e)[4], float& a, float& b) {
     using O = OcPl<C, SHARED>;
     const float *p0 = pl + O::at(t), *p1 = p0 + O::PL, *p2 = p1 + O::PL, *p3 = p2 + O::PL;
     if (col == 0) {
@@ -367,7 +257,7 @@ __device__ __forceinline__ void diag_h(const Patch2& k, float (&d)[4]) {
 
 // Pre-smoothing from e = 0 and the sum of the red cells' residuals (the black ones' are zero).
 template <int C, bool SHARED>
-__device__ __forceinline__ float pre_h(float* sm, float* pl, OcPos<C>& t, int nu, const Patch2& k, const float4 inv, const float (&r)[4], float (&e)[4]) {
+__device__ __forceinline__ float pre_h(float* sm, float* pl, OcPos<OcMem<C>>& t, int nu, const Patch2& k, const float4 inv, const float (&r)[4], float (&e)[4]) {
     float a, b;
 #pragma unroll 1
     for (int sw = 0; sw < nu; ++sw) {
@@ -380,12 +270,12 @@ __device__ __forceinline__ float pre_h(float* sm, float* pl, OcPos<C>& t, int nu
             e[3] = (r[3] + b) * inv.w;
         }
         pub_h<C, SHARED>(pl, t, 0, e);
-        if (SHARED) nb_sync<C>(sm, t, 4 * OcMem<C>::W); else __syncthreads();
+        if (SHARED) nb_sync(sm, t, 4 * OcMem<C>::W); else __syncthreads();
         nb_h<C, SHARED>(pl, t, 1, k, e, a, b);
         e[1] = (r[1] + a) * inv.y;
         e[2] = (r[2] + b) * inv.z;
         pub_h<C, SHARED>(pl, t, 1, e);
-        if (SHARED) nb_sync<C>(sm, t, 4 * OcMem<C>::W); else __syncthreads();
+        if (SHARED) nb_sync(sm, t, 4 * OcMem<C>::W); else __syncthreads();
     }
     nb_h<C, SHARED>(pl, t, 0, k, e, a, b);
     float d[4];
@@ -394,17 +284,17 @@ __device__ __forceinline__ float pre_h(float* sm, float* pl, OcPos<C>& t, int nu
 }
 // e already holds the corrected values; post-smoothing (black, red); the last red values are not published.
 template <int C, bool SHARED>
-__device__ __forceinline__ void post_h(float* sm, float* pl, OcPos<C>& t, int nu, const Patch2& k, const float4 inv, const float (&r)[4], float (&e)[4]) {
+__device__ __forceinline__ void post_h(float* sm, float* pl, OcPos<OcMem<C>>& t, int nu, const Patch2& k, const float4 inv, const float (&r)[4], float (&e)[4]) {
     float a, b;
 #pragma unroll 1
     for (int sw = 0; sw < nu; ++sw) {
         pub_h<C, SHARED>(pl, t, 0, e);
-        if (SHARED) nb_sync<C>(sm, t, 4 * OcMem<C>::W); else __syncthreads();
+        if (SHARED) nb_sync(sm, t, 4 * OcMem<C>::W); else __syncthreads();
         nb_h<C, SHARED>(pl, t, 1, k, e, a, b);
         e[1] = (r[1] + a) * inv.y;
         e[2] = (r[2] + b) * inv.z;
         pub_h<C, SHARED>(pl, t, 1, e);
-        if (SHARED) nb_sync<C>(sm, t, 4 * OcMem<C>::W); else __syncthreads();
+        if (SHARED) nb_sync(sm, t, 4 * OcMem<C>::W); else __syncthreads();
         nb_h<C, SHARED>(pl, t, 0, k, e, a, b);
         e[0] = (r[0] + a) * inv.x;
         e[3] = (r[3] + b) * inv.w;
@@ -414,24 +304,24 @@ __device__ __forceinline__ void post_h(float* sm, float* pl, OcPos<C>& t, int nu
 // ---- a level with one cell per thread; red: tx + ty even ----
 struct Cell1 { float w, e, s, n; };
 template <int C, bool SHARED>
-__device__ __forceinline__ void pub_q(float* pl, const OcPos<C>& t, float e) {
+__device__ __forceinline__ void pub_q(float* pl, const OcPos<OcMem<C>>& t, float e) {
     if (SHARED && C > 1 && t.nbase) {
         using M = OcMem<C>;
-        oc_store(t.nbase + 4 * (M::QP + (t.lower ? (M::H + 1) * M::PT : 0) + t.tx + 1), e, t.nbase + 4 * nb_bar(t, !t.lower));
+        oc_store(t.nbase + 4 * (M::QP + (t.lower ? (M::H + 1) * M::PT : 0) + t.tx + 1), e, t.nbase + nb_bar(t, !t.lower));
     }
     pl[OcPl<C, SHARED>::at(t)] = e;
 }
 template <int C, bool SHARED>
-__device__ __forceinline__ float nb_q(const float* pl, const OcPos<C>& t, const Cell1& k) {
+__device__ __forceinline__ float nb_q(const float* pl, const OcPos<OcMem<C>>& t, const Cell1& k) {
     using O = OcPl<C, SHARED>;
     const float* p = pl + O::at(t);
     return fmaf(k.w, p[-1], fmaf(k.e, p[1], fmaf(k.s, p[-O::PT], k.n * p[O::PT])));
 }
 template <int C, bool SHARED>
-__device__ __forceinline__ bool red_q(const OcPos<C>& t) { return ((SHARED ? t.tx + t.ty : t.lx + t.ly) & 1) == 0; }
+__device__ __forceinline__ bool red_q(const OcPos<OcMem<C>>& t) { return ((SHARED ? t.tx + t.ty : t.lx + t.ly) & 1) == 0; }
 // Pre-smoothing from e = 0; returns the residual of a red cell, 0 for a black one.
 template <int C, bool SHARED>
-__device__ __forceinline__ float pre_q(float* sm, float* pl, OcPos<C>& t, int nu, const Cell1& k, float inv, float r, float& e) {
+__device__ __forceinline__ float pre_q(float* sm, float* pl, OcPos<OcMem<C>>& t, int nu, const Cell1& k, float inv, float r, float& e) {
     const bool red = red_q<C, SHARED>(t);
 #pragma unroll 1
     for (int sw = 0; sw < nu; ++sw) {
@@ -439,27 +329,27 @@ __device__ __forceinline__ float pre_q(float* sm, float* pl, OcPos<C>& t, int nu
             e = (sw == 0 ? r : r + nb_q<C, SHARED>(pl, t, k)) * inv;
             pub_q<C, SHARED>(pl, t, e);
         }
-        if (SHARED) nb_sync<C>(sm, t, 2 * OcMem<C>::W); else __syncthreads();
+        if (SHARED) nb_sync(sm, t, 2 * OcMem<C>::W); else __syncthreads();
         if (!red) {
             e = (r + nb_q<C, SHARED>(pl, t, k)) * inv;
             pub_q<C, SHARED>(pl, t, e);
         }
-        if (SHARED) nb_sync<C>(sm, t, 2 * OcMem<C>::W); else __syncthreads();
+        if (SHARED) nb_sync(sm, t, 2 * OcMem<C>::W); else __syncthreads();
     }
     return red ? r + fmaf(-((k.w + k.e) + (k.s + k.n)), e, nb_q<C, SHARED>(pl, t, k)) : 0.f;
 }
 template <int C, bool SHARED>
-__device__ __forceinline__ void post_q(float* sm, float* pl, OcPos<C>& t, int nu, const Cell1& k, float inv, float r, float& e) {
+__device__ __forceinline__ void post_q(float* sm, float* pl, OcPos<OcMem<C>>& t, int nu, const Cell1& k, float inv, float r, float& e) {
     const bool red = red_q<C, SHARED>(t);
 #pragma unroll 1
     for (int sw = 0; sw < nu; ++sw) {
         if (red) pub_q<C, SHARED>(pl, t, e);
-        if (SHARED) nb_sync<C>(sm, t, 2 * OcMem<C>::W); else __syncthreads();
+        if (SHARED) nb_sync(sm, t, 2 * OcMem<C>::W); else __syncthreads();
         if (!red) {
             e = (r + nb_q<C, SHARED>(pl, t, k)) * inv;
             pub_q<C, SHARED>(pl, t, e);
         }
-        if (SHARED) nb_sync<C>(sm, t, 2 * OcMem<C>::W); else __syncthreads();
+        if (SHARED) nb_sync(sm, t, 2 * OcMem<C>::W); else __syncthreads();
         if (red) e = (r + nb_q<C, SHARED>(pl, t, k)) * inv;
     }
 }
@@ -483,7 +373,7 @@ __device__ __forceinline__ Cell1 coarse_faces(const Cell1& k, int tx, int ty) {
 // Gauss-Jordan elimination in registers: thread (row, quarter) holds 16 columns of a row, the
 // pivot row and column go through shared memory, one barrier per step.  Stored symmetrised.
 template <int C>
-__device__ __forceinline__ void build_inv8(float* sm, const OcPos<C>& t, const Cell1& k8) {
+__device__ __forceinline__ void build_inv8(float* sm, const OcPos<OcMem<C>>& t, const Cell1& k8) {
     using M = OcMem<C>;
     float* M8 = sm + M::INV8;
     float* fa = M8;                                         // 4 x 64 faces first
@@ -546,7 +436,7 @@ __device__ __forceinline__ void build_inv8(float* sm, const OcPos<C>& t, const C
 
 // The 16^2 level (one cell per thread, its plane pl) with the dense solve of the 8^2 level below it.
 template <int C, bool SHARED>
-__device__ __forceinline__ void level16(float* sm, float* pl, OcPos<C>& t, int nu, float cc, const Cell1& k, float inv, float r, float& e) {
+__device__ __forceinline__ void level16(float* sm, float* pl, OcPos<OcMem<C>>& t, int nu, float cc, const Cell1& k, float inv, float r, float& e) {
     using M = OcMem<C>;
     const float res = quad_sum(pre_q<C, SHARED>(sm, pl, t, nu, k, inv, r, e));
     if (((t.lx | t.ly) & 1) == 0) sm[M::R8 + (t.ly >> 1) * 8 + (t.lx >> 1)] = res;
@@ -649,18 +539,10 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     extern __shared__ __align__(16) float sm[];
     const int n = 64 * C;
     const int p = blockIdx.x / M::CC;
-    OcPos<C> t;
-    t.tid = threadIdx.x;
-    t.tx = t.tid % M::W; t.ty = t.tid / M::W;
-    t.lx = t.tid & 15; t.ly = t.tid >> 4;
-    t.rank = C == 1 ? 0u : oc_rank();
-    t.seq = 0; t.par = 0; t.polls = OC_POLLS;
-    t.nbase = 0;
-    t.lower = t.ty == 0;
-    if (C > 1) {
-        if (t.ty == 0 && t.rank > 0) t.nbase = oc_map(sm, t.rank - 1);
-        if (t.ty == M::H - 1 && t.rank < M::CC - 1) t.nbase = oc_map(sm, t.rank + 1);
-    }
+    OcPos<OcMem<C>> t;
+    oc_place(t, sm, (int)threadIdx.x % M::W, (int)threadIdx.x / M::W);
+    t.lx = t.tid & 15;
+    t.ly = t.tid >> 4;
     const int gx = 4 * t.tx, gy = 4 * ((int)t.rank * M::H + t.ty);
     const size_t base = (size_t)p * n * n;
     const double b2 = A.b2pp ? A.b2pp[p] : A.b2const;
@@ -678,12 +560,8 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     const float scale = __int_as_float((127 + sexp) << 23);
     const float b2s = (float)(b2 * (double)scale * (double)scale);
     // guards and planes
-    for (int i = M::SIDE + t.tid; i < M::BARS; i += OC_T) sm[i] = 0.f;
-    if (C > 1 && t.tid == 0) {
-        for (int k = 0; k < 8; ++k)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(sm + M::BARS + 2 * k)) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    for (int i = M::SIDE + t.tid; i < M::ENDF; i += OC_T) sm[i] = 0.f;
+    if (C > 1 && t.tid == 0) oc_init_bars<M>(sm);
     // faces of the patch: west faces 4 x 5, south faces 5 x 4
     float kw[20], ks[20];
     {
@@ -738,9 +616,9 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                 const int f = i / part, c = i % part, I = c % (M::W / 2), J = c / (M::W / 2);
                 const float* q = st + f * OC_T + 2 * J * M::W + 2 * I;
                 const float v = f == 0 ? q[0] + q[M::W] : f == 1 ? q[1] + q[M::W + 1] : f == 2 ? q[0] : q[M::W];
-                for (int d0 = 0; d0 < M::CC; ++d0) oc_push(fb + f * all + (int)t.rank * part + c, (uint32_t)d0, v, all_bar<C>(sm, OC_GATHER));
+                for (int d0 = 0; d0 < M::CC; ++d0) oc_push(fb + f * all + (int)t.rank * part + c, (uint32_t)d0, v, all_bar<OcMem<C>>(sm, OC_GATHER));
             }
-            all_sync<C>(sm, t, OC_GATHER, all * 16);
+            all_sync(sm, t, OC_GATHER, all * 16);
             Cell1 k16;
             if (C == 4) {
                 float* lf = sm + M::LF + t.tid;
@@ -809,11 +687,11 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                 if (sw > 0) {
                     sweep_f<C, 0>(sm, t, kw, ks, r, e, false);
                     pub_f<C, 0>(sm, t, e);
-                    nb_sync<C>(sm, t, 8 * M::W);
+                    nb_sync(sm, t, 8 * M::W);
                 }
                 sweep_f<C, 1>(sm, t, kw, ks, r, e, false);
                 pub_f<C, 1>(sm, t, e);
-                nb_sync<C>(sm, t, 8 * M::W);
+                nb_sync(sm, t, 8 * M::W);
             }
             float rh[4], eh[4];
             {
@@ -853,9 +731,9 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                         const float4 u = *reinterpret_cast<const float4*>(sm + M::STG + 2 * J * (M::W / 2) + I);
                         const float4 v = *reinterpret_cast<const float4*>(sm + M::STG + (2 * J + 1) * (M::W / 2) + I);
                         oc_push4(sm + M::RB + (int)t.rank * part + c, (uint32_t)(t.tid / (part / 4)),
-                                 make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w), all_bar<C>(sm, OC_GATHER));
+                                 make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w), all_bar<OcMem<C>>(sm, OC_GATHER));
                     }
-                    all_sync<C>(sm, t, OC_GATHER, m * m * 4);
+                    all_sync(sm, t, OC_GATHER, m * m * 4);
                     const int px = t.tx >> 1, py = (int)t.rank * (M::H / 2) + (t.ty >> 1);   // the parent on the gathered level
                     const float* sf = sm + M::SF + t.tid;
                     const Cell1 k16{sf[0], sf[OC_T], sf[2 * OC_T], sf[3 * OC_T]};
@@ -900,10 +778,10 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
 #pragma unroll 1
             for (int sw = 0; sw < A.nu_f; ++sw) {
                 pub_f<C, 0>(sm, t, e);
-                nb_sync<C>(sm, t, 8 * M::W);
+                nb_sync(sm, t, 8 * M::W);
                 sweep_f<C, 1>(sm, t, kw, ks, r, e, false);
                 pub_f<C, 1>(sm, t, e);
-                nb_sync<C>(sm, t, 8 * M::W);
+                nb_sync(sm, t, 8 * M::W);
                 sweep_f<C, 0>(sm, t, kw, ks, r, e, false);
             }
             // beta, p = z + beta p
@@ -911,7 +789,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
 #pragma unroll
             for (int c = 0; c < 16; ++c) s = fmaf(r[c], e[c], s);
             red_put<C>(sm, t, OC_RZ, s);
-            all_sync<C>(sm, t, OC_RZ, 32 * M::CC);
+            all_sync(sm, t, OC_RZ, 32 * M::CC);
             const float rzn = red_get<C>(sm, t, 1);
             if (!first) {
                 const float beta = rzn / rz;
@@ -929,7 +807,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             for (int j = 0; j < 4; ++j) P4[j * OC_T] = make_float4(e[4 * j], e[4 * j + 1], e[4 * j + 2], e[4 * j + 3]);
             pub_f<C, 0>(sm, t, e);
             pub_f<C, 1>(sm, t, e);
-            nb_sync<C>(sm, t, 16 * M::W);
+            nb_sync(sm, t, 16 * M::W);
             // q = A p in flux form, p.q
             float q[16];
             s = 0.f;
@@ -956,7 +834,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) xv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            all_sync<C>(sm, t, OC_PQ, 32 * M::CC);
+            all_sync(sm, t, OC_PQ, 32 * M::CC);
             const float pq = red_get<C>(sm, t, 2);
             const float alpha = pq > 0.f ? rz / pq : 0.f;
 #pragma unroll
@@ -1063,7 +941,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             }
         }
         red_put<C>(sm, t, OC_RZ, s);
-        all_sync<C>(sm, t, OC_RZ, 32 * M::CC);
+        all_sync(sm, t, OC_RZ, 32 * M::CC);
         if (C > 1 && __syncthreads_or(t.polls == 0)) break;
         const float res2 = red_get<C>(sm, t, OC_RZ);
         if (res2 <= A.tolout2 * b2s) { converged = true; break; }
@@ -1120,11 +998,12 @@ static bool oc_fits() {
     return nc > 0;
 }
 
-// Whether the context's solves run on chip: mixed precision, the default tile kernels, a grid of 64,
+// Whether the context's solves run on chip: the default tile kernels and, in mixed precision (onchip64.cu: FP64), a grid of 64,
 // 128 or 256 cells per side (a 512^2 strip would not fit a cluster of 16; at each of the three this is
 // the faster solver from 2 particles to thousands), and clusters of that size on this device.
 bool onchip_supported(const Ctx& c) {
-    if (c.dim != 2 || !mixed_precision(c.cfg) || c.cfg.tile_kernel != 0) return false;
+    if (c.dim != 2 || c.cfg.tile_kernel != 0) return false;
+    if (!mixed_precision(c.cfg)) return onchip64_supported(c);
     if (c.n == 64) return oc_fits<1>();
     if (c.n == 128) return oc_fits<2>();
     if (c.n == 256) return oc_fits<4>();
@@ -1139,8 +1018,7 @@ static void oc_launch(Ctx& c, const OcArgs& A, int count) {
     check(cudaLaunchKernelEx(&cfg, k_onchip<C>, A), "on-chip solve"); ++c.pc.launches;
 }
 
-// Solves a batch into W; the counters accumulate in c.gcnt (fold_onchip_counters reads them).
-void solve_batch_onchip(Ctx& c, int count, const Rhs& R, double* W) {
+static void solve_batch_onchip32(Ctx& c, int count, const Rhs& R, double* W) {
     InnerSolver<float>& s = c.s32;
     LevelArrays<float>& f = s.lv[0];
     OcArgs A{};
@@ -1159,11 +1037,18 @@ void solve_batch_onchip(Ctx& c, int count, const Rhs& R, double* W) {
     A.badp = c.lenient ? c.badp : nullptr;
     A.cnt = c.gcnt;
     A.err = c.dev_err;
-    if (c.prof) check(cudaEventRecord(c.ev0, c.stream), "event");
     if (c.n == 64) oc_launch<1>(c, A, count);
     else if (c.n == 128) oc_launch<2>(c, A, count);
     else oc_launch<4>(c, A, count);
-    if (c.prof) {   // profiling: this kernel is the dominant one (faces' two parts in, w out per cell)
+}
+
+// Solves a batch into W; the counters accumulate in c.gcnt (OnchipCounters reads them).
+void solve_batch_onchip(Ctx& c, int count, const Rhs& R, double* W) {
+    const bool mixed = mixed_precision(c.cfg);
+    if (c.prof) check(cudaEventRecord(c.ev0, c.stream), "event");
+    if (mixed) solve_batch_onchip32(c, count, R, W);
+    else solve_batch_onchip64(c, count, R, W);
+    if (c.prof) {   // profiling: this kernel is the dominant one (faces in, as two parts or with 1/D and the coarser levels; w out)
         check(cudaEventRecord(c.ev1, c.stream), "event");
         check(cudaEventSynchronize(c.ev1), "event wait");
         float ms = 0.f;
@@ -1171,7 +1056,7 @@ void solve_batch_onchip(Ctx& c, int count, const Rhs& R, double* W) {
         c.pc.dom_ms += ms;
         c.pc.dom_launches += 1;
         c.pc.dom_particles += count;
-        c.pc.dom_bytes += 24.0 * c.n * c.n * count;
+        c.pc.dom_bytes += (mixed ? 24.0 : 40.0) * c.n * c.n * count;
     }
 }
 

@@ -176,6 +176,8 @@ Rhs shared_rhs(const Ctx& c);
 int solve_batch(Ctx& c, int count, const Rhs& R, double* W);   // W: the FP64 solutions (count x n x n)
 bool onchip_supported(const Ctx& c);
 void solve_batch_onchip(Ctx& c, int count, const Rhs& R, double* W);
+bool onchip64_supported(const Ctx& c);   // onchip64.cu: the FP64 solver's part of the two
+void solve_batch_onchip64(Ctx& c, int count, const Rhs& R, double* W);
 void forward_solve_graph(Ctx& c, const double* X, int count, double* Phi_out);   // into the graph being captured
 void capture_move_steps(Ctx& c, int steps, int* acc_count);                      // into the graph being captured
 void launch_mark_out_of_range(Ctx& c, int count, double* Phi);

@@ -1795,7 +1795,7 @@ int solve_batch(Ctx& c, int count, const Rhs& R, double* W) {
     if (c.onchip) {                       // counted and checked by the caller's OnchipCounters
         c.pc.solves += count;
         c.pc.cells = c.n * c.n;
-        c.pc.word_bytes = 4;
+        c.pc.word_bytes = mixed_precision(c.cfg) ? 4 : 8;
         solve_batch_onchip(c, count, R, W);
         return 0;
     }
