@@ -133,6 +133,20 @@ __device__ inline void ld2(const T* p, T& a, T& b) {
     a = v.x;
     b = v.y;
 }
+__device__ inline void ld4(const float* p, float* v) {
+    const float4 u = *reinterpret_cast<const float4*>(p);
+    v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+}
+__device__ inline void ld4(const double* p, double* v) {
+    const double2 u = reinterpret_cast<const double2*>(p)[0], t = reinterpret_cast<const double2*>(p)[1];
+    v[0] = u.x; v[1] = u.y; v[2] = t.x; v[3] = t.y;
+}
+__device__ inline void st4(float* p, const float* v) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ inline void st4(double* p, const double* v) {
+    reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
+}
+
 template <typename T>
 __device__ inline void st2(T* p, T a, T b) {
     typename Vec2<T>::type v;
@@ -662,31 +676,25 @@ struct WApplyArgs {
     int first;
 };
 
-// p <- z + beta p on the tile plus a one-cell ring, then q = A p and p.q on the tile.
-// Lane l covers column l % 16 of rows l / 16 + 2 k (k < 8), so one warp access
-// touches 16 consecutive words of two rows: in global memory two 64-byte row
-// segments, in the staged p (row stride 48 = 16 mod 32) 32 distinct banks.
-// All global loads (z, p, ring, faces) are issued before any is used.
+// p <- z + beta p, then q = A p and p.q, on a tile of 32 x 8 cells per warp: lane l holds columns 4 (l % 8) .. + 3 of
+// rows 2 (l / 8) and + 1, so every access is a 16-byte load or store of whole 128-byte lines, neighbours' values come
+// by shuffle and the ring of p is formed by the lanes at the tile's edges.  All global loads (z, p, ring,
+// faces) are issued before any is used.  Bound by HBM in FP32 (24 bytes per cell) and by the FP64 unit in FP64; on
+// 16 x 16 tiles with scalar loads and a staged p it was the L1's request rate (82 % busy, two lines per
+// request): 125 particles of 512^2 170 us, now 137 (5.7 TB/s).  In FP64 both take 306 us for 256 of 256^2.
 // q is formed as the sum of the face fluxes k_f (p_c - p_nb), not as
 // diag p_c - sum k_f p_nb: for a smooth p the differences are exact and the
 // rounding error stays at the size of the fluxes, where the diagonal form
 // loses it to cancellation.  CG's recursive residual r - alpha q then tracks
 // the true residual of the FP32 iterate closely, and each refinement phase's
 // reduction holds for the FP64 residual too.
-// MINB: resident blocks per SM asked of the register allocator (7 for FP32:
-// 72 registers without spills, 28 warps per SM to cover the load latency;
-// 4 for FP64: 128 registers).
-constexpr int WAPPLY_PW = 48;                 // staged p row stride (tile + ring: 18 columns used)
-constexpr int WAPPLY_PR = WT + 2;             // staged rows
-
+// MINB: resident blocks per SM asked of the register allocator.
 template <typename T>
-__device__ inline void wapply_item(const WApplyArgs<T>& A, T* sp, int lane, int item) {
-    constexpr int PW = WAPPLY_PW;
-    constexpr int PR = WAPPLY_PR;
-    const int n = A.a.n;
-    int pi, tile, tx, ty;
-    item_tile(A.a, item, pi, tile, tx, ty);
-    const int p = A.a.list[pi];
+__device__ inline void wapply_item(const WApplyArgs<T>& A, int lane, int item) {
+    const int n = A.a.n, lt = A.a.lg_tpr, lx = lt - 1;     // n / 32 tiles per row, n / 8 rows of them
+    const int p = A.a.list[item >> (2 * lt)], tile = item & ((1 << (2 * lt)) - 1);
+    const int cq = lane & 7, ry = lane >> 3;
+    const int x = (tile & ((1 << lx) - 1)) * 32 + 4 * cq, y = (tile >> lx) * 8 + 2 * ry;
     const size_t base = (size_t)p * n * n;
     const T* zg = A.z + base;
     const T* pg = A.pin + base;
@@ -694,63 +702,61 @@ __device__ inline void wapply_item(const WApplyArgs<T>& A, T* sp, int lane, int 
     const T* ks = A.Ks + base;
     const bool first = A.first != 0;
     const T b = first ? T(0) : (T)A.betac[p];
-    const int cx = lane & 15, ry = lane >> 4;
-    const int gx = tx * WT + cx;
+    const int gi = y * n + x;
     // phase 1: loads
-    T pv[8], pold[8], fw[8], fe[8], fs[8], fn[8], rz[2], rp[2];
-    int rgi[2];
-    bool rin[2];
+    T pv[2][4], po[2][4] = {}, w[2][5], s[3][4], rv[3] = {}, ro[3] = {};
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int gy = ty * WT + ry + 2 * k;
-        const int gi = gy * n + gx;
-        pv[k] = zg[gi];
-        pold[k] = first ? T(0) : pg[gi];
-        fw[k] = kw[gi];
-        fe[k] = gx + 1 < n ? kw[gi + 1] : A.E[(size_t)p * n + gy];
-        fs[k] = ks[gi];
-        fn[k] = gy + 1 < n ? ks[gi + n] : A.Nn[(size_t)p * n + gx];
+    for (int j = 0; j < 2; ++j) {
+        ld4(zg + gi + j * n, pv[j]);
+        if (!first) ld4(pg + gi + j * n, po[j]);
+        ld4(kw + gi + j * n, w[j]);
+        ld4(ks + gi + j * n, s[j]);
+    }
+    ld4(y + 2 < n ? ks + gi + 2 * n : A.Nn + (size_t)p * n + x, s[2]);
+    // the ring: a cell of the row below and of the row above per lane, and of the columns beside (lanes 0 - 7 west, 8 - 15 east)
+    const int x0 = x - 4 * cq, y0 = y - 2 * ry;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int xr = k < 2 ? x0 + lane : lane < 8 ? x0 - 1 : x0 + 32, yr = k == 0 ? y0 - 1 : k == 1 ? y0 + 8 : y0 + (lane & 7);
+        if ((k < 2 || lane < 16) && xr >= 0 && xr < n && yr >= 0 && yr < n) {
+            rv[k] = zg[yr * n + xr];
+            if (!first) ro[k] = pg[yr * n + xr];
+        }
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int i = lane + 32 * h;
-        const int side = i / WT, j = i % WT;
-        int gxx, gyy;
-        if (side == 0) { gxx = tx * WT - 1; gyy = ty * WT + j; }
-        else if (side == 1) { gxx = tx * WT + WT; gyy = ty * WT + j; }
-        else if (side == 2) { gxx = tx * WT + j; gyy = ty * WT - 1; }
-        else { gxx = tx * WT + j; gyy = ty * WT + WT; }
-        rin[h] = gxx >= 0 && gxx < n && gyy >= 0 && gyy < n;
-        rgi[h] = gyy * n + gxx;
-        rz[h] = rin[h] ? zg[rgi[h]] : T(0);
-        rp[h] = (rin[h] && !first) ? pg[rgi[h]] : T(0);
+    for (int j = 0; j < 2; ++j) {
+        w[j][4] = T(0);
+        if (cq == 7) w[j][4] = x + 4 < n ? kw[gi + j * n + 4] : A.E[(size_t)p * n + y + j];
     }
-    // phase 2: p_new into shared memory
+    // phase 2: the new p
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        pv[k] += b * pold[k];
-        sp[(ry + 2 * k + 1) * PW + cx + 1] = pv[k];
+    for (int i = 0; i < 4; ++i) {
+        pv[0][i] += b * po[0][i];
+        pv[1][i] += b * po[1][i];
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int i = lane + 32 * h;
-        const int side = i / WT, j = i % WT;
-        const int lx = side == 0 ? 0 : side == 1 ? PR - 1 : j + 1;
-        const int ly = side == 2 ? 0 : side == 3 ? PR - 1 : j + 1;
-        sp[ly * PW + lx] = rz[h] + b * rp[h];
-    }
-    __syncwarp();
+    for (int k = 0; k < 3; ++k) rv[k] += b * ro[k];
     T pq = T(0);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int yy = ry + 2 * k;
-        const int c = (yy + 1) * PW + cx + 1;
-        const T q = fw[k] * (pv[k] - sp[c - 1]) + fe[k] * (pv[k] - sp[c + 1]) + fs[k] * (pv[k] - sp[c - PW]) +
-                    fn[k] * (pv[k] - sp[c + PW]);
-        const size_t gi = base + (size_t)(ty * WT + yy) * n + gx;
-        A.pout[gi] = pv[k];
-        A.q[gi] = q;
-        pq += pv[k] * q;
+    for (int j = 0; j < 2; ++j) {
+        T pw = __shfl_up_sync(0xffffffffu, pv[j][3], 1), pe = __shfl_down_sync(0xffffffffu, pv[j][0], 1);
+        const T we = __shfl_down_sync(0xffffffffu, w[j][0], 1), beside = __shfl_sync(0xffffffffu, rv[2], (cq == 7 ? 8 : 0) + 2 * ry + j);
+        if (cq == 0) pw = beside;
+        if (cq == 7) pe = beside;
+        else w[j][4] = we;
+        T q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            T v = j == 0 ? __shfl_up_sync(0xffffffffu, pv[1][i], 8) : __shfl_down_sync(0xffffffffu, pv[0][i], 8);
+            const T u = __shfl_sync(0xffffffffu, rv[j], 4 * cq + i);
+            if (ry == (j == 0 ? 0 : 3)) v = u;
+            const T c = pv[j][i], west = i == 0 ? pw : pv[j][i - 1], east = i == 3 ? pe : pv[j][i + 1];
+            const T south = j == 0 ? v : pv[0][i], north = j == 0 ? pv[1][i] : v;
+            q[i] = w[j][i] * (c - west) + w[j][i + 1] * (c - east) + s[j][i] * (c - south) + s[j + 1][i] * (c - north);
+            pq += c * q[i];
+        }
+        st4(A.pout + base + gi + j * n, pv[j]);
+        st4(A.q + base + gi + j * n, q);
     }
     const double tot = warp_sum<T>(pq);
     if (lane == 0) A.part_pq[(size_t)p * A.a.ntiles + tile] = tot;
@@ -758,11 +764,10 @@ __device__ inline void wapply_item(const WApplyArgs<T>& A, T* sp, int lane, int 
 
 template <typename T, int MINB>
 __global__ void __launch_bounds__(32 * WPB, MINB) k_wapply(WApplyArgs<T> A) {
-    __shared__ T smp[WPB][WAPPLY_PR * WAPPLY_PW];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int item = blockIdx.x * WPB + warp;
     if (item >= work_total(A.a)) return;
-    wapply_item<T>(A, smp[warp], lane, item);
+    wapply_item<T>(A, lane, item);
 }
 
 }  // namespace smcgm
