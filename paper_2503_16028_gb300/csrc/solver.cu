@@ -731,17 +731,17 @@ __global__ void __launch_bounds__(256) k_residual(int n, const double* __restric
 // Mixed precision: the FP64-accurate residual b - A w, with w in FP64 and the
 // faces and b as df32 pairs, evaluated as b - sum over faces of the fluxes
 // k_f (w_c - w_nb) (w_nb = 0 beyond a wall).  Only the differences w_c - w_nb
-// use the FP64 unit (exact for neighbouring values, by Sterbenz's lemma), and
-// each face's flux is formed once: a 32 x 32 tile puts the west and south
-// fluxes of its cells, plus those of the next column and row, into shared
-// memory as df32 (the difference split by bit manipulation, the product in
-// df32), and every cell takes its east / north flux from its neighbour's west
-// / south one.  Products and sums run in df32 on the FP32 pipes (error ~2^-47
+// use the FP64 unit (exact for neighbouring values, by Sterbenz's lemma; the difference
+// split by bit manipulation, the product in df32), and each face's flux is formed once.
+// Products and sums run in df32 on the FP32 pipes (error ~2^-47
 // of the face fluxes, whose sum is ~200 |b| at 256^2).  Stored in FP32 with the
 // partial |res|^2 per tile, summed in FP32 (a convergence test needs no more,
 // and the FP64 unit, ~1/64 of the FP32 rate here, is left to the differences).
-// RES_THREADS per 32 x 32 tile: 128 (four rows of threads) measured faster than 256 (+0.6 % for the
-// whole move) and 512.
+// A block of four warps per 32 x 32 tile, 8 rows a warp: lane l forms the west and south fluxes of columns
+// 4 (l % 8) .. + 3 of rows 2 (l / 8) and + 1 and takes the others' by shuffle; the tile's last
+// column and a warp's last row of faces are one more flux per lane.  Issue slots bound it (166
+// instructions per cell) beside the FP64 unit: 24 particles of 512^2 72 us with the fluxes staged in
+// shared memory (261 instructions per cell, the edge faces a divergent third flux per row), now 48.
 constexpr int RES_THREADS = 128;
 __global__ void __launch_bounds__(RES_THREADS) k_residual_mix(int n, const float* __restrict__ Kwh, const float* __restrict__ Kwl,
                                                       const float* __restrict__ Ksh, const float* __restrict__ Ksl,
@@ -751,45 +751,75 @@ __global__ void __launch_bounds__(RES_THREADS) k_residual_mix(int n, const float
                                                       size_t bstride, float* __restrict__ rout,
                                                       double* __restrict__ part_res, const int* __restrict__ act) {
     __shared__ float red[RES_THREADS / 32];
-    __shared__ float2 FW[TILE][TILE + 1];   // FW[j][i]: flux of the west face of cell (x0 + i, y0 + j); column TILE: the east edge
-    __shared__ float2 FS[TILE + 1][TILE];   // FS[j][i]: south face; row TILE: the north edge
     const int pb = blockIdx.y;
     if (!act[pb]) return;
-    const int tpr = n / TILE;
-    const int tx = blockIdx.x % tpr, ty = blockIdx.x / tpr;
-    const int x0 = tx * TILE, y0 = ty * TILE;
-    const size_t nn = (size_t)n * n, base = (size_t)pb * nn;
+    const int tpr = n / TILE, lane = threadIdx.x & 31, cq = lane & 7, ry = lane >> 3;
+    const int x0 = (blockIdx.x % tpr) * TILE, y0 = (blockIdx.x / tpr) * TILE + 8 * (threadIdx.x >> 5);   // the warp's 32 x 8 cells
+    const int x = x0 + 4 * cq, y = y0 + 2 * ry;
+    const size_t base = (size_t)pb * n * n;
     const double* wp = w + base;
     const float *kwh = Kwh + base, *kwl = Kwl + base, *ksh = Ksh + base, *ksl = Ksl + base;
-    const int li = threadIdx.x % TILE, lj0 = threadIdx.x / TILE;   // RES_THREADS / 32 rows of threads
-    auto flux = [](float kh, float kl, double d) {
-        const df32 v = df_mul(df32{kh, kl}, df_from_double_bits(d));
-        return make_float2(v.hi, v.lo);
-    };
-    for (int lj = lj0; lj < TILE; lj += blockDim.x / TILE) {
-        const int i = x0 + li, j = y0 + lj;
-        const int c = j * n + i;
-        const double wc = wp[c];
-        FW[lj][li] = flux(kwh[c], kwl[c], i > 0 ? wc - wp[c - 1] : wc);
-        FS[lj][li] = flux(ksh[c], ksl[c], j > 0 ? wc - wp[c - n] : wc);
-        if (li == TILE - 1)
-            FW[lj][TILE] = i + 1 < n ? flux(kwh[c + 1], kwl[c + 1], wp[c + 1] - wc)
-                                     : flux(Eh[(size_t)pb * n + j], El[(size_t)pb * n + j], -wc);
-        if (lj == TILE - 1)
-            FS[TILE][li] = j + 1 < n ? flux(ksh[c + n], ksl[c + n], wp[c + n] - wc)
-                                     : flux(Nh[(size_t)pb * n + i], Nl[(size_t)pb * n + i], -wc);
+    auto flux = [](float kh, float kl, double d) { return df_mul(df32{kh, kl}, df_from_double_bits(d)); };
+    auto shfl = [](df32 v, int from) { return df32{__shfl_sync(0xffffffffu, v.hi, from), __shfl_sync(0xffffffffu, v.lo, from)}; };
+    const int gi = y * n + x;
+    double wv[3][4] = {};                   // rows y - 1, y, y + 1
+    if (y > 0) ld4(wp + gi - n, wv[0]);
+    ld4(wp + gi, wv[1]);
+    ld4(wp + gi + n, wv[2]);
+    df32 east, north;                       // the tile's east face of row y0 + lane % 8; the warp's north face of column x0 + lane
+    {
+        const int c = (y0 + (lane & 7)) * n + x0 + TILE, e = pb * n + y0 + (lane & 7);
+        const bool in = x0 + TILE < n;
+        const double wn = in ? wp[c] : 0.0;
+        east = flux(in ? kwh[c] : Eh[e], in ? kwl[c] : El[e], wn - wp[c - 1]);
     }
-    __syncthreads();
+    {
+        const int c = (y0 + 8) * n + x0 + lane, e = pb * n + x0 + lane;
+        const bool in = y0 + 8 < n;
+        const double wn = in ? wp[c] : 0.0;
+        north = flux(in ? ksh[c] : Nh[e], in ? ksl[c] : Nl[e], wn - wp[c - n]);
+    }
+    df32 fs[2][4];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        float kh[4], kl[4];
+        ld4(ksh + gi + j * n, kh);
+        ld4(ksl + gi + j * n, kl);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) fs[j][i] = flux(kh[i], kl[i], wv[j + 1][i] - wv[j][i]);
+    }
     float acc2 = 0.f;                       // |r|^2 of a thread's cells
-    for (int lj = lj0; lj < TILE; lj += blockDim.x / TILE) {
-        const int c = (y0 + lj) * n + x0 + li;
-        const float2 fw = FW[lj][li], fe = FW[lj][li + 1], fs = FS[lj][li], fn = FS[lj + 1][li];
-        const df32 aw = df_add(df_add(df32{fw.x, fw.y}, df32{-fe.x, -fe.y}), df_add(df32{fs.x, fs.y}, df32{-fn.x, -fn.y}));
-        const float2 bb = bdf[(size_t)pb * bstride + c];
-        const df32 res = df_sub_acc(df32{bb.x, bb.y}, aw);
-        const float r = __fadd_rn(res.hi, res.lo);
-        rout[base + c] = r;
-        acc2 = fmaf(r, r, acc2);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        float kh[4], kl[4], b[8], r[4];
+        ld4(kwh + gi + j * n, kh);
+        ld4(kwl + gi + j * n, kl);
+        const float* bp = reinterpret_cast<const float*>(bdf + (size_t)pb * bstride + gi + j * n);
+        ld4(bp, b);
+        ld4(bp + 4, b + 4);
+        double wl = __shfl_up_sync(0xffffffffu, wv[j + 1][3], 1);
+        if (cq == 0) wl = x > 0 ? wp[gi + j * n - 1] : 0.0;
+        df32 fw[5];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            fw[i] = flux(kh[i], kl[i], wv[j + 1][i] - wl);
+            wl = wv[j + 1][i];
+        }
+        const df32 next = shfl(fw[0], lane + 1), edge = shfl(east, 2 * ry + j);
+        fw[4] = cq == 7 ? edge : next;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            df32 fn = fs[1][i];
+            if (j == 1) {
+                const df32 above = shfl(fs[0][i], lane + 8), top = shfl(north, 4 * cq + i);
+                fn = ry == 3 ? top : above;
+            }
+            const df32 aw = df_add(df_add(fw[i], df_neg(fw[i + 1])), df_add(fs[j][i], df_neg(fn)));
+            const df32 res = df_sub_acc(df32{b[2 * i], b[2 * i + 1]}, aw);
+            r[i] = __fadd_rn(res.hi, res.lo);
+            acc2 = fmaf(r[i], r[i], acc2);
+        }
+        st4(rout + base + gi + j * n, r);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc2 += __shfl_down_sync(0xffffffffu, acc2, o);
