@@ -596,6 +596,8 @@ __global__ void __launch_bounds__(256) k_resp(int N, int K, double* __restrict__
 // mean, with sum_n g_nj (x_n - c_j) and N_j, over one chunk of the particles (grid z): each thread
 // holds one 4 x 4 tile of the lower triangle (136 tiles at r = 64: 5 % more products than the triangle
 // itself; 32 x 32 tiles took 48 % more), 16 particles' deviations staged in shared memory per step.
+// 136 tiles are four warps and a quarter: the lanes of the partial warp divide each step's particles among
+// them, so that it costs the FP64 pipe a quarter of a warp (173 -> 154 us at N = 4096, K = 8, r = 64).
 // k_cov_finish adds the chunks in a fixed order.
 constexpr int COV_PN = 16;
 __host__ __device__ inline int cov_tiles(int r) { const int R = row_blocks(r); return R * (R + 1) / 2; }
@@ -615,7 +617,14 @@ __global__ void __launch_bounds__(256) k_cov_acc(int N, int r, const double* __r
     double* D = csm;                      // [COV_PN][rp] deviations
     double* Wd = D + COV_PN * rp;         // [COV_PN][rp] weighted deviations
     double* gs = Wd + COV_PN * rp;
-    const int t = blockIdx.x * 256 + tid, T = cov_tiles(r);
+    const int T = cov_tiles(r), base = T & ~31, left = T - base;
+    // a tile per thread; the last, partial warp's `left` tiles with S lanes each, which share a step's particles
+    int t = blockIdx.x * 256 + tid, S = 1, slice = 0;
+    if (left && (t & ~31) == base) {
+        while (2 * S * left <= 32 && 2 * S <= COV_PN) S *= 2;
+        slice = (tid & 31) / left;
+        t = slice < S ? base + (tid & 31) % left : T;
+    }
     int ta = 0, tb = 0;
     if (t < T) {
         ta = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
@@ -637,10 +646,11 @@ __global__ void __launch_bounds__(256) k_cov_acc(int N, int r, const double* __r
         }
         __syncthreads();
         if (t < T) {
+            const double *wa = Wd + slice * rp + 4 * ta, *db = D + slice * rp + 4 * tb;
 #pragma unroll 4
-            for (int p = 0; p < COV_PN; ++p) {
-                const double2 a01 = *reinterpret_cast<const double2*>(Wd + p * rp + 4 * ta), a23 = *reinterpret_cast<const double2*>(Wd + p * rp + 4 * ta + 2);
-                const double2 b01 = *reinterpret_cast<const double2*>(D + p * rp + 4 * tb), b23 = *reinterpret_cast<const double2*>(D + p * rp + 4 * tb + 2);
+            for (int p = slice; p < COV_PN; p += S, wa += S * rp, db += S * rp) {
+                const double2 a01 = *reinterpret_cast<const double2*>(wa), a23 = *reinterpret_cast<const double2*>(wa + 2);
+                const double2 b01 = *reinterpret_cast<const double2*>(db), b23 = *reinterpret_cast<const double2*>(db + 2);
                 const double a[4] = {a01.x, a01.y, a23.x, a23.y}, b[4] = {b01.x, b01.y, b23.x, b23.y};
 #pragma unroll
                 for (int x = 0; x < 4; ++x)
@@ -657,7 +667,12 @@ __global__ void __launch_bounds__(256) k_cov_acc(int N, int r, const double* __r
         __syncthreads();
     }
     double* out = part + ((size_t)j * nch + chunk) * cov_row(r);
-    if (t < T)
+    for (int h = S / 2; h > 0; h >>= 1)       // the slices of a tile (S differs from 1 in whole warps)
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) acc[x][y] += __shfl_down_sync(0xffffffffu, acc[x][y], h * left);
+    if (t < T && slice == 0)
 #pragma unroll
         for (int x = 0; x < 4; ++x)
 #pragma unroll
