@@ -684,40 +684,40 @@ __global__ void __launch_bounds__(256) k_cov_acc(int N, int r, const double* __r
 }
 
 // Adds the chunks and writes C_j (both triangles), its diagonal, m_j and the weights; a component with
-// N_j < 2 is re-seeded at the particle with the lowest largest responsibility.
+// N_j < 2 is re-seeded at the particle with the lowest largest responsibility.  Latency: every chunk is requested
+// before the first barrier (one sum after the other 35 us, so 19, caches cold).
 __global__ void __launch_bounds__(256) k_cov_finish(int N, int K, int r, int nch, const double* __restrict__ part, const double* __restrict__ gmax,
                                                     const double* __restrict__ xsT, const double* __restrict__ pooled,
                                                     const double* __restrict__ lamS, double floor_frac, double* __restrict__ w,
                                                     double* __restrict__ m, double* __restrict__ lam, double* __restrict__ cov) {
     // four threads per element (and per mode, component) share the chunks
-    __shared__ double dm[MAXR], s_nj[MAXK], s_v[256];
+    __shared__ double dm[MAXR], s_nj[MAXK], s_v[2 + MAXR / 64][256];
     __shared__ int s_i[256];
     const int j = blockIdx.y, tid = threadIdx.x, T = cov_tiles(r), cg = tid >> 6, el = tid & 63;
     const size_t row = cov_row(r);
     const double* pj = part + (size_t)j * nch * row;
-    auto chunk_sum = [&](const double* p0, bool on) {       // the sum over the chunks of p0[c * row], in the first 64 threads
+    auto partial = [&](const double* p0, bool on) {         // a quarter of the sum over the chunks of p0[c * row]
         double a = 0.0;
         if (on)
 #pragma unroll 5
             for (int c = cg; c < nch; c += 4) a += p0[c * row];
-        __syncthreads();
-        s_v[tid] = a;
-        __syncthreads();
-        return (s_v[el] + s_v[64 + el]) + (s_v[128 + el] + s_v[192 + el]);
+        return a;
     };
-    {
-        const double a = chunk_sum(part + (size_t)min(el, K - 1) * nch * row + (size_t)T * 16 + r, el < K);
-        if (tid < K) s_nj[tid] = a;
-        __syncthreads();
-    }
+    auto whole = [&](int k) { return (s_v[k][el] + s_v[k][64 + el]) + (s_v[k][128 + el] + s_v[k][192 + el]); };
+    const size_t e = (size_t)blockIdx.x * 64 + el;
+    // every load before the first barrier: the kernel is their latency
+    s_v[0][tid] = partial(part + (size_t)min(el, K - 1) * nch * row + (size_t)T * 16 + r, el < K);
+    s_v[1][tid] = partial(pj + e, e < (size_t)T * 16);
+    for (int k = 0; 64 * k < r; ++k) s_v[2 + k][tid] = partial(pj + (size_t)T * 16 + 64 * k + el, 64 * k + el < r);
+    __syncthreads();
+    if (tid < K) s_nj[tid] = whole(0);
+    __syncthreads();
     const double nj = s_nj[j];
     const bool low = nj < 2.0;
-    for (int m0 = 0; m0 < r; m0 += 64) {
-        const double a = chunk_sum(pj + (size_t)T * 16 + m0 + el, m0 + el < r);
-        if (tid < 64 && m0 + tid < r) dm[m0 + tid] = a / nj;
-    }
-    const size_t e = (size_t)blockIdx.x * 64 + el;
-    const double s = chunk_sum(pj + e, e < (size_t)T * 16);
+    if (tid < 64)
+        for (int k = 0; 64 * k + tid < r; ++k) dm[64 * k + tid] = whole(2 + k) / nj;
+    const double s = whole(1);
+    __syncthreads();
     if (tid < 64 && e < (size_t)T * 16) {
         const int t = (int)(e >> 4), q = (int)(e & 15);
         int ta = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
@@ -739,12 +739,12 @@ __global__ void __launch_bounds__(256) k_cov_finish(int N, int K, int r, int nch
         int bi = N;
         for (int n = tid; n < N; n += 256)
             if (gmax[n] < best) { best = gmax[n]; bi = n; }
-        s_v[tid] = best;
+        s_v[0][tid] = best;
         s_i[tid] = bi;
         __syncthreads();
         if (tid == 0)
             for (int k = 1; k < 256; ++k)
-                if (s_v[k] < s_v[0] || (s_v[k] == s_v[0] && s_i[k] < s_i[0])) { s_v[0] = s_v[k]; s_i[0] = s_i[k]; }
+                if (s_v[0][k] < s_v[0][0] || (s_v[0][k] == s_v[0][0] && s_i[k] < s_i[0])) { s_v[0][0] = s_v[0][k]; s_i[0] = s_i[k]; }
         __syncthreads();
         if (tid < r) m[(size_t)j * r + tid] = xsT[(size_t)tid * N + s_i[0]];
     } else if (tid < r) {
