@@ -380,9 +380,9 @@ __global__ void k_sum(int N, const double* __restrict__ a, double* __restrict__ 
 // An iteration is k_chol, k_estep_full, k_resp, k_cov_acc, k_cov_finish.  The E-step and the
 // contraction are N K r^2 / 2 FP64 multiply-adds each (108 us at N = 4096, K = 8, r = 64 on the
 // FP64 pipes), everything else should stay small beside them.  Measured per 50-iteration fit
-// there: 70.2 -> 22 ms (one block per particle reading rows of L^-1 uncoalesced 631 -> 150 us, FP64
-// pipe 76 % busy; the factor with its column sums in global memory 416 -> 79 us; the contraction on
-// 32 x 32 tiles 292 -> 173 us, FP64 pipe 87 %).
+// there: 70.2 -> 20.4 ms (one block per particle reading rows of L^-1 uncoalesced 631 -> 150 us, FP64
+// pipe 76 % busy: 1.7 warps per scheduler, so some have two; the factor with its column sums in global memory
+// 416 -> 71 us; the contraction on 32 x 32 tiles 292 -> 154 us, the pipe all but full).
 // ------------------------------------------------------------------------
 
 // Rows in blocks of four: block I holds L[4I + q][k] at 8 I (I + 1) + 4 k + q, k < 4 I + 4, with
@@ -393,11 +393,13 @@ __host__ __device__ inline int lb_size(int r) { const int R = row_blocks(r); ret
 size_t cov_lb_doubles(int K, int r) { return (size_t)K * lb_size(r) + K; }
 
 // Cholesky factor L_j (lower), log det L_j and the blocked rows above of every C_j, one block per
-// component, FP64: right-looking, W_ic -= W_ik W_ck / W_kk on the trailing triangle (all threads),
-// L_ik = W_ik / sqrt(W_kk) at the end; in shared memory while it fits (r <= CHOL_SMEM_R), else in
+// component, FP64: right-looking in panels of four columns, W_ic -= sum W_ik W_ck / W_kk on the trailing triangle (all
+// threads), L_ik = W_ik / sqrt(W_kk) at the end; in shared memory while it fits (r <= CHOL_SMEM_R), else in
 // L_j's own storage.  A pivot that is not positive (C_j not positive definite) sets *bad and counts
 // as 1 so the rest stays finite.  cst_j = log w_j - r/2 log(2 pi) - log det L_j when w is given.
-// Bound by the FP64 pipe of one SM (r^3 / 6 multiply-adds, 11 us at r = 64) and 2 r barriers.
+// Bound by the FP64 pipe of one SM and the pivots' chain: about 48 operations of 64 cycles per panel and
+// scheduler, then the update (r^3 / 6 multiply-adds, 11 us at r = 64).  With a column per step, two barriers
+// and a pivot chain each: 79 us at r = 64, K = 8; in panels 71.
 constexpr int CHOL_SMEM_R = 160;
 
 // 1 / d for a positive normal d to ~1 ulp: the hardware's approximate FP64 reciprocal (full exponent range) and two
@@ -413,52 +415,69 @@ __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ 
                                               double* __restrict__ Lb, double* __restrict__ logdet, double* __restrict__ cst,
                                               int* __restrict__ bad) {
     extern __shared__ __align__(16) double chsm[];
-    __shared__ double T[MAXR], rs[MAXR], red[32], s_rinv;
+    __shared__ double T[4][MAXR], rs[MAXR], red[32];
     const int j = blockIdx.x, tid = threadIdx.x;
     const size_t rr = (size_t)r * r;
     const double* A = cov + j * rr;
     double* Lj = L + j * rr;
     double* Wk = SMEM ? chsm : Lj;
     const int ws = SMEM ? r + 1 : r;
-    for (int e = tid; e < (int)rr; e += 256) {
-        const int i = e / r, c = e % r;
-        if (c <= i) Wk[i * ws + c] = A[e];
-    }
+    for (int i = tid >> 5; i < r; i += 8)
+        for (int c = tid & 31; c <= i; c += 32) Wk[i * ws + c] = A[i * r + c];
     __syncthreads();
     const int tx = tid & 15, ty = tid >> 4;
-    // the pivot's reciprocal is formed by the thread that finishes it, while the others update
-    auto pivot = [&](double d, int k) {
-        if (!(d > 0.0)) {
-            d = 1.0;
-            atomicExch(bad, 1);
-        }
-        rs[k] = d;
-        s_rinv = rcp_newton(d);
-    };
-    if (tid == 0) pivot(Wk[0], 0);
-    __syncthreads();
-    for (int k = 0; k < r; ++k) {
-        if (k + 1 + tid < r) T[k + 1 + tid] = Wk[(k + 1 + tid) * ws + k] * s_rinv;   // r <= 256 = the threads
-        __syncthreads();
-        if (tid == 0 && k + 1 < r) {                      // the next pivot first
-            const double v = fma(-Wk[(k + 1) * ws + k], T[k + 1], Wk[(k + 1) * ws + k + 1]);
-            Wk[(k + 1) * ws + k + 1] = v;
-            pivot(v, k + 1);
-        }
-        // rows from the longest down, four of a thread's elements at a time
-        for (int c0 = k + 1 + tx; c0 < r; c0 += 16) {
-            const double tc = T[c0];
-            int i = c0 + ((ty - c0) & 15);                // the first row >= c0 of this thread's rows (ty mod 16)
-            for (; i + 48 < r; i += 64) {
-                double w[4], v[4];
+    for (int k = 0; k < r; k += 4) {
+        // columns k .. k + 3 (beyond r: those of the identity): a thread per row eliminates the 4 x 4 diagonal block, then its row
+        const int ri = k + tid;                               // r <= 256 = the threads
+        double w[4];
+        if (ri < r) {
+            double d[4][4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) { w[q] = Wk[(i + 16 * q) * ws + k]; v[q] = Wk[(i + 16 * q) * ws + c0]; }
+            for (int a = 0; a < 4; ++a) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (q > 0 || i != k + 1) Wk[(i + 16 * q) * ws + c0] = fma(-w[q], tc, v[q]);
+                for (int b = 0; b <= a; ++b) d[a][b] = k + a < r ? Wk[(k + a) * ws + k + b] : a == b ? 1.0 : 0.0;
+                w[a] = a <= tid ? Wk[ri * ws + k + a] : 0.0;
             }
-            for (; i < r; i += 16)
-                if (i != k + 1) Wk[i * ws + c0] = fma(-Wk[i * ws + k], tc, Wk[i * ws + c0]);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const bool pos = d[c][c] > 0.0;
+                const double dc = pos ? d[c][c] : 1.0, rinv = rcp_newton(dc);
+                if (tid == 0 && k + c < r) {
+                    rs[k + c] = dc;
+                    if (!pos) atomicExch(bad, 1);
+                }
+#pragma unroll
+                for (int b = c + 1; b < 4; ++b) {
+                    const double tb = d[b][c] * rinv;
+#pragma unroll
+                    for (int a = b; a < 4; ++a) d[a][b] = fma(-d[a][c], tb, d[a][b]);
+                    w[b] = fma(-w[c], tb, w[b]);
+                }
+                T[c][ri] = w[c] * rinv;
+            }
+            if (tid >= 4)
+#pragma unroll
+                for (int a = 0; a < 4; ++a) Wk[ri * ws + k + a] = w[a];
+        }
+        __syncthreads();
+        if (tid < 4 && ri < r)                                // the diagonal block's rows, which every row's thread has read
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+                if (a <= tid) Wk[ri * ws + k + a] = w[a];
+        // the trailing triangle, two of a thread's elements at a time
+        for (int c0 = k + 4 + tx; c0 < r; c0 += 16) {
+            const double t0 = T[0][c0], t1 = T[1][c0], t2 = T[2][c0], t3 = T[3][c0];
+            auto upd = [&](int i) {
+                const double* q = Wk + i * ws + k;
+                return fma(-q[0], t0, fma(-q[1], t1, fma(-q[2], t2, fma(-q[3], t3, Wk[i * ws + c0]))));
+            };
+            int i = c0 + ((ty - c0) & 15);                    // the first row >= c0 of this thread's rows (ty mod 16)
+            for (; i + 16 < r; i += 32) {
+                const double u = upd(i), v = upd(i + 16);
+                Wk[i * ws + c0] = u;
+                Wk[(i + 16) * ws + c0] = v;
+            }
+            if (i < r) Wk[i * ws + c0] = upd(i);
         }
         __syncthreads();
     }
@@ -466,7 +485,7 @@ __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ 
     for (int k = tid; k < r; k += 256) {
         const double sq = sqrt(rs[k]);
         rs[k] = 1.0 / sq;
-        T[k] = sq;
+        T[0][k] = sq;
         ld += log(sq);
     }
     ld = block_sum(ld, red);                 // its barriers also publish rs and T
@@ -477,22 +496,21 @@ __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ 
     __syncthreads();
     double* Lbj = Lb + (size_t)j * lb_size(r);
     const int R = row_blocks(r);
-    for (int e = tid; e < 16 * R * R; e += 256) {
-        const int i = e / (4 * R), c = e % (4 * R);
-        if (c > (i | 3)) continue;
-        double v = 0.0;
-        if (c == i) v = i < r ? rs[i] : 1.0;
-        else if (c < i && i < r) v = Wk[i * ws + c] * rs[c];
-        Lbj[8 * (i >> 2) * ((i >> 2) + 1) + 4 * c + (i & 3)] = v;
-    }
+    for (int i = tid >> 5; i < 4 * R; i += 8)
+        for (int c = tid & 31; c <= (i | 3); c += 32) {
+            double v = 0.0;
+            if (c == i) v = i < r ? rs[i] : 1.0;
+            else if (c < i && i < r) v = Wk[i * ws + c] * rs[c];
+            Lbj[8 * (i >> 2) * ((i >> 2) + 1) + 4 * c + (i & 3)] = v;
+        }
     __syncthreads();
-    for (int e = tid; e < (int)rr; e += 256) {
-        const int i = e / r, c = e % r;
-        double v = 0.0;
-        if (c == i) v = T[i];
-        else if (c < i) v = Wk[i * ws + c] * rs[c];
-        Lj[e] = v;                            // in place when the work array is L_j itself
-    }
+    for (int i = tid >> 5; i < r; i += 8)
+        for (int c = tid & 31; c < r; c += 32) {
+            double v = 0.0;
+            if (c == i) v = T[0][i];
+            else if (c < i) v = Wk[i * ws + c] * rs[c];
+            Lj[i * r + c] = v;                // in place when the work array is L_j itself
+        }
 }
 
 // Forward substitution L y = rhs for 32 right-hand sides, one per lane; ys[i][lane] in shared memory,
