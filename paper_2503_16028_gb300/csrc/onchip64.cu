@@ -41,6 +41,11 @@ struct O6Args {
     double* W;
     GraphCounters* cnt;
     int* err;
+    const double* inv4;          // per particle: the dense inverse of the 4^2 level, 16 x 16
+    // the V-cycle alone: right-hand sides, corrections, the active particles
+    const double* vr;
+    double* ve;
+    const int *list, *nact;
 };
 
 // Shared memory, in doubles.
@@ -249,19 +254,21 @@ __device__ __forceinline__ bool sum6(double* sm, OcPos<M>& t, int slot, const do
     return false;
 }
 
-template <int C>
+// V: one V-cycle only, for the levels from 128^2 down of a larger grid's multi-pass solver.
+template <int C, bool V>
 __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
     using M = O6Mem<C>;
     extern __shared__ __align__(16) double sm6[];
     double* sm = sm6;
     constexpr int n = 64 * C;
-    const int p = blockIdx.x / M::CC;
+    if (V && A.nact && (int)(blockIdx.x / M::CC) >= *A.nact) return;
+    const int p = V ? A.list[blockIdx.x / M::CC] : (int)(blockIdx.x / M::CC);
     OcPos<M> t;
     oc_place(t, sm, Lev6<M, 0>::x(threadIdx.x), Lev6<M, 0>::y(threadIdx.x));
     const int gx = 2 * t.tx, gy = 2 * ((int)t.rank * M::H + t.ty);
     const size_t base = (size_t)p * n * n;
-    const double b2 = A.b2pp ? A.b2pp[p] : A.b2const;
-    double* W = A.W + base + (size_t)gy * n + gx;
+    const double b2 = V ? 1.0 : A.b2pp ? A.b2pp[p] : A.b2const;
+    double* W = (V ? A.ve : A.W) + base + (size_t)gy * n + gx;
     if (!(b2 > 0.0)) {                                      // not solved: w = 0 (the whole cluster alike)
         *reinterpret_cast<double2*>(W) = *reinterpret_cast<double2*>(W + n) = make_double2(0.0, 0.0);
         return;
@@ -273,21 +280,29 @@ __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
         const O6Level& L = A.lv[0];
         const double *Kw = L.Kw + base, *Ks = L.Ks + base, *inv = L.inv + base;
         const size_t c = (size_t)gy * n + gx;
+        auto two = [](const double* q) { return *reinterpret_cast<const double2*>(q); };
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            kw[3 * j] = Kw[c + j * n];
-            kw[3 * j + 1] = Kw[c + j * n + 1];
+            const double2 k = two(Kw + c + j * n), v = two(inv + c + j * n);
+            kw[3 * j] = k.x;
+            kw[3 * j + 1] = k.y;
             kw[3 * j + 2] = gx + 2 < n ? Kw[c + j * n + 2] : L.E[(size_t)p * n + gy + j];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) sm[M::INVF + (2 * j + i) * O6_T + t.tid] = inv[c + j * n + i];
+            sm[M::INVF + 2 * j * O6_T + t.tid] = v.x;
+            sm[M::INVF + (2 * j + 1) * O6_T + t.tid] = v.y;
         }
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
+        for (int j = 0; j < 3; ++j) {
+            const double2 k = two(gy + j < n ? Ks + c + (size_t)j * n : L.Nn + (size_t)p * n + gx);
+            ks[2 * j] = k.x;
+            ks[2 * j + 1] = k.y;
+        }
+        const double* B = V ? A.vr + base + c : A.b + (size_t)p * A.bstride + c;
 #pragma unroll
-            for (int i = 0; i < 2; ++i) ks[2 * j + i] = gy + j < n ? Ks[c + (size_t)j * n + i] : L.Nn[(size_t)p * n + gx + i];
-        const double* B = A.b + (size_t)p * A.bstride + c;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) r[k] = B[(k >> 1) * n + (k & 1)];
+        for (int j = 0; j < 2; ++j) {
+            const double2 v = two(B + j * n);
+            r[2 * j] = v.x;
+            r[2 * j + 1] = v.y;
+        }
     }
     // the coarser levels' faces: cell (x, y) of a level of side m
     auto load_level = [&](const O6Level& L, int m, int x, int y, double* f, int nt) {
@@ -303,34 +318,7 @@ __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
     constexpr int l16 = C == 1 ? 2 : 3;
     if (t.tid < 256) load_level(A.lv[l16], 16, Lev6<M, 16>::x(t.tid), Lev6<M, 16>::y(t.tid), sm + M::F16 + t.tid, 256);
     if (t.tid < 64) load_level(A.lv[l16 + 1], 8, Lev6<M, 8>::x(t.tid), Lev6<M, 8>::y(t.tid), sm + M::F8 + t.tid, 64);
-    // dense inverse of the 4^2 level by Gauss-Jordan elimination (symmetric positive definite: no pivoting), an entry
-    // per thread of the first 256
-    if (t.tid < 256) {
-        double* a = sm + M::RES;                             // 16 x 16 work matrix
-        const int i = t.tid >> 4, j = t.tid & 15;
-        {
-            const O6Level& L = A.lv[l16 + 2];
-            const int x = i & 3, y = i >> 2;
-            const size_t c = (size_t)p * 16 + i;
-            const double kE = x < 3 ? L.Kw[c + 1] : L.E[(size_t)p * 4 + y], kN = y < 3 ? L.Ks[c + 4] : L.Nn[(size_t)p * 4 + x];
-            double v = 0.0;
-            if (j == i) v = (L.Kw[c] + kE) + (L.Ks[c] + kN);
-            else if (j == i - 1 && x > 0) v = -L.Kw[c];
-            else if (j == i + 1 && x < 3) v = -kE;
-            else if (j == i - 4) v = -L.Ks[c];
-            else if (j == i + 4) v = -kN;
-            a[t.tid] = v;
-        }
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-#pragma unroll 1
-        for (int k = 0; k < 16; ++k) {
-            const double pv = 1.0 / a[17 * k], f = a[16 * i + k], rk = a[16 * k + j] * pv, v = a[t.tid];
-            asm volatile("bar.sync 1, 256;" ::: "memory");
-            a[t.tid] = i == k ? (j == k ? pv : rk) : (j == k ? -f * pv : fma(-f, rk, v));
-            asm volatile("bar.sync 1, 256;" ::: "memory");
-        }
-        sm[M::INV4 + t.tid] = 0.5 * (a[t.tid] + a[16 * j + i]);
-    }
+    if (t.tid < 256) sm[M::INV4 + t.tid] = A.inv4[(size_t)p * 256 + t.tid];
     oc_sync<C>();                                            // every block of the cluster runs, its mbarriers are ready
     const size_t pb = (size_t)blockIdx.x * 2 * O6_T + t.tid;   // this thread's patch rows in x, p and q
     double *HPL = sm + M::HPL, *P32 = sm + M::P32, *P16 = sm + M::P16, *P8 = sm + M::P8;
@@ -346,18 +334,22 @@ __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
         double thr = 0.0, rz = 0.0, al = 0.0;
         bool first = true, dead = false;
         for (;;) {
-            const double s[1] = {fma(r[0], r[0], r[1] * r[1]) + fma(r[2], r[2], r[3] * r[3])};
             e[0] = r[0] * sm[M::INVF + t.tid];
             e[3] = r[3] * sm[M::INVF + 3 * O6_T + t.tid];
             pub_f6(sm, t, 0, e);
-            if (!first) ++iters;
-            dead = sum6(sm, t, OC_RR, s, 8 * M::W, [&](const double (&v)[1]) {
-                const double rr = v[0];
-                if (first) thr = fmax(A.tol2 * rr, A.floor2 * b2);
-                SC[0] = first ? (rr > 0.0 ? 1.0 : 0.0) : (rr <= thr || iters >= A.maxit || !(rr == rr)) ? 0.0 : 1.0;
-            });
-            if (dead || SC[0] == 0.0) break;
-            if (first) ++inner;
+            if (V) {
+                nb_sync(sm, t, 8 * M::W);
+            } else {
+                const double s[1] = {fma(r[0], r[0], r[1] * r[1]) + fma(r[2], r[2], r[3] * r[3])};
+                if (!first) ++iters;
+                dead = sum6(sm, t, OC_RR, s, 8 * M::W, [&](const double (&v)[1]) {
+                    const double rr = v[0];
+                    if (first) thr = fmax(A.tol2 * rr, A.floor2 * b2);
+                    SC[0] = first ? (rr > 0.0 ? 1.0 : 0.0) : (rr <= thr || iters >= A.maxit || !(rr == rr)) ? 0.0 : 1.0;
+                });
+                if (dead || SC[0] == 0.0) break;
+                if (first) ++inner;
+            }
             // V-cycle: z = M r in e
             double nb0 = 0.0, nb3 = 0.0;                      // red cells: D e = r + nb
 #pragma unroll 1
@@ -454,6 +446,7 @@ __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
                 nb_sync(sm, t, 8 * M::W);
                 sweep_f6(sm, t, 0, kw, ks, r, e);
             }
+            if (V) break;
             // A z: r on the red cells, in flux form on the black ones
             pub_f6(sm, t, 0, e);
             nb_sync(sm, t, 8 * M::W);
@@ -499,6 +492,11 @@ __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
             r[2] = fma(-alpha, q1.x, r[2]); r[3] = fma(-alpha, q1.y, r[3]);
             first = false;
         }
+        if (V) {
+            *reinterpret_cast<double2*>(W) = make_double2(e[0], e[1]);
+            *reinterpret_cast<double2*>(W + n) = make_double2(e[2], e[3]);
+            break;
+        }
         // ---- w += x; residual b - A w in flux form, the neighbours' w through the finest planes ----
         ++phases;
         {
@@ -533,7 +531,7 @@ __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
         if (SC[0] == 1.0) { converged = true; break; }
         __syncthreads();                                     // SC[0] is read before the next phase writes it
     }
-    if (t.rank == 0 && t.tid == 0) {
+    if (!V && t.rank == 0 && t.tid == 0) {
         GraphCounters* g = A.cnt;
         atomicAdd(&g->cg_iterations, (unsigned long long)iters);
         atomicAdd(&g->inner_solves, (unsigned long long)inner);
@@ -545,9 +543,46 @@ __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
     if (C > 1) oc_sync<C>();                                  // no block leaves while another may still store into it
 }
 
-template <int C>
+// Dense inverses of the 4^2 level's operators, a warp per particle: lane l holds half a row, Gauss-Jordan
+// elimination (symmetric positive definite: no pivoting) by shuffles.  A block of the solver's 1024 threads took 15 us for
+// it, on one entry a thread; 14 operations a step of one warp cost the FP64 pipe an eighth of that.
+__global__ void __launch_bounds__(128) k_inv4(int count, const double* __restrict__ Kw, const double* __restrict__ Ks, const double* __restrict__ E,
+                                              const double* __restrict__ Nn, double* __restrict__ out) {
+    __shared__ double T[4][16][17];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, p = blockIdx.x * 4 + wp;
+    if (p >= count) return;
+    const int i = lane >> 1, h = lane & 1, x = i & 3, y = i >> 2, c = p * 16 + i;
+    const double kW = Kw[c], kS = Ks[c], kE = x < 3 ? Kw[c + 1] : E[p * 4 + y], kN = y < 3 ? Ks[c + 4] : Nn[p * 4 + x];
+    double a[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int j = 8 * h + q;
+        a[q] = j == i ? (kW + kE) + (kS + kN) : j == i - 1 && x > 0 ? -kW : j == i + 1 && x < 3 ? -kE : j == i - 4 ? -kS : j == i + 4 ? -kN : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        const double rp = 1.0 / __shfl_sync(0xffffffffu, a[k & 7], 2 * k + (k >> 3)), f = __shfl_sync(0xffffffffu, a[k & 7], 2 * i + (k >> 3));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const double rk = __shfl_sync(0xffffffffu, a[q], 2 * k + h) * rp;
+            const bool col = 8 * h + q == k;
+            a[q] = i == k ? (col ? rp : rk) : col ? -f * rp : fma(-f, rk, a[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) T[wp][i][8 * h + q] = a[q];
+    __syncwarp();
+    for (int k = lane; k < 256; k += 32) out[(size_t)p * 256 + k] = 0.5 * (T[wp][k >> 4][k & 15] + T[wp][k & 15][k >> 4]);
+}
+
+void launch_inv4(Ctx& c, int count) {
+    const LevelArrays<double>& L = c.s64.lv[c.s64.nlev - 3];
+    k_inv4<<<(count + 3) / 4, 128, 0, c.stream>>>(count, L.Kw, L.Ks, L.E, L.Nn, c.s64.inv4); ++c.pc.launches;
+}
+
+template <int C, bool V>
 static void o6_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int count, cudaStream_t st) {
-    check(cudaFuncSetAttribute(k_onchip64<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)O6Mem<C>::BYTES), "attr");
+    check(cudaFuncSetAttribute(k_onchip64<C, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)O6Mem<C>::BYTES), "attr");
     cfg = cudaLaunchConfig_t{};
     cfg.gridDim = dim3((unsigned)(count * C * C));
     cfg.blockDim = dim3(O6_T);
@@ -561,53 +596,81 @@ static void o6_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int co
     cfg.numAttrs = C > 1 ? 1 : 0;
 }
 
-// Whether the FP64 solves run on chip: 64^2 or 128^2, the sizes whose faces fit the registers of one block or of a
-// cluster of 4 with one block per SM (both measured faster than the passes from 2 particles to thousands, above).
-bool onchip64_supported(const Ctx& c) {
-    if (c.dim != 2 || mixed_precision(c.cfg) || c.cfg.tile_kernel != 0 || (c.n != 64 && c.n != 128)) return false;
+template <int C, bool V>
+static bool o6_fits() {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     int nc = 0;
-    if (c.n == 64) {
-        o6_config<1>(cfg, attr, 1, nullptr);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nc, k_onchip64<1>, O6_T, O6Mem<1>::BYTES) != cudaSuccess) nc = 0;
-    } else {
-        o6_config<2>(cfg, attr, 1, nullptr);
-        if (cudaOccupancyMaxActiveClusters(&nc, k_onchip64<2>, &cfg) != cudaSuccess) nc = 0;
+    o6_config<C, V>(cfg, attr, 1, nullptr);
+    if (C == 1) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nc, k_onchip64<C, V>, O6_T, O6Mem<C>::BYTES) != cudaSuccess) nc = 0;
+    } else if (cudaOccupancyMaxActiveClusters(&nc, k_onchip64<C, V>, &cfg) != cudaSuccess) {
+        nc = 0;
     }
     (void)cudaGetLastError();
     return nc > 0;
+}
+
+// Whether the FP64 solves run on chip: 64^2 or 128^2, the sizes whose faces fit the registers of one block or of a
+// cluster of 4 with one block per SM (both measured faster than the passes from 2 particles to thousands, above).
+bool onchip64_supported(const Ctx& c) {
+    if (c.dim != 2 || mixed_precision(c.cfg) || c.cfg.tile_kernel != 0) return false;
+    return c.n == 64 ? o6_fits<1, false>() : c.n == 128 && o6_fits<2, false>();
+}
+
+// Whether the multi-pass FP64 solver of a larger grid runs its levels from 128^2 down on chip: the cluster's V-cycle does 33 operations per cell
+// of 128^2 where the passes smooth 2.25 times the cells (256 particles of 256^2: 540 -> 395 us per V-cycle below 256^2).
+bool onchip64_vcycle_supported(const Ctx& c) {
+    return c.dim == 2 && !mixed_precision(c.cfg) && c.cfg.tile_kernel == 0 && c.n > 128 && o6_fits<2, true>();
+}
+
+template <int C, bool V>
+static void o6_launch(Ctx& c, O6Args& A, int top, int count) {
+    InnerSolver<double>& s = c.s64;
+    A.cc = c.cfg.coarse_scale;
+    A.nu_c = c.cfg.smooth_sweeps;
+    A.n = s.lv[top].n;
+    for (int l = 0; l < 6 && (A.n >> l) >= 4; ++l) {
+        const LevelArrays<double>& L = s.lv[top + l];
+        A.lv[l] = O6Level{L.Kw, L.Ks, L.E, L.Nn, L.inv};
+    }
+    A.inv4 = s.inv4;
+    A.err = c.dev_err;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    o6_config<C, V>(cfg, attr, count, c.stream);
+    check(cudaLaunchKernelEx(&cfg, k_onchip64<C, V>, A), "on-chip FP64 solve");
+    ++c.pc.launches;
 }
 
 // Solves a batch into W; the counters accumulate in c.gcnt.
 void solve_batch_onchip64(Ctx& c, int count, const Rhs& R, double* W) {
     InnerSolver<double>& s = c.s64;
     O6Args A{};
-    A.n = c.n; A.max_outer = c.cfg.max_refine < 2 ? 2 : c.cfg.max_refine; A.maxit = c.cfg.max_iter;
-    A.nu_f = c.cfg.fine_sweeps; A.nu_c = c.cfg.smooth_sweeps;
-    A.cc = c.cfg.coarse_scale;
+    A.max_outer = c.cfg.max_refine < 2 ? 2 : c.cfg.max_refine; A.maxit = c.cfg.max_iter;
+    A.nu_f = c.cfg.fine_sweeps;
     A.tol2 = A.tolout2 = c.cfg.tol_outer * c.cfg.tol_outer;
     A.floor2 = 0.25 * A.tolout2;
     A.b2const = R.b2const; A.b2pp = R.b2pp;
-    for (int l = 0; l < 6 && (c.n >> l) >= 4; ++l) {
-        const LevelArrays<double>& L = s.lv[l];
-        A.lv[l] = O6Level{L.Kw, L.Ks, L.E, L.Nn, L.inv};
-    }
     A.b = R.b64; A.bstride = R.stride;
     A.x = reinterpret_cast<double2*>(s.x); A.p = reinterpret_cast<double2*>(s.p[0]); A.q = reinterpret_cast<double2*>(s.q);
     A.W = W;
     A.cnt = c.gcnt;
-    A.err = c.dev_err;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[1];
-    if (c.n == 64) {
-        o6_config<1>(cfg, attr, count, c.stream);
-        check(cudaLaunchKernelEx(&cfg, k_onchip64<1>, A), "on-chip FP64 solve");
-    } else {
-        o6_config<2>(cfg, attr, count, c.stream);
-        check(cudaLaunchKernelEx(&cfg, k_onchip64<2>, A), "on-chip FP64 solve");
-    }
-    ++c.pc.launches;
+    if (c.n == 64) o6_launch<1, false>(c, A, 0, count);
+    else o6_launch<2, false>(c, A, 0, count);
+}
+
+// The V-cycle from the level of 128^2 down (r to e2 there) for the active particles.
+void launch_vcycle64(Ctx& c, int level, int nact) {
+    InnerSolver<double>& s = c.s64;
+    O6Args A{};
+    A.max_outer = 1;
+    A.nu_f = c.cfg.smooth_sweeps;
+    A.vr = s.lv[level].r;
+    A.ve = s.lv[level].e2;
+    A.list = s.list;
+    A.nact = c.graph ? s.nact : nullptr;
+    o6_launch<2, true>(c, A, level, nact);
 }
 
 }  // namespace smcgm

@@ -141,6 +141,7 @@ struct InnerSolver {
     std::vector<LevelArrays<T>> lv;
     T *r[2] = {nullptr, nullptr}, *p[2] = {nullptr, nullptr};
     T *x = nullptr, *q = nullptr, *z = nullptr;
+    T* inv4 = nullptr;       // FP64: dense inverses of the 4 x 4 level's operators (256 per particle), for onchip64.cu
 };
 
 struct Partials { double *rr, *rz, *pq, *res; int ntiles; };
@@ -178,6 +179,9 @@ bool onchip_supported(const Ctx& c);
 void solve_batch_onchip(Ctx& c, int count, const Rhs& R, double* W);
 bool onchip64_supported(const Ctx& c);   // onchip64.cu: the FP64 solver's part of the two
 void solve_batch_onchip64(Ctx& c, int count, const Rhs& R, double* W);
+bool onchip64_vcycle_supported(const Ctx& c);
+void launch_vcycle64(Ctx& c, int level, int nact);
+void launch_inv4(Ctx& c, int count);
 void forward_solve_graph(Ctx& c, const double* X, int count, double* Phi_out);   // into the graph being captured
 void capture_move_steps(Ctx& c, int steps, int* acc_count);                      // into the graph being captured
 void launch_mark_out_of_range(Ctx& c, int count, double* Phi);
@@ -286,6 +290,7 @@ struct Ctx {
     cudaStream_t gaux[4] = {nullptr, nullptr, nullptr, nullptr};
     GraphCounters* gcnt = nullptr;    // device counters of graph-mode and on-chip solves
     bool onchip = false;              // the solves run in onchip.cu's kernel (decided at smc_init)
+    bool vchip = false;               // FP64 passes: the levels from 128^2 down in onchip64.cu's V-cycle (decided at smc_init)
     bool onchip_open = false;         // an OnchipCounters scope is collecting their counters
     int* gouter = nullptr;            // device: [0] refinement phase, [1] particles entering it
     MoveSched* msched = nullptr;      // device schedule of a graph-mode move

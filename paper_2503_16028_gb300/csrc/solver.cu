@@ -1269,12 +1269,18 @@ struct Passes {
             if (c.cfg.smooth_sweeps == 2) run_vcycle_lower<T, 2>(c, s, nact);
             else run_vcycle_lower<T, 1>(c, s, nact);
         } else if (path == 2) {
-            for (int l = 1; l < s.ntile_levels; ++l) {
+            // the levels of the tiled passes; from 128^2 down in one launch on chip where the FP64 solver may
+            const bool chip = sizeof(T) == 8 && c.vchip;
+            int top = s.ntile_levels;
+            if (chip)
+                for (top = 1; s.lv[top].n > 128;) ++top;
+            for (int l = 1; l < top; ++l) {
                 if (level_halo(c, l) == 4) launch_wpre<T, 4>(c, s, l, nact, s.lv[l].r, nullptr, 0, 0, nullptr);
                 else launch_wpre<T, 2>(c, s, l, nact, s.lv[l].r, nullptr, 0, 0, nullptr);
             }
-            launch_coarse<T>(c, s, nact);
-            for (int l = s.ntile_levels - 1; l >= 1; --l) {
+            if (chip) launch_vcycle64(c, top, nact);
+            else launch_coarse<T>(c, s, nact);
+            for (int l = top - 1; l >= 1; --l) {
                 if (level_halo(c, l) == 4) launch_wpost<T, 4>(c, s, l, nact, s.lv[l].r, s.lv[l].e2, 0);
                 else launch_wpost<T, 2>(c, s, l, nact, s.lv[l].r, s.lv[l].e2, 0);
             }
@@ -1414,6 +1420,7 @@ void launch_coarsen_all(Ctx& c, InnerSolver<T>& s, int count) {
             const size_t total = (size_t)A.n * A.n * count;
             k_inv_diag<T><<<grid_for(total), 256, 0, c.stream>>>(A.n, total, A.Kw, A.Ks, A.E, A.Nn, A.inv); ++c.pc.launches;
         }
+    if (sizeof(T) == 8 && (c.onchip || c.vchip)) launch_inv4(c, count);
 }
 template void launch_coarsen_all<float>(Ctx&, InnerSolver<float>&, int);
 template void launch_coarsen_all<double>(Ctx&, InnerSolver<double>&, int);

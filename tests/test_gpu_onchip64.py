@@ -71,3 +71,30 @@ def test_particles_do_not_depend_on_their_batch(n, N):
         out.append(s.particles())
         s.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("n,fine,coarse", [(256, 1, 2), (256, 2, 1)])
+def test_vcycle_below_the_passes(n, fine, coarse):
+    """Larger grids run their levels from 128^2 down on chip: the solution against the oracle, and a captured move
+    (ragged solve batches of 3) bit for bit against the host loop's."""
+    wl = dict(inputs.load_workload("darcy64_bimodal"), n=n)
+    pair = [smcgm.Sampler(smcgm.make_config(wl, n_particles=7, n_components=1, gm_rank=4, precision=0, solve_batch=3, fine_sweeps=fine,
+                                            smooth_sweeps=coarse)) for _ in range(2)]
+    for s in pair:
+        s.smc_temper_step()
+        s.smc_resample()
+        s.gm_fit()
+    X, _ = pair[0].particles()
+    W = torch.empty(7, n * n, dtype=torch.float64, device="cuda")
+    P = torch.empty(7, dtype=torch.float64, device="cuda")
+    pair[0].smc_forward(torch.tensor(X, device="cuda"), P, W)
+    w = oproblem.from_workload(wl).solve(X[5]).reshape(-1)
+    assert _rel(W[5].cpu().numpy(), w) < 1e-10
+    b = smcgm.Batch([pair[1]], steps=1)
+    acc, _ = pair[0].smc_move(1)
+    assert b.move()[0] == acc
+    for u, v in zip(pair[0].particles(), pair[1].particles()):
+        assert np.array_equal(u, v)
+    b.close()
+    for s in pair:
+        s.close()
