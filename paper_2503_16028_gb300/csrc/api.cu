@@ -126,7 +126,7 @@ static void plan_inner(Planner& P, InnerSolver<T>& s, int n, int B, int coarse_t
     s.r[0] = P.take<T>(nn); s.r[1] = P.take<T>(nn);
     s.p[0] = P.take<T>(nn); s.p[1] = P.take<T>(nn);
     s.x = P.take<T>(nn); s.q = P.take<T>(nn); s.z = P.take<T>(nn);
-    if (sizeof(T) == 8) s.inv4 = P.take<T>((size_t)256 * B);
+    if (sizeof(T) == 8 || n > 256) s.binv = P.take<T>((size_t)(sizeof(T) == 8 ? 256 : 4096) * B);
 }
 
 // Lays out every device array; with base == nullptr only sizes them.
@@ -496,7 +496,7 @@ smc_status smc_init(const smc_config* cfg, void* d_ws, size_t bytes, void* strea
         if (mixed_precision(c.cfg)) build_tma_maps<float>(c, c.s32);
         else build_tma_maps<double>(c, c.s64);
         c.onchip = onchip_supported(c);
-        c.vchip = onchip64_vcycle_supported(c);
+        c.vchip = vcycle_supported(c);
     }
     set_prior_mixture(c);
     c.fitted = (c.cfg.kernel == SMC_K_PCN || c.cfg.kernel == SMC_K_PCNL);

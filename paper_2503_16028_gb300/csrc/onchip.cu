@@ -54,6 +54,11 @@ struct OcArgs {
     const int* badp;
     GraphCounters* cnt;
     int* err;
+    // the V-cycle alone: right-hand sides, corrections, the active particles, the 8^2 level's dense inverses (`build`: form them)
+    const float* vr;
+    float *ve, *inv8;
+    const int *list, *nact;
+    int build;
 };
 
 // A block covers 64 C x 64 / C cells (a strip of rows): W x H threads, a 4 x 4 patch each.
@@ -532,21 +537,23 @@ __device__ __forceinline__ double tri_to_double(float h, float m, float l, int a
     return I ? __hiloint2double(__double2hiint(d) + ((eh - 186 + add) << 20), __double2loint(d)) : 0.0;
 }
 
-// One particle per cluster of C x C blocks, n = 64 C.
-template <int C>
+// One particle per cluster of C x C blocks, n = 64 C.  V: one V-cycle only, for the levels from n down of a larger grid's
+// multi-pass solver (or, at set-up, only the dense inverse that it uses).
+template <int C, bool V>
 __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     using M = OcMem<C>;
     extern __shared__ __align__(16) float sm[];
     const int n = 64 * C;
-    const int p = blockIdx.x / M::CC;
+    if (V && A.nact && (int)(blockIdx.x / M::CC) >= *A.nact) return;
+    const int p = V && A.list ? A.list[blockIdx.x / M::CC] : (int)(blockIdx.x / M::CC);
     OcPos<OcMem<C>> t;
     oc_place(t, sm, (int)threadIdx.x % M::W, (int)threadIdx.x / M::W);
     t.lx = t.tid & 15;
     t.ly = t.tid >> 4;
     const int gx = 4 * t.tx, gy = 4 * ((int)t.rank * M::H + t.ty);
     const size_t base = (size_t)p * n * n;
-    const double b2 = A.b2pp ? A.b2pp[p] : A.b2const;
-    if (!(b2 > 0.0) || (A.badp && A.badp[p])) {             // not solved: w = 0 (the whole cluster alike)
+    const double b2 = V ? 1.0 : A.b2pp ? A.b2pp[p] : A.b2const;
+    if (!V && (!(b2 > 0.0) || (A.badp && A.badp[p]))) {             // not solved: w = 0 (the whole cluster alike)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             double2* o = reinterpret_cast<double2*>(A.W + base + (size_t)(gy + j) * n + gx);
@@ -643,19 +650,38 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             sf[0] = k16.w; sf[OC_T] = k16.e; sf[2 * OC_T] = k16.s; sf[3 * OC_T] = k16.n;
             const Cell1 k8 = coarse_faces(k16, t.lx, t.ly);
             __syncthreads();
-            build_inv8<C>(sm, t, k8);
+            if (V && !A.build) {
+                const float4* g = reinterpret_cast<const float4*>(A.inv8 + (size_t)p * 4096);
+                for (int i = t.tid; i < 1024; i += OC_T) reinterpret_cast<float4*>(sm + M::INV8)[i] = g[i];
+                __syncthreads();
+            } else {
+                build_inv8<C>(sm, t, k8);
+            }
         }
     }
+    if (V && A.build) {
+        if (t.rank == 0)
+            for (int i = t.tid; i < 4096; i += OC_T) A.inv8[(size_t)p * 4096 + i] = sm[M::INV8 + i];
+        if (t.polls == 0) atomicExch(A.err, 1);
+        oc_sync<C>();
+        return;
+    }
     // r = scaled b
-    const float2* B = A.bdf + (size_t)p * A.bstride;
+    const float2* B = V ? nullptr : A.bdf + (size_t)p * A.bstride;
     float r[16], e[16];
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < 4; ++j) {
+        if (V) {
+            const float4 v = *reinterpret_cast<const float4*>(A.vr + base + (size_t)(gy + j) * n + gx);
+            r[4 * j] = v.x; r[4 * j + 1] = v.y; r[4 * j + 2] = v.z; r[4 * j + 3] = v.w;
+            continue;
+        }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float2 v = B[(size_t)(gy + j) * n + gx + i];
             r[4 * j + i] = __fadd_rn(v.x, v.y) * scale;
         }
+    }
     const size_t pb = (size_t)blockIdx.x * 4 * OC_T + t.tid;   // this thread's patch rows in x, wh, wm, wl
     int iters = 0, phases = 0, inner = 0;
     bool converged = false, wset = false;
@@ -666,20 +692,26 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
         bool first = true;
         for (;;) {
             float s = 0.f;
+            if (!V) {
 #pragma unroll
-            for (int c = 0; c < 16; ++c) s = fmaf(r[c], r[c], s);
-            red_put<C>(sm, t, 0, s);
+                for (int c = 0; c < 16; ++c) s = fmaf(r[c], r[c], s);
+                red_put<C>(sm, t, 0, s);
+            }
             sweep_f<C, 0>(sm, t, kw, ks, r, e, true);
             pub_f<C, 0>(sm, t, e);
-            if (rr_sync<C>(sm, t)) break;
-            const float rr = red_get<C>(sm, t, 0);
-            if (first) {
-                thr = fmaxf(A.tol2 * rr, A.floor2 * b2s);
-                if (!(rr > 0.f)) break;
-                ++inner;
+            if (V) {
+                nb_sync(sm, t, 8 * M::W);
             } else {
-                ++iters;
-                if (rr <= thr || iters >= A.maxit || !(rr == rr)) break;
+                if (rr_sync<C>(sm, t)) break;
+                const float rr = red_get<C>(sm, t, 0);
+                if (first) {
+                    thr = fmaxf(A.tol2 * rr, A.floor2 * b2s);
+                    if (!(rr > 0.f)) break;
+                    ++inner;
+                } else {
+                    ++iters;
+                    if (rr <= thr || iters >= A.maxit || !(rr == rr)) break;
+                }
             }
             // V-cycle: z = M r in e
 #pragma unroll 1
@@ -784,6 +816,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                 nb_sync(sm, t, 8 * M::W);
                 sweep_f<C, 0>(sm, t, kw, ks, r, e, false);
             }
+            if (V) break;
             // beta, p = z + beta p
             s = 0.f;
 #pragma unroll
@@ -848,6 +881,12 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
 #pragma unroll
             for (int c = 0; c < 16; ++c) r[c] = fmaf(-alpha, q[c], r[c]);
             first = false;
+        }
+        if (V) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                *reinterpret_cast<float4*>(A.ve + base + (size_t)(gy + j) * n + gx) = make_float4(e[4 * j], e[4 * j + 1], e[4 * j + 2], e[4 * j + 3]);
+            break;
         }
         // ---- w += x; FP64-accurate residual ----
         ++phases;
@@ -947,14 +986,14 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
         if (res2 <= A.tolout2 * b2s) { converged = true; break; }
     }
 #pragma unroll 1
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; !V && j < 4; ++j) {
         const size_t at = pb + j * OC_T;
         const float4 h = A.wh[at], m = A.wm[at], l = A.wl[at];
         double2* o = reinterpret_cast<double2*>(A.W + base + (size_t)(gy + j) * n + gx);
         o[0] = make_double2(tri_to_double(h.x, m.x, l.x, -sexp), tri_to_double(h.y, m.y, l.y, -sexp));
         o[1] = make_double2(tri_to_double(h.z, m.z, l.z, -sexp), tri_to_double(h.w, m.w, l.w, -sexp));
     }
-    if (t.rank == 0 && t.tid == 0) {
+    if (!V && t.rank == 0 && t.tid == 0) {
         GraphCounters* g = A.cnt;
         atomicAdd(&g->cg_iterations, (unsigned long long)iters);
         atomicAdd(&g->inner_solves, (unsigned long long)inner);
@@ -966,10 +1005,10 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     if (C > 1) oc_sync<C>();                                    // no block leaves while another may still store into it
 }
 
-template <int C>
+template <int C, bool V>
 static void oc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int count, cudaStream_t st) {
-    check(cudaFuncSetAttribute(k_onchip<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OcMem<C>::BYTES), "attr");
-    if (C == 4) check(cudaFuncSetAttribute(k_onchip<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "attr");
+    check(cudaFuncSetAttribute(k_onchip<C, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OcMem<C>::BYTES), "attr");
+    if (C == 4) check(cudaFuncSetAttribute(k_onchip<C, V>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "attr");
     cfg = cudaLaunchConfig_t{};
     cfg.gridDim = dim3((unsigned)(count * C * C));
     cfg.blockDim = dim3(OC_T);
@@ -983,15 +1022,15 @@ static void oc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int co
     cfg.numAttrs = C > 1 ? 1 : 0;
 }
 
-template <int C>
+template <int C, bool V>
 static bool oc_fits() {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    oc_config<C>(cfg, attr, 1, nullptr);
+    oc_config<C, V>(cfg, attr, 1, nullptr);
     int nc = 0;
     if (C == 1) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nc, k_onchip<C>, OC_T, OcMem<C>::BYTES) != cudaSuccess) nc = 0;
-    } else if (cudaOccupancyMaxActiveClusters(&nc, k_onchip<C>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nc, k_onchip<C, V>, OC_T, OcMem<C>::BYTES) != cudaSuccess) nc = 0;
+    } else if (cudaOccupancyMaxActiveClusters(&nc, k_onchip<C, V>, &cfg) != cudaSuccess) {
         nc = 0;
     }
     (void)cudaGetLastError();
@@ -1004,18 +1043,29 @@ static bool oc_fits() {
 bool onchip_supported(const Ctx& c) {
     if (c.dim != 2 || c.cfg.tile_kernel != 0) return false;
     if (!mixed_precision(c.cfg)) return onchip64_supported(c);
-    if (c.n == 64) return oc_fits<1>();
-    if (c.n == 128) return oc_fits<2>();
-    if (c.n == 256) return oc_fits<4>();
+    if (c.n == 64) return oc_fits<1, false>();
+    if (c.n == 128) return oc_fits<2, false>();
+    if (c.n == 256) return oc_fits<4, false>();
     return false;
 }
 
-template <int C>
+// Whether the mixed-precision multi-pass solver of a larger grid (512^2) runs its levels from 128^2 down on chip: per V-cycle
+// of 250 particles 126 us in five launches, which smooth 2.25 times the cells they own, and 50 in one.  Not from 256^2
+// down: 14 clusters of 16 at a time would take longer (about 430 us) than its two passes and this (310).
+static bool onchip32_vcycle_supported(const Ctx& c) { return c.n > 256 && oc_fits<2, true>(); }
+
+// Whether the passes of a larger grid's solver leave the levels from 128^2 down to launch_vcycle.
+bool vcycle_supported(const Ctx& c) {
+    if (c.dim != 2 || c.cfg.tile_kernel != 0 || c.onchip) return false;
+    return mixed_precision(c.cfg) ? onchip32_vcycle_supported(c) : onchip64_vcycle_supported(c);
+}
+
+template <int C, bool V>
 static void oc_launch(Ctx& c, const OcArgs& A, int count) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    oc_config<C>(cfg, attr, count, c.stream);
-    check(cudaLaunchKernelEx(&cfg, k_onchip<C>, A), "on-chip solve"); ++c.pc.launches;
+    oc_config<C, V>(cfg, attr, count, c.stream);
+    check(cudaLaunchKernelEx(&cfg, k_onchip<C, V>, A), "on-chip solve"); ++c.pc.launches;
 }
 
 static void solve_batch_onchip32(Ctx& c, int count, const Rhs& R, double* W) {
@@ -1037,9 +1087,39 @@ static void solve_batch_onchip32(Ctx& c, int count, const Rhs& R, double* W) {
     A.badp = c.lenient ? c.badp : nullptr;
     A.cnt = c.gcnt;
     A.err = c.dev_err;
-    if (c.n == 64) oc_launch<1>(c, A, count);
-    else if (c.n == 128) oc_launch<2>(c, A, count);
-    else oc_launch<4>(c, A, count);
+    if (c.n == 64) oc_launch<1, false>(c, A, count);
+    else if (c.n == 128) oc_launch<2, false>(c, A, count);
+    else oc_launch<4, false>(c, A, count);
+}
+
+// The V-cycle from the level of 128^2 down (r to e2 there) for the active particles; with `build` the dense
+// inverses of the 8^2 level that it uses, for the first `nact` particles.
+static void vcycle32(Ctx& c, int level, int nact, bool build) {
+    InnerSolver<float>& s = c.s32;
+    LevelArrays<float>& f = s.lv[level];
+    OcArgs A{};
+    A.n = f.n; A.max_outer = 1; A.nu_f = A.nu_c = c.cfg.smooth_sweeps;
+    A.cc = (float)c.cfg.coarse_scale;
+    A.Kw = f.Kw; A.Ks = f.Ks; A.E = f.E; A.Nn = f.Nn;
+    A.vr = f.r; A.ve = f.e2; A.inv8 = s.binv;
+    A.build = build;
+    if (!build) {
+        A.list = s.list;
+        A.nact = c.graph ? s.nact : nullptr;
+    }
+    A.err = c.dev_err;
+    oc_launch<2, true>(c, A, nact);
+}
+void launch_vcycle(Ctx& c, InnerSolver<float>&, int level, int nact) { vcycle32(c, level, nact, false); }
+void launch_vcycle(Ctx& c, InnerSolver<double>&, int level, int nact) { launch_vcycle64(c, level, nact); }
+// At set-up, after the coarser levels: the dense inverses of the on-chip solvers' smallest level.
+void launch_dense_inverses(Ctx& c, InnerSolver<double>&, int count) {
+    if (c.onchip || c.vchip) launch_inv4(c, count);
+}
+void launch_dense_inverses(Ctx& c, InnerSolver<float>& s, int count) {
+    int l = 0;
+    while (s.lv[l].n > 128) ++l;
+    if (c.vchip) vcycle32(c, l, count, true);
 }
 
 // Solves a batch into W; the counters accumulate in c.gcnt (OnchipCounters reads them).

@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(128) k_inv4(int count, const double* __restric
 
 void launch_inv4(Ctx& c, int count) {
     const LevelArrays<double>& L = c.s64.lv[c.s64.nlev - 3];
-    k_inv4<<<(count + 3) / 4, 128, 0, c.stream>>>(count, L.Kw, L.Ks, L.E, L.Nn, c.s64.inv4); ++c.pc.launches;
+    k_inv4<<<(count + 3) / 4, 128, 0, c.stream>>>(count, L.Kw, L.Ks, L.E, L.Nn, c.s64.binv); ++c.pc.launches;
 }
 
 template <int C, bool V>
@@ -621,7 +621,7 @@ bool onchip64_supported(const Ctx& c) {
 // Whether the multi-pass FP64 solver of a larger grid runs its levels from 128^2 down on chip: the cluster's V-cycle does 33 operations per cell
 // of 128^2 where the passes smooth 2.25 times the cells (256 particles of 256^2: 540 -> 395 us per V-cycle below 256^2).
 bool onchip64_vcycle_supported(const Ctx& c) {
-    return c.dim == 2 && !mixed_precision(c.cfg) && c.cfg.tile_kernel == 0 && c.n > 128 && o6_fits<2, true>();
+    return c.n > 128 && o6_fits<2, true>();
 }
 
 template <int C, bool V>
@@ -634,7 +634,7 @@ static void o6_launch(Ctx& c, O6Args& A, int top, int count) {
         const LevelArrays<double>& L = s.lv[top + l];
         A.lv[l] = O6Level{L.Kw, L.Ks, L.E, L.Nn, L.inv};
     }
-    A.inv4 = s.inv4;
+    A.inv4 = s.binv;
     A.err = c.dev_err;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];

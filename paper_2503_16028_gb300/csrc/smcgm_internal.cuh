@@ -141,7 +141,7 @@ struct InnerSolver {
     std::vector<LevelArrays<T>> lv;
     T *r[2] = {nullptr, nullptr}, *p[2] = {nullptr, nullptr};
     T *x = nullptr, *q = nullptr, *z = nullptr;
-    T* inv4 = nullptr;       // FP64: dense inverses of the 4 x 4 level's operators (256 per particle), for onchip64.cu
+    T* binv = nullptr;       // dense inverses of the on-chip solvers' smallest level (FP64: 4^2; FP32, grids above 256^2: 8^2)
 };
 
 struct Partials { double *rr, *rz, *pq, *res; int ntiles; };
@@ -182,6 +182,12 @@ void solve_batch_onchip64(Ctx& c, int count, const Rhs& R, double* W);
 bool onchip64_vcycle_supported(const Ctx& c);
 void launch_vcycle64(Ctx& c, int level, int nact);
 void launch_inv4(Ctx& c, int count);
+// the multi-pass solvers' levels from 128^2 down in one launch (onchip.cu, onchip64.cu)
+bool vcycle_supported(const Ctx& c);
+void launch_vcycle(Ctx& c, InnerSolver<float>& s, int level, int nact);
+void launch_vcycle(Ctx& c, InnerSolver<double>& s, int level, int nact);
+void launch_dense_inverses(Ctx& c, InnerSolver<float>& s, int count);
+void launch_dense_inverses(Ctx& c, InnerSolver<double>& s, int count);
 void forward_solve_graph(Ctx& c, const double* X, int count, double* Phi_out);   // into the graph being captured
 void capture_move_steps(Ctx& c, int steps, int* acc_count);                      // into the graph being captured
 void launch_mark_out_of_range(Ctx& c, int count, double* Phi);
@@ -290,7 +296,7 @@ struct Ctx {
     cudaStream_t gaux[4] = {nullptr, nullptr, nullptr, nullptr};
     GraphCounters* gcnt = nullptr;    // device counters of graph-mode and on-chip solves
     bool onchip = false;              // the solves run in onchip.cu's kernel (decided at smc_init)
-    bool vchip = false;               // FP64 passes: the levels from 128^2 down in onchip64.cu's V-cycle (decided at smc_init)
+    bool vchip = false;               // the passes leave the levels from 128^2 down to launch_vcycle (decided at smc_init)
     bool onchip_open = false;         // an OnchipCounters scope is collecting their counters
     int* gouter = nullptr;            // device: [0] refinement phase, [1] particles entering it
     MoveSched* msched = nullptr;      // device schedule of a graph-mode move

@@ -1236,6 +1236,14 @@ static int tile_path(const Ctx& c, bool fp32) {
     return path;
 }
 
+// The first level below the tiled passes: the coarse kernel's, or 128^2 where the rest of the V-cycle runs on chip.
+template <typename T>
+static int lower_top(const Ctx& c, const InnerSolver<T>& s) {
+    int top = c.vchip ? 1 : s.ntile_levels;
+    while (c.vchip && s.lv[top].n > 128) ++top;
+    return top;
+}
+
 // The passes of one CG iteration on the finest level and the V-cycle below it.
 template <typename T>
 struct Passes {
@@ -1269,16 +1277,12 @@ struct Passes {
             if (c.cfg.smooth_sweeps == 2) run_vcycle_lower<T, 2>(c, s, nact);
             else run_vcycle_lower<T, 1>(c, s, nact);
         } else if (path == 2) {
-            // the levels of the tiled passes; from 128^2 down in one launch on chip where the FP64 solver may
-            const bool chip = sizeof(T) == 8 && c.vchip;
-            int top = s.ntile_levels;
-            if (chip)
-                for (top = 1; s.lv[top].n > 128;) ++top;
+            const int top = lower_top(c, s);
             for (int l = 1; l < top; ++l) {
                 if (level_halo(c, l) == 4) launch_wpre<T, 4>(c, s, l, nact, s.lv[l].r, nullptr, 0, 0, nullptr);
                 else launch_wpre<T, 2>(c, s, l, nact, s.lv[l].r, nullptr, 0, 0, nullptr);
             }
-            if (chip) launch_vcycle64(c, top, nact);
+            if (c.vchip) launch_vcycle(c, s, top, nact);
             else launch_coarse<T>(c, s, nact);
             for (int l = top - 1; l >= 1; --l) {
                 if (level_halo(c, l) == 4) launch_wpost<T, 4>(c, s, l, nact, s.lv[l].r, s.lv[l].e2, 0);
@@ -1322,12 +1326,14 @@ static void staged_lower(Ctx& c, InnerSolver<float>& s, int nact) {
     // The coarser tiled levels keep the warp kernels loading from global memory:
     // without the CG vectors their registers allow 16 warps per SM, which
     // measured faster than the staged form there.
-    for (int l = 1; l < s.ntile_levels; ++l) {
+    const int top = lower_top(c, s);
+    for (int l = 1; l < top; ++l) {
         if (level_halo(c, l) == 4) launch_wpre<float, 4>(c, s, l, nact, s.lv[l].r, nullptr, 0, 0, nullptr);
         else launch_wpre<float, 2>(c, s, l, nact, s.lv[l].r, nullptr, 0, 0, nullptr);
     }
-    launch_coarse<float>(c, s, nact);
-    for (int l = s.ntile_levels - 1; l >= 1; --l) {
+    if (c.vchip) launch_vcycle(c, s, top, nact);
+    else launch_coarse<float>(c, s, nact);
+    for (int l = top - 1; l >= 1; --l) {
         if (level_halo(c, l) == 4) launch_wpost<float, 4>(c, s, l, nact, s.lv[l].r, s.lv[l].e2, 0);
         else launch_wpost<float, 2>(c, s, l, nact, s.lv[l].r, s.lv[l].e2, 0);
     }
@@ -1420,7 +1426,7 @@ void launch_coarsen_all(Ctx& c, InnerSolver<T>& s, int count) {
             const size_t total = (size_t)A.n * A.n * count;
             k_inv_diag<T><<<grid_for(total), 256, 0, c.stream>>>(A.n, total, A.Kw, A.Ks, A.E, A.Nn, A.inv); ++c.pc.launches;
         }
-    if (sizeof(T) == 8 && (c.onchip || c.vchip)) launch_inv4(c, count);
+    launch_dense_inverses(c, s, count);
 }
 template void launch_coarsen_all<float>(Ctx&, InnerSolver<float>&, int);
 template void launch_coarsen_all<double>(Ctx&, InnerSolver<double>&, int);

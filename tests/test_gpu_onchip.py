@@ -73,3 +73,17 @@ def test_particles_do_not_depend_on_their_batch():
         out.append(s.particles())
         s.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("fine,coarse", [(1, 2), (2, 1)])
+def test_vcycle_below_the_passes(fine, coarse):
+    """512^2 runs its levels from 128^2 down on chip (populations in ragged solve batches)."""
+    wl = dict(inputs.load_workload("darcy64_bimodal"), n=512)
+    s = smcgm.Sampler(smcgm.make_config(wl, n_particles=7, n_components=1, gm_rank=4, solve_batch=3, fine_sweeps=fine, smooth_sweeps=coarse))
+    X, _ = s.particles()
+    W = torch.empty(7, 512 * 512, dtype=torch.float64, device="cuda")
+    P = torch.empty(7, dtype=torch.float64, device="cuda")
+    s.smc_forward(torch.tensor(X, device="cuda"), P, W)
+    w = oproblem.from_workload(wl).solve(X[5]).reshape(-1)
+    assert _rel(W[5].cpu().numpy(), w) < 1e-10
+    s.close()
