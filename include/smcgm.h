@@ -79,16 +79,18 @@ typedef enum { SMC_K_PCN = 0, SMC_K_PCN_GM = 1, SMC_K_GM_INDEP = 2, SMC_K_PCNL =
  * are formed in double-float (pairs of FP32) arithmetic, ~1e-14 relative, and
  * need |u| < 64 (else the call fails; use SMC_P_FP64).
  * SMC_P_BF16SMOOTH_REFINE: SMC_P_FP32_REFINE with the multigrid smoother's
- * face coefficients stored in BF16 on every tiled level (n_l > 32): the
- * red-black Gauss-Seidel sweeps, the V-cycle residuals and the restriction
- * read the interior west / south faces as BF16 (8-bit significand, converted
- * to FP32 as they are read; FP32 arithmetic throughout), the wall faces,
- * right-hand sides and corrections stay FP32.  The faces are fixed during a
- * solve, so the V-cycle stays a fixed symmetric positive definite
- * preconditioner of the FP32 CG operator, which keeps its FP32 faces; the
- * coarse levels (n_l <= 32) keep FP32 faces; the FP64-accurate refinement
- * is unchanged, so w and Phi meet the same tol_outer.  The paper specifies
- * no solver: this is a storage precision choice of the preconditioner. */
+ * face coefficients stored in BF16 on the finest level where the solver runs in
+ * passes (cfg.tile_kernel; solves kept on chip read no faces during their
+ * iterations and stay in FP32): the red-black Gauss-Seidel sweeps, the
+ * residual and the restriction there read the interior west / south faces as
+ * BF16 (8-bit significand, converted to FP32 as they are read; FP32
+ * arithmetic throughout), the wall faces, right-hand sides and corrections
+ * stay FP32.  The faces are fixed during a solve, so the V-cycle stays a
+ * fixed symmetric positive definite preconditioner of the FP32 CG operator,
+ * which keeps its FP32 faces; the coarser levels keep FP32 faces; the
+ * FP64-accurate refinement is unchanged, so w and Phi meet the same
+ * tol_outer.  The paper specifies no solver: this is a storage precision
+ * choice of the preconditioner. */
 typedef enum { SMC_P_FP64 = 0, SMC_P_FP32_REFINE = 1, SMC_P_BF16SMOOTH_REFINE = 2 } smc_precision;
 
 typedef struct smc_config {
@@ -128,9 +130,10 @@ typedef struct smc_config {
                            modes (EM with the ridge var_floor * diag(lambda_S)); 0: diagonal
                            lambda_j as in Sec. 2.3.  pCN-GM and independence kernels only */
     int tile_kernel;    /* stencil tiles of the multigrid / CG passes on the tiled levels:
-                           0 = the default: the mixed-precision solver on grids up to
-                           256^2 keeps each particle's whole solve on chip (FP32
-                           faces throughout), anything else as 2; 1 = 32 x 32 tiles, one thread block each;
+                           0 = the default: grids up to 256^2 (in FP64 up to
+                           128^2) keep each particle's whole solve on chip (FP32 or
+                           FP64 faces throughout); larger grids run as 2 with the
+                           levels from 128^2 down on chip; 1 = 32 x 32 tiles, one thread block each;
                            2 = 16 x 16 tiles, one warp each, the finest level's inputs staged
                            by TMA (FP32; the FP64 solver uses 3); 3 = 16 x 16 tiles, one warp
                            each, loading from global memory; 4 = the finest level as 2, the
@@ -269,9 +272,10 @@ void smc_destroy(smc_ctx* ctx);
 
 /* Solver counters for throughput and roofline accounting (host-side
  * bookkeeping; the CUDA-event timing of the dominant kernel is taken only
- * while profiling is enabled).  The dominant kernel is the finest-level
- * pass that applies the CG update and runs the multigrid pre-smoothing,
- * residual and restriction. */
+ * while profiling is enabled).  The dominant kernel is the on-chip solve where
+ * solves run on chip (cfg.tile_kernel), else the finest-level pass that applies
+ * the CG update and runs the multigrid pre-smoothing, residual and
+ * restriction. */
 typedef struct smc_profile {
     long long solves;          /* forward solves (particle-solves) */
     long long cg_iterations;   /* inner CG iterations summed over particles */

@@ -21,7 +21,8 @@
 // lanes store together, and only the edge rows' warps wait for a neighbour (squares: 2048 of 256^2
 // 48.7 ms).  Below that every block of a cluster holds the whole coarse problem (32^2 for 16
 // blocks, 16^2 for 4) and solves it redundantly, which costs less than sharing it; the 8^2 level is
-// solved with its dense inverse, formed once per solve.
+// solved with its dense inverse, formed once per solve.  A larger grid's passes use the 128^2 form for
+// one V-cycle per launch, with the dense inverses formed at set-up.
 //
 // The V-cycle is otherwise that of solver.cu (symmetric red-black Gauss-Seidel, the same sweeps,
 // Galerkin coarsening, scaled correction).  The residual after a pre-smoothing that ends with the

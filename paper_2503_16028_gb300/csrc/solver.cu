@@ -18,7 +18,10 @@
 // shared memory (the halo shrinks by one cell per half-sweep), so each
 // multigrid pass reads its inputs from HBM once.  Levels at or below
 // `coarse_top` cells per side run the rest of the V-cycle in one block per
-// particle entirely in shared memory.
+// particle entirely in shared memory.  These passes solve the grids that
+// onchip.cu and onchip64.cu do not hold on chip (and any grid whose
+// configuration names a tile kernel); with the default one the levels from
+// 128^2 down are one on-chip V-cycle of those files.
 #include <cstdio>
 #include <algorithm>
 #include <cudaTypedefs.h>
