@@ -80,65 +80,72 @@ __global__ void k_faces(int n, int count, const double* __restrict__ s, FaceOut 
 }
 
 // Mixed precision: s = exp(-u) and the harmonic faces in df32 (FP32 pipes
-// only; the FP64 unit of GB300 is ~58x slower).  A block covers a 32 x 8 tile
-// of one particle: s on the tile plus its west column and south row goes to
-// shared memory, then each thread forms its cell's west and south faces
-// 2 / (s_c + s_nb) (2 / s_c on a wall) and the east / north wall faces.  The
+// only; the FP64 unit of GB300 is ~58x slower).  A warp covers 32 columns and R
+// rows of one particle, a row at a time: each lane forms its cell's s, then the west
+// and south faces 2 / (s_c + s_nb) (2 / s_c on a wall), with the west neighbour's s
+// by shuffle, the south one's from the row before; the column west of the strip is one
+// more exponential per lane, the row south of it another.  The east / north wall faces are
+// formed by the strips that lie there.  The
 // high parts are the inner solver's FP32 faces, the low parts complete them
 // to ~1e-14 relative for the FP64-accurate residual.  |u| >= 64 (beyond the
 // FP32 range of e^u) sets err[1] and is reported by the host.  With Kwb, Ksb
 // (the BF16 smoother faces) the interior faces are also stored rounded to BF16.
+// Bound by issue slots (about 190 instructions per cell).  A block per 32 x 8 tile with s staged in shared memory
+// spent a quarter more on the 41 halo exponentials, which two of its eight warps formed in a second round, and
+// waited for them: 4096 fields of 256^2 2962 us, so 1834; 1024 of 64^2 51 and 42.
 constexpr int FX = 32, FY = 8;
-__global__ void __launch_bounds__(FX * FY) k_faces_df(int n, const float2* __restrict__ u, const float2* __restrict__ exptab,
-                                                      ExpConsts ec, float* __restrict__ Kwh, float* __restrict__ Kwl,
-                                                      float* __restrict__ Ksh, float* __restrict__ Ksl, float* __restrict__ Eh,
-                                                      float* __restrict__ El, float* __restrict__ Nh, float* __restrict__ Nl,
-                                                      __nv_bfloat16* __restrict__ Kwb, __nv_bfloat16* __restrict__ Ksb,
-                                                      int* __restrict__ err, int* __restrict__ badp) {
+template <int R>
+__global__ void __launch_bounds__(128) k_faces_df(int n, const float2* __restrict__ u, const float2* __restrict__ exptab,
+                                                  ExpConsts ec, float* __restrict__ Kwh, float* __restrict__ Kwl,
+                                                  float* __restrict__ Ksh, float* __restrict__ Ksl, float* __restrict__ Eh,
+                                                  float* __restrict__ El, float* __restrict__ Nh, float* __restrict__ Nl,
+                                                  __nv_bfloat16* __restrict__ Kwb, __nv_bfloat16* __restrict__ Ksb,
+                                                  int* __restrict__ err, int* __restrict__ badp) {
     __shared__ float2 tab[64];
-    __shared__ float2 S[FY + 1][FX + 1];
-    const int p = blockIdx.y;
-    const int tpr = n / FX;
-    const int tx = blockIdx.x % tpr, ty = blockIdx.x / tpr;
+    const int p = blockIdx.y, lane = threadIdx.x & 31;
     if (threadIdx.x < 64) tab[threadIdx.x] = exptab[threadIdx.x];
     __syncthreads();
-    const size_t nn = (size_t)n * n, base = (size_t)p * nn;
+    const int strip = blockIdx.x * 4 + (threadIdx.x >> 5), x0 = strip % (n / FX) * FX, y0 = strip / (n / FX) * R, x = x0 + lane;
+    const size_t base = (size_t)p * n * n;
     const float2* up = u + base;
     bool bad = false;
-    for (int idx = threadIdx.x; idx < (FY + 1) * (FX + 1); idx += blockDim.x) {
-        const int ly = idx / (FX + 1), lx = idx % (FX + 1);
-        const int gi = tx * FX + lx - 1, gj = ty * FY + ly - 1;
-        float2 v = make_float2(1.f, 0.f);
-        if (gi >= 0 && gj >= 0) {
-            const float2 uv = up[(size_t)gj * n + gi];
-            if (!(fabsf(uv.x) < 64.f)) {
-                bad = true;
-            } else {
-                const df32 sv = df_exp(df32{-uv.x, -uv.y}, tab, ec);
-                v = make_float2(sv.hi, sv.lo);
-            }
+    auto s_of = [&](float2 uv) {
+        const bool ok = fabsf(uv.x) < 64.f;
+        bad = bad || !ok;
+        return ok ? df_exp(df32{-uv.x, -uv.y}, tab, ec) : df32{1.f, 0.f};
+    };
+    df32 west{1.f, 0.f}, south{1.f, 0.f};                     // lane r: the cell west of row y0 + r; the row before
+    if (x0 > 0) west = s_of(up[(size_t)(y0 + lane % R) * n + x0 - 1]);
+    if (y0 > 0) south = s_of(up[(size_t)(y0 - 1) * n + x]);
+    float2 next = up[(size_t)y0 * n + x];
+#pragma unroll 2
+    for (int r = 0; r < R; ++r) {
+        const int j = y0 + r;
+        const float2 uv = next;
+        if (r + 1 < R) next = up[(size_t)(j + 1) * n + x];
+        const df32 sc = s_of(uv);
+        df32 w{__shfl_up_sync(0xffffffffu, sc.hi, 1), __shfl_up_sync(0xffffffffu, sc.lo, 1)};
+        const df32 w0{__shfl_sync(0xffffffffu, west.hi, r), __shfl_sync(0xffffffffu, west.lo, r)};
+        if (lane == 0) w = w0;
+        const df32 kw = df_two_over(x > 0 ? df_add(sc, w) : sc), ks = df_two_over(j > 0 ? df_add(sc, south) : sc);
+        const size_t t = base + (size_t)j * n + x;
+        Kwh[t] = kw.hi; Kwl[t] = kw.lo;
+        Ksh[t] = ks.hi; Ksl[t] = ks.lo;
+        if (Kwb) { Kwb[t] = __float2bfloat16_rn(kw.hi); Ksb[t] = __float2bfloat16_rn(ks.hi); }
+        if (x == n - 1) {
+            const df32 wall = df_two_over(sc);
+            Eh[(size_t)p * n + j] = wall.hi; El[(size_t)p * n + j] = wall.lo;
         }
-        S[ly][lx] = v;
+        south = sc;
+    }
+    if (y0 + R == n) {
+        const df32 wall = df_two_over(south);
+        Nh[(size_t)p * n + x] = wall.hi; Nl[(size_t)p * n + x] = wall.lo;
     }
     if (bad) {
         atomicExch(&err[1], 1);
         badp[p] = 1;                          // the particle (batch index) whose field is out of range
     }
-    __syncthreads();
-    const int lx = threadIdx.x % FX, ly = threadIdx.x / FX;
-    const int i = tx * FX + lx, j = ty * FY + ly;
-    const size_t t = base + (size_t)j * n + i;
-    const float2 c2 = S[ly + 1][lx + 1];
-    const df32 sc{c2.x, c2.y};
-    const df32 wall = df_two_over(sc);
-    df32 kw = wall, ks = wall;
-    if (i > 0) { const float2 w2 = S[ly + 1][lx]; kw = df_two_over(df_add(sc, df32{w2.x, w2.y})); }
-    if (j > 0) { const float2 s2 = S[ly][lx + 1]; ks = df_two_over(df_add(sc, df32{s2.x, s2.y})); }
-    Kwh[t] = kw.hi; Kwl[t] = kw.lo;
-    Ksh[t] = ks.hi; Ksl[t] = ks.lo;
-    if (Kwb) { Kwb[t] = __float2bfloat16_rn(kw.hi); Ksb[t] = __float2bfloat16_rn(ks.hi); }
-    if (i == n - 1) { Eh[(size_t)p * n + j] = wall.hi; El[(size_t)p * n + j] = wall.lo; }
-    if (j == n - 1) { Nh[(size_t)p * n + i] = wall.hi; Nl[(size_t)p * n + i] = wall.lo; }
 }
 
 // Galerkin coarsening for piecewise-constant prolongation; with Kwcb, Kscb the
@@ -1441,7 +1448,9 @@ void launch_setup_coeffs(Ctx& c, int count) {
     if (mixed && n % FX == 0 && n % FY == 0) {
         LevelArrays<float>& f0 = c.s32.lv[0];
         check(cudaMemsetAsync(c.badp, 0, count * sizeof(int), c.stream), "memset badp");
-        k_faces_df<<<dim3((n / FX) * (n / FY), count), FX * FY, 0, c.stream>>>(
+        // strips of 32 rows while they fill the SMs (sixteen warps each), else of 8 for the latency of a few particles
+        const bool tall = (size_t)(n / FX) * (n / 32) * count >= (size_t)16 * c.sm_count;
+        (tall ? k_faces_df<32> : k_faces_df<FY>)<<<dim3((n / FX) * (n / (tall ? 32 : FY)) / 4, count), 128, 0, c.stream>>>(
             n, reinterpret_cast<const float2*>(c.u64), reinterpret_cast<const float2*>(c.exptab), c.expc, f0.Kw, c.Kwlo, f0.Ks, c.Kslo, f0.E, c.Elo, f0.Nn, c.Nlo,
             c.onchip ? nullptr : f0.Kwb, c.onchip ? nullptr : f0.Ksb, c.dev_err, c.badp); ++c.pc.launches;
         if (!c.onchip) launch_coarsen_all<float>(c, c.s32, count);
