@@ -387,7 +387,6 @@ __device__ inline typename O::V* fct_warp_t(typename O::V* b0, typename O::V* b1
     using V = typename O::V;
     V* src = b0;
     V* dst = b1;
-    const int half = N >> 1;
     const int c = lgN - 3;                              // butterfly levels lgN .. 4
     int lm = lgN - 1;
     for (int k = 0; k < c / 2; ++k, lm -= 2) {
@@ -428,27 +427,29 @@ __device__ inline typename O::V* fct_warp_t(typename O::V* b0, typename O::V* b1
                 b[2 * j] = O::add(a, bb);
                 b[2 * j + 1] = O::mul(O::sub(a, bb), t1);
             }
-            // splitting, size 4 on each half: [a0, a2 + a3, a1, a3]
-            const V e0 = b[0], e1 = O::add(b[2], b[3]), e2 = b[1], e3 = b[3];
-            const V e4 = b[4], e5 = O::add(b[6], b[7]), e6 = b[5], e7 = b[7];
-            // splitting, size 8: [e0, e4 + e5, e1, e5 + e6, e2, e6 + e7, e3, e7]
+            // splitting, size 4 on each half: [a0, a2 + a3, a1, .]
+            const V e0 = b[0], e1 = O::add(b[2], b[3]), e2 = b[1];
+            const V e4 = b[4], e5 = O::add(b[6], b[7]), e6 = b[5];
+            // splitting, size 8: [e0, e4 + e5, e1, e5 + e6, e2, . . .]
             O::store_pair(dst + fct_swz(o + 0), e0, O::add(e4, e5));
             O::store_pair(dst + fct_swz(o + 2), e1, O::add(e5, e6));
-            O::store_pair(dst + fct_swz(o + 4), e2, O::add(e6, e7));
-            O::store_pair(dst + fct_swz(o + 6), e3, e7);
+            dst[fct_swz(o + 4)] = e2;
         }
         __syncwarp();
         V* t = src; src = dst; dst = t;
     }
+    // only the outputs below N/2 are used (Km <= n/2), so only the values 0 .. M/2 of a segment: 2048 gradients of
+    // 128^2 13.88 -> 13.82 ms; of 64^2 (half a warp at N = 64) no slower: 1024 of them 1.353 -> 1.351
+    const int quarter = N >> 2;
     for (int ls = 4; ls <= lgN; ++ls) {
-        const int M = 1 << ls, h = M >> 1, lh = ls - 1;
+        const int h = 1 << (ls - 1), q = h >> 1;
         const bool first = ls == 4;                      // reads the register pass's rotated chunks
-        for (int idx = lane; idx < half; idx += 32) {
-            const int o = (idx >> lh) << ls, m = idx & (h - 1);
-            const V ev = src[first ? fct_swz(o + m) : o + m];
+        for (int idx = lane; idx < quarter; idx += 32) {
+            const int o = (idx >> (ls - 2)) << ls, m = idx & (q - 1);
             const V y0 = src[first ? fct_swz(o + h + m) : o + h + m];
-            dst[o + 2 * m] = ev;
-            dst[o + 2 * m + 1] = m + 1 < h ? O::add(y0, src[first ? fct_swz(o + h + m + 1) : o + h + m + 1]) : y0;
+            dst[o + 2 * m] = src[first ? fct_swz(o + m) : o + m];
+            dst[o + 2 * m + 1] = O::add(y0, src[first ? fct_swz(o + h + m + 1) : o + h + m + 1]);
+            if (m == q - 1) dst[o + h] = src[first ? fct_swz(o + q) : o + q];
         }
         __syncwarp();
         V* t = src; src = dst; dst = t;
