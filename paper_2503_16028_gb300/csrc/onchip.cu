@@ -85,7 +85,8 @@ struct OcMem {
     static constexpr int QP = HP + 4 * PL;
     static constexpr int LP = QP + PL;                      // C = 4: as HP for the 32^2 level (16 x 16 threads)
     static constexpr int SP = LP + (C == 4 ? 4 * 324 : 0);  // C > 1: as QP for the 16^2 level
-    static constexpr int ENDF = (SP + (C > 1 ? 324 : 0) + 1) / 2 * 2;   // C > 1: 2 x 2 + 4 mbarriers (8 bytes each)
+    static constexpr int TOK = SP + (C > 1 ? 324 : 0);      // C > 1: where the words of w_sync land
+    static constexpr int ENDF = (TOK + 2 + 1) / 2 * 2;      // C > 1: 2 x 2 + 4 mbarriers (8 bytes each)
     static constexpr int BARS = 4 * ENDF;                   // bytes
     static constexpr int TOTAL = ENDF + (C > 1 ? 16 : 0);
     static constexpr size_t BYTES = (size_t)TOTAL * 4;
@@ -107,11 +108,26 @@ __device__ __forceinline__ bool rr_sync(float* sm, OcPos<OcMem<C>>& t) {
         __syncthreads();
         return false;
     }
-    if (t.tid == 0) oc_expect(all_bar<OcMem<C>>(sm, OC_RR), 32 * OcMem<C>::CC);
+    if (t.tid == 0) oc_expect(t, all_bar<OcMem<C>>(sm, OC_RR), 32 * OcMem<C>::CC);
     nb_wait(sm, t, 8 * OcMem<C>::W);
     oc_wait(t, all_bar<OcMem<C>>(sm, OC_RR), (t.par >> OC_RR) & 1);
     t.par ^= 1u << OC_RR;
-    return __syncthreads_or(t.polls == 0);
+    return __syncthreads_or(t.dead);
+}
+
+// The solution's parts in global memory are written: visible to the block and, for the edge rows, the neighbours' too.
+// Not a cluster barrier: those have no bound, and a block whose wait ran out must meet the others at the last one
+// only.  A word to either neighbour follows the block's writes instead, counted like an edge exchange.
+template <int C>
+__device__ __forceinline__ void w_sync(float* sm, OcPos<OcMem<C>>& t) {
+    using M = OcMem<C>;
+    if (C > 1) __threadfence();
+    __syncthreads();
+    if (C > 1) {
+        if (t.nbase && t.tx == 0) oc_store(t.nbase + 4 * (M::TOK + (t.lower ? 1 : 0)), 0.f, t.nbase + nb_bar(t, !t.lower));
+        nb_wait(sm, t, 4);
+        __threadfence();
+    }
 }
 
 // ---- sums over the particle's cells: every thread of every block ends with the same bits ----
@@ -663,8 +679,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     if (V && A.build) {
         if (t.rank == 0)
             for (int i = t.tid; i < 4096; i += OC_T) A.inv8[(size_t)p * 4096 + i] = sm[M::INV8 + i];
-        if (t.polls == 0) atomicExch(A.err, 1);
-        oc_sync<C>();
+        oc_leave(t, A.err);
         return;
     }
     // r = scaled b
@@ -685,7 +700,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     }
     const size_t pb = (size_t)blockIdx.x * 4 * OC_T + t.tid;   // this thread's patch rows in x, wh, wm, wl
     int iters = 0, phases = 0, inner = 0;
-    bool converged = false, wset = false;
+    bool converged = false, wset = false, dead = false;
 #pragma unroll 1
     for (int o = 0; o < A.max_outer; ++o) {
         // ---- CG on A x = r from x = 0 ----
@@ -703,7 +718,8 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             if (V) {
                 nb_sync(sm, t, 8 * M::W);
             } else {
-                if (rr_sync<C>(sm, t)) break;
+                dead = rr_sync<C>(sm, t);
+                if (dead) break;
                 const float rr = red_get<C>(sm, t, 0);
                 if (first) {
                     thr = fmaxf(A.tol2 * rr, A.floor2 * b2s);
@@ -889,6 +905,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
                 *reinterpret_cast<float4*>(A.ve + base + (size_t)(gy + j) * n + gx) = make_float4(e[4 * j], e[4 * j + 1], e[4 * j + 2], e[4 * j + 3]);
             break;
         }
+        if (dead) break;
         // ---- w += x; FP64-accurate residual ----
         ++phases;
 #pragma unroll
@@ -904,7 +921,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             A.wh[at] = h; A.wm[at] = m; A.wl[at] = l;
         }
         wset = true;
-        oc_sync<C>();
+        w_sync<C>(sm, t);
         float s = 0.f;
         {
             const float *Kwl = A.Kwl + base, *Ksl = A.Ksl + base;
@@ -982,14 +999,15 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
         }
         red_put<C>(sm, t, OC_RZ, s);
         all_sync(sm, t, OC_RZ, 32 * M::CC);
-        if (C > 1 && __syncthreads_or(t.polls == 0)) break;
+        if (C > 1 && __syncthreads_or(t.dead)) break;
         const float res2 = red_get<C>(sm, t, OC_RZ);
         if (res2 <= A.tolout2 * b2s) { converged = true; break; }
     }
 #pragma unroll 1
     for (int j = 0; !V && j < 4; ++j) {
         const size_t at = pb + j * OC_T;
-        const float4 h = A.wh[at], m = A.wm[at], l = A.wl[at];
+        float4 h = make_float4(0.f, 0.f, 0.f, 0.f), m = h, l = h;
+        if (wset) { h = A.wh[at]; m = A.wm[at]; l = A.wl[at]; }
         double2* o = reinterpret_cast<double2*>(A.W + base + (size_t)(gy + j) * n + gx);
         o[0] = make_double2(tri_to_double(h.x, m.x, l.x, -sexp), tri_to_double(h.y, m.y, l.y, -sexp));
         o[1] = make_double2(tri_to_double(h.z, m.z, l.z, -sexp), tri_to_double(h.w, m.w, l.w, -sexp));
@@ -1002,8 +1020,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
         if (!converged) atomicAdd(&g->nonconv, 1ull);
         atomicMax(&g->itmax, iters);
     }
-    if (C > 1 && t.polls == 0) atomicExch(A.err, 1);
-    if (C > 1) oc_sync<C>();                                    // no block leaves while another may still store into it
+    oc_leave(t, A.err);
 }
 
 template <int C, bool V>

@@ -204,7 +204,7 @@ __device__ __forceinline__ bool sum6(double* sm, OcPos<M>& t, int slot, const do
     double* buf = sm + M::BUF;
 #pragma unroll
     for (int k = 0; k < NV; ++k) buf[k * O6_T + t.tid] = v[k];
-    if (M::C > 1 && t.tid == 0) oc_expect(all_bar<M>(sm, slot), 8 * NV * M::CC);
+    if (M::C > 1 && t.tid == 0) oc_expect(t, all_bar<M>(sm, slot), 8 * NV * M::CC);
     __syncthreads();
     if (t.tid < 128 * NV) {                    // per value one warp per scheduler: 8 values each, then the warp
         const double* q = buf + (t.tid >> 7) * O6_T + (t.tid & 127);
@@ -248,7 +248,7 @@ __device__ __forceinline__ bool sum6(double* sm, OcPos<M>& t, int slot, const do
             }
         }
         t.par ^= 1u << slot;
-        return __syncthreads_or(t.polls == 0);
+        return __syncthreads_or(t.dead);
     }
     __syncthreads();
     return false;
@@ -539,8 +539,7 @@ __global__ void __launch_bounds__(O6_T, 1) k_onchip64(const O6Args A) {
         if (!converged) atomicAdd(&g->nonconv, 1ull);
         atomicMax(&g->itmax, iters);
     }
-    if (C > 1 && t.polls == 0) atomicExch(A.err, 1);
-    if (C > 1) oc_sync<C>();                                  // no block leaves while another may still store into it
+    oc_leave(t, A.err);
 }
 
 // Dense inverses of the 4^2 level's operators, a warp per particle: lane l holds half a row, Gauss-Jordan
