@@ -1,7 +1,8 @@
 // The exchange helpers of the on-chip solvers (csrc/onchip.cuh) in a small kernel of their own: clusters of
-// four blocks trade edge rows and sums for some rounds.  With `drop` one block leaves out one word of one sum, as
-// a lost message would: the receiver's wait runs out, it leaves, the others' next waits run out too, and
-// the kernel ends with its error flag set.
+// four blocks trade edge rows and sums for some rounds.  With `drop` one block leaves out one word of one edge row, as
+// a lost message would: the receiver's wait runs out and it leaves after that round's sum, which the others have in
+// full; their waits of the next round run out, and the kernel ends with its error flag set.  (An edge
+// row, whose mbarriers no later round reaches without the receiver: the sums' one would count the next round's words.)
 #include <cstdio>
 #include <cuda_runtime.h>
 #define OC_WAIT_NS 20000000u
@@ -25,10 +26,10 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(Mem::T) k_rounds(int
     int rounds = 0;
     float sum = 0.f;
     for (; rounds < ROUNDS; ++rounds) {
-        if (t.nbase) oc_store(t.nbase + 4 * (Mem::ROW + (t.lower ? Mem::W : 0) + t.tx), (float)(t.rank + 1), t.nbase + nb_bar(t, !t.lower));
+        const bool lost = drop && t.rank == 1 && t.lower && t.tx == 0 && rounds == DROP_ROUND;
+        if (t.nbase && !lost) oc_store(t.nbase + 4 * (Mem::ROW + (t.lower ? Mem::W : 0) + t.tx), (float)(t.rank + 1), t.nbase + nb_bar(t, !t.lower));
         nb_sync(sm, t, 4 * Mem::W);
-        const bool lost = drop && t.rank == 2 && rounds == DROP_ROUND;
-        if (t.tid < Mem::CC && !(lost && t.tid == 0))
+        if (t.tid < Mem::CC)
             oc_push(&sm[Mem::SUM + t.rank], (uint32_t)t.tid, (float)(t.rank + rounds), all_bar<Mem>(sm, OC_RR));
         all_sync(sm, t, OC_RR, 4 * Mem::CC);
         if (__syncthreads_or(t.dead)) break;
