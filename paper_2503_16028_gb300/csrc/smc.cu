@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(SMC_THREADS) k_temper(int N, const double* __r
     __syncthreads();
     const double phimin = tot[0];
     const double rest = 1.0 - t;
-    double lo = 0.0, hi = rest, ess_lo = (double)N, h;
+    double lo = 0.0, hi = rest, ess_lo = 0.0, h;
     for (int round = 0;; ++round) {
         // cand[m], m = 1 .. 15: the midpoint of cand[m - s] and cand[m + s], s the lowest set bit of m (cand[0] = lo,
         // cand[16] = hi), level by level as the halvings would form them; slot 0 then holds 1 - t
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(SMC_THREADS) k_temper(int N, const double* __r
     for (int i = n0 + tid; i < n1; i += SMC_THREADS) logw[i] = -h * phi[i] - lse;
     if (blockIdx.x == 0 && tid == 0) {
         out[0] = h;
-        out[1] = ess_lo;
+        out[1] = h > 0.0 ? ess_lo : s;   // at h = 0 the sum of N ones, or NaN with a potential that is not finite
         out[2] = lse - log((double)N);
         out[3] = (h == rest) ? 1.0 : t + h;
     }
