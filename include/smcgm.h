@@ -325,7 +325,11 @@ smc_status smc_copy_to_host(smc_ctx* ctx, void* dst, const void* src, size_t byt
  * current device (so a device reset in between does no harm); the first call
  * on a device also loads the array there, so make it before capturing work
  * into a stream graph.  All calls share the array: calls that overlap on the
- * GPU race and must be serialised by the caller (e.g. one stream).  Returns
+ * GPU race and must be serialised by the caller (e.g. one stream); the kernel's
+ * blocks wait for one another, so a call that another one disturbs may also hold
+ * its SMs for a few seconds.  Such a wait that runs out (two seconds) leaves indices
+ * of -1, which no completed call writes: the call itself has returned SMC_OK
+ * long before.  Returns
  * SMC_EINVAL for n_particles outside [1, SMC_STATIC_RESAMPLE_MAX] or a
  * d_logw / d_indices that CUDA reports as unregistered host memory or as
  * memory of another GPU than the current one (message in

@@ -68,9 +68,12 @@ __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;" :
 // Barrier over all blocks of a cooperative launch (all of them resident): every block adds
 // one arrival to *count (zeroed before the launch) and waits until `target` arrivals have
 // been counted (gridDim.x times the number of barriers so far).  The wait is bounded: after
-// GRID_SPINS polls the block sets *err and returns false, and the caller returns.  What
-// other blocks wrote before the barrier must be read with __ldcg (their L2 copies).
-constexpr unsigned GRID_SPINS = 1u << 23;
+// GRID_SPINS polls and GRID_WAIT_NS nanoseconds more the block sets *err and returns false, and the caller
+// returns.  What other blocks wrote before the barrier must be read with __ldcg (their L2 copies).
+#ifndef GRID_WAIT_NS
+#define GRID_WAIT_NS 2000000000u
+#endif
+constexpr unsigned GRID_SPINS = 1024;
 // The two halves of the barrier: work that needs no other block's results goes between them.
 __device__ inline void grid_arrive(unsigned* count) {
     __syncthreads();
@@ -82,10 +85,17 @@ __device__ inline void grid_arrive(unsigned* count) {
 __device__ inline bool grid_wait(unsigned* count, unsigned target, int* err) {
     __shared__ int ok;
     if (threadIdx.x == 0) {
-        unsigned seen = 0, spins = 0;
-        do {
+        unsigned seen = 0, since = 0;
+        for (unsigned spins = 0;; ++spins) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-        } while (seen < target && ++spins < GRID_SPINS);
+            if (seen >= target) break;
+            if (spins >= GRID_SPINS) {
+                unsigned now;
+                asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(now));
+                if (spins == GRID_SPINS) since = now;
+                if (now - since >= GRID_WAIT_NS) break;
+            }
+        }
         ok = seen >= target;
         if (!ok) atomicExch(err, 1);
         __threadfence();

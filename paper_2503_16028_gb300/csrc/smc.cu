@@ -168,6 +168,11 @@ __global__ void __launch_bounds__(SMC_THREADS) k_resample(int N, const double* _
     const int i = blockIdx.x * SMC_THREADS + tid;
     const bool on = i < N;
     unsigned arrivals = 0;
+    auto meet = [&] {                                        // a wait that ran out leaves the error flag and -1, never an old index
+        const bool ok = grid_barrier(bar, arrivals += G, err);
+        if (!ok && on) idx[i] = -1;
+        return ok;
+    };
     const double lw = on ? logw[i] : -1.0 / 0.0;
     auto gather = [&](const double* p, bool maximum) {      // the blocks' values p[g], combined alike in every block
         double a = maximum ? -1.0 / 0.0 : 0.0;
@@ -181,11 +186,11 @@ __global__ void __launch_bounds__(SMC_THREADS) k_resample(int N, const double* _
     };
     double v = block_max(lw, red);
     if (tid == 0) part[blockIdx.x] = v;
-    if (!grid_barrier(bar, arrivals += G, err)) return;
+    if (!meet()) return;
     const double mx = gather(part, true);
     v = block_sum(on ? exp(lw - mx) : 0.0, red);
     if (tid == 0) part[SMC_BLOCKS + blockIdx.x] = v;
-    if (!grid_barrier(bar, arrivals += G, err)) return;
+    if (!meet()) return;
     const double lse = mx + log(gather(part + SMC_BLOCKS, false));
     const double w = on ? exp(lw - lse) : -1.0;
     unsigned long long q = on ? (unsigned long long)floor(w * (double)T) : 0;
@@ -213,7 +218,7 @@ __global__ void __launch_bounds__(SMC_THREADS) k_resample(int N, const double* _
             pb[2] = (double)ib;
         }
     }
-    if (!grid_barrier(bar, arrivals += G, err)) return;
+    if (!meet()) return;
     if (wid == 0) {                              // total, prefix of the earlier blocks, and the largest weight
         unsigned long long tot = 0, off = 0;
         double wb = -2.0;
@@ -254,7 +259,7 @@ __global__ void __launch_bounds__(SMC_THREADS) k_resample(int N, const double* _
     run += s_off;
     for (int k = 0; k < wid; ++k) run += s_q[k];
     if (on) cdf[i] = run;
-    if (!grid_barrier(bar, arrivals += G, err)) return;
+    if (!meet()) return;
     // particle k: smallest i with N * CDF_i > k T + u48
     if (on) {
         const unsigned long long target = (unsigned long long)i * T + u48;
@@ -421,7 +426,7 @@ void launch_grid_moments(Ctx& c, const double* mean_kl, double* mean_grid, doubl
 // the library allocates nothing.
 // ---------------------------------------------------------------------------
 constexpr int STATIC_PART = 6 * SMC_BLOCKS;   // the blocks' partials
-// the CDF, the partials, then the grid barrier's counter and its error flag
+// the CDF, the partials, then the grid barrier's counter and its error flag (which nobody reads: the indices of -1 say it)
 static __device__ __align__(256) unsigned long long g_static_scratch[SMC_STATIC_RESAMPLE_MAX + STATIC_PART + 1];
 
 // Device address of g_static_scratch on the current device.  It is looked up on every
