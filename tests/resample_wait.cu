@@ -11,7 +11,7 @@ using namespace smcgm;
 int main() {
     int N = 500;                                             // two blocks, the second one in part
     double *logw, *part;
-    unsigned long long *cdf, u48 = 12345;
+    unsigned long long *cdf, u48 = 1ull << 47;     // half a step: no index depends on how the rounded weights add up
     int *idx, *flags;                                        // flags: the barrier's counter, the error flag
     if (cudaMalloc(&logw, N * sizeof(double)) || cudaMalloc(&part, smc_partial_doubles() * sizeof(double)) ||
         cudaMalloc(&cdf, N * sizeof(*cdf)) || cudaMalloc(&idx, 512 * sizeof(int)) || cudaMalloc(&flags, 2 * sizeof(int))) return 2;
