@@ -153,7 +153,7 @@ static size_t plan(const smc_config& cfg, Ctx* c, char* base) {
     C.dim = dim; C.n = n; C.Km = Km; C.d = d; C.N = N; C.K = K; C.r = r; C.B = B; C.nobs = cfg.n_obs;
     C.lam = P.take<double>(d); C.sqrtlam = P.take<double>(d);
     C.basis = P.take<double>((size_t)n * Km);
-    C.b64 = P.take<double>(dim == 2 ? cells : (size_t)(2 * n - 1));   // 1D: b_1 .. b_{n-1}, then B_0 .. B_{n-1}
+    C.b64 = P.take<double>(dim == 2 ? cells : (size_t)(2 * n));   // 1D: b_1 .. b_{n-1}, then the table of host_tables
     C.obs = P.take<double>((size_t)cfg.n_obs * dim); C.data = P.take<double>(cfg.n_obs);
     C.S = P.take<int>(r); C.slot = P.take<int>(d);
     C.X = P.take<double>((size_t)N * d); C.X2 = P.take<double>((size_t)N * d); C.V = P.take<double>((size_t)N * d);
@@ -271,8 +271,12 @@ static void host_tables(Ctx& c, std::vector<double>& lam, std::vector<double>& b
             if (cfg.source_kind == 1) f = cfg.src_amp * std::exp(-cfg.src_width * (x - 0.5) * (x - 0.5));
             b[i - 1] = f / ((double)n * n);
         }
-        b.push_back(0.0);                              // the partial sums B_m = b_1 + .. + b_m, m = 0 .. n - 1
-        for (int i = 1; i < n; ++i) b.push_back(b.back() + b[i - 1]);
+        // the partial sums B_m = b_1 + .. + b_m of the cells m < n / 2, B_m - B_{n-1} of the others, then B_{n-1}
+        std::vector<double> sum(n + 1, 0.0);
+        for (int m = 1; m < n / 2; ++m) sum[m] = sum[m - 1] + b[m - 1];
+        for (int m = n - 2; m >= n / 2; --m) sum[m] = sum[m + 1] - b[m];
+        sum[n] = (sum[n / 2 - 1] + b[n / 2 - 1]) - sum[n / 2];
+        b.insert(b.end(), sum.begin(), sum.end());
         S.resize(c.r);
         std::iota(S.begin(), S.end(), 0);
     }

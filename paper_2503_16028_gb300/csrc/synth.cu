@@ -597,13 +597,18 @@ void launch_observe(Ctx& c, const double* w, int count, double* Phi) {
 // 1D forward map, one block per particle: u at the n midpoints from the sine KL
 // expansion (the basis table holds S[i][k] = sqrt(2) sin((k+1) pi (i+1/2)/n)), then
 // the nodal FD system.  With the flux D_i = K_{i+1/2} (w_{i+1} - w_i) its equations
-// read D_{i-1} - D_i = b_i, so D_i = g - B_i with B_i = b_1 + .. + b_i (a table) and,
-// from w_0 = w_n = 0 and R_i = 1 / K_{i+1/2} = e^{-u_i},
-//   g = sum_i B_i R_i / sum_i R_i,   w_i = sum_{m < i} (g - B_m) R_m.
+// read D_{i-1} - D_i = b_i, so D_i = D_k - C_i with C_i = b_{k+1} + .. + b_i (i > k; negated sums below k) for any
+// cell k and, from w_0 = w_n = 0 and R_i = 1 / K_{i+1/2} = e^{-u_i},
+//   D_k = sum_i C_i R_i / sum_i R_i,   w_i = sum_{m < i} D_m R_m.
 // Sums and scans over the block replace the elimination along the grid, which one
 // thread per particle did with n dependent divisions after n Km products of its own:
-// 256 particles, n = 128, 64 modes: 737 -> 15.7 us.  w is summed from the nearer
-// wall, so values next to either wall keep their relative accuracy.  FP64 throughout.
+// 256 particles, n = 128, 64 modes: 737 us for that.  FP64 throughout.
+// Behind a thin barrier (a cell or a few of very low permeability) D is small there and R huge, so D must not be a
+// difference of large numbers at that cell: k is the cell of the largest R, whose own C is zero, and the C_i are
+// differences within a half of the grid's partial sums, so a source that fades towards the walls keeps its digits too.
+// And w is summed from the wall on its side of its maximum (the source has one sign, so D changes sign
+// once), where all terms of a sum have one sign.  Relative error ~1e-15 for barriers of any height, where sums
+// about cell 0 split at n / 2 lost 1e-10 at e^-20 and 1e-4 at e^-30 (and the elimination 1e-13 to 1e-2).
 // ------------------------------------------------------------------------
 constexpr int F1_THREADS = 128;
 constexpr int F1_SMEM_N = 8192;    // larger grids keep R and w in the batch's global scratch (and more modes stay in X)
@@ -629,12 +634,15 @@ __device__ inline double block_scan_excl(double v, double* sh) {
     return base + e;
 }
 
+// bsum: the partial sums B_m = b_1 + .. + b_m of the lower half of the cells (m < n / 2), B_m - B_{n-1} of the upper
+// half, then B_{n-1}.
 __global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const double* __restrict__ X, const double* __restrict__ S,
                                                           const double* __restrict__ bsum, int nobs, const double* __restrict__ obs,
                                                           const double* __restrict__ data, double inv2s2, double* __restrict__ Phi,
                                                           double* __restrict__ wout, double* __restrict__ scratch) {
     extern __shared__ __align__(16) double f1sm[];
-    __shared__ double red[32], s_g;
+    __shared__ double red[32], s_g, s_u[F1_THREADS / 32];
+    __shared__ int s_k[F1_THREADS / 32];
     const int p = blockIdx.x, tid = threadIdx.x;
     const int kv = Km <= F1_SMEM_N ? Km : 0;       // modes held in shared memory
     const double* v = kv ? f1sm : X + (size_t)p * Km;
@@ -642,7 +650,9 @@ __global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const d
     double* w = R + n;                             // [n + 1], w[0] = w[n] = 0
     for (int k = tid; k < kv; k += F1_THREADS) f1sm[k] = X[(size_t)p * Km + k];
     __syncthreads();
-    double t1 = 0.0, t2 = 0.0;
+    double umin = 1.0 / 0.0;
+    int ku = n - 1;                                // the cell of the least u, the lowest on ties
+    auto least = [&](double u, int i) { if (u < umin || (u == umin && i < ku)) { umin = u; ku = i; } };
     for (int i = tid; i < n; i += F1_THREADS) {
         const double2* Si = reinterpret_cast<const double2*>(S + (size_t)i * Km);   // Km is even
         double u0 = 0.0, u1 = 0.0;
@@ -652,28 +662,46 @@ __global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const d
             u0 = fma(v[2 * k], sv.x, u0);
             u1 = fma(v[2 * k + 1], sv.y, u1);
         }
-        const double r = exp(-(u0 + u1));
-        R[i] = r;
-        t1 += r;
-        t2 = fma(bsum[i], r, t2);
+        const double u = u0 + u1;
+        least(u, i);
+        R[i] = exp(-u);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double ou = __shfl_xor_sync(0xffffffffu, umin, o);
+        const int ok = __shfl_xor_sync(0xffffffffu, ku, o);
+        least(ou, ok);
+    }
+    if ((tid & 31) == 0) { s_u[tid >> 5] = umin; s_k[tid >> 5] = ku; }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < F1_THREADS / 32; ++q) least(s_u[q], s_k[q]);
+    const double bk = bsum[ku], btot = bsum[n], up = ku < n / 2 ? btot : 0.0, down = ku < n / 2 ? 0.0 : -btot;
+    auto C = [&](int m) { return (bsum[m] - bk) + (m < n / 2 ? down : up); };
+    double t1 = 0.0, t2 = 0.0;
+    for (int i = tid; i < n; i += F1_THREADS) {
+        t1 += R[i];
+        t2 = fma(C(i), R[i], t2);
     }
     t1 = block_sum(t1, red);
     t2 = block_sum(t2, red);
     if (tid == 0) s_g = t2 / t1;
     __syncthreads();
     const double g = s_g;
+    auto D = [&](int m) { return g - C(m); };
+    auto from_left = [&](int m) { return m == 0 || (btot < 0.0 ? D(m - 1) <= 0.0 : D(m - 1) >= 0.0); };
     // thread t's cells are [m0, m1): the sum of its increments, the sums of all before and after it
     const int ch = (n + F1_THREADS - 1) / F1_THREADS, m0 = min(n, tid * ch), m1 = min(n, m0 + ch);
     double loc = 0.0;
-    for (int m = m0; m < m1; ++m) loc = fma(g - bsum[m], R[m], loc);
+    for (int m = m0; m < m1; ++m) loc = fma(D(m), R[m], loc);
     double L = block_scan_excl<false>(loc, red);
     double Q = block_scan_excl<true>(loc, red);
-    for (int m = m0; m < m1 && m <= n / 2; ++m) {   // left half: w_m = sum of the increments before m
+    for (int m = m0; m < m1 && from_left(m); ++m) {   // up to the maximum: w_m = sum of the increments before m
         w[m] = L;
-        L = fma(g - bsum[m], R[m], L);
+        L = fma(D(m), R[m], L);
     }
-    for (int m = m1 - 1; m >= m0 && m > n / 2; --m) {
-        Q = fma(g - bsum[m], R[m], Q);
+    for (int m = m1 - 1; m >= m0 && !from_left(m); --m) {
+        Q = fma(D(m), R[m], Q);
         w[m] = -Q;
     }
     if (tid == 0) w[n] = 0.0;
