@@ -121,12 +121,12 @@ __device__ __forceinline__ bool rr_sync(float* sm, OcPos<OcMem<C>>& t) {
 template <int C>
 __device__ __forceinline__ void w_sync(float* sm, OcPos<OcMem<C>>& t) {
     using M = OcMem<C>;
-    if (C > 1) __threadfence();
+    if (C > 1 && t.nbase) __threadfence();
     __syncthreads();
     if (C > 1) {
         if (t.nbase && t.tx == 0) oc_store(t.nbase + 4 * (M::TOK + (t.lower ? 1 : 0)), 0.f, t.nbase + nb_bar(t, !t.lower));
         nb_wait(sm, t, 4);
-        __threadfence();
+        if (t.nbase) __threadfence();
     }
 }
 
