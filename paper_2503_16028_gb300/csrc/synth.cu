@@ -611,6 +611,7 @@ void launch_observe(Ctx& c, const double* w, int count, double* Phi) {
 // about cell 0 split at n / 2 lost 1e-10 at e^-20 and 1e-4 at e^-30 (and the elimination 1e-13 to 1e-2).
 // ------------------------------------------------------------------------
 constexpr int F1_THREADS = 128;
+constexpr double F1_MAX_LOG_R = 600.0;   // beyond it R is kept in units of the excess: e^709 overflows, and the sums before it (w itself may still fit)
 constexpr int F1_SMEM_N = 8192;    // larger grids keep R and w in the batch's global scratch (and more modes stay in X)
 
 // Exclusive scan of v over the block in thread order (REV: from the last thread down).
@@ -653,7 +654,7 @@ __global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const d
     double umin = 1.0 / 0.0;
     int ku = n - 1;                                // the cell of the least u, the lowest on ties
     auto least = [&](double u, int i) { if (u < umin || (u == umin && i < ku)) { umin = u; ku = i; } };
-    for (int i = tid; i < n; i += F1_THREADS) {
+    auto field = [&](int i) {
         const double2* Si = reinterpret_cast<const double2*>(S + (size_t)i * Km);   // Km is even
         double u0 = 0.0, u1 = 0.0;
 #pragma unroll 8
@@ -662,7 +663,10 @@ __global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const d
             u0 = fma(v[2 * k], sv.x, u0);
             u1 = fma(v[2 * k + 1], sv.y, u1);
         }
-        const double u = u0 + u1;
+        return u0 + u1;
+    };
+    for (int i = tid; i < n; i += F1_THREADS) {
+        const double u = field(i);
         least(u, i);
         R[i] = exp(-u);
     }
@@ -676,6 +680,12 @@ __global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const d
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < F1_THREADS / 32; ++q) least(s_u[q], s_k[q]);
+    double unit = 1.0;                             // of R and w
+    if (-umin > F1_MAX_LOG_R) {
+        const double shift = -umin - F1_MAX_LOG_R;
+        unit = exp(shift);
+        for (int i = tid; i < n; i += F1_THREADS) R[i] = exp(-field(i) - shift);
+    }
     const double bk = bsum[ku], btot = bsum[n], up = ku < n / 2 ? btot : 0.0, down = ku < n / 2 ? 0.0 : -btot;
     auto C = [&](int m) { return (bsum[m] - bk) + (m < n / 2 ? down : up); };
     double t1 = 0.0, t2 = 0.0;
@@ -689,7 +699,9 @@ __global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const d
     __syncthreads();
     const double g = s_g;
     auto D = [&](int m) { return g - C(m); };
-    auto from_left = [&](int m) { return m == 0 || (btot < 0.0 ? D(m - 1) <= 0.0 : D(m - 1) >= 0.0); };
+    auto along = [&](int m) { return btot < 0.0 ? D(m) <= 0.0 : D(m) >= 0.0; };      // the flux has its sign at the left wall
+    // a maximum beside cell k leaves that cell out: D_k may underflow where R_k is e^700 of the others
+    auto from_left = [&](int m) { return m == 0 || (along(m - 1) && (m - 1 != ku || along(m))); };
     // thread t's cells are [m0, m1): the sum of its increments, the sums of all before and after it
     const int ch = (n + F1_THREADS - 1) / F1_THREADS, m0 = min(n, tid * ch), m1 = min(n, m0 + ch);
     double loc = 0.0;
@@ -697,12 +709,12 @@ __global__ void __launch_bounds__(F1_THREADS) k_forward1d(int n, int Km, const d
     double L = block_scan_excl<false>(loc, red);
     double Q = block_scan_excl<true>(loc, red);
     for (int m = m0; m < m1 && from_left(m); ++m) {   // up to the maximum: w_m = sum of the increments before m
-        w[m] = L;
+        w[m] = L * unit;
         L = fma(D(m), R[m], L);
     }
     for (int m = m1 - 1; m >= m0 && !from_left(m); --m) {
         Q = fma(D(m), R[m], Q);
-        w[m] = -Q;
+        w[m] = -Q * unit;
     }
     if (tid == 0) w[n] = 0.0;
     __syncthreads();
