@@ -67,8 +67,9 @@ __global__ void k_em_init(int N, int K, int r, EmPicks init, const double* __res
 //      component's current mean, to `part` (one row of 2 K r + K values per block);
 //   2. each block adds the rows for its slice of the (j, s) pairs, in a fixed order, and
 //      writes m = c + S1 / N_j and lambda = max(S2 / N_j - (S1 / N_j)^2, floor lambda_s).
-// The pivot moves with the fit, so the subtraction loses nothing once the means settle
-// (|m - c|^2 << lambda), and a component's next iteration starts from the new mean.
+// The pivot moves with the fit, so the subtraction loses nothing once the means settle.  Where a mean moved by more
+// than half a standard deviation it could cancel digits (all but 1 / N of S2 at worst), so in such an iteration,
+// mostly the first few, all blocks form the sums about the new means again, with two barriers more.
 // A collapsed component (N_j < 2) is found by every block alike (same sums, same order).
 // Measured (r = 64, 50 iterations, ncu): N = 1024, K = 4 9.0 -> 0.9 ms, N = 256, K = 2 7.2 -> 0.77 ms
 // (what is left is the chain of FP64 latencies through an iteration, 15 us: an exponential takes 1250
@@ -94,9 +95,10 @@ struct EmArgs {
     double *w, *m, *lam;          // in: the initial mixture; out: the fitted one
     double *part;                 // two buffers of gridDim rows (S1, S2: K r; N_j: K; min of gmax, its particle), then 1 / (2 lambda): K r
     double *loglik;
-    unsigned* bar;
+    unsigned *bar, *again;        // the barrier's counter; the last iteration whose variances need the sums about the new means, plus one
     int* err;
 };
+constexpr double EM_AGAIN = 0.25;   // |m - c|^2 / lambda above which they do: below it the subtraction costs at most a third of a bit
 
 // Division of a small index (< 2^16) by a divisor known per launch: the high word of a product.
 struct EmDiv {
@@ -213,41 +215,44 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
         __syncthreads();
         double* part = A.part + (size_t)(it & 1) * G * row;   // the other buffer may still be read
         double* out = part + (size_t)b * row;
-        if (split > 1) {                   // few pairs: groups of Kr threads share the particles
-            const int h = tid / Kr, q = tid - h * Kr, j = by_r.quot(q), s = q - j * r;
-            double s1 = 0.0, s2 = 0.0;
-            if (h < split) {
-                const double c = sm[(size_t)j * rp + s];
-                const double* g = lp + (size_t)j * per;
-                for (int p = h; p < np; p += split) {
-                    const double e = X(p, s) - c, ge = g[p] * e;
-                    s1 += ge;
-                    s2 = fma(ge, e, s2);
-                }
-                spl[tid] = s1;
-                spl[EM_THREADS + tid] = s2;
-            }
-            __syncthreads();
-            if (h == 0) {
-                for (int k = 1; k < split; ++k) { s1 += spl[k * Kr + q]; s2 += spl[EM_THREADS + k * Kr + q]; }
-                out[q] = s1;
-                out[Kr + q] = s2;
-            }
-        } else {
-            for (int t = tid; t < Kr; t += EM_THREADS) {
-                const int j = by_r.quot(t), s = t - j * r;
-                const double c = sm[(size_t)j * rp + s];
-                const double* g = lp + (size_t)j * per;
+        auto sums = [&] {                  // of g (x - c) and g (x - c)^2 about the means c in shared memory
+            if (split > 1) {                   // few pairs: groups of Kr threads share the particles
+                const int h = tid / Kr, q = tid - h * Kr, j = by_r.quot(q), s = q - j * r;
                 double s1 = 0.0, s2 = 0.0;
-                for (int p = 0; p < np; ++p) {
-                    const double e = X(p, s) - c, ge = g[p] * e;
-                    s1 += ge;
-                    s2 = fma(ge, e, s2);
+                if (h < split) {
+                    const double c = sm[(size_t)j * rp + s];
+                    const double* g = lp + (size_t)j * per;
+                    for (int p = h; p < np; p += split) {
+                        const double e = X(p, s) - c, ge = g[p] * e;
+                        s1 += ge;
+                        s2 = fma(ge, e, s2);
+                    }
+                    spl[tid] = s1;
+                    spl[EM_THREADS + tid] = s2;
                 }
-                out[t] = s1;
-                out[Kr + t] = s2;
+                __syncthreads();
+                if (h == 0) {
+                    for (int k = 1; k < split; ++k) { s1 += spl[k * Kr + q]; s2 += spl[EM_THREADS + k * Kr + q]; }
+                    out[q] = s1;
+                    out[Kr + q] = s2;
+                }
+            } else {
+                for (int t = tid; t < Kr; t += EM_THREADS) {
+                    const int j = by_r.quot(t), s = t - j * r;
+                    const double c = sm[(size_t)j * rp + s];
+                    const double* g = lp + (size_t)j * per;
+                    double s1 = 0.0, s2 = 0.0;
+                    for (int p = 0; p < np; ++p) {
+                        const double e = X(p, s) - c, ge = g[p] * e;
+                        s1 += ge;
+                        s2 = fma(ge, e, s2);
+                    }
+                    out[t] = s1;
+                    out[Kr + t] = s2;
+                }
             }
-        }
+        };
+        sums();
         for (int j = tid >> 5; j < K; j += EM_THREADS / 32) {
             double a = 0.0;
             for (int p = tid & 31; p < np; p += 32) a += lp[(size_t)j * per + p];
@@ -295,6 +300,7 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
                 n += __shfl_xor_sync(0xffffffffu, n, o);
             }
             double mv, lv;
+            bool jump = false;
             if (n < 2.0) {                  // rare: re-seeded at the particle with the lowest max_j g
                 double bg = 1.0 / 0.0, bi = (double)N;
                 for (int k = 0; k < G; ++k) {
@@ -307,9 +313,11 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
                 const double dm = s1 / n;
                 mv = sm[(size_t)j * rp + s] + dm;
                 lv = fmax(s2 / n - dm * dm, A.floor_frac * A.lamS[s]);
+                jump = dm * dm > EM_AGAIN * lv;
             }
             if (lane == 0) {
                 A.m[q] = mv;
+                if (jump) atomicExch(A.again, (unsigned)it + 1u);
                 A.lam[q] = lv;
                 g_si[q] = 1.0 / (2.0 * lv);
             }
@@ -327,10 +335,43 @@ __global__ void __launch_bounds__(EM_THREADS) k_em(EmArgs A) {
             sw[tid] = (nj[tid] < 2.0 ? 1.0 : nj[tid]) / tot;
         }
         if (!grid_wait(A.bar, arrivals += G, A.err)) return;
+        const bool again = __ldcg(A.again) == (unsigned)it + 1u;   // the same in every block: written before the barrier
         for (int t = tid; t < Kr; t += EM_THREADS) {
             const int j = by_r.quot(t), s = t - j * r;
             sm[(size_t)j * rp + s] = __ldcg(&A.m[t]);
             si[(size_t)j * rp + s] = __ldcg(&g_si[t]);
+        }
+        if (again) {
+            // means and variances once more, about the new means: the sums' part of the rows is free (N_j, beside it, may still be read)
+            __syncthreads();
+            sums();
+            if (!grid_barrier(A.bar, arrivals += G, A.err)) return;
+            for (int q = lo + wid; q < hi; q += EM_THREADS / 32) {
+                const int j = by_r.quot(q), s = q - j * r;
+                double s1 = 0.0, s2 = 0.0;
+                for (int k = lane; k < G; k += 32) {
+                    const double* pr = part + (size_t)k * row;
+                    s1 += __ldcg(&pr[q]);
+                    s2 += __ldcg(&pr[Kr + q]);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+                    s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+                }
+                if (lane == 0 && !(nj[j] < 2.0)) {
+                    const double n = nj[j], dm = s1 / n, lv = fmax(s2 / n - dm * dm, A.floor_frac * A.lamS[s]);
+                    A.m[q] = sm[(size_t)j * rp + s] + dm;
+                    A.lam[q] = lv;
+                    g_si[q] = 1.0 / (2.0 * lv);
+                }
+            }
+            if (!grid_barrier(A.bar, arrivals += G, A.err)) return;
+            for (int t = tid; t < Kr; t += EM_THREADS) {
+                const int j = by_r.quot(t), s = t - j * r;
+                sm[(size_t)j * rp + s] = __ldcg(&A.m[t]);
+                si[(size_t)j * rp + s] = __ldcg(&g_si[t]);
+            }
         }
         // sum_s log lambda_js as one logarithm per component: the product of the mantissas (in [1, 2), at most 256 of
         // them: no overflow) and the sum of the exponents
@@ -863,7 +904,7 @@ static void em_diag(Ctx& c, const double* lamS, double* ll) {
     EmArgs A{};
     A.N = N; A.K = K; A.r = r; A.iters = c.cfg.em_iters; A.lg_lanes = 2; A.floor_frac = c.cfg.var_floor;
     A.xsT = c.xsT; A.pooled = c.pooled; A.lamS = lamS; A.w = c.gw; A.m = c.gmu; A.lam = c.glam;
-    A.part = c.empart; A.loglik = ll; A.bar = reinterpret_cast<unsigned*>(c.icount + 44); A.err = c.dev_err;
+    A.part = c.empart; A.loglik = ll; A.bar = reinterpret_cast<unsigned*>(c.icount + 44); A.again = A.bar + 1; A.err = c.dev_err;
     const int G = std::max(1, std::min({EM_BLOCKS, c.sm_count, (N + EM_MINP - 1) / EM_MINP}));
     const int per = (N + G - 1) / G;
     while (A.lg_lanes < 5 && (per * K << (A.lg_lanes + 1)) <= EM_ETHREADS) ++A.lg_lanes;   // the chain of FP64 latencies is what bounds small fits
@@ -872,7 +913,7 @@ static void em_diag(Ctx& c, const double* lamS, double* ll) {
     const size_t sm = em_smem(K, r, per, xs);
     const void* fn = xs ? reinterpret_cast<const void*>(&k_em<true>) : reinterpret_cast<const void*>(&k_em<false>);
     check(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LIMIT), "attr");
-    check(cudaMemsetAsync(A.bar, 0, sizeof(unsigned), c.stream), "memset");
+    check(cudaMemsetAsync(A.bar, 0, 2 * sizeof(unsigned), c.stream), "memset");
     void* args[] = {&A};
     check(cudaLaunchCooperativeKernel(fn, dim3(G), dim3(EM_THREADS), args, sm, c.stream), "EM launch"); ++c.pc.launches;
 }
