@@ -418,7 +418,7 @@ __global__ void k_sum(int N, const double* __restrict__ a, double* __restrict__ 
 //   E-step: log p_nj = log w_j - r/2 log(2 pi) - log det L_j - |L_j^{-1}(x_n - m_j)|^2 / 2,
 //   M-step: C_j = sum_n g_nj (x_n - m_j)(x_n - m_j)^T / N_j + floor diag(lambda_S),
 //   initial and re-seeded covariances diag(pooled variances).
-// An iteration is k_chol, k_estep_full, k_resp, k_cov_acc, k_cov_finish.  The E-step and the
+// An iteration is k_chol, k_estep_full, k_resp, k_cov_mean, k_cov_acc, k_cov_finish.  The E-step and the
 // contraction are N K r^2 / 2 FP64 multiply-adds each (108 us at N = 4096, K = 8, r = 64 on the
 // FP64 pipes), everything else should stay small beside them.  Measured per 50-iteration fit
 // there: 70.2 -> 20.4 ms (one block per particle reading rows of L^-1 uncoalesced 631 -> 150 us, FP64
@@ -651,8 +651,29 @@ __global__ void __launch_bounds__(256) k_resp(int N, int K, double* __restrict__
     }
 }
 
-// The contraction sum_n g_nj (x_n - c_j)(x_n - c_j)^T about the pivot c_j = the component's current
-// mean, with sum_n g_nj (x_n - c_j) and N_j, over one chunk of the particles (grid z): each thread
+// The pivots of the contraction: sums_j[s] = sum_n g_nj x_ns, sums_j[r] = N_j, a block each.  Their quotient is the new mean to
+// rounding (about the old one the subtraction of (m - c)(m - c)^T cancels digits where a mean jumps, all but
+// 1 / N at worst); k_cov_finish corrects it by the sums about itself.  One FP64 operation per element, 4 us at
+// N = 4096, K = 8, r = 64 on the pipe; 8 us per iteration in the fit.
+__global__ void __launch_bounds__(256) k_cov_mean(int N, int r, const double* __restrict__ xsT, const double* __restrict__ resp,
+                                                  double* __restrict__ sums) {
+    __shared__ double red[32];
+    const int s = blockIdx.x, j = blockIdx.y;
+    const double *x = xsT + (size_t)s * N, *g = resp + (size_t)j * N;
+    double b = 0.0;
+    if (s < r) {
+#pragma unroll 8
+        for (int n = threadIdx.x; n < N; n += 256) b = fma(g[n], x[n], b);
+    } else {
+#pragma unroll 8
+        for (int n = threadIdx.x; n < N; n += 256) b += g[n];
+    }
+    b = block_sum(b, red);
+    if (threadIdx.x == 0) sums[(size_t)j * (r + 1) + s] = b;
+}
+
+// The contraction sum_n g_nj (x_n - c_j)(x_n - c_j)^T about the pivot c_j of k_cov_mean,
+// with sum_n g_nj (x_n - c_j) and N_j, over one chunk of the particles (grid z): each thread
 // holds one 4 x 4 tile of the lower triangle (136 tiles at r = 64: 5 % more products than the triangle
 // itself; 32 x 32 tiles took 48 % more), 16 particles' deviations staged in shared memory per step.
 // 136 tiles are four warps and a quarter: the lanes of the partial warp divide each step's particles among
@@ -666,16 +687,19 @@ __host__ __device__ inline int cov_chunks(int K, int r) {
     const int c = 304 / (K * ((cov_tiles(r) + 255) / 256));
     return c < 1 ? 1 : c > 64 ? 64 : c;
 }
-size_t cov_partial_doubles(int K, int r) { return (size_t)K * cov_chunks(K, r) * cov_row(r); }
-static size_t cov_smem(int r) { return sizeof(double) * (2 * (size_t)COV_PN * 4 * row_blocks(r) + COV_PN); }
+static size_t cov_sums_at(int K, int r) { return (size_t)K * cov_chunks(K, r) * cov_row(r); }   // k_cov_mean's sums, after the chunks
+size_t cov_partial_doubles(int K, int r) { return cov_sums_at(K, r) + (size_t)K * (r + 1); }
+static size_t cov_smem(int r) { return sizeof(double) * ((2 * (size_t)COV_PN + 1) * 4 * row_blocks(r) + COV_PN); }
 
 __global__ void __launch_bounds__(256) k_cov_acc(int N, int r, const double* __restrict__ xsT, const double* __restrict__ resp,
-                                                 const double* __restrict__ m, double* __restrict__ part) {
+                                                 const double* __restrict__ sums, double* __restrict__ part) {
     extern __shared__ __align__(16) double csm[];
     const int j = blockIdx.y, chunk = blockIdx.z, nch = gridDim.z, tid = threadIdx.x, rp = 4 * row_blocks(r);
     double* D = csm;                      // [COV_PN][rp] deviations
     double* Wd = D + COV_PN * rp;         // [COV_PN][rp] weighted deviations
-    double* gs = Wd + COV_PN * rp;
+    double* pv = Wd + COV_PN * rp;        // [rp] pivots
+    double* gs = pv + rp;
+    if (tid < r) pv[tid] = sums[(size_t)j * (r + 1) + tid] / sums[(size_t)j * (r + 1) + r];
     const int T = cov_tiles(r), base = T & ~31, left = T - base;
     // a tile per thread; the last, partial warp's `left` tiles with S lanes each, which share a step's particles
     int t = blockIdx.x * 256 + tid, S = 1, slice = 0;
@@ -699,7 +723,7 @@ __global__ void __launch_bounds__(256) k_cov_acc(int N, int r, const double* __r
         __syncthreads();
         for (int e = tid; e < COV_PN * rp; e += 256) {
             const int s = e / COV_PN, p = e % COV_PN;
-            const double dv = (s < r && n0 + p < n_hi) ? xsT[(size_t)s * N + n0 + p] - m[(size_t)j * r + s] : 0.0;
+            const double dv = (s < r && n0 + p < n_hi) ? xsT[(size_t)s * N + n0 + p] - pv[s] : 0.0;
             D[p * rp + s] = dv;
             Wd[p * rp + s] = gs[p] * dv;
         }
@@ -745,8 +769,8 @@ __global__ void __launch_bounds__(256) k_cov_acc(int N, int r, const double* __r
 // Adds the chunks and writes C_j (both triangles), its diagonal, m_j and the weights; a component with
 // N_j < 2 is re-seeded at the particle with the lowest largest responsibility.  Latency: every chunk is requested
 // before the first barrier (one sum after the other 35 us, so 19, caches cold).
-__global__ void __launch_bounds__(256) k_cov_finish(int N, int K, int r, int nch, const double* __restrict__ part, const double* __restrict__ gmax,
-                                                    const double* __restrict__ xsT, const double* __restrict__ pooled,
+__global__ void __launch_bounds__(256) k_cov_finish(int N, int K, int r, int nch, const double* __restrict__ part, const double* __restrict__ sums,
+                                                    const double* __restrict__ gmax, const double* __restrict__ xsT, const double* __restrict__ pooled,
                                                     const double* __restrict__ lamS, double floor_frac, double* __restrict__ w,
                                                     double* __restrict__ m, double* __restrict__ lam, double* __restrict__ cov) {
     // four threads per element (and per mode, component) share the chunks
@@ -807,7 +831,7 @@ __global__ void __launch_bounds__(256) k_cov_finish(int N, int K, int r, int nch
         __syncthreads();
         if (tid < r) m[(size_t)j * r + tid] = xsT[(size_t)tid * N + s_i[0]];
     } else if (tid < r) {
-        m[(size_t)j * r + tid] += dm[tid];
+        m[(size_t)j * r + tid] = sums[(size_t)j * (r + 1) + tid] / sums[(size_t)j * (r + 1) + r] + dm[tid];
     }
     if (j == 0 && tid == 0) {
         double tot = 0.0;
@@ -876,6 +900,7 @@ static void em_full(Ctx& c, const double* lamS, double* ll) {
     check(cudaFuncSetAttribute(k_estep_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * ESF_WARPS * 32 * MAXR)), "attr");
     check(cudaFuncSetAttribute(k_cov_acc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cov_smem(MAXR)), "attr");
     const double* cst = c.gLb + (size_t)K * lb_size(r);
+    double* sums = c.covpart + cov_sums_at(K, r);
     auto estep = [&] {
         k_estep_full<<<dim3((N + 32 * ESF_WARPS - 1) / (32 * ESF_WARPS), K), 32 * ESF_WARPS, esm, c.stream>>>(N, r, c.xsT, c.gmu, c.gLb, cst, c.resp);
         k_resp<<<(N + P - 1) / P, 256, 0, c.stream>>>(N, K, c.resp, c.lse, c.gmax);
@@ -886,10 +911,11 @@ static void em_full(Ctx& c, const double* lamS, double* ll) {
     for (int it = 0; it < c.cfg.em_iters; ++it) {
         launch_chol(c, true);
         estep();
-        k_cov_acc<<<dim3(tg, K, nch), 256, csm, c.stream>>>(N, r, c.xsT, c.resp, c.gmu, c.covpart);
-        k_cov_finish<<<dim3((cov_tiles(r) * 16 + 63) / 64, K), 256, 0, c.stream>>>(N, K, r, nch, c.covpart, c.gmax, c.xsT, c.pooled, lamS,
+        k_cov_mean<<<dim3(r + 1, K), 256, 0, c.stream>>>(N, r, c.xsT, c.resp, sums);
+        k_cov_acc<<<dim3(tg, K, nch), 256, csm, c.stream>>>(N, r, c.xsT, c.resp, sums, c.covpart);
+        k_cov_finish<<<dim3((cov_tiles(r) * 16 + 63) / 64, K), 256, 0, c.stream>>>(N, K, r, nch, c.covpart, sums, c.gmax, c.xsT, c.pooled, lamS,
                                                                                    c.cfg.var_floor, c.gw, c.gmu, c.glam, c.gcov);
-        c.pc.launches += 2;
+        c.pc.launches += 3;
     }
     launch_chol(c, true);
     estep();

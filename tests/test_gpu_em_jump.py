@@ -14,7 +14,7 @@ from paper_2503_16028_gb300 import inputs, smcgm  # noqa: E402
 from oracle import gm, prior  # noqa: E402
 
 
-@pytest.mark.parametrize("full", [0])
+@pytest.mark.parametrize("full", [0, 1])
 @pytest.mark.parametrize("N,r", [(32768, 16), (32767, 5), (4099, 64)])
 def test_variances_after_a_jump(full, N, r):
     if not torch.cuda.is_available():
