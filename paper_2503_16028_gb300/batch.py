@@ -95,8 +95,9 @@ def run_batch(samplers, mcmc_steps, max_layers=200, concurrent=True):
 
 
 DEFAULT_CANDIDATES = (
-    dict(),                                            # the library defaults
+    dict(),                                            # the library defaults (solves on chip where they fit)
     dict(tile_kernel=1),                               # 32 x 32 block tiles
+    dict(tile_kernel=2),                               # 16 x 16 warp tiles, the finest level staged by TMA
     dict(tile_kernel=3),                               # 16 x 16 warp tiles, global loads
     dict(tile_kernel=4),                               # warp tiles on the finest level, block tiles below
     dict(smooth_sweeps=1),
