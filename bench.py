@@ -214,8 +214,8 @@ class ClockSampler:
                     reasons=sorted(reasons), samples=len(sm), power_w_max=max(power) if power else None)
 
 
-def make_sampler(wl, precision, N, smcgm):
-    cfg = smcgm.make_config(wl, precision=precision, n_particles=N)
+def make_sampler(wl, precision, N, smcgm, **over):
+    cfg = smcgm.make_config(wl, precision=precision, n_particles=N, **over)
     s = smcgm.Sampler(cfg)
     # a realistic state: one tempering layer (reweight, resample, mixture fit)
     s.smc_temper_step()
@@ -564,9 +564,8 @@ def time_moves(s, steps, warmup, torch, barrier):
 
 
 def on_chip(prof):
-    """Whether the profiled solves ran in the on-chip kernel (its algorithmic bytes: 24 per cell and solve)."""
-    cells = prof.get("dom_particles", 0) * prof["cells"]
-    return cells > 0 and abs(prof["dom_bytes"] / cells - 24.0) < 1e-6
+    """Whether the profiled solves ran in an on-chip kernel (smc_solver of the sampler that ran them)."""
+    return prof.get("solver", "").startswith("k_onchip")
 
 
 def model_bytes_per_solve(prof, n, d):
@@ -655,6 +654,7 @@ def run_native(args, rank, world, local):
     d = s.d
     clocks = ClockSampler(local)
     ms, prof = time_moves(s, args.steps, args.warmup, torch, barrier)
+    prof["solver"] = s.smc_solver()
     clk = clocks.stop()
     ms_max = max_over_ranks(ms, world, "cuda")
     value = whole_job_rate(N * args.steps, world, ms_max)
@@ -667,7 +667,7 @@ def run_native(args, rank, world, local):
     traffic = tb * 65536 * prof["dom_particles"] / max(1, prof["dom_launches"]) if tb else None
     roof = dict(bound="latency" if chip else "hbm", achieved=dom_ach, peak=hbm_peak, unit="GB/s", frac=dom_ach / hbm_peak, traffic=traffic,
                 algorithmic_bytes_per_launch=prof["dom_bytes"] / max(1, prof["dom_launches"]),
-                kernel="k_onchip<4> (whole solve of a particle on a cluster of 16 blocks; HBM only for its faces and its solution)" if chip else
+                kernel="%s (whole solve of a particle on chip; HBM only for its faces and its solution)" % prof["solver"] if chip else
                 "k_tpre<2,CG> (finest level, CG update + pre-smoothing + restriction, TMA-staged; %s smoother faces)"
                 % args.smoother.upper(), peak_source=peak_src,
                 launches=prof["dom_launches"], ms_per_launch=prof["dom_ms"] / max(1, prof["dom_launches"]))
@@ -688,20 +688,25 @@ def run_native(args, rank, world, local):
     s.close()
     del s
     torch.cuda.empty_cache()
-    alt_leg = None
-    if not args.no_alt_smoother:
-        sb = make_sampler(wl, prec_of[alt], N, smcgm)
+    def smoother_leg(smoother, **over):
+        sb = make_sampler(wl, prec_of[smoother], N, smcgm, **over)
         msb, profb = time_moves(sb, args.steps, args.warmup, torch, barrier)
+        solver = sb.smc_solver()
         sb.close()
+        torch.cuda.empty_cache()
         msb = max_over_ranks(msb, world, "cuda")
         dom_b = profb["dom_bytes"] / (profb["dom_ms"] / 1000.0) / 1e9 if profb["dom_ms"] > 0 else 0.0
-        alt_leg = dict(smoother=alt, value=whole_job_rate(N * args.steps, world, msb), unit=UNIT, ms_per_step=msb / args.steps,
-                       cg_per_solve=profb["cg_iterations"] / max(1, profb["solves"]),
-                       inner_solves_per_solve=profb["inner_solves"] / max(1, profb["solves"]),
-                       dominant_kernel=dict(achieved=dom_b, frac=dom_b / hbm_peak,
-                                            algorithmic_bytes_per_launch=profb["dom_bytes"] / max(1, profb["dom_launches"]),
-                                            ms_per_launch=profb["dom_ms"] / max(1, profb["dom_launches"])))
-        torch.cuda.empty_cache()
+        return dict(smoother=smoother, solver=solver, value=whole_job_rate(N * args.steps, world, msb), unit=UNIT, ms_per_step=msb / args.steps,
+                    cg_per_solve=profb["cg_iterations"] / max(1, profb["solves"]),
+                    inner_solves_per_solve=profb["inner_solves"] / max(1, profb["solves"]),
+                    dominant_kernel=dict(achieved=dom_b, frac=dom_b / hbm_peak,
+                                         algorithmic_bytes_per_launch=profb["dom_bytes"] / max(1, profb["dom_launches"]),
+                                         ms_per_launch=profb["dom_ms"] / max(1, profb["dom_launches"])))
+
+    alt_leg = None
+    if not args.no_alt_smoother:
+        # on chip no smoother reads faces from memory: the two storages are compared in the passes (tile_kernel = 2)
+        alt_leg = [smoother_leg(x, tile_kernel=2) for x in ("fp32", "bf16")] if chip else smoother_leg(alt)
     fp64 = agree = None
     if not args.no_fp64:
         s64 = make_sampler(wl, smcgm.SMC_P_FP64, N, smcgm)

@@ -300,6 +300,12 @@ typedef struct smc_profile {
  * events cannot be created. */
 smc_status smc_profile_query(smc_ctx* ctx, int enable, smc_profile* out, int reset);
 
+/* Which kernel solves this context's forward problems, chosen at smc_init from the grid, the precision, cfg.tile_kernel
+ * and the device: "k_onchip<C>" or "k_onchip64<C>" (mixed precision, FP64: a particle's whole solve in one launch, on
+ * a cluster of C * C blocks), "passes" (one launch per multigrid or CG pass), "k_forward1d" (dim = 1).  "" for NULL.
+ * Static storage. */
+const char* smc_solver(const smc_ctx* ctx);
+
 /* Copies `bytes` from device address `src` (e.g. a view returned above) to
  * host memory `dst` on the context's stream and waits for it: a helper for
  * bindings that have no CUDA runtime of their own.  Both buffers stay the

@@ -527,6 +527,15 @@ const char* smc_last_error(const smc_ctx* ctx) {
     return ctx->c.err.c_str();
 }
 
+const char* smc_solver(const smc_ctx* ctx) {
+    if (!ctx) return "";
+    const Ctx& c = ctx->c;
+    if (c.dim == 1) return "k_forward1d";
+    if (!c.onchip) return "passes";
+    if (!mixed_precision(c.cfg)) return c.n == 64 ? "k_onchip64<1>" : "k_onchip64<2>";
+    return c.n == 64 ? "k_onchip<1>" : c.n == 128 ? "k_onchip<2>" : "k_onchip<4>";
+}
+
 void smc_destroy(smc_ctx* ctx) {
     if (!ctx) return;
     if (ctx->c.ev0) cudaEventDestroy(ctx->c.ev0);

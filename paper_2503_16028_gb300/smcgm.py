@@ -73,6 +73,7 @@ EXPORTS = {
     "smc_version": (ctypes.c_char_p, []),
     "smc_config_size": (ctypes.c_size_t, []),
     "smc_profile_query": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.POINTER(smc_profile), ctypes.c_int]),
+    "smc_solver": (ctypes.c_char_p, [_vp]),
     "smc_copy_to_host": (ctypes.c_int, [_vp, _vp, _vp, ctypes.c_size_t]),
     "smc_resample_indices_static": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_ulonglong, ctypes.c_int, _vp, _vp]),
     "smc_batch_create": (ctypes.c_int, [ctypes.POINTER(_vp), ctypes.c_int, ctypes.c_int, ctypes.POINTER(_vp)]),
@@ -364,6 +365,10 @@ class Sampler:
         lw = self.to_host(ptrs[3].value, self.N)
         idx = self.to_host(ptrs[4].value, self.N, np.int32)
         return dict(log_alpha=la, accepted=acc.astype(bool), phi_proposed=pv, logw=lw, indices=idx)
+
+    def smc_solver(self):
+        """Name of the kernel that solves the context's forward problems ("passes" for the multi-pass solvers)."""
+        return self.lib.smc_solver(self.ctx).decode()
 
     def smc_profile_query(self, enable=-1, reset=False):
         out = smc_profile()
