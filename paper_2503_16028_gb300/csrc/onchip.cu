@@ -44,7 +44,9 @@ constexpr int OC_T = 256;
 
 struct OcArgs {
     int n, max_outer, maxit, nu_f, nu_c;
-    float cc, tol2, floor2, tolout2;
+    float cc;
+    float2 tol2;                 // the pair of the squared reduction per phase
+    double floor2, tolout2;
     double b2const;
     const double* b2pp;
     const float *Kw, *Ks, *E, *Nn, *Kwl, *Ksl, *El, *Nl;   // faces: high and low parts
@@ -77,8 +79,9 @@ struct OcMem {
     static constexpr int INV8 = SF + (C > 1 ? 4 * OC_T : 0);   // dense inverse of the 8^2 level, [k][row]
     static constexpr int R8 = INV8 + 4096;
     static constexpr int PART8 = R8 + 64;
-    static constexpr int RED = PART8 + 256;                 // 3 slots of 8 CC warp sums
-    static constexpr int RB = RED + 3 * 8 * CC;             // gathered right-hand side of the first local level
+    static constexpr int RED = PART8 + 256;                 // 3 slots of 8 CC warp sums (df32)
+    static constexpr int THR = RED + 3 * 16 * CC;           // |r|^2 no phase need go below, |r|^2 at which the solve ends (df32)
+    static constexpr int RB = THR + 4;                      // gathered right-hand side of the first local level
     static constexpr int STG = PART8;                       // C > 1: pair sums of a block's part of it, H x W / 2
     static constexpr int SIDE = RB + (C == 4 ? 1024 : C == 2 ? 256 : 0);   // 4 sides x 2 colours
     static constexpr int HP = SIDE + 8 * (SZH + SZV);       // 4 planes: cell (i, j) of each 2 x 2 patch
@@ -94,12 +97,6 @@ struct OcMem {
     static_assert(STG % 4 == 0 && RB % 4 == 0 && SIDE % 2 == 0 && RED % 4 == 0, "vector alignment");
 };
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // The exchange that starts an iteration: |r|^2 and the first red edges.  True if a wait ran out in any thread
 // of the block, which then leaves the loops alike (threads must not decide on sums that others did not see).
 template <int C>
@@ -108,7 +105,7 @@ __device__ __forceinline__ bool rr_sync(float* sm, OcPos<OcMem<C>>& t) {
         __syncthreads();
         return false;
     }
-    if (t.tid == 0) oc_expect(t, all_bar<OcMem<C>>(sm, OC_RR), 32 * OcMem<C>::CC);
+    if (t.tid == 0) oc_expect(t, all_bar<OcMem<C>>(sm, OC_RR), 64 * OcMem<C>::CC);
     nb_wait(sm, t, 8 * OcMem<C>::W);
     oc_wait(t, all_bar<OcMem<C>>(sm, OC_RR), (t.par >> OC_RR) & 1);
     t.par ^= 1u << OC_RR;
@@ -131,35 +128,69 @@ __device__ __forceinline__ void w_sync(float* sm, OcPos<OcMem<C>>& t) {
 }
 
 // ---- sums over the particle's cells: every thread of every block ends with the same bits ----
+// FP32 within 256 cells (half a warp); these sums (in a cluster: the exact sums of a warp's two) are added as fixed-point numbers, 44
+// bits below the largest, whose integer sums do not depend on an order.  So the sum over 65536 cells has the error of its
+// 256-cell terms, as the passes' sums have (FP32 in a tile, FP64 across tiles).  Two integer additions over a warp take
+// little more than the five FP32 additions by shuffle of a plain sum: a gradient call of 2048 particles of 128^2 13.90 ms with FP32
+// sums throughout, 14.04 so, 14.67 with pairs of FP32 by shuffle; a move of 4096 of 256^2 83.7, 86.3, 88.0.
 template <int C>
 __device__ __forceinline__ void red_put(float* sm, const OcPos<OcMem<C>>& t, int slot, float v) {
     using M = OcMem<C>;
-    v = warp_sum(v);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     const int lane = t.tid & 31, wid = t.tid >> 5;
-    float* dst = sm + M::RED + slot * 8 * M::CC + (int)t.rank * 8 + wid;
+    float* dst = sm + M::RED + slot * 16 * M::CC + 2 * ((int)t.rank * 8 + wid);
     if (C == 1) {
-        if (lane == 0) *dst = v;
-    } else if (lane < M::CC) {
-        oc_push(dst, (uint32_t)lane, v, all_bar<OcMem<C>>(sm, slot));
+        if ((lane & 15) == 0) dst[lane >> 4] = v;
+        return;
     }
+    float2 w;
+    two_sum(v, __shfl_xor_sync(0xffffffffu, v, 16), w.x, w.y);
+    if (lane < M::CC) oc_store2(oc_map(dst, (uint32_t)lane), w, oc_map(all_bar<OcMem<C>>(sm, slot), (uint32_t)lane));
 }
 template <int C>
-__device__ __forceinline__ float red_get(const float* sm, const OcPos<OcMem<C>>& t, int slot) {
+__device__ __forceinline__ df32 red_get(const float* sm, const OcPos<OcMem<C>>& t, int slot) {
     using M = OcMem<C>;
-    const float* s = sm + M::RED + slot * 8 * M::CC;
-    if (C == 1) {
-        const float4 a = *reinterpret_cast<const float4*>(s), b = *reinterpret_cast<const float4*>(s + 4);
-        return ((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w));
-    }
+    constexpr int NV = C == 4 ? 4 : 1;                       // sums per lane
+    const float* s = sm + M::RED + slot * 16 * M::CC;
     const int lane = t.tid & 31;
-    float v;
-    if (C == 2) {
-        v = s[lane];
-    } else {
-        const float4 a = *reinterpret_cast<const float4*>(s + 4 * lane);
-        v = (a.x + a.y) + (a.z + a.w);
+    float2 v[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+        v[k] = C > 1 ? reinterpret_cast<const float2*>(s)[32 * k + lane] : make_float2(lane < 16 ? s[lane] : 0.f, 0.f);
+    unsigned top = 0;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) top = max(top, __float_as_uint(v[k].x) & 0x7fffffffu);
+    top = __reduce_max_sync(0xffffffffu, top);
+    const int ex = max((int)(top >> 23), 24);                // sums below 2^-103 count as that
+    const float up = __int_as_float((275 - ex) << 23), down = __int_as_float((ex - 21) << 23);   // to |v| < 2^22 and back
+    constexpr float RINT = 12582912.f;                       // 1.5 2^23: x + RINT holds rint(x) in its last bits
+    int q = 0, r = 0;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        const float a = fmaf(v[k].x, up, RINT), f = fmaf(v[k].x, up, -__fsub_rn(a, RINT));   // the integer part; the rest, exact
+        q += __float_as_int(a) - 0x4b400000;
+        r += __float_as_int(fmaf(C > 1 ? fmaf(v[k].y, up, f) : f, 4194304.f, RINT)) - 0x4b400000;
     }
-    return warp_sum(v);
+    q = __reduce_add_sync(0xffffffffu, q);                   // at most 128 of 2^22 each (r: of 0.75 2^22)
+    r = __reduce_add_sync(0xffffffffu, r);
+    df32 d;
+    two_sum((float)(q >> 12) * 4096.f, (float)(q & 4095), d.hi, d.lo);
+    two_sum(d.hi, fmaf((float)r, 1.f / 4194304.f, d.lo), d.hi, d.lo);
+    d.hi *= down;
+    d.lo *= down;
+    if (top >= 0x7f800000u) d.hi = __int_as_float(0x7fffffff);   // infinities and NaN
+    return d;
+}
+__host__ __device__ __forceinline__ float2 pair_of(double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+}
+__device__ __forceinline__ bool at_most(df32 a, df32 b) { return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo); }
+// a / b to FP32: the remainder of a first quotient, formed exactly, corrects it.
+__device__ __forceinline__ float quotient(df32 a, df32 b) {
+    const float inv = 1.f / b.hi, q = a.hi * inv;
+    return fmaf((fmaf(-q, b.hi, a.hi) + a.lo) - q * b.lo, inv, q);
 }
 
 // ---- the finest level: a 4 x 4 patch, e[4 j + i] of cell (i, j); red: i + j even ----
@@ -582,7 +613,11 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
     int sexp = -((int)((__double2hiint(b2) >> 20) & 0x7ff) - 1023 >> 1);
     sexp = max(-100, min(100, sexp));
     const float scale = __int_as_float((127 + sexp) << 23);
-    const float b2s = (float)(b2 * (double)scale * (double)scale);
+    if (!V && t.tid == 0) {                                          // read after the barriers of the set-up
+        const double b2s = b2 * (double)scale * (double)scale;
+        reinterpret_cast<float2*>(sm + M::THR)[0] = pair_of(A.floor2 * b2s);
+        reinterpret_cast<float2*>(sm + M::THR)[1] = pair_of(A.tolout2 * b2s);
+    }
     // guards and planes
     for (int i = M::SIDE + t.tid; i < M::ENDF; i += OC_T) sm[i] = 0.f;
     if (C > 1 && t.tid == 0) oc_init_bars<M>(sm);
@@ -704,7 +739,7 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
 #pragma unroll 1
     for (int o = 0; o < A.max_outer; ++o) {
         // ---- CG on A x = r from x = 0 ----
-        float thr = 0.f, rz = 0.f;
+        df32 thr{0.f, 0.f}, rz{0.f, 0.f};
         bool first = true;
         for (;;) {
             float s = 0.f;
@@ -720,14 +755,15 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             } else {
                 dead = rr_sync<C>(sm, t);
                 if (dead) break;
-                const float rr = red_get<C>(sm, t, 0);
+                const df32 rr = red_get<C>(sm, t, 0);
                 if (first) {
-                    thr = fmaxf(A.tol2 * rr, A.floor2 * b2s);
-                    if (!(rr > 0.f)) break;
+                    const df32 part = df_mul(df32{A.tol2.x, A.tol2.y}, rr), least{sm[M::THR], sm[M::THR + 1]};
+                    thr = at_most(part, least) ? least : part;
+                    if (!(rr.hi > 0.f)) break;
                     ++inner;
                 } else {
                     ++iters;
-                    if (rr <= thr || iters >= A.maxit || !(rr == rr)) break;
+                    if (at_most(rr, thr) || iters >= A.maxit || !(rr.hi == rr.hi)) break;
                 }
             }
             // V-cycle: z = M r in e
@@ -839,10 +875,10 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
 #pragma unroll
             for (int c = 0; c < 16; ++c) s = fmaf(r[c], e[c], s);
             red_put<C>(sm, t, OC_RZ, s);
-            all_sync(sm, t, OC_RZ, 32 * M::CC);
-            const float rzn = red_get<C>(sm, t, 1);
+            all_sync(sm, t, OC_RZ, 64 * M::CC);
+            const df32 rzn = red_get<C>(sm, t, 1);
             if (!first) {
-                const float beta = rzn / rz;
+                const float beta = quotient(rzn, rz);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const float4 v = P4[j * OC_T];
@@ -884,9 +920,9 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) xv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            all_sync(sm, t, OC_PQ, 32 * M::CC);
-            const float pq = red_get<C>(sm, t, 2);
-            const float alpha = pq > 0.f ? rz / pq : 0.f;
+            all_sync(sm, t, OC_PQ, 64 * M::CC);
+            const df32 pq = red_get<C>(sm, t, 2);
+            const float alpha = pq.hi > 0.f ? quotient(rz, pq) : 0.f;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 xv[j].x = fmaf(alpha, e[4 * j], xv[j].x);
@@ -998,10 +1034,9 @@ __global__ void __launch_bounds__(OC_T, 2) k_onchip(const OcArgs A) {
             }
         }
         red_put<C>(sm, t, OC_RZ, s);
-        all_sync(sm, t, OC_RZ, 32 * M::CC);
+        all_sync(sm, t, OC_RZ, 64 * M::CC);
         if (C > 1 && __syncthreads_or(t.dead)) break;
-        const float res2 = red_get<C>(sm, t, OC_RZ);
-        if (res2 <= A.tolout2 * b2s) { converged = true; break; }
+        if (at_most(red_get<C>(sm, t, OC_RZ), df32{sm[M::THR + 2], sm[M::THR + 3]})) { converged = true; break; }
     }
 #pragma unroll 1
     for (int j = 0; !V && j < 4; ++j) {
@@ -1092,9 +1127,9 @@ static void solve_batch_onchip32(Ctx& c, int count, const Rhs& R, double* W) {
     OcArgs A{};
     A.n = c.n; A.max_outer = c.cfg.max_refine; A.maxit = c.cfg.max_iter; A.nu_f = c.cfg.fine_sweeps; A.nu_c = c.cfg.smooth_sweeps;
     A.cc = (float)c.cfg.coarse_scale;
-    A.tol2 = (float)(c.cfg.tol_inner * c.cfg.tol_inner);
-    A.tolout2 = (float)(c.cfg.tol_outer * c.cfg.tol_outer);
-    A.floor2 = (float)(0.25 * c.cfg.tol_outer * c.cfg.tol_outer);   // no phase need reduce |r| below half the final tolerance
+    A.tol2 = pair_of(c.cfg.tol_inner * c.cfg.tol_inner);
+    A.tolout2 = c.cfg.tol_outer * c.cfg.tol_outer;
+    A.floor2 = 0.25 * A.tolout2;   // no phase need reduce |r| below half the final tolerance
     A.b2const = R.b2const; A.b2pp = R.b2pp;
     A.Kw = f.Kw; A.Ks = f.Ks; A.E = f.E; A.Nn = f.Nn;
     A.Kwl = c.Kwlo; A.Ksl = c.Kslo; A.El = c.Elo; A.Nl = c.Nlo;
