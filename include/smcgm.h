@@ -155,7 +155,8 @@ smc_status smc_workspace_size(const smc_config* cfg, size_t* bytes);
  * beta = beta0.  d_workspace: the caller's device buffer of `bytes` >=
  * smc_workspace_size() bytes, 256-byte aligned, kept until smc_destroy().
  * On success *out is the new context (release it with smc_destroy()).
- * SMC_EINVAL for an invalid cfg (reason in smc_last_error(NULL)), SMC_ENOMEM
+ * SMC_EINVAL for an invalid cfg or a prior draw outside the mixed solver's
+ * range |u| < 64 (reason in smc_last_error(NULL)), SMC_ENOMEM
  * when bytes is too small (checked before the GPU is touched), SMC_ECUDA if a
  * CUDA call fails. */
 smc_status smc_init(const smc_config* cfg, void* d_workspace, size_t bytes, void* stream, smc_ctx** out);

@@ -515,10 +515,20 @@ smc_status smc_init(const smc_config* cfg, void* d_ws, size_t bytes, void* strea
     *out = ctx;
     return SMC_OK;
     }
+    catch (const InputError& ie) {
+        g_init_error = ie.what;
+        delete ctx;
+        return SMC_EINVAL;
+    }
     catch (const CudaError& ce) {
         g_init_error = std::string(ce.what) + ": " + cudaGetErrorString(ce.e);
         delete ctx;
         return SMC_ECUDA;
+    }
+    catch (const std::bad_alloc&) {
+        g_init_error = "host allocation failed";
+        delete ctx;
+        return SMC_ENOMEM;
     }
 }
 
