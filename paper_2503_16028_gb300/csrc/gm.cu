@@ -443,14 +443,17 @@ size_t cov_lb_doubles(int K, int r) { return (size_t)K * lb_size(r) + K; }
 // and a pivot chain each: 79 us at r = 64, K = 8; in panels 71.
 constexpr int CHOL_SMEM_R = 160;
 
-// 1 / d for a positive normal d to ~1 ulp: the hardware's approximate FP64 reciprocal (full exponent range) and two
-// Newton steps, half the latency of a rounded division.
+// 1 / d to an ulp for d in [2^-1000, 2^1000]: the Newton-Raphson iteration y <- y + y (1 - d y) from the hardware's approximate
+// reciprocal (some 20 bits), which squares the relative error at each of its two steps; half the latency of a rounded
+// division.
 __device__ __forceinline__ double rcp_newton(double d) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
     y = fma(y, fma(-d, y, 1.0), y);
     return fma(y, fma(-d, y, 1.0), y);
 }
+// Pivots at the ends of the range, subnormal ones included: a call, so that the common path has no instruction of it.
+__device__ __noinline__ double divide(double a, double b) { return a / b; }
 template <bool SMEM>
 __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ cov, const double* __restrict__ w, double* __restrict__ L,
                                               double* __restrict__ Lb, double* __restrict__ logdet, double* __restrict__ cst,
@@ -482,19 +485,22 @@ __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ 
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const bool pos = d[c][c] > 0.0;
-                const double dc = pos ? d[c][c] : 1.0, rinv = rcp_newton(dc);
+                const double dc = pos ? d[c][c] : 1.0;
+                const bool far = !(dc >= 0x1p-1000 && dc <= 0x1p1000);
+                const double rinv = rcp_newton(dc);
+                auto over = [&](double x) { return far ? divide(x, dc) : x * rinv; };
                 if (tid == 0 && k + c < r) {
                     rs[k + c] = dc;
                     if (!pos) atomicExch(bad, 1);
                 }
 #pragma unroll
                 for (int b = c + 1; b < 4; ++b) {
-                    const double tb = d[b][c] * rinv;
+                    const double tb = over(d[b][c]);
 #pragma unroll
                     for (int a = b; a < 4; ++a) d[a][b] = fma(-d[a][c], tb, d[a][b]);
                     w[b] = fma(-w[c], tb, w[b]);
                 }
-                T[c][ri] = w[c] * rinv;
+                T[c][ri] = over(w[c]);
             }
             if (tid >= 4)
 #pragma unroll
