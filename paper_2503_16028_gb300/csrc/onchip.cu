@@ -43,7 +43,7 @@ namespace smcgm {
 constexpr int OC_T = 256;
 
 struct OcArgs {
-    int n, max_outer, maxit, nu_f, nu_c;
+    int max_outer, maxit, nu_f, nu_c;
     float cc;
     float2 tol2;                 // the pair of the squared reduction per phase
     double floor2, tolout2;
@@ -1125,7 +1125,7 @@ static void solve_batch_onchip32(Ctx& c, int count, const Rhs& R, double* W) {
     InnerSolver<float>& s = c.s32;
     LevelArrays<float>& f = s.lv[0];
     OcArgs A{};
-    A.n = c.n; A.max_outer = c.cfg.max_refine; A.maxit = c.cfg.max_iter; A.nu_f = c.cfg.fine_sweeps; A.nu_c = c.cfg.smooth_sweeps;
+    A.max_outer = c.cfg.max_refine; A.maxit = c.cfg.max_iter; A.nu_f = c.cfg.fine_sweeps; A.nu_c = c.cfg.smooth_sweeps;
     A.cc = (float)c.cfg.coarse_scale;
     A.tol2 = pair_of(c.cfg.tol_inner * c.cfg.tol_inner);
     A.tolout2 = c.cfg.tol_outer * c.cfg.tol_outer;
@@ -1151,7 +1151,7 @@ static void vcycle32(Ctx& c, int level, int nact, bool build) {
     InnerSolver<float>& s = c.s32;
     LevelArrays<float>& f = s.lv[level];
     OcArgs A{};
-    A.n = f.n; A.max_outer = 1; A.nu_f = A.nu_c = c.cfg.smooth_sweeps;
+    A.max_outer = 1; A.nu_f = A.nu_c = c.cfg.smooth_sweeps;
     A.cc = (float)c.cfg.coarse_scale;
     A.Kw = f.Kw; A.Ks = f.Ks; A.E = f.E; A.Nn = f.Nn;
     A.vr = f.r; A.ve = f.e2; A.inv8 = s.binv;
