@@ -187,10 +187,12 @@ __host__ __device__ __forceinline__ float2 pair_of(double v) {
     return make_float2(h, (float)(v - (double)h));
 }
 __device__ __forceinline__ bool at_most(df32 a, df32 b) { return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo); }
-// a / b to FP32: the remainder of a first quotient, formed exactly, corrects it.
+// a / b to FP32: the remainder of a first quotient, formed exactly, corrects it.  In a field of u = 50 r.z and p.Ap are subnormal, whose
+// reciprocal overflows: both are brought up first.
 __device__ __forceinline__ float quotient(df32 a, df32 b) {
-    const float inv = 1.f / b.hi, q = a.hi * inv;
-    return fmaf((fmaf(-q, b.hi, a.hi) + a.lo) - q * b.lo, inv, q);
+    const float up = fabsf(b.hi) < 0x1p-96f ? 0x1p64f : 1.f, c = b.hi * up, d = a.hi * up;
+    const float inv = 1.f / c, q = d * inv;
+    return fmaf((fmaf(-q, c, d) + a.lo * up) - q * (b.lo * up), inv, q);
 }
 
 // ---- the finest level: a 4 x 4 patch, e[4 j + i] of cell (i, j); red: i + j even ----
