@@ -71,8 +71,8 @@ __global__ void k_em_init(int N, int K, int r, EmPicks init, const double* __res
 // than half a standard deviation it could cancel digits (all but 1 / N of S2 at worst), so in such an iteration,
 // mostly the first few, all blocks form the sums about the new means again, with two barriers more.
 // A collapsed component (N_j < 2) is found by every block alike (same sums, same order).
-// Measured (r = 64, 50 iterations, ncu): N = 1024, K = 4 9.0 -> 0.9 ms, N = 256, K = 2 7.2 -> 0.77 ms
-// (what is left is the chain of FP64 latencies through an iteration, 15 us: an exponential takes 1250
+// Measured (r = 64, 50 iterations, the whole fit): N = 1024, K = 4 9.0 -> 0.97 ms, N = 256, K = 2 7.2 -> 0.84 ms
+// (what is left is the chain of FP64 latencies through an iteration, 16 us: an exponential takes 1250
 // cycles, a logarithm 2200, a division 500; the FP64 pipe is 6 % busy).
 // ------------------------------------------------------------------------
 constexpr int EM_THREADS = 256;
@@ -421,9 +421,9 @@ __global__ void k_sum(int N, const double* __restrict__ a, double* __restrict__ 
 // An iteration is k_chol, k_estep_full, k_resp, k_cov_mean, k_cov_acc, k_cov_finish.  The E-step and the
 // contraction are N K r^2 / 2 FP64 multiply-adds each (108 us at N = 4096, K = 8, r = 64 on the
 // FP64 pipes), everything else should stay small beside them.  Measured per 50-iteration fit
-// there: 70.2 -> 20.4 ms (one block per particle reading rows of L^-1 uncoalesced 631 -> 150 us, FP64
-// pipe 76 % busy: 1.7 warps per scheduler, so some have two; the factor with its column sums in global memory
-// 416 -> 71 us; the contraction on 32 x 32 tiles 292 -> 154 us, the pipe all but full).
+// there: 70.2 -> 20.7 ms (one block per particle reading rows of L^-1 uncoalesced 631 -> 150 us, FP64
+// pipe 81 % busy: 1.7 warps per scheduler, so some have two; the factor with its column sums in global memory
+// 416 -> 69 us; the contraction on 32 x 32 tiles 292 -> 152 us, the pipe all but full).
 // ------------------------------------------------------------------------
 
 // Rows in blocks of four: block I holds L[4I + q][k] at 8 I (I + 1) + 4 k + q, k < 4 I + 4, with
@@ -440,7 +440,7 @@ size_t cov_lb_doubles(int K, int r) { return (size_t)K * lb_size(r) + K; }
 // as 1 so the rest stays finite.  cst_j = log w_j - r/2 log(2 pi) - log det L_j when w is given.
 // Bound by the FP64 pipe of one SM and the pivots' chain: about 48 operations of 64 cycles per panel and
 // scheduler, then the update (r^3 / 6 multiply-adds, 11 us at r = 64).  With a column per step, two barriers
-// and a pivot chain each: 79 us at r = 64, K = 8; in panels 71.
+// and a pivot chain each: 79 us at r = 64, K = 8; in panels 69.
 constexpr int CHOL_SMEM_R = 160;
 
 // 1 / d to an ulp for d in [2^-1000, 2^1000]: the Newton-Raphson iteration y <- y + y (1 - d y) from the hardware's approximate
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(256) k_chol(int r, const double* __restrict__ 
             for (int c = 0; c < 4; ++c) {
                 const bool pos = d[c][c] > 0.0;
                 const double dc = pos ? d[c][c] : 1.0;
-                const bool far = !(dc >= 0x1p-1000 && dc <= 0x1p1000);
+                const bool far = (unsigned)((__double2hiint(dc) >> 20) - 23) >= 2000u;    // not in [2^-1000, 2^1000); no FP64 operation
                 const double rinv = rcp_newton(dc);
                 auto over = [&](double x) { return far ? divide(x, dc) : x * rinv; };
                 if (tid == 0 && k + c < r) {
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(256) k_cov_mean(int N, int r, const double* __
 // holds one 4 x 4 tile of the lower triangle (136 tiles at r = 64: 5 % more products than the triangle
 // itself; 32 x 32 tiles took 48 % more), 16 particles' deviations staged in shared memory per step.
 // 136 tiles are four warps and a quarter: the lanes of the partial warp divide each step's particles among
-// them, so that it costs the FP64 pipe a quarter of a warp (173 -> 154 us at N = 4096, K = 8, r = 64).
+// them, so that it costs the FP64 pipe a quarter of a warp (173 -> 152 us at N = 4096, K = 8, r = 64).
 // k_cov_finish adds the chunks in a fixed order.
 constexpr int COV_PN = 16;
 __host__ __device__ inline int cov_tiles(int r) { const int R = row_blocks(r); return R * (R + 1) / 2; }

@@ -9,7 +9,7 @@
 // residual and correction stay in registers for the whole solve, CG's p and the reciprocal
 // diagonals in shared memory, and only the solution's three FP32 parts and x go through L2.
 // Measured against it (synthesis and set-up included): 1024 solves of 64^2 4.17 -> 0.66 ms, 2048 of
-// 128^2 15.7 -> 6.6 ms, 2048 of 256^2 54.9 -> 42.0 ms, 2 of 256^2 2.35 -> 0.30 ms.
+// 128^2 15.7 -> 6.5 ms, 2048 of 256^2 54.9 -> 41.3 ms, 2 of 256^2 2.35 -> 0.34 ms.
 //
 // Layout: a block covers a strip of 64 C x 64 / C cells (C = n / 64) with 16 C x 16 / C threads, a
 // 4 x 4 patch each; a thread also owns the 2 x 2 cells below its patch on the next level and the
@@ -29,8 +29,8 @@
 // black cells vanishes there, so only the red cells are restricted.
 //
 // What bounds it: the latency of about 30 barrier-separated phases per CG iteration (45 and 25
-// remote exchanges of 324 cycles each at 256^2), not HBM: two blocks per SM (128 registers a
-// thread, 80 to 113 KB) reach 0.53 (64^2) and 0.35 (256^2) issued instructions per scheduler cycle.
+// remote exchanges at 256^2 and 128^2), not HBM: two blocks per SM (128 registers a
+// thread, 80 to 113 KB) reach 0.53 (64^2) and 0.38 (256^2) issued instructions per scheduler cycle.
 // 14 clusters of 16 fit the GPU at a time (112 of 152 SMs).
 #include <cstdio>
 #include "smcgm_internal.cuh"
