@@ -20,7 +20,8 @@ mixed-precision path, the solver-only rate (smc_forward), the end-to-end rate
 with pinned host buffers through smc_batch_move_host (each move one CUDA graph;
 the smc_move_host form beside it), the adjoint-gradient rate, a whole SMC
 run to t = 1 timed layer by layer with an FP64 run of the same seed in lockstep
-(the posterior error of the mixed-precision run against it), the 64^2 workload on
+(the posterior error of the mixed-precision run against it), the passes with FP32 and BF16
+smoother faces (the other storage alone where the headline runs in passes), the 64^2 workload on
 the GPU (host-driven and as one CUDA graph) and on the CPU oracle, the 32-problem
 batching workload (one after another, a host thread each, one CUDA graph), the SM
 clocks sampled during the timed region and the CPU oracle baseline.
